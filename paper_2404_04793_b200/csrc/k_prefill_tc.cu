@@ -5,17 +5,26 @@
 // is two sweeps over 128x128 tiles of the score matrix, each tile one tcgen05.mma chain
 // (M = N = 128, K = head_dim, bf16 in, fp32 accumulators in tensor memory):
 //   sweep 1, CTA = (sequence, query head, 128 query rows): S = Q_tile K_tile^T for the key tiles
-//     up to the diagonal; thread r of the four softmax warps owns TMEM lane r = one query row and
+//     up to the diagonal; a drain thread owns one TMEM lane = one query row and
 //     keeps its running max / sum -> row log-sum-exp.
-//   sweep 2, CTA = (sequence, KV head, 128 keys): the operands swap, S^T = K_tile Q_tile^T for all
-//     query tiles from the diagonal down and all heads of the group; thread t owns one key and
-//     adds exp2(s*scale - lse[row]) over the tile's columns -> the key's column sum, with no
-//     cross-thread reduction and no atomics (deterministic).
-// Roles per CTA (6 warps): warp 0 issues TMA tile loads (128-byte swizzle, every CTA its own tiles) into
-// a ring of shared-memory stages; warp 1 allocates tensor memory and issues the MMAs, signalling
-// completion through tcgen05.commit -> mbarrier; warps 2-5 drain the accumulators with
-// tcgen05.ld.  Two accumulator buffers let the next tile's MMA run under this tile's exponentials.
+//   sweep 2, CTA = (sequence, KV head, 128 keys, some heads of the group): the operands swap,
+//     S^T = K_tile Q_tile^T for all query tiles from the diagonal down and the CTA's heads; thread t
+//     owns one key and adds exp2(s*scale - lse[row]) over the tile's columns -> the key's column sum,
+//     with no cross-thread reduction and no atomics; a key tile cut into several CTAs by heads is
+//     added up, in head order, by the one that finishes last (deterministic).
+// Roles per CTA (10 warps): warp 0 issues TMA tile loads (128-byte swizzle, every CTA its own tiles)
+// into a ring of shared-memory stages; warp 1 allocates tensor memory, issues the MMAs, signalling
+// completion through tcgen05.commit -> mbarrier, and stages the row log-sum-exps of sweep 2; warps 2-9
+// drain the accumulators with tcgen05.ld.  Two accumulator buffers let the next tile's MMA run under
+// this tile's exponentials.
+// Built to parity and measured slower (us of sweeps 1 / 2, 4 sequences of 4096, 32 / 8 heads of 128,
+// against 321 / 374): queries on the lanes in both sweeps with one register per key in sweep 2, which
+// takes the log-sum-exps out of shared memory (315 / 416 as one persistent CTA per SM with 128x256
+// tiles, 326 / 449 with the next tile's load in flight across the tile boundary, 334 / 511 as two CTAs
+// of nine warps); no issuing warps, the last warp to empty a buffer issues its MMAs (413 / 481: an MMA
+// holds the thread that issues it for about 80 cycles).
 // Every mbarrier wait is bounded: on expiry the CTA raises a status bit and winds down.
+#include <algorithm>
 #include <type_traits>
 
 #include "sq_internal.h"
@@ -32,11 +41,53 @@ using namespace tc;
 // warps wait for an accumulator or a tensor-memory load.
 constexpr int kPrefillThreads = 64 + 256;
 
+// exp2 of a pair on the FMA pipe: x = n + f with n the nearest integer (the usual 1.5 * 2^23
+// addition), 2^f for |f| <= 1/2 from a degree-5 polynomial (fitted here by a Remez exchange on the
+// relative error; in fp32 within 2.1e-7 of the exact value, ex2.approx's own bound is 1.7e-7), the
+// exponent added to the bits.  Arguments below -126 give 2^-126 (times at most sqrt 2) instead of a
+// smaller number or 0.
+__device__ __forceinline__ unsigned long long ex2_pair_fma(unsigned long long x2) {
+  constexpr float kMagic = 12582912.f;
+  float x0, x1;
+  f32x2_split(x2, x0, x1);
+  x2 = f32x2(fmaxf(x0, -126.f), fmaxf(x1, -126.f));
+  const unsigned long long t2 = add_f32x2(x2, f32x2(kMagic, kMagic));
+  const unsigned long long n2 = add_f32x2(t2, f32x2(-kMagic, -kMagic));
+  const unsigned long long f2 = fma_f32x2(n2, f32x2(-1.f, -1.f), x2);
+  unsigned long long p2 = f32x2(1.3276472454890609e-3f, 1.3276472454890609e-3f);
+  p2 = fma_f32x2(p2, f2, f32x2(9.675540961325169e-3f, 9.675540961325169e-3f));
+  p2 = fma_f32x2(p2, f2, f32x2(5.550713092088699e-2f, 5.550713092088699e-2f));
+  p2 = fma_f32x2(p2, f2, f32x2(2.4022120237350464e-1f, 2.4022120237350464e-1f));
+  p2 = fma_f32x2(p2, f2, f32x2(6.931469440460205e-1f, 6.931469440460205e-1f));
+  p2 = fma_f32x2(p2, f2, f32x2(1.f, 1.f));
+  float t0, t1, p0, p1;
+  f32x2_split(t2, t0, t1);
+  f32x2_split(p2, p0, p1);
+  return f32x2(__uint_as_float(__float_as_uint(p0) + (__float_as_uint(t0) << 23)),
+               __uint_as_float(__float_as_uint(p1) + (__float_as_uint(t1) << 23)));
+}
+__device__ __forceinline__ unsigned long long ex2_pair_sfu(unsigned long long x2) {
+  float x0, x1;
+  f32x2_split(x2, x0, x1);
+  return f32x2(ex2(x0), ex2(x1));
+}
+// Of every eight pairs of score elements this many take the FMA-pipe form, spread evenly.  The drain
+// is bound by the special-function unit (16 exponentials per cycle and SM: 1024 cycles per 128x128
+// tile) with none of them, by issue slots and the FMA pipe (two cycles per packed instruction) from
+// three of eight on.  Measured on B200, us per layer of sweep 1 / sweep 2 with 0, 1, 2, 3, 4 of eight:
+// head_dim 128 (4 sequences of 4096, 32 / 8 heads) 334/395, 321/374, 322/377, 337/380, 380/402;
+// head_dim 64 (2 sequences of 5003, 71 / 1 heads) 539/559, 512/520, 506/513, 533/523, 610/579.
+template <int D>
+__device__ __forceinline__ constexpr bool on_fma(int pair) {
+  constexpr int n = D == 64 ? 2 : 1;
+  return ((pair & 7) * n) % 8 + n >= 8;  // `pair` is a constant after unrolling
+}
+
 // SWEEP 1: rows = queries, streamed tiles = keys; SWEEP 2: rows = keys, streamed tiles = queries.
 template <int D, int STAGES, int SWEEP>
 __global__ void __launch_bounds__(kPrefillThreads, 2)
     prefill_scores_tc_kernel(const __grid_constant__ CUtensorMap tm_rows, const __grid_constant__ CUtensorMap tm_stream,
-                             ScoreArgs a, float scale_log2, int* status) {
+                             ScoreArgs a, ScorePieces pc, float scale_log2, int* status) {
   constexpr int SUB = D / 64;                  // 64-column sub-tiles per operand tile
   constexpr int TILE_BYTES = SUB * kSubBytes;  // one operand tile
   constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTM >> 3) << 17) | ((uint32_t)(kTM >> 4) << 24);
@@ -55,7 +106,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
   auto bar_lse = [&](int b) { return s_u32(bars + 5 + 2 * STAGES + b); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* lse_s = reinterpret_cast<float*>(tmem_slot + 4);  // [2][128], sweep 2 only
+  float* lse_s = reinterpret_cast<float*>(tmem_slot + 4);  // [2][128]: sweep 2, minus the row log-sum-exps
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int P = a.prompt, g = a.n_q_head / a.n_kv_head;
@@ -63,7 +114,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
   // grid = (head, sequence, tile): the tile index varies slowest, so the CTAs with the most streamed
   // tiles of every head and sequence start first and the short ones fill the tail of the launch
   const int bi = blockIdx.y;
-  int row_tile, n_stream;
+  int row_tile, n_stream, piece = 0, head0 = 0;
   long long rows0;  // first row of this CTA's fixed tile in the rows tensor
   int hq = 0, hk = 0;
   if (SWEEP == 1) {
@@ -74,21 +125,34 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
     rows0 = ((long long)bi * a.n_q_head + hq) * P + (long long)row_tile * kTM;
   } else {
     hk = blockIdx.x;
-    row_tile = blockIdx.z;               // key tile 0 sees every query tile: longest first
-    n_stream = g * (n_tile - row_tile);
+    row_tile = blockIdx.z / pc.n_piece;  // key tile 0 sees every query tile: longest first
+    piece = blockIdx.z - row_tile * pc.n_piece;
+    head0 = piece * pc.heads;            // this piece's heads of the group
+    n_stream = min(pc.heads, g - head0) * (n_tile - row_tile);
     rows0 = ((long long)bi * a.n_kv_head + hk) * P + (long long)row_tile * kTM;
   }
-  // first row of streamed tile i, and (sweep 2) its head / query tile
-  auto stream_row0 = [&](int i, int& h_out, int& qt_out) -> long long {
-    if (SWEEP == 1) {
-      h_out = 0;
-      qt_out = i;
-      return ((long long)bi * a.n_kv_head + hk) * P + (long long)i * kTM;
+  // Walks the streamed tiles in order: (sweep 1) key tiles 0..row_tile, (sweep 2) per head of the
+  // piece the query tiles from the diagonal down.
+  struct Walk {
+    int h, qt;
+    long long row0;
+  };
+  auto walk_begin = [&]() {
+    Walk w;
+    w.h = head0;
+    w.qt = SWEEP == 1 ? 0 : row_tile;
+    w.row0 = SWEEP == 1 ? ((long long)bi * a.n_kv_head + hk) * P
+                        : ((long long)bi * a.n_q_head + hk * g + head0) * P + (long long)row_tile * kTM;
+    return w;
+  };
+  auto walk_next = [&](Walk& w) {
+    ++w.qt;
+    w.row0 += kTM;
+    if (SWEEP == 2 && w.qt == n_tile) {
+      w.qt = row_tile;
+      ++w.h;
+      w.row0 += P - (long long)(n_tile - row_tile) * kTM;
     }
-    const int per = n_tile - row_tile;
-    h_out = i / per;
-    qt_out = row_tile + (i - h_out * per);
-    return ((long long)bi * a.n_q_head + hk * g + h_out) * P + (long long)qt_out * kTM;
   };
 
   if (tid == 0) {
@@ -99,8 +163,8 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar_sfull(b), 1);
-      mbar_init(bar_sfree(b), 256);
-      mbar_init(bar_lse(b), 256);
+      mbar_init(bar_sfree(b), 8);  // one arrival per drain warp
+      mbar_init(bar_lse(b), 1);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -121,16 +185,16 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
 #pragma unroll
       for (int sb = 0; sb < SUB; ++sb) tma_load_2d(s_u32(a_s + sb * kSubBytes), &tm_rows, sb * 64, (int)rows0, bar_a);
       int issued = 0;
+      Walk w = walk_begin();
       for (int i = 0; i < n_stream; ++i) {
         const int st = i % STAGES;
         if (i >= STAGES && !mbar_wait(bar_empty(st), ((i / STAGES) - 1) & 1, abort_flag)) break;
-        int h, qt;
-        const long long r0 = stream_row0(i, h, qt);
         mbar_expect_tx(bar_full(st), TILE_BYTES);
 #pragma unroll
         for (int sb = 0; sb < SUB; ++sb)
-          tma_load_2d(s_u32(b_s + st * TILE_BYTES + sb * kSubBytes), &tm_stream, sb * 64, (int)r0, bar_full(st));
+          tma_load_2d(s_u32(b_s + st * TILE_BYTES + sb * kSubBytes), &tm_stream, sb * 64, (int)w.row0, bar_full(st));
         issued = i + 1;
+        walk_next(w);
       }
       if (*abort_flag) {
         // winding down early: let the copies already in flight land before the CTA exits
@@ -142,15 +206,34 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
       }
     }
   } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
+    // ---------------- MMA issuer; sweep 2: also stages the tile's row log-sum-exps ----------------
+    // (fetched one tile ahead, so that the trip to memory runs under the tile before)
+    auto fetch_lse = [&](const Walk& w) {
+      const float* src = a.lse2 + ((size_t)bi * a.n_q_head + hk * g + w.h) * P;
+      const int q = w.qt * kTM + lane * 4;
+      float4 v;
+      v.x = (q + 0 < P) ? -src[q + 0] : -INFINITY;  // a query past the end attends to nothing
+      v.y = (q + 1 < P) ? -src[q + 1] : -INFINITY;
+      v.z = (q + 2 < P) ? -src[q + 2] : -INFINITY;
+      v.w = (q + 3 < P) ? -src[q + 3] : -INFINITY;
+      return v;
+    };
+    Walk w = walk_begin();
+    float4 lse_next = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (SWEEP == 2) lse_next = fetch_lse(w);
     bool ok = mbar_wait(bar_a, 0, abort_flag);
     for (int i = 0; ok && i < n_stream; ++i) {
       const int st = i % STAGES, buf = i & 1;
       ok = mbar_wait(bar_full(st), (i / STAGES) & 1, abort_flag);
       if (ok && i >= 2) ok = mbar_wait(bar_sfree(buf), ((i >> 1) - 1) & 1, abort_flag);
       if (!ok) break;
+      if (SWEEP == 2) {
+        *reinterpret_cast<float4*>(lse_s + buf * kTM + lane * 4) = lse_next;
+        __syncwarp();
+      }
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (lane == 0) {
+        if (SWEEP == 2) mbar_arrive(bar_lse(buf));
         const uint32_t d_tmem = tmem_base + buf * kTM;
 #pragma unroll
         for (int k = 0; k < D / 16; ++k) {
@@ -162,6 +245,10 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
         umma_commit(bar_sfull(buf)); // the accumulator buffer is complete
       }
       __syncwarp();
+      if (SWEEP == 2 && i + 1 < n_stream) {
+        walk_next(w);
+        lse_next = fetch_lse(w);
+      }
     }
   } else {
     // ---------------- accumulator drain: thread = one row of the fixed tile ----------------
@@ -169,90 +256,108 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
     const int half = (warp - 2) >> 2;  // which 64 columns of every tile this warp drains
     const int row = quarter * 32 + lane;
     const int row_idx = row_tile * kTM + row;  // query index (sweep 1) / key index (sweep 2)
-    const int t256 = (warp - 2) * 32 + lane;
-    float m = -INFINITY, l = 0.f, colsum = 0.f;
+    const uint32_t s_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * 64;
+    const unsigned long long scale2 = f32x2(scale_log2, scale_log2);
+    // sweep 1: running reference of the row and its sum; sweep 2: the key's sum (even and odd columns)
+    float m = -INFINITY, l = 0.f;
+    unsigned long long acc_a = f32x2(0.f, 0.f), acc_b = acc_a;
     bool ok = true;
-    // sweep 2: the row log-sum-exp of query t256 of streamed tile i; fetched one tile ahead, so
-    // that its trip to memory runs under the previous tile's arithmetic
-    auto fetch_lse = [&](int i) -> float {
-      int h, qt;
-      stream_row0(i, h, qt);
-      const int q = qt * kTM + t256;
-      return (q < P) ? a.lse2[((size_t)bi * a.n_q_head + hk * g + h) * P + q] : INFINITY;
-    };
-    float lse_next = 0.f;
-    if (SWEEP == 2 && t256 < kTM && n_stream > 0) lse_next = fetch_lse(0);
+    Walk w = walk_begin();
     for (int i = 0; ok && i < n_stream; ++i) {
       const int buf = i & 1;
-      int h, qt;
-      stream_row0(i, h, qt);
-      if (SWEEP == 2) {
-        if (t256 < kTM) {
-          lse_s[buf * kTM + t256] = lse_next;
-          if (i + 1 < n_stream) lse_next = fetch_lse(i + 1);
-        }
-        mbar_arrive(bar_lse(buf));  // all 128 row sums of this query tile are staged
-        ok = mbar_wait(bar_lse(buf), (i >> 1) & 1, abort_flag);
-      }
+      const bool diag = w.qt == row_tile;
+      walk_next(w);
+      if (SWEEP == 2) ok = mbar_wait(bar_lse(buf), (i >> 1) & 1, abort_flag);
       if (ok) ok = mbar_wait(bar_sfull(buf), (i >> 1) & 1, abort_flag);
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       // The tile on the diagonal masks half of its elements; every other tile masks none.  The two
-      // cases are separate instantiations of the drain loop, so that tiles off the diagonal (all
-      // but one per row of tiles) carry no compare / select per element.
-      auto drain_tile = [&](auto diag_c) {
+      // cases are separate instantiations of the drain, so that tiles off the diagonal (all but one
+      // per row of tiles) carry no compare / select per element.
+      auto chunk = [&](auto diag_c, uint32_t (&r)[32], int c0) {  // columns c0 .. c0+31 of the tile
         constexpr bool DIAG = decltype(diag_c)::value;
-#pragma unroll 1
-        for (int c = 2 * half; c < 2 * half + 2; ++c) {
-          float v[32];
-          tmem_ld32(tmem_base + ((uint32_t)(quarter * 32) << 16) + buf * kTM + c * 32, v);
-          if (SWEEP == 1) {
-            if (DIAG) {
+        if (SWEEP == 1) {
+          if (DIAG) {
 #pragma unroll
-              for (int j = 0; j < 32; ++j)
-                if (c * 32 + j > row) v[j] = -INFINITY;  // key after the query
-            }
-            float mx = v[0];
+            for (int j = 0; j < 32; ++j)
+              if (c0 + j > row) r[j] = 0xff800000u;  // key after the query: -inf
+          }
+          float mx = __uint_as_float(r[0]);
 #pragma unroll
-            for (int j = 1; j < 32; ++j) mx = fmaxf(mx, v[j]);
-            const float m_new = fmaxf(m, mx * scale_log2);
-            if (m_new > -INFINITY) {
-              float sum = 0.f;
+          for (int j = 1; j + 1 < 32; j += 2) mx = max3(mx, __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
+          mx = fmaxf(mx, __uint_as_float(r[31]));
+          const float m_new = fmaxf(m, mx * scale_log2);
+          if (DIAG && m_new == -INFINITY) return;  // nothing of the row so far (second half of the first rows)
+          if (m_new > m) {
+            const float f = ex2(m - m_new);
+            const unsigned long long f2 = f32x2(f, f), zero = f32x2(0.f, 0.f);
+            acc_a = fma_f32x2(acc_a, f2, zero);
+            acc_b = fma_f32x2(acc_b, f2, zero);
+            m = m_new;
+          }
+          const unsigned long long neg_m2 = f32x2(-m, -m);
 #pragma unroll
-              for (int j = 0; j < 32; ++j) sum += ex2(fmaf(v[j], scale_log2, -m_new));
-              l = l * ex2(m - m_new) + sum;
-              m = m_new;
-            }
-          } else {
-            const float4* ls = reinterpret_cast<const float4*>(lse_s + buf * kTM + c * 32);
+          for (int jp = 0; jp < 16; ++jp) {
+            const unsigned long long x2 =
+                fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])), scale2, neg_m2);
+            // (the masked tile keeps to the form that gives an exact 0)
+            const unsigned long long e2 = !DIAG && on_fma<D>(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
+            if (jp & 1) acc_b = add_f32x2(acc_b, e2);
+            else acc_a = add_f32x2(acc_a, e2);
+          }
+        } else {
+          const ulonglong2* ls = reinterpret_cast<const ulonglong2*>(lse_s + buf * kTM + c0);
 #pragma unroll
-            for (int j4 = 0; j4 < 8; ++j4) {
-              const float4 lv = ls[j4];
-              const float e0 = ex2(fmaf(v[4 * j4 + 0], scale_log2, -lv.x));
-              const float e1 = ex2(fmaf(v[4 * j4 + 1], scale_log2, -lv.y));
-              const float e2 = ex2(fmaf(v[4 * j4 + 2], scale_log2, -lv.z));
-              const float e3 = ex2(fmaf(v[4 * j4 + 3], scale_log2, -lv.w));
-              if (DIAG) {
-                const int q0 = c * 32 + 4 * j4;  // query before the key: no attention
-                colsum += (q0 + 0 >= row ? e0 : 0.f) + (q0 + 1 >= row ? e1 : 0.f) + (q0 + 2 >= row ? e2 : 0.f) +
-                          (q0 + 3 >= row ? e3 : 0.f);
-              } else {
-                colsum += (e0 + e1) + (e2 + e3);
+          for (int j4 = 0; j4 < 8; ++j4) {
+            const ulonglong2 lv = ls[j4];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+              const int jp = 2 * j4 + q;
+              const unsigned long long x2 = fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])),
+                                                      scale2, q ? lv.y : lv.x);
+              unsigned long long e2 = on_fma<D>(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
+              if (DIAG) {  // query before the key: no attention
+                float e0, e1;
+                f32x2_split(e2, e0, e1);
+                e2 = f32x2(c0 + 2 * jp >= row ? e0 : 0.f, c0 + 2 * jp + 1 >= row ? e1 : 0.f);
               }
+              if (q) acc_b = add_f32x2(acc_b, e2);
+              else acc_a = add_f32x2(acc_a, e2);
             }
           }
         }
       };
-      if (qt == row_tile) drain_tile(std::true_type{});
+      auto hand_back = [&]() {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_sfree(buf));
+      };
+      auto drain_tile = [&](auto diag_c) {
+        uint32_t ra[32], rb[32];
+        tmem_ld32_nowait(s_addr + buf * kTM, ra);
+        tmem_wait_ld(ra);
+        tmem_ld32_nowait(s_addr + buf * kTM + 32, rb);
+        chunk(diag_c, ra, half * 64);
+        __syncwarp();
+        tmem_wait_ld(rb);
+        if (SWEEP == 1) hand_back();  // the tile is in registers: the tensor core may have the buffer back
+        chunk(diag_c, rb, half * 64 + 32);
+        if (SWEEP == 2) hand_back();  // the buffer's lse staging is in use until here
+      };
+      if (diag) drain_tile(std::true_type{});
       else drain_tile(std::false_type{});
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      mbar_arrive(bar_sfree(buf));
+    }
+    {
+      float a0, a1, b0, b1;
+      f32x2_split(acc_a, a0, a1);
+      f32x2_split(acc_b, b0, b1);
+      l = (a0 + a1) + (b0 + b1);
     }
     // the two halves of a row meet in shared memory (the staging area is free once every drain
     // thread is past its last tile); every drain thread reaches both barriers, aborted or not
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (half == 1) {
-      lse_s[2 * row] = (SWEEP == 1) ? m : colsum;
+      lse_s[2 * row] = m;
       lse_s[2 * row + 1] = l;
     }
     asm volatile("bar.sync 1, 256;" ::: "memory");
@@ -264,7 +369,8 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
         const float ll = l * ex2(m - mm) + o1 * ex2(o0 - mm);
         a.lse2[((size_t)bi * a.n_q_head + hq) * P + row_idx] = mm + log2f(ll);
       } else {
-        a.acc_prompt[((size_t)bi * a.n_kv_head + hk) * P + row_idx] = colsum + o0;
+        float* dst = pc.n_piece == 1 ? a.acc_prompt : pc.partial + (size_t)piece * a.batch * a.n_kv_head * P;
+        dst[((size_t)bi * a.n_kv_head + hk) * P + row_idx] = l + o1;
       }
     }
   }
@@ -275,6 +381,26 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem_base) : "memory");
   }
   if (tid == 0 && *abort_flag) atomicOr(status, kStatusTimeout);
+  if (SWEEP == 2 && pc.n_piece > 1) {
+    // the key tile's last piece to finish adds all pieces up, in head order (no piece waits)
+    __shared__ int s_last;
+    if (tid == 0) {
+      int* ticket = pc.tickets + ((size_t)bi * a.n_kv_head + hk) * n_tile + row_tile;
+      __threadfence();
+      s_last = atomicAdd(ticket, 1) == pc.n_piece - 1;
+      if (s_last) *ticket = 0;
+    }
+    __syncthreads();
+    const int key = row_tile * kTM + tid;
+    if (s_last && tid < kTM && key < P) {
+      __threadfence();
+      const size_t at = ((size_t)bi * a.n_kv_head + hk) * P + key, stride = (size_t)a.batch * a.n_kv_head * P;
+      float sum = 0.f;
+#pragma unroll 8
+      for (int p = 0; p < pc.n_piece; ++p) sum += __ldcg(pc.partial + at + p * stride);
+      a.acc_prompt[at] = sum;
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -328,10 +454,26 @@ static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) 
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  k1<<<dim3(a.n_q_head, a.batch, n_tile), kPrefillThreads, smem, s>>>(tm_q, tm_k, a, scale_log2, status);
+  // Sweep 2 walks the heads of a group one after the other.  A launch of few key tiles and many heads
+  // (71 heads on one KV head) would be over when its longest CTA is: it is cut into pieces of `heads`
+  // heads so that the longest CTA has at most about a quarter of a CTA slot's share of the work.
+  // Measured, us per layer, one CTA per key tile / cut: 2 sequences of 5003 tokens, 71 heads on one KV
+  // head (80 key tiles): 3283 / 559; 1 sequence of 777, 32 on 8: 37 / 15; 4 of 4096, 32 on 8: 410 / 395.
+  ScorePieces pc;
+  const int g = a.n_q_head / a.n_kv_head;
+  const long long units = (long long)a.batch * a.n_kv_head;
+  constexpr long long kSlots = 2 * 148;  // two CTAs per SM
+  long long heads = std::max(1LL, std::min((long long)g, units * g * (n_tile + 1) / (8 * kSlots)));
+  auto pieces = [&](long long h) { return (g + h - 1) / h; };
+  while (heads < g && (pieces(heads) * units * a.prompt > (long long)a.partial_floats || pieces(heads) * n_tile > 65535)) ++heads;
+  pc.heads = (int)heads;
+  pc.n_piece = (int)pieces(heads);
+  pc.partial = a.partial;
+  pc.tickets = a.tickets;
+  k1<<<dim3(a.n_q_head, a.batch, n_tile), kPrefillThreads, smem, s>>>(tm_q, tm_k, a, pc, scale_log2, status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k2<<<dim3(a.n_kv_head, a.batch, n_tile), kPrefillThreads, smem, s>>>(tm_k, tm_q, a, scale_log2, status);
+  k2<<<dim3(a.n_kv_head, a.batch, n_tile * pc.n_piece), kPrefillThreads, smem, s>>>(tm_k, tm_q, a, pc, scale_log2, status);
   return cudaGetLastError();
 }
 

@@ -21,7 +21,7 @@ inline int elem_bytes(int dtype) { return dtype == SQ_F32 ? 4 : 2; }
 constexpr int kMaxImportanceCtas = 4096;
 
 struct WsLayout {
-  size_t cos_sum, tok_count, cta_partial, ticket, cos_sim, budget, is_g3, status, tickets, layers, order, order_by_layer,
+  size_t cos_sum, tok_count, cta_partial, ticket, cos_sim, budget, is_g3, status, tickets, score_tickets, layers, order, order_by_layer,
       evict_tab;
   size_t part_stat, part_o, logits, acc_prompt, lse2, total;
   size_t items_cap, logits_floats, lse_floats, n_desc_cap;
@@ -137,6 +137,7 @@ WsLayout ws_layout(const sq_config& c, int64_t b_init) {
   w.is_g3 = take(ND);
   w.status = take(4);
   w.tickets = take(4 * L * U);
+  w.score_tickets = take(c.policy == SQ_POLICY_H2O ? 4 * U * (((size_t)c.max_prompt + 127) / 128) : 0);
   w.layers = take(sizeof(LayerDesc) * ND);
   w.order = take(4 * ND);
   w.order_by_layer = take(4 * ND);
@@ -490,6 +491,9 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
       s.n_kv_head = c->cfg.n_kv_head;
       s.prompt = P;
       s.head_dim = c->cfg.head_dim;
+      s.partial = ws_ptr<float>(c, c->wl.part_o);  // the decode partials are idle during prefill
+      s.partial_floats = c->wl.items_cap * (c->cfg.n_q_head / c->cfg.n_kv_head) * c->cfg.head_dim;
+      s.tickets = ws_ptr<int>(c, c->wl.score_tickets);
       SQ_CUDA(c, launch_prefill_scores(s, c->cfg.dtype, ws_ptr<int>(c, c->wl.status), st));
       acc = s.acc_prompt;
     }

@@ -69,6 +69,16 @@ struct ScoreArgs {  // H2O prompt scores of one layer
   float* lse2;        // [B, Hq, P]  log2-domain row log-sum-exp
   float* acc_prompt;  // [B, Hkv, P]
   int batch, n_q_head, n_kv_head, prompt, head_dim;
+  float* partial;       // scratch for column sums of some heads (tcgen05 kernels), partial_floats of it
+  size_t partial_floats;
+  int* tickets;         // [B * Hkv][ceil(P / 128)] arrival counters, zero between launches
+};
+// How sweep 2 of the prompt scores is cut: pieces of `heads` query heads of a group; with more than
+// one piece, piece p's column sums go to partial + p * B * Hkv * P and the last to finish adds them.
+struct ScorePieces {
+  int heads, n_piece;
+  float* partial;
+  int* tickets;
 };
 
 // "Layer" below means one cache descriptor: a layer of the whole batch, or, with per-sequence
