@@ -40,6 +40,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   const int unit = it.local / it.n_split, split = it.local - unit * it.n_split;
   const int len = min(a.n_tok + 1, b);
   const bool h2o = (a.policy == SQ_POLICY_H2O);
+  if (!a.early) grid_wait();
   int w;  // slot that receives the new token
   if (h2o) {
     w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
@@ -63,6 +64,36 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   float* stat = a.part_stat + (size_t)blockIdx.x * a.group * kStatStride;
   float* po = a.part_o + (size_t)blockIdx.x * a.group * D;
 
+  // One batch of this lane's rows; the new token's come from k_new / v_new (`fresh`) or, ahead of
+  // grid_wait(), not at all (the cached row its slot still holds, replaced afterwards).
+  uint4 kq[U], vq[U];
+  bool ok[U];
+  auto load_rows = [&](int r0, bool fresh) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int row = r0 + u * RPW + rg;
+      ok[u] = row < t1;
+      const int rr = ok[u] ? row : t0;
+      const T* kp = (fresh && rr == w) ? kn : Kb + (size_t)rr * D;
+      const T* vp = (fresh && rr == w) ? vn : Vb + (size_t)rr * D;
+      kq[u] = ld_stream(kp + sub * EPV);
+      vq[u] = ld_stream(vp + sub * EPV);
+    }
+  };
+  if (a.early) {
+    const int r0 = t0 + warp * (U * RPW);
+    load_rows(r0, false);
+    grid_wait();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int row = r0 + u * RPW + rg, rr = ok[u] ? row : t0;
+      if (rr == w) {
+        kq[u] = ld_stream(kn + sub * EPV);
+        vq[u] = ld_stream(vn + sub * EPV);
+      }
+    }
+  }
+
   for (int hb = 0; hb < a.group; hb += GT) {
     float qr[GT][EPV], o[GT][EPV], m[GT], l[GT];
 #pragma unroll
@@ -82,18 +113,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
       }
     }
     for (int r0 = t0 + warp * (U * RPW); r0 < t1; r0 += NW * U * RPW) {
-      uint4 kq[U], vq[U];
-      bool ok[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int row = r0 + u * RPW + rg;
-        ok[u] = row < t1;
-        const int rr = ok[u] ? row : t0;
-        const T* kp = (rr == w) ? kn : Kb + (size_t)rr * D;
-        const T* vp = (rr == w) ? vn : Vb + (size_t)rr * D;
-        kq[u] = ld_stream(kp + sub * EPV);
-        vq[u] = ld_stream(vp + sub * EPV);
-      }
+      if (!(a.early && hb == 0 && r0 == t0 + warp * (U * RPW))) load_rows(r0, true);
       float s[U][GT];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -235,6 +255,7 @@ __global__ void __launch_bounds__(kSelThreads, 5) decode_combine_kernel(DecodeAr
   if (!locate_desc(a, blockIdx.x / a.n_unit, it)) return;
   const int layer = it.layer;
   const int tid = threadIdx.x, D = a.head_dim, G = a.group, ns = it.n_split;
+  grid_wait();
   const LayerDesc* ldp = a.layers + layer;
   const int b = ldp->b, cap = ldp->cap;
   const size_t item0 = (size_t)it.base + (size_t)unit * ns;
@@ -358,6 +379,7 @@ __global__ void __launch_bounds__(32 * kWarpUpdWarps, 3) h2o_update_warp_kernel(
   const LayerDesc* ldp = a.layers + layer;
   const int b = ldp->b, cap = ldp->cap;
   const float* stat = a.part_stat + ((size_t)k * a.n_unit + unit) * G * kStatStride;
+  grid_wait();
   if (lane < G) {
     const float2 ml = *reinterpret_cast<const float2*>(stat + lane * kStatStride);
     s_M[wib][lane] = ml.x;
@@ -447,18 +469,18 @@ __global__ void __launch_bounds__(32 * kWarpUpdWarps, 3) h2o_update_warp_kernel(
 }
 
 template <typename T, int D>
-static void launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t s) {
+static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t s) {
+  const DecodeArgsBase& base = a;
   if (a.group == 1) {
-    // the register-capped kernel gets its own build for launches without split-K
+    // the register-capped kernel gets its own build for launches without split-K (which takes no table)
     // few unsplit units (at most two 16-warp CTAs per SM, all resident at once): 16 warps per unit
-    if (a.uniform && n_items <= 2 * 148) decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16><<<n_items, 512, 0, s>>>(a);
-    else if (a.uniform) decode_attn_kernel<T, D, 1, 1, DecodeArgsBase><<<n_items, 128, 0, s>>>(a);  // sliced: no table
-    else decode_attn_kernel<T, D, 1, 0, DecodeArgs><<<n_items, 128, 0, s>>>(a);
-  } else if (a.group <= 4) {
-    decode_attn_kernel<T, D, 4, -1, DecodeArgs><<<n_items, 128, 0, s>>>(a);
-  } else {
-    decode_attn_kernel<T, D, 8, -1, DecodeArgs><<<n_items, 128, 0, s>>>(a);
+    if (a.uniform && n_items <= 2 * 148)
+      return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16>, n_items, 512, 0, s, base);
+    if (a.uniform) return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase>, n_items, 128, 0, s, base);
+    return launch_chained(decode_attn_kernel<T, D, 1, 0, DecodeArgs>, n_items, 128, 0, s, a);
   }
+  if (a.group <= 4) return launch_chained(decode_attn_kernel<T, D, 4, -1, DecodeArgs>, n_items, 128, 0, s, a);
+  return launch_chained(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, n_items, 128, 0, s, a);
 }
 
 // Which attention kernel serves a shape: wide bf16 groups at head_dim 64 go to the tcgen05
@@ -489,29 +511,23 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need
     if (e == cudaSuccess) done = true;
     else if (e != cudaErrorNotSupported) return e;
   }
-  if (done) {
-  } else if (dtype == SQ_F32) {
-    if (a.head_dim == 64) launch_attn_g<float, 64>(a, n_items, s);
-    else launch_attn_g<float, 128>(a, n_items, s);
-  } else {
-    if (a.head_dim == 64) launch_attn_g<__nv_bfloat16, 64>(a, n_items, s);
-    else launch_attn_g<__nv_bfloat16, 128>(a, n_items, s);
+  if (!done) {
+    cudaError_t e;
+    if (dtype == SQ_F32) e = a.head_dim == 64 ? launch_attn_g<float, 64>(a, n_items, s) : launch_attn_g<float, 128>(a, n_items, s);
+    else e = a.head_dim == 64 ? launch_attn_g<__nv_bfloat16, 64>(a, n_items, s) : launch_attn_g<__nv_bfloat16, 128>(a, n_items, s);
+    if (e != cudaSuccess) return e;
   }
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || !need_combine) return e;
+  if (!need_combine) return cudaSuccess;
   const int n_cta = a.n_layer_total * a.n_unit;
   // More units than the CTA-per-unit kernel holds in one wave (5 CTAs per SM), and nothing to
   // merge: only the scores and the next victim remain, one warp per unit.  Smaller launches
   // (one layer of a small batch) finish sooner with a CTA per unit.
   if (a.policy == SQ_POLICY_H2O && a.uniform && a.group <= 32 && n_cta > 148 * 5) {
-    h2o_update_warp_kernel<<<(n_cta + kWarpUpdWarps - 1) / kWarpUpdWarps, 32 * kWarpUpdWarps, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_chained(h2o_update_warp_kernel, (n_cta + kWarpUpdWarps - 1) / kWarpUpdWarps, 32 * kWarpUpdWarps, 0, s,
+                          static_cast<const DecodeArgsBase&>(a));
   }
-  if (dtype == SQ_F32)
-    decode_combine_kernel<float><<<n_cta, kSelThreads, 0, s>>>(a);
-  else
-    decode_combine_kernel<__nv_bfloat16><<<n_cta, kSelThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  if (dtype == SQ_F32) return launch_chained(decode_combine_kernel<float>, n_cta, kSelThreads, 0, s, a);
+  return launch_chained(decode_combine_kernel<__nv_bfloat16>, n_cta, kSelThreads, 0, s, a);
 }
 
 }  // namespace sq

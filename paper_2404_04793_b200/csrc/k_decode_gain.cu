@@ -19,6 +19,7 @@
 // Split-K pieces of a unit leave their candidate in global memory; the piece that arrives last
 // (atomic ticket, nobody waits) picks the winner.  Every barrier wait is bounded.
 #include "sq_decode_common.cuh"
+#include "sq_device.cuh"
 #include "sq_internal.h"
 #include "sq_select.cuh"
 #include "sq_tc.cuh"
@@ -97,32 +98,46 @@ __global__ void __launch_bounds__(64 + 128 * SETS, CTAS)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+
+  // fetch of K tile i (its stage is free); rows of this unit in the [rows][64] view of the pool
+  auto load_tile = [&](int i) {
+    const int st = i % STAGES;
+    const long long k_row0 = ldp->k_off / (kD * 2) + (long long)unit * cap;
+    mbar_expect_tx(bar_full(st), kTileBytes);
+    tma_load_2d(s_u32(k_s + st * kTileBytes), &tm_k, 0, (int)(k_row0 + t0 + i * kTM), bar_full(st));
+  };
+  // The attention launch ahead changes one row of a unit's K, the new token's: the first tiles are
+  // fetched while it runs out, up to the one that holds that row.  (The victim table still says which
+  // one it is: a unit's victim is replaced by this kernel, after the unit's last piece has read it here.)
+  int issued = 0;
+  if (tid == 0) {
+    const int w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
+    const int n_pre = min(min(STAGES, n_tiles), (w >= t0 && w < t1) ? (w - t0) / kTM : STAGES);
+    for (; issued < n_pre; ++issued) load_tile(issued);
+  }
+  grid_wait();
   if (tid >= 64 && tid < 64 + kTM) {
     const int h = tid - 64;
     const float* lse = a.logits + ldp->lse_off + (size_t)unit * G;
     // columns past the group read +inf here, so their weight is exp2(-inf) = 0
     s_nlse[h] = (h < G) ? -lse[h] : -INFINITY;
   }
-  tc_fence_before();
   __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_slot;
 
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      // rows of this unit in the [rows][64] views of the pool and of q (tensor maps)
-      const long long k_row0 = ldp->k_off / (kD * 2) + (long long)unit * cap;
       const long long q_row0 = (long long)(tok * a.n_q_head + (size_t)kvh * G);
       mbar_expect_tx(bar_q, n_cols * 128);
       tma_load_2d(s_u32(q_s), &tm_q, 0, (int)q_row0, bar_q);
-      int issued = 0;
-      for (int i = 0; i < n_tiles; ++i) {
-        const int st = i % STAGES;
-        if (i >= STAGES && !mbar_wait(bar_empty(st), ((i / STAGES) - 1) & 1, abort_flag)) break;
-        mbar_expect_tx(bar_full(st), kTileBytes);
-        tma_load_2d(s_u32(k_s + st * kTileBytes), &tm_k, 0, (int)(k_row0 + t0 + i * kTM), bar_full(st));
-        issued = i + 1;
+      for (; issued < n_tiles; ++issued) {
+        const int i = issued;
+        if (i >= STAGES && !mbar_wait(bar_empty(i % STAGES), ((i / STAGES) - 1) & 1, abort_flag)) break;
+        load_tile(i);
       }
       if (*abort_flag) {
         // copies in flight must land before the CTA's shared memory is released
@@ -316,9 +331,9 @@ cudaError_t launch_h2o_gain_tc(const DecodeArgs& a, int n_items, size_t pool_byt
     configured = true;
   }
   const int n_buf = kTmemCols == 128 ? 1 : (3 * n_cols <= kTmemCols ? 3 : 2);
-  if (a.uniform) kern_u<<<n_items, 64 + 128 * kSets, smem, s>>>(tm_q, tm_k, a, n_cols, n_buf);  // sliced: no table
-  else kern_s<<<n_items, 64 + 128 * kSets, smem, s>>>(tm_q, tm_k, a, n_cols, n_buf);
-  return cudaGetLastError();
+  const DecodeArgsBase& base = a;  // without split-K: no table
+  if (a.uniform) return launch_chained(kern_u, n_items, 64 + 128 * kSets, smem, s, tm_q, tm_k, base, n_cols, n_buf);
+  return launch_chained(kern_s, n_items, 64 + 128 * kSets, smem, s, tm_q, tm_k, a, n_cols, n_buf);
 }
 
 }  // namespace sq

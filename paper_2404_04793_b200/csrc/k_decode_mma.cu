@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
   const int unit = it.local / it.n_split, split = it.local - unit * it.n_split;
   const int len = min(a.n_tok + 1, b);
   const bool h2o = (a.policy == SQ_POLICY_H2O);
+  if (!a.early) grid_wait();
   int w;
   if (h2o) {
     w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
@@ -113,13 +114,42 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
   float* stat = a.part_stat + (size_t)blockIdx.x * G * kStatStride;
   float* po = a.part_o + (size_t)blockIdx.x * G * D;
 
-  // the CTA whose range holds slot w stores the new token first, then reads it like any other
+  const int n_tiles = (t1 - t0 + kTile - 1) / kTile;
+  // `skip`: a row that is left out (the new token's, in the tiles fetched before it is in the cache)
+  auto load_tile = [&](int tile, int skip) {
+    if (tile < n_tiles) {
+      const int stage = tile % STAGES;
+      const int row0 = t0 + tile * kTile;
+      const uint32_t kdst = smem_u32(k_s + stage * TILE_BYTES), vdst = smem_u32(v_s + stage * TILE_BYTES);
+      for (int i = tid; i < kTile * CH; i += NT) {
+        const int r = i / CH, c = i - r * CH;
+        if (row0 + r == skip) continue;
+        const bool ok = row0 + r < t1;
+        const size_t src = (size_t)(ok ? row0 + r : t0) * D + c * 8;
+        const uint32_t off = swz<D>(r, c);
+        cp_async16(kdst + off, Kb + src, ok);
+        cp_async16(vdst + off, Vb + src, ok);
+      }
+    }
+    cp_async_commit();
+  };
+  // The first tiles of the cache, but for the new token's row, are under way before the launch ahead
+  // is done (a.early) and before q is read.
+#pragma unroll
+  for (int s = 0; s < STAGES - 1; ++s) load_tile(s, w);
+  if (a.early) grid_wait();
+
+  // the CTA whose range holds slot w stores the new token: in the cache, where later tiles read it
+  // like any other row, and in the tile already fetched around it
   if (w >= t0 && w < t1) {
     if (tid < 2 * CH) {
       const bool is_v = tid >= CH;
       const int c = is_v ? tid - CH : tid;
       const uint4 val = *reinterpret_cast<const uint4*>((is_v ? vn : kn) + c * 8);
       *reinterpret_cast<uint4*>((is_v ? Vb : Kb) + (size_t)w * D + c * 8) = val;
+      const int tile = (w - t0) / kTile;
+      if (tile < STAGES - 1)
+        *reinterpret_cast<uint4*>((is_v ? v_s : k_s) + tile * TILE_BYTES + swz<D>((w - t0) % kTile, c)) = val;
     }
     if (tid == 2 * CH) {
       reinterpret_cast<int*>(a.pool + ldp->pos_off)[(size_t)unit * cap + w] = a.n_tok;
@@ -135,26 +165,6 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
     *reinterpret_cast<uint4*>(q_s + swz<D>(row, c)) = val;
   }
   __syncthreads();
-
-  const int n_tiles = (t1 - t0 + kTile - 1) / kTile;
-  auto load_tile = [&](int tile) {
-    if (tile < n_tiles) {
-      const int stage = tile % STAGES;
-      const int row0 = t0 + tile * kTile;
-      const uint32_t kdst = smem_u32(k_s + stage * TILE_BYTES), vdst = smem_u32(v_s + stage * TILE_BYTES);
-      for (int i = tid; i < kTile * CH; i += NT) {
-        const int r = i / CH, c = i - r * CH;
-        const bool ok = row0 + r < t1;
-        const size_t src = (size_t)(ok ? row0 + r : t0) * D + c * 8;
-        const uint32_t off = swz<D>(r, c);
-        cp_async16(kdst + off, Kb + src, ok);
-        cp_async16(vdst + off, Vb + src, ok);
-      }
-    }
-    cp_async_commit();
-  };
-#pragma unroll
-  for (int s = 0; s < STAGES - 1; ++s) load_tile(s);
 
   // A fragments of Q, kept for the whole item
   uint32_t qa[MT][KS][4];
@@ -186,7 +196,7 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
   for (int tile = 0; tile < n_tiles; ++tile) {
     cp_async_wait<STAGES - 2>();
     __syncthreads();
-    load_tile(tile + STAGES - 1);
+    load_tile(tile + STAGES - 1, -1);
     const int stage = tile % STAGES;
     const uint32_t kst = smem_u32(k_s + stage * TILE_BYTES), vst = smem_u32(v_s + stage * TILE_BYTES);
     const int tok0 = t0 + tile * kTile + wn * 16;  // first token of this warp's 16
@@ -382,8 +392,7 @@ static cudaError_t launch_cfg(const DecodeArgs& a, int n_items, cudaStream_t s) 
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  kern<<<n_items, 32 * WM * WN, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(kern, n_items, 32 * WM * WN, smem, s, a);
 }
 
 // Returns cudaErrorNotSupported when no tensor-core configuration covers the shape.

@@ -33,6 +33,7 @@
 #include <type_traits>
 
 #include "sq_decode_common.cuh"
+#include "sq_device.cuh"
 #include "sq_internal.h"
 #include "sq_tc.cuh"
 #include "sq_tc_quad.cuh"
@@ -87,6 +88,7 @@ __global__ void __launch_bounds__(192, 2)
   const int b = ldp->b, cap = ldp->cap, G = a.group;
   const int unit = it.local / it.n_split, split = it.local - unit * it.n_split;
   const int len = min(a.n_tok + 1, b);
+  if (!a.early) grid_wait();
   int w;
   if (H2O) {
     w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
@@ -104,26 +106,6 @@ __global__ void __launch_bounds__(192, 2)
   using bf16 = __nv_bfloat16;
   // (pointers are formed where they are used: the softmax loop needs the registers)
 
-  // the CTA whose range holds slot w stores the new token first (generic proxy), then lets
-  // the TMA reads (async proxy) see it
-  if (w >= t0 && w < t1) {
-    if (tid < 16) {
-      bf16* Kb = reinterpret_cast<bf16*>(a.pool + ldp->k_off) + (size_t)unit * cap * kD;
-      bf16* Vb = reinterpret_cast<bf16*>(a.pool + ldp->v_off) + (size_t)unit * cap * kD;
-      const bf16* kn = reinterpret_cast<const bf16*>(a.k_new) + (tok * a.n_kv_head + kvh) * kD;
-      const bf16* vn = reinterpret_cast<const bf16*>(a.v_new) + (tok * a.n_kv_head + kvh) * kD;
-      const bool is_v = tid >= 8;
-      const int c = tid & 7;
-      const uint4 val = *reinterpret_cast<const uint4*>((is_v ? vn : kn) + c * 8);
-      *reinterpret_cast<uint4*>((is_v ? Vb : Kb) + (size_t)w * kD + c * 8) = val;
-    }
-    if (tid == 16) {
-      reinterpret_cast<int*>(a.pool + ldp->pos_off)[(size_t)unit * cap + w] = a.n_tok;
-      if (H2O) reinterpret_cast<float*>(a.pool + ldp->acc_off)[(size_t)unit * cap + w] = 0.f;
-    }
-    __threadfence();
-    fence_proxy_async();
-  }
   if (tid == 0) {
     mbar_init(bar_q, 1);
     mbar_init(bar_odone, 1);
@@ -148,23 +130,56 @@ __global__ void __launch_bounds__(192, 2)
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  // fetch of K and V tile i (its stage is free); rows of this unit in the [rows][64] view of the pool
+  auto load_tile = [&](int i) {
+    const int st = i % STAGES;
+    const long long k_row0 = ldp->k_off / (kD * 2) + (long long)unit * cap;
+    const long long v_row0 = ldp->v_off / (kD * 2) + (long long)unit * cap;
+    mbar_expect_tx(bar_full(st), 2 * kTileBytes);
+    tma_load_2d(s_u32(k_s + st * kTileBytes), &tm_k, 0, (int)(k_row0 + t0 + i * kTM), bar_full(st));
+    tma_load_2d(s_u32(v_s + st * kTileBytes), &tm_v, 0, (int)(v_row0 + t0 + i * kTM), bar_full(st));
+  };
+  // The first tiles are under way before the launch ahead is done, up to the one that holds slot w
+  int issued = 0;
+  if (a.early) {
+    if (tid == 0) {
+      const int n_pre = min(min(STAGES, n_tiles), (w >= t0 && w < t1) ? (w - t0) / kTM : STAGES);
+      for (; issued < n_pre; ++issued) load_tile(issued);
+    }
+    grid_wait();
+  }
+  // the CTA whose range holds slot w stores the new token (generic proxy), then lets the TMA reads
+  // (async proxy) see it
+  if (w >= t0 && w < t1) {
+    if (tid < 16) {
+      bf16* Kb = reinterpret_cast<bf16*>(a.pool + ldp->k_off) + (size_t)unit * cap * kD;
+      bf16* Vb = reinterpret_cast<bf16*>(a.pool + ldp->v_off) + (size_t)unit * cap * kD;
+      const bf16* kn = reinterpret_cast<const bf16*>(a.k_new) + (tok * a.n_kv_head + kvh) * kD;
+      const bf16* vn = reinterpret_cast<const bf16*>(a.v_new) + (tok * a.n_kv_head + kvh) * kD;
+      const bool is_v = tid >= 8;
+      const int c = tid & 7;
+      const uint4 val = *reinterpret_cast<const uint4*>((is_v ? vn : kn) + c * 8);
+      *reinterpret_cast<uint4*>((is_v ? Vb : Kb) + (size_t)w * kD + c * 8) = val;
+    }
+    if (tid == 16) {
+      reinterpret_cast<int*>(a.pool + ldp->pos_off)[(size_t)unit * cap + w] = a.n_tok;
+      if (H2O) reinterpret_cast<float*>(a.pool + ldp->acc_off)[(size_t)unit * cap + w] = 0.f;
+    }
+    __threadfence();
+    fence_proxy_async();
+  }
+  __syncthreads();
+
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      // rows of this unit in the [rows][64] views of the pool (tensor maps) and of q
-      const long long k_row0 = ldp->k_off / (kD * 2) + (long long)unit * cap;
-      const long long v_row0 = ldp->v_off / (kD * 2) + (long long)unit * cap;
       const long long q_row0 = (long long)(tok * a.n_q_head + (size_t)kvh * G);
       mbar_expect_tx(bar_q, kQBytes);
       tma_load_2d(s_u32(q_s), &tm_q, 0, (int)q_row0, bar_q);
-      int issued = 0;
-      for (int i = 0; i < n_tiles; ++i) {
-        const int st = i % STAGES;
-        if (i >= STAGES && !mbar_wait(bar_empty(st), ((i / STAGES) - 1) & 1, abort_flag)) break;
-        mbar_expect_tx(bar_full(st), 2 * kTileBytes);
-        tma_load_2d(s_u32(k_s + st * kTileBytes), &tm_k, 0, (int)(k_row0 + t0 + i * kTM), bar_full(st));
-        tma_load_2d(s_u32(v_s + st * kTileBytes), &tm_v, 0, (int)(v_row0 + t0 + i * kTM), bar_full(st));
-        issued = i + 1;
+      for (; issued < n_tiles; ++issued) {
+        const int i = issued;
+        if (i >= STAGES && !mbar_wait(bar_empty(i % STAGES), ((i / STAGES) - 1) & 1, abort_flag)) break;
+        load_tile(i);
       }
       if (*abort_flag) {
         mbar_wait(bar_q, 0, abort_flag);
@@ -470,8 +485,7 @@ static cudaError_t launch_tc_cfg(const DecodeArgs& a, int n_items, const CUtenso
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  kern<<<n_items, 192, smem, s>>>(tq, tk, tv, a);
-  return cudaGetLastError();
+  return launch_chained(kern, n_items, 192, smem, s, tq, tk, tv, a);
 }
 
 // Returns cudaErrorNotSupported when the shape is outside this kernel's range.

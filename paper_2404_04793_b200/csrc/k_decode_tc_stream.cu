@@ -44,6 +44,7 @@
 #include <type_traits>
 
 #include "sq_decode_common.cuh"
+#include "sq_device.cuh"
 #include "sq_internal.h"
 #include "sq_stream.cuh"
 #include "sq_tc.cuh"
@@ -182,6 +183,7 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
   SegIter it;
   it.init(a, blockIdx.x);
 
+  if (warp != 0 || !a.early) grid_wait();  // (the producer: once its first tiles are under way)
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     int g = 0;          // tiles issued so far
@@ -203,6 +205,23 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
         }
       } else {
         w = ring_slot(a.n_tok, b, ldp->ring_base, ldp->ring_origin);
+      }
+      // rows of this unit in the [rows][64] views of the pool (tensor maps) and of q
+      const long long k_row0 = ldp->k_off / (kD * 2) + (long long)unit * cap + t0;
+      const long long v_row0 = ldp->v_off / (kD * 2) + (long long)unit * cap + t0;
+      auto load_tile = [&](int i) {
+        const int st = g % STAGES;
+        mbar_expect_tx(bar_full(st), 2 * kTileBytes);
+        tma_load_2d(s_u32(k_s + st * kTileBytes), &tm_k, 0, (int)(k_row0 + i * kTM), bar_full(st));
+        tma_load_2d(s_u32(v_s + st * kTileBytes), &tm_v, 0, (int)(v_row0 + i * kTM), bar_full(st));
+      };
+      int i0 = 0;  // tiles of the segment already under way
+      if (a.early && it.seg == 0) {
+        // the CTA's first tiles do not wait for the launch ahead, up to the one that holds slot w
+        const int n_pre = min(min(STAGES, it.ntile), (w >= t0 && w < t1) ? (w - t0) / kTM : STAGES);
+        for (; i0 < n_pre; ++i0, ++g)
+          if (lane == 0) load_tile(i0);
+        grid_wait();
       }
       if (w >= t0 && w < t1) {
         // this segment fetches the tile that holds slot w: store the new row first (generic
@@ -228,23 +247,15 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
       // Q has one buffer: the previous segment's last S product must have read it
       if (it.seg >= 1) ok = warp_wait(bar_qempty, (it.seg - 1) & 1, abort_flag);
       if (!ok) break;
-      // rows of this unit in the [rows][64] views of the pool (tensor maps) and of q
-      const long long k_row0 = ldp->k_off / (kD * 2) + (long long)unit * cap + t0;
-      const long long v_row0 = ldp->v_off / (kD * 2) + (long long)unit * cap + t0;
       if (lane == 0) {
         mbar_expect_tx(bar_qfull, kQBytes);
         tma_load_2d(s_u32(q_s), &tm_q, 0, (int)(tok * a.n_q_head + (size_t)kvh * G), bar_qfull);
       }
       q_issued = it.seg + 1;
-      for (int i = 0; ok && i < it.ntile; ++i, ++g) {
-        const int st = g % STAGES;
-        if (g >= STAGES) ok = warp_wait(bar_empty(st), ((g / STAGES) - 1) & 1, abort_flag);
+      for (int i = i0; ok && i < it.ntile; ++i, ++g) {
+        if (g >= STAGES) ok = warp_wait(bar_empty(g % STAGES), ((g / STAGES) - 1) & 1, abort_flag);
         if (!ok) break;
-        if (lane == 0) {
-          mbar_expect_tx(bar_full(st), 2 * kTileBytes);
-          tma_load_2d(s_u32(k_s + st * kTileBytes), &tm_k, 0, (int)(k_row0 + i * kTM), bar_full(st));
-          tma_load_2d(s_u32(v_s + st * kTileBytes), &tm_v, 0, (int)(v_row0 + i * kTM), bar_full(st));
-        }
+        if (lane == 0) load_tile(i);
       }
     }
     if (*abort_flag && lane == 0) {
@@ -556,8 +567,7 @@ static cudaError_t launch_tc_stream_cfg(const StreamArgs& t, int n_cta, const CU
     if (e != cudaSuccess) return e;
     configured = true;
   }
-  kern<<<n_cta, 192, smem, s>>>(tq, tk, tv, t);
-  return cudaGetLastError();
+  return launch_chained(kern, n_cta, 192, smem, s, tq, tk, tv, t);
 }
 
 // desc_tiles[k]: 128-token tiles per unit of the k-th descriptor of the launch (launch order).

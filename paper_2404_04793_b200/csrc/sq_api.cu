@@ -66,6 +66,10 @@ struct sq_ctx {
   long long imp_tokens[kMaxLayers];  // tokens of a layer seen by sq_layer_importance so far
   bool prefilled[kMaxLayers];
   bool importance_seen[kMaxLayers];
+  // The context's last launch, if it was a decode launch: its layers [last_begin, last_end) and stream.
+  // Any other call that launches something on the caches clears it (last_end = 0).
+  int last_begin, last_end;
+  void* last_stream;
   std::string err;
 };
 
@@ -286,6 +290,8 @@ int sq_ctx_create(const sq_config* cfg, int64_t b_init, void* pool, size_t pool_
   c->per_seq = cfg->per_sequence_budgets != 0;
   c->begun = false;
   c->budget_state = 0;
+  c->last_begin = c->last_end = 0;
+  c->last_stream = nullptr;
   // one pinned block, carved into the staging arrays (largest alignment first)
   const size_t nd = wl.n_desc_cap;
   const size_t bytes = nd * (sizeof(LayerDesc) + sizeof(EvictLayer) + 8 + 4 + 4 + 4 + 4 + 1) + 64;
@@ -331,6 +337,7 @@ const char* sq_last_error(sq_ctx* c) { return c ? c->err.c_str() : "context is N
 int sq_begin_sequence_batch(sq_ctx* c, int32_t batch, int32_t prompt_len, void* stream) {
   if (!c) return SQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  c->last_end = 0;
   if (batch < 1 || batch > c->cfg.max_batch) return fail(c, SQ_ERR_INVALID_ARG, "batch out of range");
   if (prompt_len < 1 || prompt_len > c->cfg.max_prompt) return fail(c, SQ_ERR_INVALID_ARG, "prompt_len out of range");
   c->batch = batch;
@@ -411,6 +418,7 @@ int sq_layer_importance_fused(sq_ctx* c, int32_t layer, const void* resid, const
 int sq_allocate_budgets(sq_ctx* c, int64_t b_init, double p, void* stream) {
   if (!c) return SQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  c->last_end = 0;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
   if (!(p > 0.0 && p <= 1.0)) return fail(c, SQ_ERR_INVALID_ARG, "p must satisfy 0 < p <= 1");
   if (b_init < 1 || b_init > c->b_init_cap) return fail(c, SQ_ERR_INVALID_ARG, "b_init must be in 1..the context's b_init");
@@ -445,6 +453,7 @@ int sq_allocate_budgets(sq_ctx* c, int64_t b_init, double p, void* stream) {
 int sq_set_budgets(sq_ctx* c, const int32_t* budgets_host, void* stream) {
   if (!c) return SQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  c->last_end = 0;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
   if (!budgets_host) return fail(c, SQ_ERR_INVALID_ARG, "budgets_host is NULL");
   if (c->budget_state == 1) SQ_CUDA(c, cudaEventSynchronize(c->ev));
@@ -466,6 +475,7 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
                         const float* acc_prompt, void* stream) {
   if (!c) return SQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  c->last_end = 0;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
   if (layer < 0 || layer >= c->cfg.n_layer) return fail(c, SQ_ERR_INVALID_ARG, "layer out of range");
   if (!k_prompt || !v_prompt || !aligned16(k_prompt) || !aligned16(v_prompt))
@@ -643,6 +653,12 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
     a.split_tokens = split;
     a.policy = cfg.policy;
     a.scale_log2 = (float)(1.4426950408889634 / std::sqrt((double)cfg.head_dim));
+    // A launch directly behind one of other layers may read its caches while that one runs out: what
+    // these layers' caches hold was written by launches before it.
+    a.early = c->last_end > 0 && c->last_stream == stream && (e <= c->last_begin || s >= c->last_end);
+    c->last_begin = s;
+    c->last_end = e;
+    c->last_stream = stream;
     const bool combine = cfg.policy == SQ_POLICY_H2O;  // other policies merge split-K pieces in the last piece
     // 128-token tiles per unit of every descriptor, in launch order (the wide-group kernel deals
     // the launch's tiles out evenly over the SMs)
@@ -660,6 +676,7 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
 int sq_evict(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const int32_t* new_budgets_host, void* stream) {
   if (!c) return SQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  c->last_end = 0;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
   if (layer_begin < 0 || layer_end > c->cfg.n_layer || layer_begin >= layer_end || !new_budgets_host)
     return fail(c, SQ_ERR_INVALID_ARG, "layer range / budgets");
@@ -907,6 +924,7 @@ int sq_ctx_export_layout(sq_ctx* c, sq_layer_layout* out) {
 int sq_ctx_import_layout(sq_ctx* c, const sq_layer_layout* in, void* stream) {
   if (!c || !in) return SQ_ERR_INVALID_ARG;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  c->last_end = 0;
   const sq_config& cfg = c->cfg;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
   if (c->budget_state == 1) SQ_CUDA(c, cudaEventSynchronize(c->ev));

@@ -69,6 +69,15 @@ __device__ __forceinline__ float to_float<__nv_bfloat16>(__nv_bfloat16 x) {
   return __bfloat162float(x);
 }
 
+// Programmatic dependent launch.  grid_wait() returns when every launch before this one in the stream
+// is complete and its writes are visible; it comes before a kernel's first global write and before it
+// reads anything the launch ahead of it may have written.  It lets the next launch start only after
+// that: so everything older than the launch directly ahead is complete when a kernel starts.
+__device__ __forceinline__ void grid_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -40,3 +40,57 @@ def test_prompt_scores_cut_by_heads(head_dim, hq, hkv, batch, prompt):
             want = O.prefill_scores(H.f64(q[s, h * g:(h + 1) * g]), H.f64(k[s, h]))
             np.testing.assert_allclose(acc, want, rtol=H.RTOL_ACC[w.dtype], atol=1e-6)
     assert ctx.status() == 0
+
+
+# Decode launches of one layer right behind one another start before the launch ahead is done and fetch
+# their first rows ahead of it, all but the new token's: its slot goes through every row of the cache,
+# and one layer behind itself (n_layer 1) or a stream change must not read ahead
+@pytest.mark.parametrize("policy", [synth.SLIDING_WINDOW, synth.H2O])
+@pytest.mark.parametrize("dtype,head_dim,hq,hkv,budget", [
+    (torch.bfloat16, 128, 2, 2, 70), (torch.bfloat16, 128, 8, 2, 200), (torch.bfloat16, 64, 40, 1, 400), (torch.bfloat16, 64, 128, 1, 140),
+    (torch.float32, 64, 6, 2, 50)])
+@pytest.mark.parametrize("n_layer", [1, 3])
+def test_layer_by_layer_launches_match_the_whole_stack(policy, dtype, head_dim, hq, hkv, budget, n_layer):
+    w = workload("chain", 9200 + budget, policy=policy, dtype=dtype, head_dim=head_dim, n_q_head=hq, n_kv_head=hkv,
+                 n_layer=n_layer, batch=2, prompt=budget + 9, steps=budget + 5, heavy_mode="none")
+    budgets = [max(8, budget - 31 * l) for l in range(n_layer)]
+    ctxs = []
+    for _ in range(2):
+        ctx = H.make_ctx(w, b_init=budget)
+        ctx.begin_sequence_batch(w.batch, w.prompt)
+        ctx.set_budgets(budgets)
+        for l in range(n_layer):
+            q, k, v = synth.prompt_qkv(w, l, DEV)
+            ctx.prefill_compress(l, k, v, q if policy == synth.H2O else None)
+        ctxs.append(ctx)
+    stack, chained = ctxs
+    side = torch.cuda.Stream()
+    for t in range(w.steps):
+        q, kn, vn = synth.decode_qkv(w, t, DEV)
+        a, b = torch.empty_like(q), torch.empty_like(q)
+        torch.cuda.synchronize()
+        stack.decode_step(0, n_layer, q, kn, vn, a)
+        if t % 7 == 3:                                # the step's last layer on another stream, behind an event
+            ev = torch.cuda.Event()
+            for l in range(n_layer - 1):
+                chained.decode_step(l, l + 1, q[l], kn[l], vn[l], b[l])
+            ev.record()
+            with torch.cuda.stream(side):
+                side.wait_event(ev)
+                l = n_layer - 1
+                chained.decode_step(l, l + 1, q[l], kn[l], vn[l], b[l])
+                ev.record(side)
+            torch.cuda.current_stream().wait_event(ev)
+        else:
+            for l in range(n_layer):
+                chained.decode_step(l, l + 1, q[l], kn[l], vn[l], b[l])
+        assert torch.allclose(a.float(), b.float(), rtol=0, atol=H.TOL_OUT[dtype])   # other split-K pieces
+    for l in range(n_layer):
+        for h in range(hkv):
+            pa, _ = stack.get_kept(l, 1, h)
+            pb, _ = chained.get_kept(l, 1, h)
+            assert pa == pb
+            ka, va = stack.get_kv(l, 1, h)
+            kb, vb = chained.get_kv(l, 1, h)
+            assert torch.equal(ka, kb) and torch.equal(va, vb)
+    assert stack.status() == 0 and chained.status() == 0
