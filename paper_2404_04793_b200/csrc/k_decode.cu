@@ -2,6 +2,7 @@
 // token into the slot C_seq frees, attend over the kept slots (split-K flash-decode, all query
 // heads of a KV head share one pass over K/V), and for H2O add the received probabilities to
 // the per-token scores and choose the slot the next append will reuse.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 
@@ -9,6 +10,7 @@
 #include "sq_internal.h"
 #include "sq_select.cuh"
 #include "sq_decode_common.cuh"
+#include "sq_scores.cuh"
 
 namespace sq {
 
@@ -22,7 +24,9 @@ namespace sq {
 // batch): those leave most warp slots of the GPU empty with 4 warps per unit, and each warp then
 // walks its rows in a chain of dependent round trips to memory; 16 warps per unit make the chain
 // a quarter as long.
-template <typename T, int D, int GT, int UNIFORM, class Args, int NW = 4>
+// SCORES: H2O with the score update in the same launch (sq_scores.cuh): the pieces of a unit are the
+// CTAs of a cluster and the logits stay in shared memory.
+template <typename T, int D, int GT, int UNIFORM, class Args, int NW = 4, bool SCORES = false>
 __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 8 : 6) : 1) : 2) decode_attn_kernel(Args a) {
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;   // lanes per row
@@ -31,19 +35,22 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   __shared__ float sm_o[NW][GT][D];
   __shared__ float sm_m[NW][GT], sm_l[NW][GT];
 
+  extern __shared__ __align__(16) float dyn[];  // SCORES: logits [token of the piece][group], partial O [group][D], its sums [group][4]
   ItemLoc it;
-  if (!locate<UNIFORM, Args>(a, blockIdx.x, it)) return;
+  int item = blockIdx.x;
+  if constexpr (SCORES) item /= cluster_size();
+  if (!locate<UNIFORM, Args>(a, item, it)) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int sub = lane % LPR, rg = lane / LPR;
   const LayerDesc* ldp = a.layers + it.layer;
   const int b = ldp->b, cap = ldp->cap;
-  const int unit = it.local / it.n_split, split = it.local - unit * it.n_split;
+  const int unit = it.local / it.n_split;
   const int len = min(a.n_tok + 1, b);
-  const bool h2o = (a.policy == SQ_POLICY_H2O);
+  const bool h2o = SCORES || (a.policy == SQ_POLICY_H2O);
   if (!a.early) grid_wait();
   int w;  // slot that receives the new token
   if (h2o) {
-    w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
+    w = (a.n_tok < b) ? a.n_tok : __ldcg(reinterpret_cast<const int*>(a.pool + ldp->victim_off) + unit);
     if (w < 0 || w >= b) {
       if (tid == 0) atomicOr(a.status, 2);
       w = 0;
@@ -51,7 +58,15 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   } else {
     w = ring_slot(a.n_tok, b, ldp->ring_base, ldp->ring_origin);
   }
-  const int t0 = split * a.split_tokens, t1 = min(len, t0 + a.split_tokens);
+  int t0, piece;
+  if constexpr (SCORES) {
+    piece = piece_slots(len, cluster_size());
+    t0 = cluster_rank() * piece;
+  } else {
+    piece = a.split_tokens;
+    t0 = (it.local - unit * it.n_split) * piece;
+  }
+  const int t1 = min(len, t0 + piece);  // (a piece may be empty under SCORES)
   const int seq = unit / a.n_kv_head, kvh = unit - seq * a.n_kv_head;
   const size_t tok = (size_t)(it.layer - a.layer_begin) * a.batch + seq;
   const T* Kb = reinterpret_cast<const T*>(a.pool + ldp->k_off) + (size_t)unit * cap * D;
@@ -60,7 +75,11 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   const T* kn = reinterpret_cast<const T*>(a.k_new) + (tok * a.n_kv_head + kvh) * D;
   const T* vn = reinterpret_cast<const T*>(a.v_new) + (tok * a.n_kv_head + kvh) * D;
   T* ob = reinterpret_cast<T*>(a.out) + (tok * a.n_q_head + (size_t)kvh * a.group) * D;
-  float* logit = a.logits + ldp->logit_off + (size_t)unit * cap * a.group;  // [slot][group]
+  float* logit;  // [slot][group]
+  if constexpr (SCORES) logit = dyn - (size_t)t0 * a.group;
+  else logit = a.logits + ldp->logit_off + (size_t)unit * cap * a.group;
+  float* part_o = dyn + ((size_t)piece * a.group + 3) / 4 * 4;  // SCORES
+  float* part_stat = part_o + (size_t)a.group * D;
   float* stat = a.part_stat + (size_t)blockIdx.x * a.group * kStatStride;
   float* po = a.part_o + (size_t)blockIdx.x * a.group * D;
 
@@ -82,12 +101,12 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   };
   if (a.early) {
     const int r0 = t0 + warp * (U * RPW);
-    load_rows(r0, false);
+    if (t0 < t1) load_rows(r0, false);
     grid_wait();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int row = r0 + u * RPW + rg, rr = ok[u] ? row : t0;
-      if (rr == w) {
+      if (t0 < t1 && rr == w) {
         kq[u] = ld_stream(kn + sub * EPV);
         vq[u] = ld_stream(vn + sub * EPV);
       }
@@ -212,6 +231,11 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
         L += sm_l[ww][g] * f;
         O += sm_o[ww][g][e] * f;
       }
+      if constexpr (SCORES) {
+        part_o[h * D + e] = O;
+        if (e == 0) *reinterpret_cast<float4*>(part_stat + h * 4) = make_float4(M, L, L, 0.f);
+        continue;
+      }
       if (it.n_split == 1)
         ob[(size_t)h * D + e] = narrow<T>(O / L);
       else
@@ -239,7 +263,12 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
       if (h2o) reinterpret_cast<float*>(a.pool + ldp->acc_off)[(size_t)unit * cap + w] = 0.f;
     }
   }
-  if (!h2o && it.n_split > 1) merge_if_last<T, (GT == 1 ? 2 : 4)>(a, it, unit);
+  if constexpr (SCORES) {
+    __shared__ ScoreShared sh;
+    finish_scores<T, D, NW * 32>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * a.group, part_o, part_stat, sh);
+  } else {
+    if (!h2o && it.n_split > 1) merge_if_last<T, (GT == 1 ? 2 : 4)>(a, it, unit);
+  }
 }
 
 // One CTA per (layer, unit): merges the split-K partials into the output and, for H2O, adds
@@ -483,11 +512,51 @@ static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t 
   return launch_chained(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, n_items, 128, 0, s, a);
 }
 
+constexpr int kScoresLimit = 96 * 1024;  // dynamic shared memory of a CTA with the score update
+template <auto KERN>
+static cudaError_t launch_scores_kernel(const DecodeArgs& a, int pieces, int n_cta, int threads, size_t smem, cudaStream_t s) {
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresLimit);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  return launch_chained_cluster(KERN, pieces, n_cta, threads, smem, s, static_cast<const DecodeArgsBase&>(a));
+}
+
+// H2O with the score update in the launch.  Returns cudaErrorNotSupported where the second launch
+// (decode_combine_kernel, h2o_update_warp_kernel) is needed: a piece's logits do not fit.
+// Measured, us per token, second launch / this form: 32 layers of 32 / 32 heads of 128, one launch per layer,
+// 1 sequence 432 / 281, 8: 615 / 485, 40: 775 / 755; all layers in one launch, 8 sequences: 176 / 171; fp32, 12
+// layers of 16 / 4 heads, 8 sequences: 331 / 271.
+template <typename T, int D>
+static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
+  const int G = a.group;
+  if (G > 32) return cudaErrorNotSupported;
+  constexpr int kSm = 148;
+  const long long units = (long long)a.n_layer_total * a.n_unit;
+  // few units: 16 warps each (two such CTAs per SM); else 4 warps, eight CTAs per SM
+  const bool wide = G == 1 && units <= 2 * kSm;
+  const long long slots = G == 1 && !wide ? 8 * kSm : 2 * kSm;
+  int pieces = (int)std::min<long long>(kMaxPieces, std::max<long long>(1, slots / units));
+  pieces = std::min(pieces, std::max(1, max_len / (wide ? 256 : 128)));
+  const size_t limit = (wide || G > 1) ? kScoresLimit : 24 * 1024;
+  auto bytes = [&](int p) { return (((size_t)piece_slots(max_len, p) * G + 3) / 4 * 4 + (size_t)G * (D + 4)) * 4; };
+  while (pieces < kMaxPieces && bytes(pieces) > limit) ++pieces;
+  const size_t smem = bytes(pieces);
+  if (smem > limit) return cudaErrorNotSupported;
+  const int n_cta = (int)(units * pieces);
+  if (wide) return launch_scores_kernel<decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16, true>>(a, pieces, n_cta, 512, smem, s);
+  if (G == 1) return launch_scores_kernel<decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
+  if (G <= 4) return launch_scores_kernel<decode_attn_kernel<T, D, 4, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
+  return launch_scores_kernel<decode_attn_kernel<T, D, 8, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
+}
+
 // Which attention kernel serves a shape: wide bf16 groups at head_dim 64 go to the tcgen05
 // kernel, other grouped bf16 heads to the mma.sync kernel, everything else (fp32, one query head
 // per KV head, shapes those do not cover) to the fp32-pipe kernel.
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
-                          size_t q_rows, const int* desc_tiles, cudaStream_t s) {
+                          size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
   bool done = false;
   if (dtype == SQ_BF16 && a.group > 32) {
@@ -506,6 +575,13 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need
   // every other kernel needs the per-slot logits for H2O: a context sized for the tcgen05 pair
   // does not hold them, and nothing may fall back silently
   if (!done && a.policy == SQ_POLICY_H2O && !a.has_logits) return cudaErrorNotSupported;
+  if (!done && a.policy == SQ_POLICY_H2O) {
+    cudaError_t e;
+    if (dtype == SQ_BF16 && a.group > 1) e = launch_decode_mma_scores(a, max_len, s);
+    else if (dtype == SQ_F32) e = a.head_dim == 64 ? launch_attn_scores<float, 64>(a, max_len, s) : launch_attn_scores<float, 128>(a, max_len, s);
+    else e = a.head_dim == 64 ? launch_attn_scores<__nv_bfloat16, 64>(a, max_len, s) : launch_attn_scores<__nv_bfloat16, 128>(a, max_len, s);
+    if (e != cudaErrorNotSupported) return e;
+  }
   if (!done && dtype == SQ_BF16 && a.group > 1) {
     cudaError_t e = launch_decode_attn_mma(a, n_items, s);
     if (e == cudaSuccess) done = true;

@@ -115,7 +115,7 @@ __global__ void __launch_bounds__(64 + 128 * SETS, CTAS)
   // one it is: a unit's victim is replaced by this kernel, after the unit's last piece has read it here.)
   int issued = 0;
   if (tid == 0) {
-    const int w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
+    const int w = (a.n_tok < b) ? a.n_tok : __ldcg(reinterpret_cast<const int*>(a.pool + ldp->victim_off) + unit);
     const int n_pre = min(min(STAGES, n_tiles), (w >= t0 && w < t1) ? (w - t0) / kTM : STAGES);
     for (; issued < n_pre; ++issued) load_tile(issued);
   }

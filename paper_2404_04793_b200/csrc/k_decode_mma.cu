@@ -8,15 +8,23 @@
 // K/V tiles of 64 tokens stream through a multi-stage cp.async pipeline (16-byte copies,
 // XOR-swizzled rows so ldmatrix is bank-conflict free).  Warps split the tile's tokens (WN)
 // and, for very wide groups, the head tiles (WM); partial results merge through shared memory.
+#include <algorithm>
+
 #include "sq_decode_common.cuh"
 #include "sq_device.cuh"
 #include "sq_internal.h"
+#include "sq_scores.cuh"
 
 namespace sq {
 
 namespace {
 
 constexpr int kTile = 64;  // tokens per pipeline stage
+constexpr int kScoresSmem = 110 * 1024;  // dynamic shared memory of a CTA with the score update: two CTAs per SM
+// tiles of a piece when a unit of `len` slots is cut into `pieces`
+__host__ __device__ inline int piece_tiles(int len, int pieces) {
+  return ((len + kTile - 1) / kTile + pieces - 1) / pieces;
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -65,8 +73,10 @@ __device__ __forceinline__ uint32_t swz(int row, int chunk) {
 
 }  // namespace
 
-template <int D, int MT, int WM, int WN, int STAGES>
-__global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArgs a) {
+// SCORES: H2O with the score update in the same launch (sq_scores.cuh): the pieces of a unit are the
+// CTAs of a cluster, piece_tiles(len) tiles each, and the logits stay in shared memory.
+template <int D, int MT, int WM, int WN, int STAGES, bool SCORES, class Args>
+__global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(Args a) {
   constexpr int NT = 32 * WM * WN;
   constexpr int CH = D / 8;            // 16-byte chunks per row
   constexpr int KS = D / 16;           // k-steps of Q K^T / pairs of output n-blocks
@@ -76,24 +86,45 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
   static_assert(kTile / WN == 16, "each warp owns 16 tokens of a tile");
   using bf16 = __nv_bfloat16;
   extern __shared__ __align__(128) unsigned char smem[];
-  unsigned char* q_s = smem;
-  unsigned char* k_s = smem + QROWS * D * 2;
+  // Q is read into registers before the last stage is filled for the first time: with SCORES, which
+  // needs the room, it starts out there
+  static_assert(!SCORES || QROWS * D * 2 <= TILE_BYTES, "Q in a stage");
+  unsigned char* k_s = smem + (SCORES ? 0 : QROWS * D * 2);
   unsigned char* v_s = k_s + STAGES * TILE_BYTES;
+  unsigned char* q_s = SCORES ? k_s + (STAGES - 1) * TILE_BYTES : smem;
 
   ItemLoc it;
-  if (!locate(a, blockIdx.x, it)) return;
+  int split;
+  if constexpr (SCORES) {
+    const int c = cluster_size(), item = blockIdx.x / c;
+    const int k = item / a.n_unit;
+    it.layer = a.order[k];
+    it.n_split = 1;
+    it.base = 0;
+    it.local = item - k * a.n_unit;
+    split = cluster_rank();
+  } else {
+    if (!locate(a, blockIdx.x, it)) return;
+  }
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int wm = warp / WN, wn = warp % WN;
   const int gq = lane >> 2, tq = lane & 3;
   const LayerDesc* ldp = a.layers + it.layer;
   const int b = ldp->b, cap = ldp->cap, G = a.group;
-  const int unit = it.local / it.n_split, split = it.local - unit * it.n_split;
+  const int unit = it.local / it.n_split;
   const int len = min(a.n_tok + 1, b);
-  const bool h2o = (a.policy == SQ_POLICY_H2O);
+  const bool h2o = SCORES || (a.policy == SQ_POLICY_H2O);
+  int piece_tokens;
+  if constexpr (SCORES) {
+    piece_tokens = piece_tiles(len, cluster_size()) * kTile;
+  } else {
+    split = it.local - unit * it.n_split;
+    piece_tokens = a.split_tokens;
+  }
   if (!a.early) grid_wait();
   int w;
   if (h2o) {
-    w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
+    w = (a.n_tok < b) ? a.n_tok : __ldcg(reinterpret_cast<const int*>(a.pool + ldp->victim_off) + unit);
     if (w < 0 || w >= b) {
       if (tid == 0) atomicOr(a.status, 2);
       w = 0;
@@ -101,7 +132,7 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
   } else {
     w = ring_slot(a.n_tok, b, ldp->ring_base, ldp->ring_origin);
   }
-  const int t0 = split * a.split_tokens, t1 = min(len, t0 + a.split_tokens);
+  const int t0 = split * piece_tokens, t1 = min(len, t0 + piece_tokens);  // (a piece may be empty under SCORES)
   const int seq = unit / a.n_kv_head, kvh = unit - seq * a.n_kv_head;
   const size_t tok = (size_t)(it.layer - a.layer_begin) * a.batch + seq;
   bf16* Kb = reinterpret_cast<bf16*>(a.pool + ldp->k_off) + (size_t)unit * cap * D;
@@ -110,8 +141,10 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
   const bf16* kn = reinterpret_cast<const bf16*>(a.k_new) + (tok * a.n_kv_head + kvh) * D;
   const bf16* vn = reinterpret_cast<const bf16*>(a.v_new) + (tok * a.n_kv_head + kvh) * D;
   bf16* ob = reinterpret_cast<bf16*>(a.out) + (tok * a.n_q_head + (size_t)kvh * G) * D;
-  float* logit = a.logits + ldp->logit_off + (size_t)unit * cap * G;
-  float* stat = a.part_stat + (size_t)blockIdx.x * G * kStatStride;
+  float* logit;  // [token][G]
+  if constexpr (SCORES) logit = reinterpret_cast<float*>(smem + 2 * STAGES * TILE_BYTES) - (size_t)t0 * G;
+  else logit = a.logits + ldp->logit_off + (size_t)unit * cap * G;
+  float* stat = a.part_stat + (size_t)blockIdx.x * G * kStatStride;  // (unused under SCORES)
   float* po = a.part_o + (size_t)blockIdx.x * G * D;
 
   const int n_tiles = (t1 - t0 + kTile - 1) / kTile;
@@ -349,6 +382,29 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(DecodeArg
     }
     __syncthreads();
   }
+  if constexpr (SCORES) {
+    // the piece's partial in shared memory, past the merge area
+    static_assert(WM == 1, "one row of warps");
+    __shared__ ScoreShared sh;
+    float* part_o = reinterpret_cast<float*>(v_s);
+    float* part_stat = part_o + MT * 16 * D;
+    static_assert(MT * 16 * (D + 4) * 4 <= STAGES * TILE_BYTES, "partial area");
+    if (wn == 0) {
+#pragma unroll
+      for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          const int h = mt * 16 + hf * 8 + gq;
+          if (h >= G) continue;
+#pragma unroll
+          for (int nb = 0; nb < NB; ++nb)
+            *reinterpret_cast<float2*>(part_o + h * D + nb * 8 + 2 * tq) = make_float2(o[mt][nb][hf * 2], o[mt][nb][hf * 2 + 1]);
+          if (tq == 0) *reinterpret_cast<float4*>(part_stat + h * 4) = make_float4(m_run[mt][hf], l_true[mt][hf], l_w[mt][hf], 0.f);
+        }
+    }
+    finish_scores<bf16, D, NT>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * G, part_o, part_stat, sh);
+    return;
+  }
   if (wn == 0) {
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
@@ -385,7 +441,7 @@ static cudaError_t launch_cfg(const DecodeArgs& a, int n_items, cudaStream_t s) 
   constexpr size_t merge = (size_t)WM * (WN / 2) * MT * 16 * (D + 4) * 4;
   static_assert(merge <= pipe, "the merge area reuses the pipeline stages");
   constexpr size_t smem = (size_t)QROWS * D * 2 + pipe;
-  auto kern = decode_attn_mma_kernel<D, MT, WM, WN, STAGES>;
+  auto kern = decode_attn_mma_kernel<D, MT, WM, WN, STAGES, false, DecodeArgs>;
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -395,6 +451,55 @@ static cudaError_t launch_cfg(const DecodeArgs& a, int n_items, cudaStream_t s) 
   return launch_chained(kern, n_items, 32 * WM * WN, smem, s, a);
 }
 
+static int sm_count() {
+  static int n_sm = 0;
+  if (n_sm == 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      n_sm = 148;
+  }
+  return n_sm;
+}
+
+template <int D, int MT, int STAGES>
+static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t logit_bytes, cudaStream_t s) {
+  const size_t smem = (size_t)2 * STAGES * kTile * D * 2 + logit_bytes;
+  auto kern = decode_attn_mma_kernel<D, MT, 1, 4, STAGES, true, DecodeArgsBase>;
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresSmem);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  return launch_chained_cluster(kern, pieces, a.n_layer_total * a.n_unit * pieces, 128, smem, s, static_cast<const DecodeArgsBase&>(a));
+}
+
+// H2O with the score update in the launch.  max_len: slots of the longest unit.  Returns
+// cudaErrorNotSupported where the second launch (decode_combine_kernel, h2o_update_warp_kernel) is the
+// better form or the logits of a piece do not fit.
+// Pieces: as many as leave all CTAs resident at once (two per SM), two tiles or more each.  Measured, us per
+// token of 32 layers of 32 / 8 heads of 128, one launch per layer, second launch / this form: 1 sequence
+// 385 / 281, 4: 451 / 391, 16: 660 / 533 (four pieces per unit, more than fit at once: 629), 64: 1060 / 983;
+// 20 / 1 heads of 64, 64 sequences: 435 / 239.  All 32 layers in one launch, 4096 units: 322 / 446.
+cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
+  const int G = a.group;
+  if (G < 2 || G > 32 || (a.head_dim != 64 && a.head_dim != 128)) return cudaErrorNotSupported;
+  const int n_sm = sm_count();
+  const long long units = (long long)a.n_layer_total * a.n_unit;
+  if (units >= 6 * n_sm) return cudaErrorNotSupported;
+  const int tiles = (max_len + kTile - 1) / kTile;
+  int pieces = (int)std::min<long long>(kMaxPieces, std::max<long long>(1, 2 * n_sm / units));
+  pieces = std::min(pieces, std::max(1, tiles / 2));
+  const int stages = a.head_dim == 128 ? 3 : 4;
+  const size_t fixed = (size_t)2 * stages * kTile * a.head_dim * 2;
+  auto logit_bytes = [&](int p) { return (size_t)piece_tiles(max_len, p) * kTile * G * 4; };
+  while (pieces < kMaxPieces && fixed + logit_bytes(pieces) > kScoresSmem) ++pieces;
+  const size_t lb = logit_bytes(pieces);
+  if (fixed + lb > kScoresSmem) return cudaErrorNotSupported;
+  if (a.head_dim == 128) return G <= 16 ? launch_scores_cfg<128, 1, 3>(a, pieces, lb, s) : launch_scores_cfg<128, 2, 3>(a, pieces, lb, s);
+  return G <= 16 ? launch_scores_cfg<64, 1, 4>(a, pieces, lb, s) : launch_scores_cfg<64, 2, 4>(a, pieces, lb, s);
+}
+
 // Returns cudaErrorNotSupported when no tensor-core configuration covers the shape.
 cudaError_t launch_decode_attn_mma(const DecodeArgs& a, int n_items, cudaStream_t s) {
   const int G = a.group;
@@ -402,13 +507,7 @@ cudaError_t launch_decode_attn_mma(const DecodeArgs& a, int n_items, cudaStream_
     // Two stages of 32 KB let three CTAs share an SM, which wins once the launch has CTAs to
     // spare (measured: Mistral- and Llama-2-70B-shaped fused steps 5-9 % faster); a launch of
     // about one wave (one layer at a time) is better off with the deeper ring per CTA.
-    static int n_sm = 0;
-    if (n_sm == 0) {
-      int dev = 0;
-      if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        n_sm = 148;
-    }
-    const bool many = n_items >= 6 * n_sm;
+    const bool many = n_items >= 6 * sm_count();
     if (G <= 16) return many ? launch_cfg<128, 1, 1, 4, 2>(a, n_items, s) : launch_cfg<128, 1, 1, 4, 3>(a, n_items, s);
     if (G <= 32) return many ? launch_cfg<128, 2, 1, 4, 2>(a, n_items, s) : launch_cfg<128, 2, 1, 4, 3>(a, n_items, s);
   } else if (a.head_dim == 64) {

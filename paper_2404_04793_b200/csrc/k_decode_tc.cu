@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(192, 2)
   if (!a.early) grid_wait();
   int w;
   if (H2O) {
-    w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
+    w = (a.n_tok < b) ? a.n_tok : __ldcg(reinterpret_cast<const int*>(a.pool + ldp->victim_off) + unit);
     if (w < 0 || w >= b) {
       if (tid == 0) atomicOr(a.status, 2);
       w = 0;

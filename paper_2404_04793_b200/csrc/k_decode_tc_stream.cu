@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
       // the slot the new token takes: the next free one while the cache grows, else the policy's victim
       int w;
       if (H2O) {
-        w = (a.n_tok < b) ? a.n_tok : reinterpret_cast<const int*>(a.pool + ldp->victim_off)[unit];
+        w = (a.n_tok < b) ? a.n_tok : __ldcg(reinterpret_cast<const int*>(a.pool + ldp->victim_off) + unit);
         if (w < 0 || w >= b) {
           if (lane == 0) atomicOr(a.status, 2);
           w = 0;

@@ -666,7 +666,7 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
     for (int k = 0; k < d1 - d0; ++k)
       desc_tiles[k] = (std::min(n_tok + 1, c->hs.layers[order_host[k]].b) + 127) / 128;
     SQ_CUDA(c, launch_decode(a, cfg.dtype, (int)n_items, combine, c->pool_bytes,
-                             (size_t)(e - s) * c->batch * cfg.n_q_head, desc_tiles.data(), st));
+                             (size_t)(e - s) * c->batch * cfg.n_q_head, desc_tiles.data(), max_len, st));
     for (int l = s; l < e; ++l) c->n_tok[l] += 1;
     s = e;
   }

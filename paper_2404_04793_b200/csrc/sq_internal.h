@@ -136,18 +136,26 @@ struct EvictArgs {
 // 128, H2O: 1 sequence 580 / 388 us, 16 sequences 825 / 661 us; 32 / 32 heads, 8 sequences 552 / 474 us; 80 layers,
 // 64 / 8 heads, 32 sequences 2651 / 2397 us; 71 / 1 heads of 64, 33 sequences, H2O 1507 / 1331 us.
 template <typename... P, typename... A>
-inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+inline cudaError_t launch_chained_cluster(void (*kern)(P...), int cluster, dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                          A&&... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = 1;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  return launch_chained_cluster(kern, 1, grid, block, smem, s, std::forward<A>(args)...);
 }
 
 // Launchers: each returns the cudaError_t of its launches.
@@ -161,14 +169,15 @@ cudaError_t launch_select_prompt(const float* acc_prompt, int n_unit, int prompt
                                  int units_per_desc, char* pool, cudaStream_t s);
 cudaError_t launch_pick_victim(char* pool, const LayerDesc* descs, int units_per_desc, int n_unit, int prompt,
                                int next_pos, cudaStream_t s);
-// desc_tiles: per descriptor of the launch (launch order) the 128-token tiles of one unit
+// desc_tiles: per descriptor of the launch (launch order) the 128-token tiles of one unit; max_len: slots of the longest unit
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
-                          size_t q_rows, const int* desc_tiles, cudaStream_t s);
+                          size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s);
 cudaError_t launch_decode_attn_tc(const DecodeArgs& a, int n_items, size_t pool_bytes, size_t q_rows, cudaStream_t s);
 cudaError_t launch_decode_attn_tc_stream(const DecodeArgs& a, const int* desc_tiles, size_t pool_bytes, size_t q_rows,
                                          cudaStream_t s);
 cudaError_t launch_h2o_gain_tc(const DecodeArgs& a, int n_items, size_t pool_bytes, size_t q_rows, cudaStream_t s);
 cudaError_t launch_decode_attn_mma(const DecodeArgs& a, int n_items, cudaStream_t s);
+cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStream_t s);
 cudaError_t launch_evict(const EvictArgs& a, cudaStream_t s);
 
 }  // namespace sq

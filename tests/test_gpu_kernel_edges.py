@@ -94,3 +94,44 @@ def test_layer_by_layer_launches_match_the_whole_stack(policy, dtype, head_dim, 
             kb, vb = chained.get_kv(l, 1, h)
             assert torch.equal(ka, kb) and torch.equal(va, vb)
     assert stack.status() == 0 and chained.status() == 0
+
+
+# H2O with the score update inside the attention launch: pieces of a unit on the CTAs of a cluster, with
+# empty and ragged pieces, short and long layers, groups that are and are not multiples of four, both
+# head dims, and units too long or too many for it
+@pytest.mark.parametrize("dtype,head_dim,hq,hkv,batch,budgets", [
+    (torch.bfloat16, 128, 8, 2, 1, [1100, 70]), (torch.bfloat16, 128, 5, 1, 2, [129, 2000]), (torch.bfloat16, 64, 32, 1, 1, [513, 64]),
+    (torch.bfloat16, 128, 24, 1, 3, [700, 1]), (torch.bfloat16, 64, 6, 3, 50, [300, 290]), (torch.float32, 64, 3, 1, 1, [1400, 33]),
+    (torch.float32, 128, 16, 2, 2, [400, 31]), (torch.bfloat16, 128, 3, 3, 2, [900, 260]), (torch.bfloat16, 64, 4, 4, 40, [200, 333]),
+    (torch.bfloat16, 128, 31, 1, 1, [9000, 50])])
+def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, budgets):
+    w = workload("fused", 9300 + budgets[0], dtype=dtype, head_dim=head_dim, n_q_head=hq, n_kv_head=hkv, n_layer=len(budgets),
+                 batch=batch, prompt=max(budgets) + 5, steps=3, heavy_mode="zipf")
+    ctx = H.make_ctx(w, b_init=max(budgets))
+    ctx.begin_sequence_batch(batch, w.prompt)
+    ctx.set_budgets(budgets)
+    g = w.group
+    units = {(l, s, h) for l in range(w.n_layer) for s in (0, batch - 1) for h in (0, hkv - 1)}
+    for l in range(w.n_layer):
+        _, k, v = synth.prompt_qkv(w, l, DEV, need_q=False)
+        ctx.prefill_compress(l, k, v, None, synth.prompt_scores_standin(w, l, DEV))
+    for t in range(w.steps):
+        q, kn, vn = synth.decode_qkv(w, t, DEV)
+        out = torch.empty_like(q)
+        # the oracle takes the library's rows and scores before the step: one step's arithmetic is compared
+        before = {u: (ctx.get_kept(*u), ctx.get_kv(*u)) for u in units}
+        for l in range(w.n_layer):
+            ctx.decode_step(l, l + 1, q[l], kn[l], vn[l], out[l])
+        for (l, s, h), ((pos, acc), (kk, vv)) in before.items():
+            u = O.UnitCache(w.policy, budgets[l], w.n_sink, w.heavy_num, w.heavy_den)
+            u.pos, u.acc, u.K, u.V = list(pos), [float(x) for x in acc], list(H.f64(kk)), list(H.f64(vv))
+            u.next_pos = w.prompt + t
+            want = u.decode_step(H.f64(q[l, s, h * g:(h + 1) * g]), H.f64(kn[l, s, h]), H.f64(vn[l, s, h]))
+            got = H.f64(out[l, s, h * g:(h + 1) * g])
+            # outputs beyond 1 meet the bf16 formats: half an ulp of the output, 2^-9 of the weights
+            bound = np.maximum(H.TOL_OUT[dtype], np.abs(want) * (2.0 ** -7 if dtype == torch.bfloat16 else 0))
+            assert np.all(np.abs(got - want) <= bound)
+            pos2, acc2 = ctx.get_kept(l, s, h)
+            assert pos2 == u.kept_positions()
+            np.testing.assert_allclose(acc2, u.acc, rtol=H.RTOL_ACC[dtype], atol=1e-6)
+    assert ctx.status() == 0
