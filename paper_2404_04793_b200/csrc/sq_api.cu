@@ -508,7 +508,7 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
       acc = s.acc_prompt;
     }
   }
-  // selection, gather and first victim: one launch each over all descriptors of the layer
+  // selection (with the first victim) and gather: one launch each over all descriptors of the layer
   const LayerDesc* descs_dev = ws_ptr<LayerDesc>(c, c->wl.layers) + layer * c->n_grp;
   const int n_unit = c->batch * c->cfg.n_kv_head;
   int max_keep = 0;
@@ -518,11 +518,10 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
     max_keep = std::max(max_keep, std::min(P, ld.b));
     any_full |= P >= ld.b;
   }
-  if (h2o) SQ_CUDA(c, launch_select_prompt(acc, n_unit, P, descs_dev, U, c->pool, st));
+  if (h2o) SQ_CUDA(c, launch_select_prompt(acc, n_unit, P, descs_dev, U, any_full, c->pool, st));
   GatherArgs ga;
   ga.k_prompt = k_prompt;
   ga.v_prompt = v_prompt;
-  ga.acc_prompt = acc;
   ga.pool = c->pool;
   ga.descs = descs_dev;
   ga.units_per_desc = U;
@@ -532,7 +531,6 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
   ga.policy = c->cfg.policy;
   ga.head_dim = c->cfg.head_dim;
   SQ_CUDA(c, launch_gather(ga, c->cfg.dtype, st));
-  if (h2o && any_full) SQ_CUDA(c, launch_pick_victim(c->pool, descs_dev, U, n_unit, P, P, st));
   c->n_tok[layer] = P;
   c->prefilled[layer] = true;
   return SQ_OK;

@@ -58,7 +58,6 @@ struct AllocateArgs {  // entry of layer i: [i * stride + blockIdx.x] (one CTA p
 struct GatherArgs {  // prompt rows -> cache slots of one layer (all its descriptors in one launch)
   const void* k_prompt;
   const void* v_prompt;
-  const float* acc_prompt;  // H2O, else null
   char* pool;
   const LayerDesc* descs;   // the layer's descriptors (device); unit u belongs to descs[u / units_per_desc]
   int units_per_desc;
@@ -166,9 +165,7 @@ cudaError_t launch_prefill_scores(const ScoreArgs& a, int dtype, int* status, cu
 cudaError_t launch_prefill_scores_alu(const ScoreArgs& a, int dtype, cudaStream_t s);
 cudaError_t launch_prefill_scores_tc(const ScoreArgs& a, int* status, cudaStream_t s);
 cudaError_t launch_select_prompt(const float* acc_prompt, int n_unit, int prompt, const LayerDesc* descs,
-                                 int units_per_desc, char* pool, cudaStream_t s);
-cudaError_t launch_pick_victim(char* pool, const LayerDesc* descs, int units_per_desc, int n_unit, int prompt,
-                               int next_pos, cudaStream_t s);
+                                 int units_per_desc, bool any_full, char* pool, cudaStream_t s);
 // desc_tiles: per descriptor of the launch (launch order) the 128-token tiles of one unit; max_len: slots of the longest unit
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
                           size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s);

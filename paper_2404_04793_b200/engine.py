@@ -154,10 +154,10 @@ class Job:
         w = self.w
         per_layer = self.per_layer_decode if per_layer_decode is None else per_layer_decode
         h2o = w.policy == synth.H2O
-        # H2O: two scoring sweeps (unless stand-in scores are given), selection, gather, first victim
-        per_layer_prefill = ((0 if inp.acc is not None else 2) + 1 + 1 + 1) if h2o else 1
+        # H2O: two scoring sweeps (unless stand-in scores are given), selection, gather
+        per_layer_prefill = ((0 if inp.acc is not None else 2) + 1 + 1) if h2o else 1
         groups = w.n_layer if per_layer else 1
-        per_step = groups * (2 if h2o else 1)
+        per_step = groups * (2 if h2o and w.group > 32 else 1)   # at least: H2O launches of many units take two as well
         return w.n_layer * inp.hidden_repeat + 1 + w.n_layer * per_layer_prefill + w.steps * per_step
 
     # ---- the same pass fed from page-locked host memory ----

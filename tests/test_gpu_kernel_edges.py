@@ -135,3 +135,45 @@ def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, bud
             assert pos2 == u.kept_positions()
             np.testing.assert_allclose(acc2, u.acc, rtol=H.RTOL_ACC[dtype], atol=1e-6)
     assert ctx.status() == 0
+
+
+# Selection over the prompt: block sizes by prompt length and the form for longer prompts, ties across the
+# threshold, equal scores everywhere, negative scores, all slots heavy but one, none heavy, budgets around the
+# prompt; the first victim shows in which token the first append replaces
+@pytest.mark.parametrize("prompt", [1, 2, 37, 1024, 1025, 4096, 4097, 9000, 16384, 16385])
+@pytest.mark.parametrize("hn,hd", [(1, 2), (0, 1), (9, 10)])
+def test_prompt_selection_edges(prompt, hn, hd):
+    batch = 6
+    w = workload("select", 9400 + prompt, dtype=torch.bfloat16, head_dim=64, n_q_head=2, n_kv_head=1, n_layer=5, batch=batch,
+                 prompt=prompt, heavy_num=hn, heavy_den=hd, heavy_mode="none")
+    budgets = [max(1, prompt // 3), max(1, prompt - 1), prompt, prompt + 3, 1]
+    ctx = H.make_ctx(w, b_init=prompt + 3)
+    ctx.begin_sequence_batch(batch, prompt)
+    ctx.set_budgets(budgets)
+    g = torch.Generator().manual_seed(prompt)
+    acc = torch.rand(batch, 1, prompt, generator=g)
+    acc[1] = 1.5                                              # all equal
+    acc[2] = torch.randint(0, 3, (1, prompt), generator=g)    # a few values, zeros among them
+    acc[3] = torch.randn(1, prompt, generator=g)              # negative scores
+    acc[4] = torch.round(acc[4] * 64) * 2.0 ** -130           # subnormal
+    acc[5, :, : prompt // 2] = -0.0
+    _, k, v = synth.prompt_qkv(w, 0, DEV, need_q=False)
+    for l in range(w.n_layer):
+        ctx.prefill_compress(l, k, v, None, acc.to(DEV))
+    for l, b in enumerate(budgets):
+        for s in range(batch):
+            keep = list(range(prompt)) if prompt <= b else \
+                O.c_seq(w.policy, list(range(prompt)), acc[s, 0].double().tolist(), b, w.n_sink, hn, hd)
+            pos, got = ctx.get_kept(l, s, 0)
+            assert pos == keep, (l, s)
+            assert got == [float(acc[s, 0, p]) for p in keep]
+    rows = ctx.get_kv(1, 3, 0)[0]
+    assert torch.equal(rows, k[3, 0].cpu()[ctx.get_kept(1, 3, 0)[0]])
+    before = {(l, s): ctx.get_kept(l, s, 0) for l in range(w.n_layer) for s in range(batch)}
+    q, kn, vn = synth.decode_qkv(w, 0, DEV)
+    ctx.decode_step(0, w.n_layer, q, kn, vn, torch.empty_like(q))
+    for (l, s), (pos, sc) in before.items():
+        keep = O.c_seq(w.policy, pos + [prompt], sc + [0.0], budgets[l], w.n_sink, hn, hd) if len(pos) + 1 > budgets[l] else \
+            list(range(len(pos) + 1))
+        assert ctx.get_kept(l, s, 0)[0] == [(pos + [prompt])[i] for i in keep], (l, s)
+    assert ctx.status() == 0
