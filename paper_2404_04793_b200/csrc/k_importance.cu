@@ -1,5 +1,7 @@
 // Layer importance (Section 3 cosine-similarity equation; Algorithm 1, steps 1-4) and the
 // layer-wise budget allocator (Algorithm 1, steps 5-12; Appendix A.2).
+#include <algorithm>
+
 #include "sq_device.cuh"
 #include "sq_internal.h"
 
@@ -12,22 +14,35 @@ namespace sq {
 // FUSED: the rows are the residual stream (a) and the attention block's output (b); the kernel
 // writes their sum, rounded to T, to sum_out and takes the cosine between a and that sum, i.e.
 // between the hidden state before and after self-attention, in the pass that produces the latter.
+// Bound by HBM: what counts is bytes in flight.  Few warps with long batches of loads (kU 16-byte pieces
+// of each row per lane) keep more in flight per SM than many warps with short ones, and leave the
+// partial sums of fewer CTAs to add up at the end.  Measured, us per layer (TB/s) of 16384 tokens of 4096
+// bf16 elements (10006 of 4544), kU x CTAs per SM: two rows read: 4 x 8 (before) 48.4 (42.2), 4 x 6 46.1 (34.3),
+// 8 x 4 43.8 (33.5), 16 x 2 41.2 (36.2), 8 x 3 42.0 = 6.4 TB/s (31.1); fused (two read, one written): 4 x 8
+// started, 5 resident (before) 83.2 (58.5), 4 x 4 72.3 (53.3), 4 x 3 70.4 (49.7), 8 x 2 67.3 = 6.0 TB/s (52.2).
+template <bool FUSED>
+struct ImportanceCfg {
+  static constexpr int kU = 8;
+  static constexpr int kCtas = FUSED ? 2 : 3;  // per SM
+};
 template <typename T, bool FUSED>
-__global__ void __launch_bounds__(256) cos_sim_reduce_kernel(ImportanceArgs a) {
+__global__ void __launch_bounds__(256, ImportanceCfg<FUSED>::kCtas) cos_sim_reduce_kernel(ImportanceArgs a) {
   constexpr int EPV = Elem<T>::kPerVec;
   const int nvec = a.hidden / EPV;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long n_warp = (long long)gridDim.x * 8;
   float wsum = 0.f;
+  grid_wait();
   for (long long row = (long long)blockIdx.x * 8 + warp; row < a.n_tok; row += n_warp) {
     const uint4* pa = reinterpret_cast<const uint4*>(a.a) + row * nvec;
     const uint4* pb = reinterpret_cast<const uint4*>(a.b) + row * nvec;
     uint4* po = FUSED ? reinterpret_cast<uint4*>(a.sum_out) + row * nvec : nullptr;
     float dot = 0.f, na = 0.f, nb = 0.f;
-    for (int v0 = lane; v0 < nvec; v0 += 128) {
-      uint4 va[4], vb[4];
+    constexpr int U = ImportanceCfg<FUSED>::kU;
+    for (int v0 = lane; v0 < nvec; v0 += 32 * U) {
+      uint4 va[U], vb[U];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < U; ++u) {
         int v = v0 + 32 * u;
         if (v < nvec) {
           va[u] = ld_stream(pa + v);
@@ -38,7 +53,7 @@ __global__ void __launch_bounds__(256) cos_sim_reduce_kernel(ImportanceArgs a) {
         }
       }
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
+      for (int u = 0; u < U; ++u) {
         float fa[EPV], fb[EPV];
         widen<T>(va[u], fa);
         widen<T>(vb[u], fb);
@@ -79,28 +94,33 @@ __global__ void __launch_bounds__(256) cos_sim_reduce_kernel(ImportanceArgs a) {
     s_last = (t == gridDim.x - 1);
   }
   __syncthreads();
-  if (s_last && warp == 0) {
+  if (s_last) {
     __threadfence();
+    __shared__ double s_acc[8];
     double acc = 0.0;
-    for (int i = lane; i < (int)gridDim.x; i += 32) acc += (double)__ldcg(a.cta_partial + i);
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) acc += (double)__ldcg(a.cta_partial + i);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) {
+    if (lane == 0) s_acc[warp] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int i = 1; i < 8; ++i) acc += s_acc[i];
       *a.cos_sum += acc;
       *a.ticket = 0u;
     }
   }
 }
 
-cudaError_t launch_importance(const ImportanceArgs& a, int dtype, int n_cta, cudaStream_t s) {
+cudaError_t launch_importance(const ImportanceArgs& a, int dtype, int n_sm, cudaStream_t s) {
+  // all CTAs resident at once; at most kMaxImportanceCtas partial sums
+  const long long slots = std::min<long long>(kMaxImportanceCtas, (long long)n_sm * (a.sum_out ? ImportanceCfg<true>::kCtas : ImportanceCfg<false>::kCtas));
+  const int n_cta = (int)std::min<long long>((a.n_tok + 7) / 8, slots);
   if (a.sum_out) {
-    if (dtype == SQ_F32) cos_sim_reduce_kernel<float, true><<<n_cta, 256, 0, s>>>(a);
-    else cos_sim_reduce_kernel<__nv_bfloat16, true><<<n_cta, 256, 0, s>>>(a);
-  } else {
-    if (dtype == SQ_F32) cos_sim_reduce_kernel<float, false><<<n_cta, 256, 0, s>>>(a);
-    else cos_sim_reduce_kernel<__nv_bfloat16, false><<<n_cta, 256, 0, s>>>(a);
+    if (dtype == SQ_F32) return launch_chained(cos_sim_reduce_kernel<float, true>, n_cta, 256, 0, s, a);
+    return launch_chained(cos_sim_reduce_kernel<__nv_bfloat16, true>, n_cta, 256, 0, s, a);
   }
-  return cudaGetLastError();
+  if (dtype == SQ_F32) return launch_chained(cos_sim_reduce_kernel<float, false>, n_cta, 256, 0, s, a);
+  return launch_chained(cos_sim_reduce_kernel<__nv_bfloat16, false>, n_cta, 256, 0, s, a);
 }
 
 // ---------------------------------------------------------------------------------------

@@ -18,7 +18,6 @@ namespace {
 constexpr size_t kAlign = 256;
 inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 inline int elem_bytes(int dtype) { return dtype == SQ_F32 ? 4 : 2; }
-constexpr int kMaxImportanceCtas = 4096;
 
 struct WsLayout {
   size_t cos_sum, tok_count, cta_partial, ticket, cos_sim, budget, is_g3, status, tickets, score_tickets, layers, order, order_by_layer,
@@ -393,9 +392,7 @@ static int importance_rows(sq_ctx* c, int32_t layer, const void* row_a, const vo
     a.cta_partial = ws_ptr<float>(c, c->wl.cta_partial);
     a.ticket = ws_ptr<unsigned int>(c, c->wl.ticket);
     a.cos_sum = ws_ptr<double>(c, c->wl.cos_sum) + d;
-    long long want = (n + 7) / 8;
-    int n_cta = (int)std::min<long long>(want, std::min(kMaxImportanceCtas, c->n_sm * 8));
-    SQ_CUDA(c, launch_importance(a, c->cfg.dtype, n_cta, static_cast<cudaStream_t>(stream)));
+    SQ_CUDA(c, launch_importance(a, c->cfg.dtype, c->n_sm, static_cast<cudaStream_t>(stream)));
     c->hs.tok_count[d] += n;
     done += n;
   }

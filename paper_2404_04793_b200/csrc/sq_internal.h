@@ -11,6 +11,7 @@
 namespace sq {
 
 constexpr int kMaxLayers = 256;
+constexpr int kMaxImportanceCtas = 4096;  // partial sums of one importance launch
 constexpr int kMaxGroup = 128;          // query heads per KV head
 constexpr int kTargetItems = 148 * 16;  // room for split-K pieces beyond one per (layer, unit)
 
@@ -158,7 +159,7 @@ inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, siz
 }
 
 // Launchers: each returns the cudaError_t of its launches.
-cudaError_t launch_importance(const ImportanceArgs& a, int dtype, int n_cta, cudaStream_t s);
+cudaError_t launch_importance(const ImportanceArgs& a, int dtype, int n_sm, cudaStream_t s);
 cudaError_t launch_allocate(const AllocateArgs& a, cudaStream_t s);
 cudaError_t launch_gather(const GatherArgs& a, int dtype, cudaStream_t s);
 cudaError_t launch_prefill_scores(const ScoreArgs& a, int dtype, int* status, cudaStream_t s);
