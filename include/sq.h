@@ -24,7 +24,7 @@
  *     workspace (sizes from sq_query_sizes); both must stay valid until sq_ctx_destroy and
  *     must not be touched by the caller in between.  sq_ctx_create allocates one small block of
  *     page-locked HOST memory (staging of the budget and layout tables, a few KB per layer) and
- *     one CUDA event; sq_ctx_destroy frees them.
+ *     three CUDA events; sq_ctx_destroy waits for what still uses the block and frees them.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Work is
  *     enqueued on it and calls return without waiting, except the sq_get_* calls and
  *     sq_status, which synchronise the device, and the first call after sq_allocate_budgets
@@ -210,7 +210,7 @@ const char* sq_last_error(sq_ctx* ctx);
  * context with the same config and b_init, sq_begin_sequence_batch with the same batch and
  * prompt_len, then sq_ctx_import_layout with the exported table; decoding continues with the
  * next token as if it had not stopped.  Export synchronises the device; import is host work plus
- * small asynchronous copies on `stream` and one wait for them.  Import lays the pool out by the
+ * one small asynchronous copy on `stream`.  Import lays the pool out by the
  * table's capacities and returns SQ_ERR_INVALID_ARG, changing nothing the caller can decode
  * from, when the table's offsets are not the ones this context gives those capacities. */
 typedef struct sq_layer_layout {

@@ -143,54 +143,79 @@ __device__ double run_cost(const double* x, int lo, int hi) {
   return c;
 }
 
-__global__ void __launch_bounds__(256) allocate_budgets_kernel(AllocateArgs a) {
+constexpr int kAllocThreads = 1024;
+
+// Smallest (cost, id) over the block, id < 0 meaning none; the result is valid in thread 0.
+__device__ __forceinline__ int block_best(double cost, int id, double* s_cost, int* s_id) {
+  auto better = [](double c1, int i1, double c2, int i2) { return i1 >= 0 && (i2 < 0 || c1 < c2 || (c1 == c2 && i1 < i2)); };
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double c2 = __shfl_xor_sync(0xffffffffu, cost, o);
+    const int i2 = __shfl_xor_sync(0xffffffffu, id, o);
+    if (better(c2, i2, cost, id)) {
+      cost = c2;
+      id = i2;
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+    s_cost[threadIdx.x >> 5] = cost;
+    s_id[threadIdx.x >> 5] = id;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0)
+    for (int w = 1; w < kAllocThreads / 32; ++w)
+      if (better(s_cost[w], s_id[w], cost, id)) {
+        cost = s_cost[w];
+        id = s_id[w];
+      }
+  return id;
+}
+
+// Bound by latency (one chain of dependent fp64 additions per run of layers): one thread per cut, nothing
+// done by a single thread that the block can share.  32 layers: 22 us with 256 threads and serial ends.
+__global__ void __launch_bounds__(kAllocThreads) allocate_budgets_kernel(AllocateArgs a) {
   __shared__ double s_x[kMaxLayers];         // sorted values
-  __shared__ int s_idx[kMaxLayers];          // layer of each sorted value
+  __shared__ int s_rank[kMaxLayers];         // rank of each layer's value
   __shared__ double s_head[kMaxLayers + 1];  // cost of run [0, i)
   __shared__ double s_tail[kMaxLayers + 1];  // cost of run [i, n)
-  __shared__ double s_best_cost[256];
-  __shared__ int s_best_id[256];
-  __shared__ int s_k, s_cut;
+  __shared__ double s_best_cost[kAllocThreads / 32];
+  __shared__ int s_best_id[kAllocThreads / 32];
+  __shared__ int s_cut;
+  __shared__ unsigned s_rest[kMaxLayers / 32];  // per 32 layers: those outside G3
   const int n = a.n_layer, tid = threadIdx.x;
   const int st = a.stride, off = blockIdx.x;  // this CTA's budget vector: entries i * st + off
+  const long long cnt = tid < n ? a.tok_count[tid * st + off] : 0;
+  grid_wait();
 
   // layer averages, rounded to fp32 (the value reported to the caller), ranked by (value, layer)
-  for (int i = tid; i < n; i += blockDim.x) {
-    long long cnt = a.tok_count[i * st + off];
-    float c = cnt > 0 ? (float)(a.cos_sum[i * st + off] / (double)cnt) : 0.f;
-    a.cos_sim[i * st + off] = c;
-    s_head[i] = (double)c;  // scratch: unsorted values
+  if (tid < n) {
+    const float c = cnt > 0 ? (float)(a.cos_sum[tid * st + off] / (double)cnt) : 0.f;
+    a.cos_sim[tid * st + off] = c;
+    s_head[tid] = (double)c;  // scratch: unsorted values
   }
   __syncthreads();
-  for (int i = tid; i < n; i += blockDim.x) {
-    double v = s_head[i];
+  if (tid < n) {
+    const double v = s_head[tid];
     int r = 0;
     for (int j = 0; j < n; ++j) {
-      double w = s_head[j];
-      r += (w < v) || (w == v && j < i);
+      const double w = s_head[j];
+      r += (w < v) || (w == v && j < tid);
     }
     s_x[r] = v;
-    s_idx[r] = i;
+    s_rank[tid] = r;
   }
   __syncthreads();
-  if (tid == 0) {
-    int distinct = 1;
-    for (int i = 1; i < n; ++i) distinct += (s_x[i] != s_x[i - 1]);
-    s_k = min(a.n_cluster, distinct);
-    s_cut = n;  // G3 = sorted ranks [cut, n)
-  }
+  const int distinct = 1 + __syncthreads_count(tid >= 1 && tid < n && s_x[tid] != s_x[tid - 1]);
+  const int k = min(a.n_cluster, distinct);
+  // heads and tails on different warps: their chains run side by side
+  if (tid <= n) s_head[tid] = (tid > 0) ? run_cost(s_x, 0, tid) : 0.0;
+  else if (tid >= 512 && tid - 512 <= n) s_tail[tid - 512] = (tid - 512 < n) ? run_cost(s_x, tid - 512, n) : 0.0;
   __syncthreads();
-  for (int i = tid; i <= n; i += blockDim.x) {
-    s_head[i] = (i > 0) ? run_cost(s_x, 0, i) : 0.0;
-    s_tail[i] = (i < n) ? run_cost(s_x, i, n) : 0.0;
-  }
-  __syncthreads();
-  const int k = s_k;
   double best = 0.0;
   int best_id = -1;
   if (k == 2) {
-    for (int i = 1 + tid; i < n; i += blockDim.x) {
-      double c = __dadd_rn(s_head[i], s_tail[i]);
+    for (int i = 1 + tid; i < n; i += kAllocThreads) {
+      const double c = __dadd_rn(s_head[i], s_tail[i]);
       if (best_id < 0 || c < best) {
         best = c;
         best_id = i;
@@ -198,63 +223,47 @@ __global__ void __launch_bounds__(256) allocate_budgets_kernel(AllocateArgs a) {
     }
   } else if (k == 3) {
     // candidate id = i * n + j, visited in increasing id per thread
-    for (int id = tid; id < n * n; id += blockDim.x) {
-      int i = id / n, j = id - i * n;
+    for (int id = tid; id < n * n; id += kAllocThreads) {
+      const int i = id / n, j = id - i * n;
       if (i < 1 || i > n - 2 || j <= i || j > n - 1) continue;
-      double c = __dadd_rn(__dadd_rn(s_head[i], run_cost(s_x, i, j)), s_tail[j]);
+      const double c = __dadd_rn(__dadd_rn(s_head[i], run_cost(s_x, i, j)), s_tail[j]);
       if (best_id < 0 || c < best) {
         best = c;
         best_id = id;
       }
     }
   }
-  s_best_cost[tid] = best;
-  s_best_id[tid] = best_id;
+  const int bi = block_best(best, best_id, s_best_cost, s_best_id);
+  if (tid == 0) s_cut = bi < 0 ? n : (k == 2 ? bi : bi % n);  // G3 = sorted ranks [cut, n)
   __syncthreads();
-  if (tid == 0) {
-    double bc = 0.0;
-    int bi = -1;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      int id = s_best_id[t];
-      if (id < 0) continue;
-      double c = s_best_cost[t];
-      if (bi < 0 || c < bc || (c == bc && id < bi)) {
-        bc = c;
-        bi = id;
-      }
-    }
-    if (k == 2 && bi >= 0) s_cut = bi;
-    if (k == 3 && bi >= 0) s_cut = bi % n;
-    // budgets (Algorithm 1, steps 6-12): G3 gets floor(b_init*p), the rest share what is left
-    const int cut = s_cut;
-    const int n3 = n - cut;
-    for (int i = 0; i < n; ++i) {
-      a.is_g3[i * st + off] = 0;
-      a.budget[i * st + off] = (int)a.b_init;
-    }
-    if (n3 > 0 && n3 < n) {
-      for (int r = cut; r < n; ++r) a.is_g3[s_idx[r] * st + off] = 1;
-      long long b_low = (long long)floor(__dmul_rn((double)a.b_init, a.p));
-      if (b_low < 1) b_low = 1;
-      long long rest = (long long)n * a.b_init - (long long)n3 * b_low;
-      long long m = n - n3;
-      long long base = rest / m, extra = rest % m;
-      long long seen = 0;
-      for (int i = 0; i < n; ++i) {
-        if (a.is_g3[i * st + off]) {
-          a.budget[i * st + off] = (int)b_low;
-        } else {
-          a.budget[i * st + off] = (int)(base + (seen < extra ? 1 : 0));
-          ++seen;
-        }
-      }
+  // budgets (Algorithm 1, steps 6-12): G3 gets floor(b_init*p), the rest share what is left
+  const int n3 = n - s_cut;
+  const bool split = n3 > 0 && n3 < n;
+  const bool g3 = split && tid < n && s_rank[tid] >= s_cut;
+  const unsigned rest_here = __ballot_sync(0xffffffffu, tid < n && !g3);
+  if (tid < kMaxLayers && (tid & 31) == 0) s_rest[tid >> 5] = rest_here;
+  __syncthreads();
+  if (tid >= n) return;
+  long long b = a.b_init;
+  if (split) {
+    long long b_low = (long long)floor(__dmul_rn((double)a.b_init, a.p));
+    if (b_low < 1) b_low = 1;
+    if (g3) {
+      b = b_low;
+    } else {
+      const long long rest = (long long)n * a.b_init - (long long)n3 * b_low;
+      const long long m = n - n3, base = rest / m, extra = rest % m;
+      long long seen = __popc(rest_here & ((1u << (tid & 31)) - 1u));  // layers outside G3 before this one
+      for (int w = 0; w < (tid >> 5); ++w) seen += __popc(s_rest[w]);
+      b = base + (seen < extra ? 1 : 0);
     }
   }
+  a.is_g3[tid * st + off] = g3 ? 1 : 0;
+  a.budget[tid * st + off] = (int)b;
 }
 
 cudaError_t launch_allocate(const AllocateArgs& a, cudaStream_t s) {
-  allocate_budgets_kernel<<<a.stride, 256, 0, s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(allocate_budgets_kernel, a.stride, kAllocThreads, 0, s, a);
 }
 
 }  // namespace sq

@@ -20,25 +20,33 @@ inline size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 inline int elem_bytes(int dtype) { return dtype == SQ_F32 ? 4 : 2; }
 
 struct WsLayout {
-  size_t cos_sum, tok_count, cta_partial, ticket, cos_sim, budget, is_g3, status, tickets, score_tickets, layers, order, order_by_layer,
-      evict_tab;
+  size_t cos_sum, cta_partial, ticket, cos_sim, status, tickets, score_tickets, layers, order, order_by_layer,
+      evict_tab, tables_end;
   size_t part_stat, part_o, logits, acc_prompt, lse2, total;
   size_t items_cap, logits_floats, lse_floats, n_desc_cap;
 };
 
-// Pinned staging for the small host <-> device tables.  "desc" = one cache descriptor: a layer
-// of the whole batch, or with per-sequence budgets a (layer, sequence) pair; arrays hold
-// n_desc_cap entries, entry of (layer, group) = layer * n_grp + group.
+// Small host <-> device tables.  "desc" = one cache descriptor: a layer of the whole batch, or with
+// per-sequence budgets a (layer, sequence) pair; arrays hold n_desc_cap entries, entry of (layer,
+// group) = layer * n_grp + group.  The host works on its own copies; what a kernel reads or a copy
+// takes is staged in one of two page-locked slots, each free again once its event has passed, so that no
+// call waits for the copies of the one before it.
+constexpr int kSlots = 2;
 struct HostStage {
-  int32_t* budget;
-  uint8_t* is_g3;
-  float* cos_sim;
-  long long* tok_count;
-  LayerDesc* layers;
-  int* order;           // all descriptors, largest budget first
-  int* order_by_layer;  // per layer its descriptors, largest budget first
-  EvictLayer* evict_tab;
-  void* block;
+  std::vector<int32_t> budget;
+  std::vector<uint8_t> is_g3;
+  std::vector<long long> tok_count;
+  std::vector<LayerDesc> layers;
+  std::vector<int> order;           // all descriptors, largest budget first
+  std::vector<int> order_by_layer;  // per layer its descriptors, largest budget first
+  std::vector<EvictLayer> evict_tab;
+  // page-locked
+  char* block;
+  int32_t* budget_down;  // written by the allocator
+  uint8_t* is_g3_down;
+  char* slot[kSlots];    // image of the workspace from WsLayout::layers on, then tok_count
+  cudaEvent_t slot_ev[kSlots];
+  int next_slot;
 };
 
 }  // namespace
@@ -132,12 +140,9 @@ WsLayout ws_layout(const sq_config& c, int64_t b_init) {
     return o;
   };
   w.cos_sum = take(8 * ND);
-  w.tok_count = take(8 * ND);
   w.cta_partial = take(4 * (size_t)kMaxImportanceCtas);
   w.ticket = take(4);
   w.cos_sim = take(4 * ND);
-  w.budget = take(4 * ND);
-  w.is_g3 = take(ND);
   w.status = take(4);
   w.tickets = take(4 * L * U);
   w.score_tickets = take(c.policy == SQ_POLICY_H2O ? 4 * U * (((size_t)c.max_prompt + 127) / 128) : 0);
@@ -145,6 +150,7 @@ WsLayout ws_layout(const sq_config& c, int64_t b_init) {
   w.order = take(4 * ND);
   w.order_by_layer = take(4 * ND);
   w.evict_tab = take(sizeof(EvictLayer) * ND);
+  w.tables_end = off;
   w.items_cap = (size_t)kTargetItems + U * L;
   w.part_stat = take(w.items_cap * G * 4 * 4);
   w.part_o = take(w.items_cap * G * c.head_dim * 4);
@@ -180,10 +186,40 @@ void sort_orders(sq_ctx* c) {
   for (int d = 0; d < nd; ++d) ord[d] = d;
   auto by_budget = [&](int x, int y) { return c->hs.budget[x] > c->hs.budget[y]; };
   std::stable_sort(ord.begin(), ord.end(), by_budget);
-  std::copy(ord.begin(), ord.end(), c->hs.order);
+  std::copy(ord.begin(), ord.end(), c->hs.order.begin());
   for (int d = 0; d < nd; ++d) ord[d] = d;
   for (int l = 0; l < c->cfg.n_layer; ++l) std::stable_sort(ord.begin() + l * ng, ord.begin() + (l + 1) * ng, by_budget);
-  std::copy(ord.begin(), ord.end(), c->hs.order_by_layer);
+  std::copy(ord.begin(), ord.end(), c->hs.order_by_layer.begin());
+}
+
+// A staging slot whose last copies or kernel are done.
+int take_slot(sq_ctx* c, int* slot) {
+  *slot = c->hs.next_slot;
+  c->hs.next_slot = (*slot + 1) % kSlots;
+  SQ_CUDA(c, cudaEventSynchronize(c->hs.slot_ev[*slot]));
+  return SQ_OK;
+}
+
+// Uploads the descriptors and launch orders, and the first n_evict entries of the eviction table: one
+// copy over that part of the workspace.
+int upload_tables(sq_ctx* c, int n_evict, cudaStream_t st) {
+  int slot;
+  const int rc = take_slot(c, &slot);
+  if (rc != SQ_OK) return rc;
+  char* img = c->hs.slot[slot];
+  const WsLayout& w = c->wl;
+  const size_t nd = c->n_desc;
+  std::memcpy(img, c->hs.layers.data(), sizeof(LayerDesc) * nd);
+  std::memcpy(img + (w.order - w.layers), c->hs.order.data(), 4 * nd);
+  std::memcpy(img + (w.order_by_layer - w.layers), c->hs.order_by_layer.data(), 4 * nd);
+  size_t end = w.order_by_layer + 4 * nd;
+  if (n_evict > 0) {
+    std::memcpy(img + (w.evict_tab - w.layers), c->hs.evict_tab.data(), sizeof(EvictLayer) * n_evict);
+    end = w.evict_tab + sizeof(EvictLayer) * n_evict;
+  }
+  SQ_CUDA(c, cudaMemcpyAsync(c->ws + w.layers, img, end - w.layers, cudaMemcpyHostToDevice, st));
+  SQ_CUDA(c, cudaEventRecord(c->hs.slot_ev[slot], st));
+  return SQ_OK;
 }
 
 // Computes the cache geometry for the budgets in hs.budget and uploads it.
@@ -224,22 +260,25 @@ int build_layout(sq_ctx* c, cudaStream_t st) {
   if (off > c->pool_bytes) return fail(c, SQ_ERR_CAPACITY, "budgets do not fit the cache pool");
   if (lfl > c->wl.logits_floats) return fail(c, SQ_ERR_CAPACITY, "budgets do not fit the workspace");
   sort_orders(c);
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<LayerDesc>(c, c->wl.layers), c->hs.layers, sizeof(LayerDesc) * c->n_desc,
-                             cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.order), c->hs.order, 4 * c->n_desc, cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.order_by_layer), c->hs.order_by_layer, 4 * c->n_desc,
-                             cudaMemcpyHostToDevice, st));
-  // the staging block is reused by later calls: make sure the copies have left it
-  SQ_CUDA(c, cudaStreamSynchronize(st));
+  const int rc = upload_tables(c, 0, st);
+  if (rc != SQ_OK) return rc;
   c->budget_state = 2;
+  return SQ_OK;
+}
+
+// Waits for the allocator's kernel, which writes its budgets to page-locked memory.
+int fetch_budgets(sq_ctx* c) {
+  SQ_CUDA(c, cudaEventSynchronize(c->ev));
+  std::copy(c->hs.budget_down, c->hs.budget_down + c->n_desc, c->hs.budget.begin());
+  std::copy(c->hs.is_g3_down, c->hs.is_g3_down + c->n_desc, c->hs.is_g3.begin());
   return SQ_OK;
 }
 
 int ensure_budgets(sq_ctx* c, cudaStream_t st) {
   if (c->budget_state == 2) return SQ_OK;
   if (c->budget_state == 0) return fail(c, SQ_ERR_STATE, "budgets not set: call sq_allocate_budgets or sq_set_budgets first");
-  SQ_CUDA(c, cudaEventSynchronize(c->ev));
-  return build_layout(c, st);
+  const int rc = fetch_budgets(c);
+  return rc != SQ_OK ? rc : build_layout(c, st);
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -291,40 +330,52 @@ int sq_ctx_create(const sq_config* cfg, int64_t b_init, void* pool, size_t pool_
   c->budget_state = 0;
   c->last_begin = c->last_end = 0;
   c->last_stream = nullptr;
-  // one pinned block, carved into the staging arrays (largest alignment first)
   const size_t nd = wl.n_desc_cap;
-  const size_t bytes = nd * (sizeof(LayerDesc) + sizeof(EvictLayer) + 8 + 4 + 4 + 4 + 4 + 1) + 64;
+  HostStage& hs = c->hs;
+  hs.budget.assign(nd, 0);
+  hs.is_g3.assign(nd, 0);
+  hs.tok_count.assign(nd, 0);
+  hs.layers.assign(nd, LayerDesc{});
+  hs.order.assign(nd, 0);
+  hs.order_by_layer.assign(nd, 0);
+  hs.evict_tab.assign(nd, EvictLayer{});
+  const size_t image = align_up(wl.tables_end - wl.layers), counts = align_up(8 * nd), down = align_up(4 * nd) + align_up(nd);
   void* blk = nullptr;
-  if (cudaHostAlloc(&blk, bytes, cudaHostAllocDefault) != cudaSuccess ||
-      cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming) != cudaSuccess) {
+  hs.next_slot = 0;
+  int n_ev = 0;
+  bool ok = cudaHostAlloc(&blk, kSlots * (image + counts) + down, cudaHostAllocDefault) == cudaSuccess;
+  if (ok) ok = cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming) == cudaSuccess;
+  const bool has_ev = ok;
+  for (; ok && n_ev < kSlots; ++n_ev) {
+    if (cudaEventCreateWithFlags(&hs.slot_ev[n_ev], cudaEventDisableTiming) != cudaSuccess) {
+      ok = false;
+      break;
+    }
+  }
+  if (!ok) {
+    for (int i = 0; i < n_ev; ++i) cudaEventDestroy(hs.slot_ev[i]);
+    if (has_ev) cudaEventDestroy(c->ev);
     if (blk) cudaFreeHost(blk);
     delete c;
     return SQ_ERR_CUDA;
   }
-  std::memset(blk, 0, bytes);
-  char* p = static_cast<char*>(blk);
-  c->hs.block = blk;
-  c->hs.layers = reinterpret_cast<LayerDesc*>(p);
-  p += nd * sizeof(LayerDesc);
-  c->hs.evict_tab = reinterpret_cast<EvictLayer*>(p);
-  p += nd * sizeof(EvictLayer);
-  c->hs.tok_count = reinterpret_cast<long long*>(p);
-  p += nd * 8;
-  c->hs.budget = reinterpret_cast<int32_t*>(p);
-  p += nd * 4;
-  c->hs.cos_sim = reinterpret_cast<float*>(p);
-  p += nd * 4;
-  c->hs.order = reinterpret_cast<int*>(p);
-  p += nd * 4;
-  c->hs.order_by_layer = reinterpret_cast<int*>(p);
-  p += nd * 4;
-  c->hs.is_g3 = reinterpret_cast<uint8_t*>(p);
+  hs.block = static_cast<char*>(blk);
+  std::memset(blk, 0, kSlots * (image + counts) + down);
+  for (int i = 0; i < kSlots; ++i) hs.slot[i] = hs.block + i * (image + counts);
+  hs.budget_down = reinterpret_cast<int32_t*>(hs.block + kSlots * (image + counts));
+  hs.is_g3_down = reinterpret_cast<uint8_t*>(reinterpret_cast<char*>(hs.budget_down) + align_up(4 * nd));
   *out = c;
   return SQ_OK;
 }
 
 int sq_ctx_destroy(sq_ctx* c) {
   if (!c) return SQ_ERR_INVALID_ARG;
+  // nothing may still read or write the page-locked block
+  cudaEventSynchronize(c->ev);
+  for (int i = 0; i < kSlots; ++i) {
+    cudaEventSynchronize(c->hs.slot_ev[i]);
+    cudaEventDestroy(c->hs.slot_ev[i]);
+  }
   cudaEventDestroy(c->ev);
   cudaFreeHost(c->hs.block);
   delete c;
@@ -424,24 +475,26 @@ int sq_allocate_budgets(sq_ctx* c, int64_t b_init, double p, void* stream) {
     if (c->per_seq && c->imp_tokens[l] != (long long)c->batch * c->prompt)
       return fail(c, SQ_ERR_STATE, "per-sequence budgets need the hidden states of every prompt token of every layer");
   }
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<long long>(c, c->wl.tok_count), c->hs.tok_count, 8 * c->n_desc, cudaMemcpyHostToDevice,
-                             st));
+  // the token counts go down and the budgets come up through page-locked memory, without copies
+  int slot;
+  const int rc = take_slot(c, &slot);
+  if (rc != SQ_OK) return rc;
+  long long* counts = reinterpret_cast<long long*>(c->hs.slot[slot] + align_up(c->wl.tables_end - c->wl.layers));
+  std::copy(c->hs.tok_count.begin(), c->hs.tok_count.begin() + c->n_desc, counts);
   AllocateArgs a;
   a.cos_sum = ws_ptr<double>(c, c->wl.cos_sum);
-  a.tok_count = ws_ptr<long long>(c, c->wl.tok_count);
+  a.tok_count = counts;
   a.n_layer = c->cfg.n_layer;
   a.n_cluster = c->cfg.n_cluster;
   a.stride = c->n_grp;
   a.b_init = b_init;
   a.p = p;
   a.cos_sim = ws_ptr<float>(c, c->wl.cos_sim);
-  a.budget = ws_ptr<int>(c, c->wl.budget);
-  a.is_g3 = ws_ptr<unsigned char>(c, c->wl.is_g3);
+  a.budget = c->hs.budget_down;
+  a.is_g3 = c->hs.is_g3_down;
   SQ_CUDA(c, launch_allocate(a, st));
-  SQ_CUDA(c, cudaMemcpyAsync(c->hs.budget, a.budget, 4 * c->n_desc, cudaMemcpyDeviceToHost, st));
-  SQ_CUDA(c, cudaMemcpyAsync(c->hs.is_g3, a.is_g3, c->n_desc, cudaMemcpyDeviceToHost, st));
-  SQ_CUDA(c, cudaMemcpyAsync(c->hs.cos_sim, a.cos_sim, 4 * c->n_desc, cudaMemcpyDeviceToHost, st));
   SQ_CUDA(c, cudaEventRecord(c->ev, st));
+  SQ_CUDA(c, cudaEventRecord(c->hs.slot_ev[slot], st));
   c->budget_state = 1;
   for (int l = 0; l < c->cfg.n_layer; ++l) c->prefilled[l] = false;
   return SQ_OK;
@@ -453,7 +506,6 @@ int sq_set_budgets(sq_ctx* c, const int32_t* budgets_host, void* stream) {
   c->last_end = 0;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
   if (!budgets_host) return fail(c, SQ_ERR_INVALID_ARG, "budgets_host is NULL");
-  if (c->budget_state == 1) SQ_CUDA(c, cudaEventSynchronize(c->ev));
   for (int l = 0; l < c->cfg.n_layer; ++l) {
     for (int g = 0; g < c->n_grp; ++g) {
       c->hs.budget[l * c->n_grp + g] = budgets_host[user_index(c, l, g)];
@@ -461,11 +513,8 @@ int sq_set_budgets(sq_ctx* c, const int32_t* budgets_host, void* stream) {
     }
     c->prefilled[l] = false;
   }
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.budget), c->hs.budget, 4 * c->n_desc, cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemsetAsync(ws_ptr<unsigned char>(c, c->wl.is_g3), 0, c->n_desc, st));
   c->budget_state = 0;
-  int rc = build_layout(c, st);
-  return rc;
+  return build_layout(c, st);
 }
 
 int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const void* v_prompt, const void* q_prompt,
@@ -607,7 +656,7 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
     }
     // the launch's descriptors in launch order: the global order for the whole stack, else layer by layer
     const bool all = (s == 0 && e == cfg.n_layer);
-    const int* order_host = all ? c->hs.order : c->hs.order_by_layer + d0;
+    const int* order_host = all ? c->hs.order.data() : c->hs.order_by_layer.data() + d0;
     DecodeArgs a;
     long long n_items = 0;
     bool any_split = false;
@@ -729,10 +778,13 @@ int sq_evict(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const int32_t* n
       c->hs.budget[d] = nb;
     }
   }
+  // all descriptors of the call in one launch, the longest caches first (their CTAs run longest)
+  std::stable_sort(c->hs.evict_tab.begin(), c->hs.evict_tab.begin() + n_active,
+                   [](const EvictLayer& x, const EvictLayer& y) { return x.len > y.len; });
+  sort_orders(c);  // the launch orders (largest budget first) may have changed
+  rc = upload_tables(c, n_active, st);
+  if (rc != SQ_OK) return rc;
   if (n_active > 0) {
-    // all descriptors of the call in one launch, the longest caches first (their CTAs run longest)
-    std::stable_sort(c->hs.evict_tab, c->hs.evict_tab + n_active,
-                     [](const EvictLayer& x, const EvictLayer& y) { return x.len > y.len; });
     EvictArgs a;
     a.pool = c->pool;
     a.tab = ws_ptr<EvictLayer>(c, c->wl.evict_tab);
@@ -743,19 +795,8 @@ int sq_evict(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const int32_t* n
     a.n_sink = cfg.n_sink;
     a.row_bytes = cfg.head_dim * elem_bytes(cfg.dtype);
     a.status = ws_ptr<int>(c, c->wl.status);
-    SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<EvictLayer>(c, c->wl.evict_tab), c->hs.evict_tab, sizeof(EvictLayer) * n_active,
-                               cudaMemcpyHostToDevice, st));
     SQ_CUDA(c, launch_evict(a, st));
   }
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<LayerDesc>(c, c->wl.layers) + layer_begin * ng, &c->hs.layers[layer_begin * ng],
-                             sizeof(LayerDesc) * nl * ng, cudaMemcpyHostToDevice, st));
-  // the launch orders (largest budget first) may have changed
-  sort_orders(c);
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.order), c->hs.order, 4 * c->n_desc, cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.order_by_layer), c->hs.order_by_layer, 4 * c->n_desc,
-                             cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.budget), c->hs.budget, 4 * c->n_desc, cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaStreamSynchronize(st));
   return SQ_OK;
 }
 
@@ -799,15 +840,14 @@ int sq_get_cos_sim(sq_ctx* c, float* cos_sim_host) {
 int sq_get_budgets(sq_ctx* c, int32_t* budgets_host, uint8_t* is_g3_host) {
   if (!c || !budgets_host) return SQ_ERR_INVALID_ARG;
   if (c->budget_state == 0) return fail(c, SQ_ERR_STATE, "budgets not set");
-  SQ_CUDA(c, cudaDeviceSynchronize());
-  std::vector<int32_t> tb(c->n_desc);
-  std::vector<uint8_t> tg(c->n_desc);
-  SQ_CUDA(c, cudaMemcpy(tb.data(), ws_ptr<int>(c, c->wl.budget), 4 * c->n_desc, cudaMemcpyDeviceToHost));
-  SQ_CUDA(c, cudaMemcpy(tg.data(), ws_ptr<unsigned char>(c, c->wl.is_g3), c->n_desc, cudaMemcpyDeviceToHost));
+  if (c->budget_state == 1) {
+    const int rc = fetch_budgets(c);
+    if (rc != SQ_OK) return rc;
+  }
   for (int l = 0; l < c->cfg.n_layer; ++l)
     for (int g = 0; g < c->n_grp; ++g) {
-      budgets_host[user_index(c, l, g)] = tb[l * c->n_grp + g];
-      if (is_g3_host) is_g3_host[user_index(c, l, g)] = tg[l * c->n_grp + g];
+      budgets_host[user_index(c, l, g)] = c->hs.budget[l * c->n_grp + g];
+      if (is_g3_host) is_g3_host[user_index(c, l, g)] = c->hs.is_g3[l * c->n_grp + g];
     }
   return SQ_OK;
 }
@@ -922,7 +962,6 @@ int sq_ctx_import_layout(sq_ctx* c, const sq_layer_layout* in, void* stream) {
   c->last_end = 0;
   const sq_config& cfg = c->cfg;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
-  if (c->budget_state == 1) SQ_CUDA(c, cudaEventSynchronize(c->ev));
   // The geometry follows the slots a layer was laid out with, not its present budget (an explicit
   // eviction lowers the budget and leaves the slots where they are): lay the pool out by the
   // exported capacities, then put the budgets back.
@@ -964,14 +1003,8 @@ int sq_ctx_import_layout(sq_ctx* c, const sq_layer_layout* in, void* stream) {
     c->n_tok[l] = n_tok >= 0 ? n_tok : 0;
   }
   sort_orders(c);
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<LayerDesc>(c, c->wl.layers), c->hs.layers, sizeof(LayerDesc) * c->n_desc,
-                             cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.order), c->hs.order, 4 * c->n_desc, cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.order_by_layer), c->hs.order_by_layer, 4 * c->n_desc,
-                             cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemcpyAsync(ws_ptr<int>(c, c->wl.budget), c->hs.budget, 4 * c->n_desc, cudaMemcpyHostToDevice, st));
-  SQ_CUDA(c, cudaMemsetAsync(ws_ptr<unsigned char>(c, c->wl.is_g3), 0, c->n_desc, st));
-  SQ_CUDA(c, cudaStreamSynchronize(st));
+  rc = upload_tables(c, 0, st);
+  if (rc != SQ_OK) return rc;
   c->budget_state = 2;
   return SQ_OK;
 }

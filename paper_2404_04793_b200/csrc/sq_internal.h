@@ -45,7 +45,7 @@ struct ImportanceArgs {
   double* cos_sum;       // += sum over tokens of the cosine
 };
 
-struct AllocateArgs {  // entry of layer i: [i * stride + blockIdx.x] (one CTA per budget vector)
+struct AllocateArgs {  // entry of layer i: [i * stride + blockIdx.x] (one CTA per budget vector); tok_count, budget, is_g3: page-locked host memory
   const double* cos_sum;
   const long long* tok_count;
   int n_layer, n_cluster, stride;
