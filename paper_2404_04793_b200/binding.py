@@ -93,16 +93,22 @@ def lib() -> ctypes.CDLL:
     return L
 
 
+# Pointers are passed as plain integers (ctypes converts them for the declared c_void_p arguments): a
+# layer's call is issued every few microseconds, and wrapping each pointer and the stream in an object
+# cost more than the launch.
 def _dptr(t):
     if t is None:
         return None
-    if not t.is_cuda or not t.is_contiguous():
-        raise ValueError("expected a contiguous CUDA tensor")
-    return c_void_p(t.data_ptr())
+    if t.is_cuda and t.is_contiguous():
+        return t.data_ptr()
+    raise ValueError("expected a contiguous CUDA tensor")
+
+
+_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
 
 
 def _stream():
-    return c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _raw_stream(_current_device())
 
 
 def make_config(*, n_layer, n_q_head, n_kv_head, head_dim, hidden, max_batch, max_prompt, max_new_tokens,
@@ -141,7 +147,8 @@ class Context:
                                      c_void_p(self.workspace.data_ptr() + wo), ws_bytes, byref(h))
         if rc != SQ_OK:
             raise SqError(rc, "sq_ctx_create")
-        self._h = h
+        self._h = h.value
+        self._decode = lib().sq_decode_step
         self.pool_bytes, self.workspace_bytes = pool_bytes, ws_bytes
         self.pool_view = self.pool[po:po + pool_bytes]     # the bytes the library was given
 
@@ -205,8 +212,10 @@ class Context:
                                            _dptr(acc_prompt), _stream()))
 
     def decode_step(self, layer_begin, layer_end, q, k_new, v_new, out):
-        self._ck(lib().sq_decode_step(self._h, layer_begin, layer_end, _dptr(q), _dptr(k_new), _dptr(v_new),
-                                      _dptr(out), _stream()))
+        rc = self._decode(self._h, layer_begin, layer_end, _dptr(q), _dptr(k_new), _dptr(v_new), _dptr(out),
+                          _raw_stream(_current_device()))
+        if rc:
+            self._ck(rc)
 
     def evict(self, layer_begin, layer_end, new_budgets):
         flat = self._flatten(new_budgets, layer_end - layer_begin)
