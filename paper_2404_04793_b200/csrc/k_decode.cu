@@ -14,6 +14,8 @@
 
 namespace sq {
 
+constexpr int kMaxPieces = 8;  // CTAs of a cluster (the portable limit)
+
 // One CTA (NW warps) per (layer, unit, split).  A K or V row is D*sizeof(T) bytes = LPR lanes
 // x 16 bytes, so a warp reads 32/LPR consecutive rows per load instruction, fully coalesced.
 // Each lane keeps its 16-byte slice of up to GT query heads (pre-scaled by log2(e)/sqrt(d))
@@ -264,8 +266,8 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
     }
   }
   if constexpr (SCORES) {
-    __shared__ ScoreShared sh;
-    finish_scores<T, D, NW * 32>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * a.group, part_o, part_stat, sh);
+    __shared__ ScoreShared<kMaxPieces> sh;
+    finish_scores<T, D, NW * 32, kMaxPieces>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * a.group, part_o, part_stat, sh, nullptr, w);
   } else {
     if (!h2o && it.n_split > 1) merge_if_last<T, (GT == 1 ? 2 : 4)>(a, it, unit);
   }

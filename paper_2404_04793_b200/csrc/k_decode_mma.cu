@@ -21,6 +21,7 @@ namespace {
 
 constexpr int kTile = 64;  // tokens per pipeline stage
 constexpr int kScoresSmem = 110 * 1024;  // dynamic shared memory of a CTA with the score update: two CTAs per SM
+constexpr int kMaxPieces = 16;           // CTAs of a cluster (above 8: opt-in)
 // tiles of a piece when a unit of `len` slots is cut into `pieces`
 __host__ __device__ inline int piece_tiles(int len, int pieces) {
   return ((len + kTile - 1) / kTile + pieces - 1) / pieces;
@@ -334,6 +335,10 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(Args a) {
       l_w[mt][hf] += __shfl_xor_sync(kFull, l_w[mt][hf], 1);
       l_w[mt][hf] += __shfl_xor_sync(kFull, l_w[mt][hf], 2);
     }
+  ScoreAhead ahead;
+  if constexpr (SCORES)
+    fetch_scores<NT>(ahead, reinterpret_cast<const float*>(a.pool + ldp->acc_off) + (size_t)unit * cap,
+                     reinterpret_cast<const int*>(a.pool + ldp->pos_off) + (size_t)unit * cap, t0 + tid, t1, len == b);
   __syncthreads();  // the pipeline buffers are free: reuse them for the merge
 
   // ---- merge the WN token groups (tree over shared memory) ----
@@ -383,12 +388,12 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(Args a) {
     __syncthreads();
   }
   if constexpr (SCORES) {
-    // the piece's partial in shared memory, past the merge area
+    // the piece's partial and the scratch of the update in shared memory, past the merge area
     static_assert(WM == 1, "one row of warps");
-    __shared__ ScoreShared sh;
     float* part_o = reinterpret_cast<float*>(v_s);
     float* part_stat = part_o + MT * 16 * D;
-    static_assert(MT * 16 * (D + 4) * 4 <= STAGES * TILE_BYTES, "partial area");
+    ScoreShared<kMaxPieces>& sh = *reinterpret_cast<ScoreShared<kMaxPieces>*>(part_stat + MT * 16 * 4);
+    static_assert(MT * 16 * (D + 4) * 4 + sizeof(sh) <= STAGES * TILE_BYTES, "partial area");
     if (wn == 0) {
 #pragma unroll
       for (int mt = 0; mt < MT; ++mt)
@@ -402,7 +407,7 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(Args a) {
           if (tq == 0) *reinterpret_cast<float4*>(part_stat + h * 4) = make_float4(m_run[mt][hf], l_true[mt][hf], l_w[mt][hf], 0.f);
         }
     }
-    finish_scores<bf16, D, NT>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * G, part_o, part_stat, sh);
+    finish_scores<bf16, D, NT, kMaxPieces>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * G, part_o, part_stat, sh, &ahead, w);
     return;
   }
   if (wn == 0) {
@@ -468,6 +473,7 @@ static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t log
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresSmem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;
     configured = true;
   }
@@ -477,10 +483,13 @@ static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t log
 // H2O with the score update in the launch.  max_len: slots of the longest unit.  Returns
 // cudaErrorNotSupported where the second launch (decode_combine_kernel, h2o_update_warp_kernel) is the
 // better form or the logits of a piece do not fit.
-// Pieces: as many as leave all CTAs resident at once (two per SM), two tiles or more each.  Measured, us per
-// token of 32 layers of 32 / 8 heads of 128, one launch per layer, second launch / this form: 1 sequence
-// 385 / 281, 4: 451 / 391, 16: 660 / 533 (four pieces per unit, more than fit at once: 629), 64: 1060 / 983;
-// 20 / 1 heads of 64, 64 sequences: 435 / 239.  All 32 layers in one launch, 4096 units: 322 / 446.
+// Pieces: as many as leave all CTAs resident at once (two per SM), a tile or more each; up to 16 where few
+// clusters of that size are enough (more of them do not all fit at once beside smaller ones).  Measured, us
+// per token of 32 layers of 32 / 8 heads of 128, one launch per layer, second launch / this form: 1 sequence
+// 385 / 266 (at most eight pieces of two tiles or more: 281), its 16384-token caches 1309 / 560 (their
+// logits do not fit eight pieces: 1138), 4: 451 / 358, 16: 660 / 534 (four pieces per unit, more than fit at
+// once: 629), 64: 1060 / 983; 20 / 1 heads of 64, 64 sequences: 435 / 237; 80 layers of 64 / 8 heads, 4 sequences:
+// 1372 / 859.  All 32 layers in one launch, 4096 units: 322 / 446.
 cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
   const int G = a.group;
   if (G < 2 || G > 32 || (a.head_dim != 64 && a.head_dim != 128)) return cudaErrorNotSupported;
@@ -488,12 +497,12 @@ cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStrea
   const long long units = (long long)a.n_layer_total * a.n_unit;
   if (units >= 6 * n_sm) return cudaErrorNotSupported;
   const int tiles = (max_len + kTile - 1) / kTile;
-  int pieces = (int)std::min<long long>(kMaxPieces, std::max<long long>(1, 2 * n_sm / units));
-  pieces = std::min(pieces, std::max(1, tiles / 2));
+  int pieces = (int)std::min<long long>(units <= 16 ? kMaxPieces : 8, std::max<long long>(1, 2 * n_sm / units));
+  pieces = std::min(pieces, tiles);
   const int stages = a.head_dim == 128 ? 3 : 4;
   const size_t fixed = (size_t)2 * stages * kTile * a.head_dim * 2;
   auto logit_bytes = [&](int p) { return (size_t)piece_tiles(max_len, p) * kTile * G * 4; };
-  while (pieces < kMaxPieces && fixed + logit_bytes(pieces) > kScoresSmem) ++pieces;
+  while (pieces < 8 && fixed + logit_bytes(pieces) > kScoresSmem) ++pieces;
   const size_t lb = logit_bytes(pieces);
   if (fixed + lb > kScoresSmem) return cudaErrorNotSupported;
   if (a.head_dim == 128) return G <= 16 ? launch_scores_cfg<128, 1, 3>(a, pieces, lb, s) : launch_scores_cfg<128, 2, 3>(a, pieces, lb, s);

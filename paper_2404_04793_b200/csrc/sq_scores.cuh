@@ -15,8 +15,6 @@
 
 namespace sq {
 
-constexpr int kMaxPieces = 8;  // CTAs of a cluster (the portable limit)
-
 __device__ __forceinline__ int cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
@@ -55,63 +53,97 @@ struct ScoreCandidate {
   unsigned long long rank;
   int slot, pad;
 };
-// Small shared scratch of finish_scores.
+// Shared scratch of finish_scores for up to PIECES CTAs per cluster.
+template <int PIECES>
 struct ScoreShared {
+  float4 stat[PIECES][32];        // the pieces' partial statistics; .w: a piece's weight in the merged row
   float m[32], inv_l[32], inv_w[32];
-  float scale[kMaxPieces][32];        // weight of a piece's partial in the merged row
-  ScoreCandidate offer[kMaxPieces];   // one per piece (the first CTA's is read)
+  ScoreCandidate offer[PIECES];   // one per piece (the first CTA's is read)
   ScoreCandidate warp_best[16];
 };
+constexpr int kScoreIl = 4;  // slots per thread in flight in the score update
+// A thread's first slots' scores and positions, which a kernel with registers to spare fetches ahead of
+// its merge so that the trip to memory runs under it (no value is looked at before the update).
+struct ScoreAhead {
+  float old[kScoreIl];
+  int p[kScoreIl];
+};
+template <int NT>
+__device__ __forceinline__ void fetch_scores(ScoreAhead& ah, const float* acc, const int* pos, int s0, int t1, bool full) {
+#pragma unroll
+  for (int u = 0; u < kScoreIl; ++u) {
+    const int slot = s0 + u * NT;
+    ah.old[u] = 0.f;
+    ah.p[u] = 0x7fffffff;
+    if (slot < t1) {
+      ah.old[u] = acc[slot];
+      if (full) ah.p[u] = pos[slot];
+    }
+  }
+}
 
 // part_o [G][D] (un-normalised) and part_stat [G][4] (maximum, sum, sum of the weights O was made with):
 // this piece's partial in shared memory, where every thread of the CTA has written it; logit [token of
-// the piece][G], log2 domain, complete too.  t0, t1: the piece's slots; len: the unit's.  NT threads.
-template <typename T, int D, int NT>
+// the piece][G], log2 domain, complete too.  t0, t1: the piece's slots; len: the unit's; w: the new
+// token's slot.  fetched: scores of the thread's first slots, or null.  NT threads.
+template <typename T, int D, int NT, int PIECES>
 __device__ __forceinline__ void finish_scores(const DecodeArgsBase& a, const LayerDesc* ldp, int unit, int t0, int t1, int len, T* ob,
-                                              const float* logit, const float* part_o, const float* part_stat, ScoreShared& sh) {
+                                              const float* logit, const float* part_o, const float* part_stat,
+                                              ScoreShared<PIECES>& sh, const ScoreAhead* fetched, int w) {
   const int tid = threadIdx.x, lane = tid & 31, G = a.group;
   const int n = cluster_size(), me = cluster_rank();
   const int b = ldp->b, cap = ldp->cap;
   const bool full = (len == b);
-  if (n > 1) cluster_sync();
-  else __syncthreads();
+  const int* pos = reinterpret_cast<const int*>(a.pool + ldp->pos_off) + (size_t)unit * cap;
+  float* acc = reinterpret_cast<float*>(a.pool + ldp->acc_off) + (size_t)unit * cap;
+  if (n > 1) {
+    cluster_sync();
+    for (int i = tid; i < n * 32; i += NT) {  // one read over the cluster per (piece, head)
+      const int r = i >> 5, h = i & 31;
+      if (h < G) sh.stat[r][h] = ld_cluster4(map_rank(part_stat + h * 4, r));
+    }
+  } else {
+    __syncthreads();
+    if (tid < G) sh.stat[0][tid] = *reinterpret_cast<const float4*>(part_stat + tid * 4);
+  }
+  __syncthreads();
   if (tid < G) {
     float M = -INFINITY;
-    float4 st[kMaxPieces];
-#pragma unroll
-    for (int r = 0; r < kMaxPieces; ++r) {
-      st[r] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
-      if (r < n) st[r] = n > 1 ? ld_cluster4(map_rank(part_stat + tid * 4, r)) : *reinterpret_cast<const float4*>(part_stat + tid * 4);
-      M = fmaxf(M, st[r].x);
-    }
+    for (int r = 0; r < n; ++r) M = fmaxf(M, sh.stat[r][tid].x);
     float L = 0.f, Lw = 0.f;
-#pragma unroll
-    for (int r = 0; r < kMaxPieces; ++r) {
-      if (r >= n) continue;
-      const float f = (st[r].x > -INFINITY) ? exp2f(st[r].x - M) : 0.f;
-      L += st[r].y * f;
-      Lw += st[r].z * f;
-      sh.scale[r][tid] = f;
+    for (int r = 0; r < n; ++r) {
+      const float4 st = sh.stat[r][tid];
+      const float f = (st.x > -INFINITY) ? exp2f(st.x - M) : 0.f;
+      L += st.y * f;
+      Lw += st.z * f;
+      sh.stat[r][tid].w = f;
     }
     sh.m[tid] = M;
     sh.inv_l[tid] = 1.f / L;
     sh.inv_w[tid] = 1.f / Lw;
   }
   __syncthreads();
-  // this CTA's share of the output, four values at a time
+  // this CTA's share of the output, four values at a time; the last CTA, whose piece is the shortest, first
   const int n4 = G * D / 4;
-  for (int i4 = me * NT + tid; i4 < n4; i4 += n * NT) {
+  for (int i4 = (n - 1 - me) * NT + tid; i4 < n4; i4 += n * NT) {
     const int h = i4 * 4 / D;
     float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r0 = 0; r0 < n; r0 += 4) {
+      float4 v[4];
 #pragma unroll
-    for (int r = 0; r < kMaxPieces; ++r) {
-      if (r >= n) break;
-      const float4 v = n > 1 ? ld_cluster4(map_rank(part_o + i4 * 4, r)) : *reinterpret_cast<const float4*>(part_o + i4 * 4);
-      const float f = sh.scale[r][h];
-      O.x += v.x * f;
-      O.y += v.y * f;
-      O.z += v.z * f;
-      O.w += v.w * f;
+      for (int u = 0; u < 4; ++u) {
+        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r0 + u < n)
+          v[u] = n > 1 ? ld_cluster4(map_rank(part_o + i4 * 4, r0 + u)) : *reinterpret_cast<const float4*>(part_o + i4 * 4);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const float f = (r0 + u < n) ? sh.stat[r0 + u][h].w : 0.f;
+        O.x += v[u].x * f;
+        O.y += v[u].y * f;
+        O.z += v[u].z * f;
+        O.w += v[u].w * f;
+      }
     }
     const float inv = sh.inv_w[h];
     if (sizeof(T) == 2) {
@@ -126,26 +158,14 @@ __device__ __forceinline__ void finish_scores(const DecodeArgsBase& a, const Lay
   }
   // scores of this piece's tokens
   const int thr = a.n_tok + 1 - ldp->b_recent;  // next step: positions <= thr are outside the recent window
-  const int* pos = reinterpret_cast<const int*>(a.pool + ldp->pos_off) + (size_t)unit * cap;
-  float* acc = reinterpret_cast<float*>(a.pool + ldp->acc_off) + (size_t)unit * cap;
   unsigned long long best = ~0ull;
   int best_slot = -1;
-  constexpr int kIl = 4;  // slots per thread in flight
-  for (int s0 = t0 + tid; s0 < t1; s0 += kIl * NT) {
-    float old[kIl];
-    int p[kIl];
+  for (int s0 = t0 + tid; s0 < t1; s0 += kScoreIl * NT) {
+    ScoreAhead ahead;
+    if (fetched && s0 < t0 + kScoreIl * NT) ahead = *fetched;
+    else fetch_scores<NT>(ahead, acc, pos, s0, t1, full);
 #pragma unroll
-    for (int u = 0; u < kIl; ++u) {
-      const int slot = s0 + u * NT;
-      old[u] = 0.f;
-      p[u] = 0x7fffffff;
-      if (slot < t1) {
-        old[u] = acc[slot];
-        if (full) p[u] = pos[slot];
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < kIl; ++u) {
+    for (int u = 0; u < kScoreIl; ++u) {
       const int slot = s0 + u * NT;
       if (slot >= t1) continue;
       const float* lg = logit + (size_t)(slot - t0) * G;
@@ -161,10 +181,12 @@ __device__ __forceinline__ void finish_scores(const DecodeArgsBase& a, const Lay
       } else {
         for (int h = 0; h < G; ++h) gain += exp2f(lg[h] - sh.m[h]) * sh.inv_l[h];
       }
-      const float v = old[u] + gain;
+      // the new token's entries may have been fetched before they were stored
+      const float v = (slot == w ? 0.f : ahead.old[u]) + gain;
+      const int p = slot == w ? a.n_tok : ahead.p[u];
       acc[slot] = v;
-      if (full && p[u] <= thr) {
-        const unsigned long long r = victim_rank(v, p[u]);
+      if (full && p <= thr) {
+        const unsigned long long r = victim_rank(v, p);
         if (r < best) {
           best = r;
           best_slot = slot;
