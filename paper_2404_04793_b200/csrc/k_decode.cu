@@ -269,7 +269,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
     __shared__ ScoreShared<kMaxPieces> sh;
     finish_scores<T, D, NW * 32, kMaxPieces>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * a.group, part_o, part_stat, sh, nullptr, w);
   } else {
-    if (!h2o && it.n_split > 1) merge_if_last<T, (GT == 1 ? 2 : 4)>(a, it, unit);
+    if (!h2o && it.n_split > 1) merge_if_last<T, (GT == 1 ? 1 : 2)>(a, it, unit, &sm_o[0][0][0]);
   }
 }
 

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(32 * WM * WN) decode_attn_mma_kernel(Args a) {
       }
     }
   }
-  if (!h2o && it.n_split > 1) merge_if_last<bf16>(a, it, unit);
+  if (!h2o && it.n_split > 1) merge_if_last<bf16>(a, it, unit, reinterpret_cast<float*>(k_s));
 }
 
 template <int D, int MT, int WM, int WN, int STAGES>

@@ -471,7 +471,7 @@ __global__ void __launch_bounds__(192, 2)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");
   }
   if (tid == 0 && *abort_flag) atomicOr(a.status, kStatusTimeout);
-  if (it.n_split > 1) merge_if_last<bf16>(a, it, unit, H2O ? a.logits + ldp->lse_off + (size_t)unit * G : nullptr);
+  if (it.n_split > 1) merge_if_last<bf16>(a, it, unit, reinterpret_cast<float*>(q_s), H2O ? a.logits + ldp->lse_off + (size_t)unit * G : nullptr);
 }
 
 template <int STAGES, int ROWS, bool H2O>

@@ -69,12 +69,13 @@ __device__ __forceinline__ bool locate(const Args& a, int idx, ItemLoc& out) {
 // output and resets the ticket.  No piece ever waits for another.  With lse_out set, the merged
 // log-sum-exp (log2 domain, from the unrounded weight sums) of every head is stored there too.
 // The merge is run by a group of nt threads (tid = index within the group) that synchronise
-// through sync(), which returns false when the group gives up.
+// through sync(), which returns false when the group gives up.  scratch: 2 * group floats of shared memory.
 template <typename T, int kBatch, typename Sync>
 __device__ __forceinline__ void merge_if_last_group(const DecodeArgsBase& a, const ItemLoc& it, int unit, float* lse_out,
-                                                    int tid, int nt, Sync sync) {
+                                                    int tid, int nt, float* scratch, Sync sync) {
   __shared__ int s_last;
-  __shared__ float s_mM[kMaxGroup], s_mInv[kMaxGroup];
+  float* s_mM = scratch;
+  float* s_mInv = scratch + a.group;
   const int G = a.group, D = a.head_dim, ns = it.n_split;
   int* ticket = a.tickets + (size_t)it.layer * a.n_unit + unit;
   if (!sync()) return;  // the group's partials are written
@@ -88,19 +89,31 @@ __device__ __forceinline__ void merge_if_last_group(const DecodeArgsBase& a, con
   if (tid == 0) *ticket = 0;
   const size_t item0 = (size_t)it.base + (size_t)unit * ns;
   const float* stat = a.part_stat + item0 * G * kStatStride;
-  // The partials were written by other SMs, so every read is an L2 round trip: the loops below
-  // keep many independent loads in flight per thread instead of one dependent chain.
+  // The partials were written by other SMs, so every read is an L2 round trip: several pieces are read at
+  // a time (one round trip per piece took longer than a piece's tiles).
+  constexpr int kP = kBatch == 1 ? 4 : 8;
   for (int h = tid; h < G; h += nt) {
-    float M = -INFINITY;
-#pragma unroll 4
-    for (int s = 0; s < ns; ++s) M = fmaxf(M, __ldcg(stat + ((size_t)s * G + h) * kStatStride));
-    float Lw = 0.f, Lt = 0.f;
-#pragma unroll 4
-    for (int s = 0; s < ns; ++s) {
-      const float4 st = __ldcg(reinterpret_cast<const float4*>(stat + ((size_t)s * G + h) * kStatStride));
-      const float f = (st.x > -INFINITY) ? exp2f(st.x - M) : 0.f;
-      Lw += st.z * f;
-      Lt += st.y * f;
+    float M = -INFINITY, Lw = 0.f, Lt = 0.f;
+    for (int s0 = 0; s0 < ns; s0 += kP) {
+      float4 st[kP];
+#pragma unroll
+      for (int p = 0; p < kP; ++p) {
+        st[p] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+        if (s0 + p < ns) st[p] = __ldcg(reinterpret_cast<const float4*>(stat + ((size_t)(s0 + p) * G + h) * kStatStride));
+      }
+      float m2 = M;
+#pragma unroll
+      for (int p = 0; p < kP; ++p) m2 = fmaxf(m2, st[p].x);
+      const float f0 = (M > -INFINITY) ? exp2f(M - m2) : 0.f;
+      Lw *= f0;
+      Lt *= f0;
+      M = m2;
+#pragma unroll
+      for (int p = 0; p < kP; ++p) {
+        const float f = (st[p].x > -INFINITY) ? exp2f(st[p].x - M) : 0.f;
+        Lw += st[p].z * f;
+        Lt += st[p].y * f;
+      }
     }
     s_mM[h] = M;
     s_mInv[h] = 1.f / Lw;
@@ -122,26 +135,30 @@ __device__ __forceinline__ void merge_if_last_group(const DecodeArgsBase& a, con
       const int i4 = base + u * nt;
       h[u] = (i4 < n4) ? (i4 * 4) / D : -1;
     }
-    for (int s = 0; s < ns; ++s) {
-      float4 v[kBatch];
-      float ms[kBatch];
+    for (int s0 = 0; s0 < ns; s0 += kP) {
+      float4 v[kP][kBatch];
+      float ms[kP][kBatch];
 #pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-        ms[u] = -INFINITY;
-        if (h[u] >= 0) {
-          v[u] = __ldcg(reinterpret_cast<const float4*>(po + (size_t)s * G * D) + base + u * nt);
-          ms[u] = __ldcg(stat + ((size_t)s * G + h[u]) * kStatStride);
+      for (int p = 0; p < kP; ++p)
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          v[p][u] = make_float4(0.f, 0.f, 0.f, 0.f);
+          ms[p][u] = -INFINITY;
+          if (h[u] >= 0 && s0 + p < ns) {
+            v[p][u] = __ldcg(reinterpret_cast<const float4*>(po + (size_t)(s0 + p) * G * D) + base + u * nt);
+            ms[p][u] = __ldcg(stat + ((size_t)(s0 + p) * G + h[u]) * kStatStride);
+          }
         }
-      }
 #pragma unroll
-      for (int u = 0; u < kBatch; ++u) {
-        const float f = (ms[u] > -INFINITY) ? exp2f(ms[u] - s_mM[max(h[u], 0)]) : 0.f;
-        O[u].x += v[u].x * f;
-        O[u].y += v[u].y * f;
-        O[u].z += v[u].z * f;
-        O[u].w += v[u].w * f;
-      }
+      for (int p = 0; p < kP; ++p)
+#pragma unroll
+        for (int u = 0; u < kBatch; ++u) {
+          const float f = (ms[p][u] > -INFINITY) ? exp2f(ms[p][u] - s_mM[max(h[u], 0)]) : 0.f;
+          O[u].x += v[p][u].x * f;
+          O[u].y += v[p][u].y * f;
+          O[u].z += v[p][u].z * f;
+          O[u].w += v[p][u].w * f;
+        }
     }
 #pragma unroll
     for (int u = 0; u < kBatch; ++u) {
@@ -165,10 +182,10 @@ __device__ __forceinline__ void merge_if_last_group(const DecodeArgsBase& a, con
 }
 
 // The whole CTA merges.
-template <typename T, int kBatch = 4>
+template <typename T, int kBatch = 2>
 __device__ __forceinline__ void merge_if_last(const DecodeArgsBase& a, const ItemLoc& it, int unit,
-                                              float* lse_out = nullptr) {
-  merge_if_last_group<T, kBatch>(a, it, unit, lse_out, (int)threadIdx.x, (int)blockDim.x, [] {
+                                              float* scratch, float* lse_out = nullptr) {
+  merge_if_last_group<T, kBatch>(a, it, unit, lse_out, (int)threadIdx.x, (int)blockDim.x, scratch, [] {
     __syncthreads();
     return true;
   });
