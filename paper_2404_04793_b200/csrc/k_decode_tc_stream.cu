@@ -20,15 +20,13 @@
 //               CTA loads its own tiles); stores the new token's row before the tile that holds
 //               its slot is fetched
 //   warp 1      MMA issue (one thread)
-//   warps 2..5  thread = one head row (TMEM lane): p = exp2(s*scale - m_ref) straight from the
-//               accumulator row, no shuffles; P is packed to bf16 and stored back to tensor
-//               memory as the A operand of the second MMA; at a segment's end the same warps
+//   warps 2..5  softmax, four threads to a head row (sq_tc_rows.cuh); at a segment's end the same warps
 //               normalise and store O (or the partial) and, if theirs was the last piece, merge
 // Measured on B200: one M=128, K=16 MMA costs 45-48 cycles for N <= 64 and 64 cycles for N = 128
 // with the A operand in tensor memory, 68 with both operands in shared memory (whatever their
 // major-ness), and operands read from shared memory compete with the TMA writes for its
 // 128 B/clk; keeping P in tensor memory removes 56 KB of shared-memory traffic per tile.
-// A row's reference m_ref is its maximum over the segment's first tile; later tiles reuse it and
+// A row's reference m_ref is its maximum over the segment's first 64 tokens; later tiles reuse it and
 // only when a weight would exceed 2^16 is the reference moved (O and the sums rescaled through
 // tcgen05.ld/st, the tile redone): every weight stays finite and the result is that of the
 // exact softmax.  Every barrier wait is bounded.
@@ -48,6 +46,7 @@
 #include "sq_internal.h"
 #include "sq_stream.cuh"
 #include "sq_tc.cuh"
+#include "sq_tc_rows.cuh"
 
 namespace sq {
 
@@ -56,18 +55,12 @@ using namespace tc;
 namespace {
 constexpr int kD = 64;
 constexpr int kTileBytes = kTM * kD * 2;  // 16 KB: one K or V tile
-constexpr float kMaxWeight = 65536.f;     // 2^16
 constexpr int kColS = 0, kColP = 128, kColO = 192, kTmemCols = 256;
 constexpr int kCtasPerSm = 2;
 
 __host__ __device__ constexpr uint32_t idesc(int n, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major ? (1u << 16) : 0u) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(128 >> 4) << 24);
-}
-__device__ __forceinline__ uint32_t pack2(float lo, float hi) {
-  uint32_t r;
-  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
 }
 // Every lane waits (a suspended try_wait wakes sooner than one polling lane plus a shuffle:
 // measured 3.73 vs 4.27 ms per decode step of the largest Falcon-shaped cell); the warp agrees
@@ -118,23 +111,25 @@ __device__ __forceinline__ void merge_pieces(const StreamArgs& a, int layer, int
     }
     const float inv = s_inv[h];
     uint2 pk;
-    pk.x = pack2(O.x * inv, O.y * inv);
-    pk.y = pack2(O.z * inv, O.w * inv);
+    pk.x = pack_bf16x2(O.x * inv, O.y * inv);
+    pk.y = pack_bf16x2(O.z * inv, O.w * inv);
     reinterpret_cast<uint2*>(ob)[i4] = pk;
   }
 }
 }  // namespace
 
-// ROWS: head rows of Q held in shared memory (96 or 128).
+// ROWS: rows of the Q tile held in shared memory (120 for up to 96 heads, else 128; see sq_tc_rows.cuh).
 template <int STAGES, int ROWS, bool H2O>
 __global__ void __launch_bounds__(192, kCtasPerSm)
     decode_attn_tc_stream_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                           const __grid_constant__ CUtensorMap tm_v, const StreamArgs a) {
   constexpr int kQBytes = ROWS * 128;
+  constexpr int kSlots = ROWS == 120 ? 3 : 4, kHeads = kSlots * 32;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  // The first MMA addresses 128 rows of Q; with ROWS = 96 rows 96..127 alias the K stage that
-  // follows (rows are independent, those accumulator rows are never read).
+  // The first MMA addresses 128 rows of Q, of which groups of eight hold heads; the others hold anything
+  // and with ROWS = 120 the last eight alias the K stage that follows (rows are independent, those
+  // accumulator rows are never read).
   unsigned char* q_s = smem;
   unsigned char* k_s = q_s + kQBytes;              // STAGES tiles
   unsigned char* v_s = k_s + STAGES * kTileBytes;  // STAGES tiles
@@ -148,8 +143,8 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* s_last = reinterpret_cast<int*>(tmem_slot + 2);
-  float* s_mm = reinterpret_cast<float*>(bars + 18);  // [128] merge scratch: maxima
-  float* s_minv = s_mm + kTM;                         // [128] merge scratch: 1 / weight sum
+  float* s_mm = reinterpret_cast<float*>(bars + 18);  // [kHeads] merge scratch: maxima
+  float* s_minv = s_mm + kHeads;                      // merge scratch: 1 / weight sums
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int G = a.group;
@@ -180,6 +175,7 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  const WideLayout layout;
   SegIter it;
   it.init(a, blockIdx.x);
 
@@ -247,10 +243,11 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
       // Q has one buffer: the previous segment's last S product must have read it
       if (it.seg >= 1) ok = warp_wait(bar_qempty, (it.seg - 1) & 1, abort_flag);
       if (!ok) break;
-      if (lane == 0) {
-        mbar_expect_tx(bar_qfull, kQBytes);
-        tma_load_2d(s_u32(q_s), &tm_q, 0, (int)(tok * a.n_q_head + (size_t)kvh * G), bar_qfull);
-      }
+      const int n_group = (G + 7) / 8;  // Q, eight heads per copy
+      if (lane == 0) mbar_expect_tx(bar_qfull, n_group * 1024);
+      __syncwarp();
+      if (lane < n_group)
+        tma_load_2d(s_u32(q_s + layout.row_of_group(lane) * 128), &tm_q, 0, (int)(tok * a.n_q_head + (size_t)kvh * G) + 8 * lane, bar_qfull);
       q_issued = it.seg + 1;
       for (int i = i0; ok && i < it.ntile; ++i, ++g) {
         if (g >= STAGES) ok = warp_wait(bar_empty(g % STAGES), ((g / STAGES) - 1) & 1, abort_flag);
@@ -325,15 +322,18 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
     }
     __syncwarp();
   } else {
-    // ---------------- softmax: thread = one head row ----------------
+    // ---------------- softmax: four threads = one head row (sq_tc_rows.cuh) ----------------
     const int quarter = warp & 3, etid = (warp - 2) * 32 + lane;
-    const int row = quarter * 32 + lane;
-    const bool live = row < G;                // this lane's row is a real head
-    const bool warp_live = quarter * 32 < G;  // tcgen05.ld/st are warp-wide: whole warps opt in or out
+    const int row = layout.head_of_lane(quarter, lane);  // the head whose row of O is this lane's
+    const bool live = row < G;
     const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
-    const uint32_t s_addr = tmem_base + lane_sel + kColS, p_addr = tmem_base + lane_sel + kColP,
-                   o_addr = tmem_base + lane_sel + kColO;
-    float m_ref = -INFINITY, l_true = 0.f, l_w = 0.f;
+    WideRows<H2O, kSlots> rows;
+    rows.s_addr = tmem_base + lane_sel + kColS;
+    rows.p_addr = tmem_base + lane_sel + kColP;
+    rows.o_addr = tmem_base + lane_sel + kColO;
+    rows.scale_log2 = a.scale_log2;
+    rows.lane = lane;
+    rows.n_slot = layout.groups(quarter, G);
     int g0 = 0;  // tiles of the CTA before the current segment
     int epi_use = 0;
     bool ok = true;
@@ -346,94 +346,19 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
       return ok;
     };
 
-    // Row maximum of the tile's valid tokens, in the log2 domain.
-    auto tile_max = [&](int n_valid) {
-      float mx = -INFINITY;
-#pragma unroll 1
-      for (int c = 0; c < 4; ++c) {
-        float v[32];
-        tmem_ld32(s_addr + c * 32, v);
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (c * 32 + j < n_valid) mx = fmaxf(mx, v[j]);
-      }
-      return mx * a.scale_log2;
-    };
-    // p = exp2(s*scale - m_ref) for the whole tile: P (bf16) to tensor memory; sums of the weights
-    // (exact fp32 for the H2O normaliser, of the bf16-rounded weights for the output) to *sum /
-    // *sum_w; returns an upper bound of the largest weight.  The role is bound by the
-    // special-function unit (one exp2 per 8 cycles per warp) and by the issue slots of one or two
-    // softmax warps per scheduler, so the scaling runs as packed fp32x2 instructions and the
-    // rounded weights are summed by mixed-precision adds: six instructions per two weights.
-    // FULL (a compile-time tag): every token of the tile is valid, so no masking code is emitted
-    // (with a run-time flag the compare / select pair ran for every weight of every tile).
-    auto tile_weights = [&](auto full_tag, int n_valid, float* sum, float* sum_w) {
-      constexpr bool full = decltype(full_tag)::value;
-      const unsigned long long scale2 = f32x2(a.scale_log2, a.scale_log2), neg_m2 = f32x2(-m_ref, -m_ref);
-      unsigned long long acc2 = f32x2(0.f, 0.f);
-      float w_a = 0.f, w_b = 0.f;
-      auto chunk = [&](const uint32_t (&r)[32], int c) {
-#pragma unroll
-        for (int hc = 0; hc < 2; ++hc) {  // P goes back sixteen tokens (eight columns) at a time
-          uint32_t pk[8];
-#pragma unroll
-          for (int jj = 0; jj < 16; jj += 2) {
-            const int j = hc * 16 + jj;
-            float p0, p1;
-            f32x2_split(fma_f32x2(f32x2(__uint_as_float(r[j]), __uint_as_float(r[j + 1])), scale2, neg_m2), p0, p1);
-            p0 = ex2(p0);
-            p1 = ex2(p1);
-            if (!full) {
-              if (c * 32 + j >= n_valid) p0 = 0.f;
-              if (c * 32 + j + 1 >= n_valid) p1 = 0.f;
-            }
-            if (H2O) acc2 = add_f32x2(acc2, f32x2(p0, p1));
-            const uint32_t u = pack2(p0, p1);  // round to nearest bf16, p0 in the low half
-            w_a = add_bf16_lo(w_a, u);
-            w_b = add_bf16_hi(w_b, u);
-            pk[jj / 2] = u;
-          }
-          tmem_st8_u32(p_addr + c * 16 + hc * 8, pk);  // tokens c*32 + hc*16 .. +15 of this row
-        }
-      };
-      // the next chunk's tensor-memory load is in flight while this one is processed
-      uint32_t ra[32], rb[32];
-      tmem_ld32_nowait(s_addr, ra);
-      tmem_wait_ld(ra);
-      tmem_ld32_nowait(s_addr + 32, rb);
-      chunk(ra, 0);
-      tmem_wait_ld(rb);
-      tmem_ld32_nowait(s_addr + 64, ra);
-      chunk(rb, 1);
-      tmem_wait_ld(ra);
-      tmem_ld32_nowait(s_addr + 96, rb);
-      chunk(ra, 2);
-      tmem_wait_ld(rb);
-      chunk(rb, 3);
-      tmem_wait_st();
-      float s0, s1;
-      f32x2_split(acc2, s0, s1);
-      *sum = s0 + s1;
-      *sum_w = w_a + w_b;
-      return w_a + w_b;  // the tile's weight sum bounds its largest weight
-    };
-
     while (ok && it.next(a)) {
       const int t0 = it.tile0 * kTM;
       t1 = min(it.len, (it.tile0 + it.ntile) * kTM);
-      m_ref = -INFINITY;
-      l_true = 0.f;
-      l_w = 0.f;
+      rows.begin();
       for (int i = 0; ok && i < it.ntile; ++i) {
         const int g = g0 + i, st = g % STAGES;
         const int n_valid = min(kTM, t1 - (t0 + i * kTM));
         ok = warp_wait(bar_sfull, g & 1, abort_flag);
-        if (ok && g >= 1) ok = warp_wait(bar_pfree, (g - 1) & 1, abort_flag);
         if (ok && n_valid < kTM) {
           // rows of the V tile past the unit's last token may hold anything: zero them
           ok = warp_wait(bar_full(st), (g / STAGES) & 1, abort_flag);
-          if (ok && row >= n_valid) {
-            uint4* vrow = reinterpret_cast<uint4*>(v_s + st * kTileBytes + row * 128);
+          if (ok && quarter * 32 + lane >= n_valid) {
+            uint4* vrow = reinterpret_cast<uint4*>(v_s + st * kTileBytes + (quarter * 32 + lane) * 128);
 #pragma unroll
             for (int c = 0; c < 8; ++c) vrow[c] = make_uint4(0, 0, 0, 0);
           }
@@ -441,45 +366,23 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
         }
         if (!ok) break;
         tc_fence_after();
-        if (warp_live) {
-          if (i == 0) m_ref = tile_max(n_valid);
-          float sum, sum_w;
-          auto weights = [&]() {
-            return (n_valid == kTM) ? tile_weights(std::true_type{}, n_valid, &sum, &sum_w)
-                                    : tile_weights(std::false_type{}, n_valid, &sum, &sum_w);
-          };
-          float pmax = weights();
-          if (__any_sync(0xffffffffu, pmax > kMaxWeight)) {
-            // rare: move the reference of the rows that need it; O and the sums (complete up to
-            // the previous tile) shrink with it, then the tile is redone.  The whole warp takes
-            // part in the TMEM round trip.
-            const float mx2 = tile_max(n_valid);
-            const bool need = pmax > kMaxWeight;
-            ok = warp_wait(bar_odone, (g - 1) & 1, abort_flag);
-            if (!ok) break;
-            tc_fence_after();
-            const float f = need ? ex2(m_ref - mx2) : 1.f;
-#pragma unroll 1
-            for (int c = 0; c < 2; ++c) {
-              float o[32];
-              tmem_ld32(o_addr + c * 32, o);
-#pragma unroll
-              for (int j = 0; j < 32; ++j) o[j] *= f;
-              tmem_st32(o_addr + c * 32, o);
-            }
-            l_true *= f;
-            l_w *= f;
-            if (need) m_ref = mx2;
-            pmax = weights();
-          }
-          l_true += sum;
-          l_w += sum_w;
+        bool s_released = rows.template tile<true>(n_valid, i == 0, bar_sfree, [&]() {
+          if (g >= 1) ok = warp_wait(bar_pfree, (g - 1) & 1, abort_flag);
+        });
+        if (!ok) break;
+        if (rows.too_large()) {
+          ok = warp_wait(bar_odone, (g - 1) & 1, abort_flag);
+          if (!ok) break;
+          tc_fence_after();
+          rows.redo(n_valid);
+          s_released = rows.template tile<true>(n_valid, false, bar_sfree, []() {});
         }
+        rows.add_tile();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) {
           mbar_arrive(bar_pready);
-          mbar_arrive(bar_sfree);
+          if (!s_released) mbar_arrive(bar_sfree);
         }
       }
       if (!ok) break;
@@ -493,7 +396,9 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
       const LayerDesc* ldp = a.layers + it.layer;
       const int c_first = it.c_first(a), n_piece = it.n_piece(a);
       float* lse = H2O ? a.logits + ldp->lse_off + (size_t)unit * G : nullptr;
-      if (warp_live) {
+      {
+        float m_ref, l_true, l_w;
+        rows.finish(&m_ref, &l_true, &l_w);
         const int seq = unit / a.n_kv_head, kvh = unit - seq * a.n_kv_head;
         const size_t tok = (size_t)(it.layer - a.layer_begin) * a.batch + seq;
         const int slot = piece_slot(c_first, (int)blockIdx.x - c_first);
@@ -503,14 +408,14 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
 #pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           float o[32];
-          tmem_ld32(o_addr + c * 32, o);
+          tmem_ld32(rows.o_addr + c * 32, o);
           if (!live) continue;
           if (n_piece == 1) {
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4)
               *reinterpret_cast<uint4*>(orow + c * 32 + q4 * 8) =
-                  make_uint4(pack2(o[q4 * 8] * inv, o[q4 * 8 + 1] * inv), pack2(o[q4 * 8 + 2] * inv, o[q4 * 8 + 3] * inv),
-                             pack2(o[q4 * 8 + 4] * inv, o[q4 * 8 + 5] * inv), pack2(o[q4 * 8 + 6] * inv, o[q4 * 8 + 7] * inv));
+                  make_uint4(pack_bf16x2(o[q4 * 8] * inv, o[q4 * 8 + 1] * inv), pack_bf16x2(o[q4 * 8 + 2] * inv, o[q4 * 8 + 3] * inv),
+                             pack_bf16x2(o[q4 * 8 + 4] * inv, o[q4 * 8 + 5] * inv), pack_bf16x2(o[q4 * 8 + 6] * inv, o[q4 * 8 + 7] * inv));
           } else {
 #pragma unroll
             for (int q4 = 0; q4 < 8; ++q4)
@@ -559,7 +464,8 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
 template <int STAGES, int ROWS, bool H2O>
 static cudaError_t launch_tc_stream_cfg(const StreamArgs& t, int n_cta, const CUtensorMap& tq, const CUtensorMap& tk,
                                  const CUtensorMap& tv, cudaStream_t s) {
-  constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 18 * 8 + 2 * kTM * 4;
+  constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 18 * 8 + 2 * (ROWS == 120 ? 96 : 128) * 4;
+  static_assert(2 * (smem + 1024) <= 228 * 1024, "two CTAs per SM");
   auto kern = decode_attn_tc_stream_kernel<STAGES, ROWS, H2O>;
   static bool configured = false;
   if (!configured) {
@@ -584,9 +490,8 @@ cudaError_t launch_decode_attn_tc_stream(const DecodeArgs& a, const int* desc_ti
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
   }
-  const int rows = a.group <= 96 ? 96 : 128;
   CUtensorMap tm_q, tm_k, tm_v;
-  if (!make_tile_map(&tm_q, a.q, (long long)q_rows, kD, rows) || !make_tile_map(&tm_k, a.pool, pool_rows, kD, kTM) ||
+  if (!make_tile_map(&tm_q, a.q, (long long)q_rows, kD, 8) || !make_tile_map(&tm_k, a.pool, pool_rows, kD, kTM) ||
       !make_tile_map(&tm_v, a.pool, pool_rows, kD, kTM))
     return cudaErrorNotSupported;
   const bool h2o = a.policy == SQ_POLICY_H2O;
@@ -608,7 +513,7 @@ cudaError_t launch_decode_attn_tc_stream(const DecodeArgs& a, const int* desc_ti
     if (n_cta < 0) return cudaErrorNotSupported;
     if (n_cta == 0) continue;
     cudaError_t e;
-    if (rows == 96) e = h2o ? launch_tc_stream_cfg<3, 96, true>(t, n_cta, tm_q, tm_k, tm_v, s) : launch_tc_stream_cfg<3, 96, false>(t, n_cta, tm_q, tm_k, tm_v, s);
+    if (a.group <= 96) e = h2o ? launch_tc_stream_cfg<3, 120, true>(t, n_cta, tm_q, tm_k, tm_v, s) : launch_tc_stream_cfg<3, 120, false>(t, n_cta, tm_q, tm_k, tm_v, s);
     else e = h2o ? launch_tc_stream_cfg<2, 128, true>(t, n_cta, tm_q, tm_k, tm_v, s) : launch_tc_stream_cfg<2, 128, false>(t, n_cta, tm_q, tm_k, tm_v, s);
     if (e != cudaSuccess) return e;
   }

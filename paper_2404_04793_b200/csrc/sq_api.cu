@@ -611,14 +611,17 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
     // Split-K plan.  A piece costs a fixed set-up plus its tiles, and pieces run in waves of
     // as many CTAs as fit the GPU at once; among the piece lengths that are whole tiles, take
     // the one with the smallest estimated time.  What a tile, a set-up (in tiles; fitted to
-    // measured step times, it includes writing and merging the partial results) and a wave are
-    // depends on the kernel the shape is served by.  The running item counts of a split launch
+    // measured step times; it includes writing and merging the partial results where `merge`, the part that
+    // only units in several pieces pay, is 0) and a wave are depends on the kernel the shape is served by.  The running item counts of a split launch
     // travel in the kernel parameters, which hold kMaxLayers descriptors: larger launches (many
     // sequences with per-sequence budgets) are not split; they have units to spare anyway.
     const bool bf16 = cfg.dtype == SQ_BF16;
-    int tile, setup, per_sm;
+    int tile, setup, per_sm, merge = 0;
+    double gain = 0.90;  // more pieces only for a clear gain
     if (bf16 && cfg.head_dim == 64 && G > 32) {  // tcgen05 kernel: 128-token tiles, 2 CTAs per SM
-      tile = 128, setup = 8, per_sm = 2;
+      // us per token, 32 layers, (setup, merge, gain) = (8, 0, 0.90) / (8, 0, 0.95) / (4, 4, 0.95): 33 sequences of
+      // 8191, 50 %, H2O 1278 / 1217 / 1217; 60 of 4000, 30 % 548 / 667 / 540; 8 of 8191, 30 %, H2O 1028 / 1098 / 1045
+      tile = 128, setup = 4, merge = 4, per_sm = 2, gain = 0.95;
     } else if (bf16 && G > 1) {                  // mma.sync kernel: 64-token tiles
       tile = 64, setup = 12, per_sm = cfg.head_dim == 64 && G <= 32 ? 3 : 2;
     } else {                                     // fp32-pipe kernel
@@ -640,16 +643,16 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
         const int len = std::min(n_tok + 1, c->hs.layers[d].b);
         const int ns = (len + cand - 1) / cand;
         items += (long long)U * ns;
-        work += (long long)U * ((long long)ns * setup + (len + tile - 1) / tile);
+        work += (long long)U * ((long long)ns * (setup + (ns > 1 ? merge : 0)) + (len + tile - 1) / tile);
       }
       if ((size_t)items > c->wl.items_cap) break;
       // CTAs start in item order, longest layers first: the makespan is about the evenly spread
       // work, but never below the longest piece, and whole waves when there are only a few
       const long long waves = (items + slots - 1) / slots;
-      const double t_max = setup + (double)std::min(cand, max_len) / tile;
+      const double t_max = setup + (cand < max_len ? merge : 0) + (double)std::min(cand, max_len) / tile;
       const double spread = (double)work / (double)slots + 0.5 * t_max;
       const double cost = items <= slots ? t_max : std::max(t_max, std::min(spread, (double)waves * t_max));
-      if (split == 0 || cost < best_cost * 0.90) {  // more pieces only for a clear gain
+      if (split == 0 || cost < best_cost * gain) {
         best_cost = cost;
         split = cand;
       }
