@@ -1,6 +1,7 @@
 // Prefill side of Algorithm 1 (step 13 with the first compression of steps 16-18 applied at
 // once): H2O prompt scores, C_seq selection over the prompt, and the gather of the kept K/V
 // rows into the layer's cache region.
+#include <algorithm>
 #include <cstdlib>
 #include <cstring>
 
@@ -11,152 +12,272 @@
 namespace sq {
 
 // ---------------------------------------------------------------------------------------
-// H2O prompt scores.  acc[t] = sum over the query heads sharing the KV head and over query
-// rows r >= t of softmax_row_r(Q K^T / sqrt(d))[t] (causal).  Two passes over 64x64 score
-// tiles: row log-sum-exp, then column sums of exp(s - lse).  Thread (tx, ty) of the 16x16
-// block owns rows ty+16r and columns tx+16c of a tile (r, c in 0..3).
+// H2O prompt scores on the fp32 pipes.  acc[t] = sum over the query heads sharing the KV head and over
+// query rows r >= t of softmax_row_r(Q K^T / sqrt(d))[t] (causal).  Two sweeps over TQ x 64 score tiles
+// (rows: queries, columns: keys): row log-sum-exp, then column sums of exp(s - lse).
+// Thread (tx, ty) of the 16 x TQ/4 block owns rows 4 ty .. +3 and columns 4 tx .. +3 of a tile.  Both
+// operands lie transposed in shared memory, so one 16-byte read of each feeds sixteen FMAs; the next
+// streamed tile is on its way to registers while this one is worked on.  Bound by the FMA pipe for large
+// prompts and by the chain of tiles of a CTA for small ones: there TQ is 32, and the second sweep's
+// stream is cut into pieces whose column sums the last to finish adds up in order (deterministic).
+// Measured, us per layer of scores, selection and gather, fp32, 64 x 64 tiles with scalar reads and one CTA per
+// key tile / this: 1 sequence of 256 tokens, 2 / 2 heads of 64: 79.6 / 25.9; 2 of 777, 16 / 4 heads of 128: 798 /
+// 286; 20 of 500, 20 / 1 heads of 64: 1627 / 585; 1 of 2048, 32 / 32 heads of 128: 2143 / 1395.
 // ---------------------------------------------------------------------------------------
-constexpr int TQ = 64, TK = 64, DC = 32;
+constexpr int TK = 64;
 
-template <typename T, int D>
-__device__ __forceinline__ void score_tile(const T* __restrict__ qbase, const T* __restrict__ kbase, int q0, int k0,
-                                           int P, float (*Qs)[DC + 1], float (*Ks)[DC + 1], float s[4][4]) {
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+// four consecutive elements of a row, widened
+template <typename T>
+__device__ __forceinline__ float4 load4(const T* p);
+template <>
+__device__ __forceinline__ float4 load4<float>(const float* p) {
+  return *reinterpret_cast<const float4*>(p);
+}
+template <>
+__device__ __forceinline__ float4 load4<__nv_bfloat16>(const __nv_bfloat16* p) {
+  const uint2 v = *reinterpret_cast<const uint2*>(p);
+  return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16),
+                     __uint_as_float(v.y & 0xffff0000u));
+}
+
+// A tile of ROWS rows of D elements on its way from global memory to shared memory, where it lies
+// transposed: element (row, e) at [e * (ROWS + 4) + row].  Rows at or past `limit` read as 0.
+template <typename T, int D, int ROWS, int NT>
+struct TileLoad {
+  static constexpr int N = ROWS * D / 4 / NT;
+  float4 v[N];
+  __device__ __forceinline__ void fetch(const T* base, int row0, int limit) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int idx = threadIdx.x + i * NT, row = idx % ROWS, e = idx / ROWS * 4;
+      v[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (row0 + row < limit) v[i] = load4<T>(base + (size_t)(row0 + row) * D + e);
+    }
+  }
+  __device__ __forceinline__ void store(float* s) const {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int idx = threadIdx.x + i * NT, row = idx % ROWS, e = idx / ROWS * 4;
+      s[(e + 0) * (ROWS + 4) + row] = v[i].x;
+      s[(e + 1) * (ROWS + 4) + row] = v[i].y;
+      s[(e + 2) * (ROWS + 4) + row] = v[i].z;
+      s[(e + 3) * (ROWS + 4) + row] = v[i].w;
+    }
+  }
+};
+
+template <int D, int TQ>
+__device__ __forceinline__ void score_tile(const float* qs, const float* ks, float (&s)[4][4]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
   for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < 4; ++c) s[r][c] = 0.f;
-  for (int dc = 0; dc < D; dc += DC) {
-    __syncthreads();
-    for (int idx = tid; idx < TQ * DC; idx += 256) {
-      int row = idx / DC, col = idx % DC;
-      int qr = q0 + row, kr = k0 + row;
-      Qs[row][col] = (qr < P) ? to_float<T>(qbase[(size_t)qr * D + dc + col]) : 0.f;
-      Ks[row][col] = (kr < P) ? to_float<T>(kbase[(size_t)kr * D + dc + col]) : 0.f;
-    }
-    __syncthreads();
 #pragma unroll 8
-    for (int dd = 0; dd < DC; ++dd) {
-      float qv[4], kv[4];
+  for (int e = 0; e < D; ++e) {
+    const float4 q = *reinterpret_cast<const float4*>(qs + e * (TQ + 4) + 4 * ty);
+    const float4 k = *reinterpret_cast<const float4*>(ks + e * (TK + 4) + 4 * tx);
+    const float qv[4] = {q.x, q.y, q.z, q.w}, kv[4] = {k.x, k.y, k.z, k.w};
 #pragma unroll
-      for (int r = 0; r < 4; ++r) qv[r] = Qs[ty + 16 * r][dd];
+    for (int r = 0; r < 4; ++r)
 #pragma unroll
-      for (int c = 0; c < 4; ++c) kv[c] = Ks[tx + 16 * c][dd];
-#pragma unroll
-      for (int r = 0; r < 4; ++r)
-#pragma unroll
-        for (int c = 0; c < 4; ++c) s[r][c] = fmaf(qv[r], kv[c], s[r][c]);
-    }
+      for (int c = 0; c < 4; ++c) s[r][c] = fmaf(qv[r], kv[c], s[r][c]);
   }
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(256) prefill_row_lse_kernel(ScoreArgs a, float scale_log2) {
-  __shared__ float Qs[TQ][DC + 1], Ks[TK][DC + 1];
+template <int D, int TQ>
+constexpr size_t score_smem() {
+  return (size_t)D * (TQ + 4 + TK + 4) * 4;
+}
+
+template <typename T, int D, int TQ>
+__global__ void __launch_bounds__(4 * TQ) prefill_row_lse_kernel(ScoreArgs a, float scale_log2) {
+  constexpr int NT = 4 * TQ;
+  extern __shared__ __align__(16) float sm[];
+  float* qs = sm;
+  float* ks = sm + D * (TQ + 4);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int qt = blockIdx.x, hq = blockIdx.y, bi = blockIdx.z;
-  const int g = a.n_q_head / a.n_kv_head, P = a.prompt;
+  const int P = a.prompt, n_qt = (P + TQ - 1) / TQ;
+  const int qt = n_qt - 1 - blockIdx.x, hq = blockIdx.y, bi = blockIdx.z;  // longest rows first
+  const int g = a.n_q_head / a.n_kv_head;
   const T* qbase = reinterpret_cast<const T*>(a.q) + ((size_t)bi * a.n_q_head + hq) * P * D;
   const T* kbase = reinterpret_cast<const T*>(a.k) + ((size_t)bi * a.n_kv_head + hq / g) * P * D;
-  const int q0 = qt * TQ;
+  const int q0 = qt * TQ, n_kt = (min(q0 + TQ, P) + TK - 1) / TK;
+  grid_wait();
+  {
+    TileLoad<T, D, TQ, NT> ql;
+    ql.fetch(qbase, q0, P);
+    ql.store(qs);
+  }
+  TileLoad<T, D, TK, NT> kl;
+  kl.fetch(kbase, 0, P);
   float m[4], l[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
     m[r] = -INFINITY;
     l[r] = 0.f;
   }
-  for (int kt = 0; kt <= qt; ++kt) {
+  for (int kt = 0; kt < n_kt; ++kt) {
     const int k0 = kt * TK;
+    __syncthreads();
+    kl.store(ks);
+    __syncthreads();
+    if (kt + 1 < n_kt) kl.fetch(kbase, k0 + TK, P);
     float s[4][4];
-    score_tile<T, D>(qbase, kbase, q0, k0, P, Qs, Ks, s);
+    score_tile<D, TQ>(qs, ks, s);
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      const int qr = q0 + ty + 16 * r;
+      const int qr = q0 + 4 * ty + r;
       float tmax = -INFINITY;
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
-        const int kr = k0 + tx + 16 * c;
+        const int kr = k0 + 4 * tx + c;
         s[r][c] = (kr <= qr && qr < P) ? s[r][c] * scale_log2 : -INFINITY;
         tmax = fmaxf(tmax, s[r][c]);
       }
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+      // every thread keeps the maximum and sum of its own columns; the row's are formed at the end
       const float m_new = fmaxf(m[r], tmax);
-      float psum = 0.f;
-      if (m_new != -INFINITY) {
+      if (m_new > -INFINITY) {
+        float sum = 0.f;
 #pragma unroll
-        for (int c = 0; c < 4; ++c) psum += exp2f(s[r][c] - m_new);
-      }
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) psum += __shfl_xor_sync(0xffffffffu, psum, o);
-      if (m_new != -INFINITY) {
-        l[r] = l[r] * exp2f(m[r] - m_new) + psum;
+        for (int c = 0; c < 4; ++c) sum += exp2f(s[r][c] - m_new);
+        l[r] = l[r] * exp2f(m[r] - m_new) + sum;
         m[r] = m_new;
       }
     }
   }
-  if (tx == 0) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int qr = q0 + ty + 16 * r;
-      if (qr < P) a.lse2[((size_t)bi * a.n_q_head + hq) * P + qr] = m[r] + log2f(l[r]);
-    }
+  for (int r = 0; r < 4; ++r) {
+    float mm = m[r];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+    float ll = (m[r] > -INFINITY) ? l[r] * exp2f(m[r] - mm) : 0.f;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
+    const int qr = q0 + 4 * ty + r;
+    if (tx == 0 && qr < P) a.lse2[((size_t)bi * a.n_q_head + hq) * P + qr] = mm + log2f(ll);
   }
 }
 
-template <typename T, int D>
-__global__ void __launch_bounds__(256) prefill_col_sum_kernel(ScoreArgs a, float scale_log2) {
-  __shared__ float Qs[TQ][DC + 1], Ks[TK][DC + 1];
-  __shared__ float red[16][TK];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int kt = blockIdx.x, hk = blockIdx.y, bi = blockIdx.z;
+// Grid: (key tile, KV head, sequence * n_piece).  The (head, query tile) pairs that a key tile sees,
+// heads outermost, go to its pieces `chunk` at a time.
+template <typename T, int D, int TQ>
+__global__ void __launch_bounds__(4 * TQ) prefill_col_sum_kernel(ScoreArgs a, float scale_log2, int n_piece, int chunk) {
+  constexpr int NT = 4 * TQ;
+  extern __shared__ __align__(16) float sm[];
+  __shared__ float red[TQ / 4][TK];
+  __shared__ int s_last;
+  float* qs = sm;
+  float* ks = sm + D * (TQ + 4);
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int kt = blockIdx.x, hk = blockIdx.y, bi = blockIdx.z / n_piece, piece = blockIdx.z - bi * n_piece;
   const int g = a.n_q_head / a.n_kv_head, P = a.prompt;
-  const int n_tile = (P + TQ - 1) / TQ;
+  const int n_qt = (P + TQ - 1) / TQ, k0 = kt * TK, qt0 = k0 / TQ, per = n_qt - qt0;
+  const int n_stream = g * per, i0 = piece * chunk, i1 = min(n_stream, i0 + chunk);
+  const int pieces_here = (n_stream + chunk - 1) / chunk;
+  if (i0 >= n_stream) return;
   const T* kbase = reinterpret_cast<const T*>(a.k) + ((size_t)bi * a.n_kv_head + hk) * P * D;
-  const int k0 = kt * TK;
+  const T* qhead0 = reinterpret_cast<const T*>(a.q) + ((size_t)bi * a.n_q_head + hk * g) * P * D;
+  const float* lse0 = a.lse2 + ((size_t)bi * a.n_q_head + hk * g) * P;
+  int h = i0 / per, qt = qt0 + (i0 - h * per);
+  {
+    TileLoad<T, D, TK, NT> kl;
+    kl.fetch(kbase, k0, P);
+    kl.store(ks);
+  }
+  TileLoad<T, D, TQ, NT> ql;
+  ql.fetch(qhead0 + (size_t)h * P * D, qt * TQ, P);
+  grid_wait();  // the inputs are older than the launch ahead, the row sums are its result
   float col[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int h = 0; h < g; ++h) {
-    const int hq = hk * g + h;
-    const T* qbase = reinterpret_cast<const T*>(a.q) + ((size_t)bi * a.n_q_head + hq) * P * D;
-    const float* lse = a.lse2 + ((size_t)bi * a.n_q_head + hq) * P;
-    for (int qt = kt; qt < n_tile; ++qt) {
-      const int q0 = qt * TQ;
-      float s[4][4];
-      score_tile<T, D>(qbase, kbase, q0, k0, P, Qs, Ks, s);
+  for (int i = i0; i < i1; ++i) {
+    const int q0 = qt * TQ;
+    float lse[4];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int qr = q0 + ty + 16 * r;
-        if (qr >= P) continue;
-        const float lr = lse[qr];
+    for (int r = 0; r < 4; ++r) {
+      const int qr = q0 + 4 * ty + r;
+      lse[r] = qr < P ? lse0[(size_t)h * P + qr] : INFINITY;  // a query past the end attends to nothing
+    }
+    __syncthreads();
+    ql.store(qs);
+    __syncthreads();
+    if (++qt == n_qt) {
+      qt = qt0;
+      ++h;
+    }
+    if (i + 1 < i1) ql.fetch(qhead0 + (size_t)h * P * D, qt * TQ, P);
+    float s[4][4];
+    score_tile<D, TQ>(qs, ks, s);
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-          const int kr = k0 + tx + 16 * c;
-          if (kr <= qr) col[c] += exp2f(s[r][c] * scale_log2 - lr);
-        }
+    for (int r = 0; r < 4; ++r) {
+      const int qr = q0 + 4 * ty + r;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const float p = exp2f(s[r][c] * scale_log2 - lse[r]);
+        if (k0 + 4 * tx + c <= qr) col[c] += p;
       }
     }
   }
-  __syncthreads();
 #pragma unroll
-  for (int c = 0; c < 4; ++c) red[ty][tx + 16 * c] = col[c];
+  for (int c = 0; c < 4; ++c) red[ty][4 * tx + c] = col[c];
   __syncthreads();
-  if (threadIdx.x < TK) {
+  const size_t unit = (size_t)bi * a.n_kv_head + hk, stride = (size_t)a.batch * a.n_kv_head * P;
+  const int kr = k0 + tid;
+  if (tid < TK && kr < P) {
     float sum = 0.f;
-    for (int y = 0; y < 16; ++y) sum += red[y][threadIdx.x];
-    const int kr = k0 + threadIdx.x;
-    if (kr < P) a.acc_prompt[((size_t)bi * a.n_kv_head + hk) * P + kr] = sum;
+    for (int y = 0; y < TQ / 4; ++y) sum += red[y][tid];
+    (pieces_here == 1 ? a.acc_prompt : a.partial + piece * stride)[unit * P + kr] = sum;
   }
+  if (pieces_here == 1) return;
+  // the key tile's last piece to finish adds all pieces up, in order (no piece waits)
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) {
+    int* ticket = a.tickets + unit * gridDim.x + kt;
+    s_last = atomicAdd(ticket, 1) == pieces_here - 1;
+    if (s_last) *ticket = 0;
+  }
+  __syncthreads();
+  if (s_last && tid < TK && kr < P) {
+    __threadfence();
+    float sum = 0.f;
+#pragma unroll 8
+    for (int p = 0; p < pieces_here; ++p) sum += __ldcg(a.partial + p * stride + unit * P + kr);
+    a.acc_prompt[unit * P + kr] = sum;
+  }
+}
+
+template <typename T, int D, int TQ>
+static cudaError_t launch_scores_tq(const ScoreArgs& a, cudaStream_t s) {
+  auto k1 = prefill_row_lse_kernel<T, D, TQ>;
+  auto k2 = prefill_col_sum_kernel<T, D, TQ>;
+  constexpr size_t smem = score_smem<D, TQ>();
+  static bool configured = false;
+  if (!configured) {
+    cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    configured = true;
+  }
+  const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
+  const int n_qt = (a.prompt + TQ - 1) / TQ, n_kt = (a.prompt + TK - 1) / TK, g = a.n_q_head / a.n_kv_head;
+  const long long units = (long long)a.batch * a.n_kv_head;
+  // pieces of about an eighth of an SM's share, as far as the scratch and the grid go
+  const long long longest = (long long)g * n_qt, tiles = units * longest * (n_kt + 1) / 2;
+  long long chunk = std::max(1LL, std::min(longest, tiles / (8 * 148)));
+  auto pieces = [&](long long c) { return (longest + c - 1) / c; };
+  while (chunk < longest && (pieces(chunk) * units * a.prompt > (long long)a.partial_floats || pieces(chunk) * a.batch > 65535))
+    chunk = std::min(longest, chunk * 2);
+  cudaError_t e = launch_chained(k1, dim3(n_qt, a.n_q_head, a.batch), 4 * TQ, smem, s, a, scale_log2);
+  if (e != cudaSuccess) return e;
+  return launch_chained(k2, dim3(n_kt, a.n_kv_head, a.batch * (unsigned)pieces(chunk)), 4 * TQ, smem, s, a, scale_log2,
+                        (int)pieces(chunk), (int)chunk);
 }
 
 template <typename T, int D>
 static cudaError_t launch_scores_t(const ScoreArgs& a, cudaStream_t s) {
-  const int n_tile = (a.prompt + TQ - 1) / TQ;
-  const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
-  prefill_row_lse_kernel<T, D><<<dim3(n_tile, a.n_q_head, a.batch), 256, 0, s>>>(a, scale_log2);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  prefill_col_sum_kernel<T, D><<<dim3(n_tile, a.n_kv_head, a.batch), 256, 0, s>>>(a, scale_log2);
-  return cudaGetLastError();
+  // small problems: more and shorter CTAs
+  const long long ctas = (long long)((a.prompt + 63) / 64) * a.n_q_head * a.batch;
+  return ctas < 2 * 148 ? launch_scores_tq<T, D, 32>(a, s) : launch_scores_tq<T, D, 64>(a, s);
 }
 
 // fp32-pipe kernels (any dtype)

@@ -145,7 +145,7 @@ WsLayout ws_layout(const sq_config& c, int64_t b_init) {
   w.cos_sim = take(4 * ND);
   w.status = take(4);
   w.tickets = take(4 * L * U);
-  w.score_tickets = take(c.policy == SQ_POLICY_H2O ? 4 * U * (((size_t)c.max_prompt + 127) / 128) : 0);
+  w.score_tickets = take(c.policy == SQ_POLICY_H2O ? 4 * U * (((size_t)c.max_prompt + 63) / 64) : 0);
   w.layers = take(sizeof(LayerDesc) * ND);
   w.order = take(4 * ND);
   w.order_by_layer = take(4 * ND);

@@ -71,9 +71,9 @@ struct ScoreArgs {  // H2O prompt scores of one layer
   float* lse2;        // [B, Hq, P]  log2-domain row log-sum-exp
   float* acc_prompt;  // [B, Hkv, P]
   int batch, n_q_head, n_kv_head, prompt, head_dim;
-  float* partial;       // scratch for column sums of some heads (tcgen05 kernels), partial_floats of it
+  float* partial;       // scratch for the column sums of a key tile's pieces, partial_floats of it (0: no pieces)
   size_t partial_floats;
-  int* tickets;         // [B * Hkv][ceil(P / 128)] arrival counters, zero between launches
+  int* tickets;         // [B * Hkv][key tiles of 64 or 128] arrival counters, zero between launches
 };
 // How sweep 2 of the prompt scores is cut: pieces of `heads` query heads of a group; with more than
 // one piece, piece p's column sums go to partial + p * B * Hkv * P and the last to finish adds them.

@@ -48,6 +48,9 @@ extern "C" int sq_prompt_scores_static(const void* q_prompt, const void* k_promp
   a.k = k_prompt;
   a.lse2 = scratch;
   a.acc_prompt = acc_out;
+  a.partial = nullptr;
+  a.partial_floats = 0;
+  a.tickets = nullptr;
   a.batch = batch;
   a.n_q_head = n_q_head;
   a.n_kv_head = n_kv_head;

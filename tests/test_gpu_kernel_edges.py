@@ -18,13 +18,14 @@ def workload(name, wid, **kw):
     return synth.Workload(name, wid, **dict(base, **kw))
 
 
-# Prompt scores on the tensor cores: key tiles cut into pieces by heads (as many pieces as heads, a last
-# piece with fewer heads, one piece), one tile, a tile of one key, full and ragged last tiles
+# Prompt scores: key tiles cut into pieces (tensor cores: by heads; as many pieces as heads, a last piece with
+# fewer heads, one piece), one tile, a tile of one key, full and ragged last tiles
 @pytest.mark.parametrize("head_dim,hq,hkv,batch,prompt", [
     (64, 71, 1, 1, 128), (64, 71, 1, 2, 385), (64, 71, 1, 9, 1155), (128, 20, 2, 1, 257), (128, 4, 1, 1, 1), (128, 6, 1, 3, 640),
     (64, 3, 3, 2, 300)])
-def test_prompt_scores_cut_by_heads(head_dim, hq, hkv, batch, prompt):
-    w = workload("edge", 9100 + prompt, head_dim=head_dim, n_q_head=hq, n_kv_head=hkv, batch=batch, prompt=prompt,
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])   # fp32: both tile heights, one and many pieces
+def test_prompt_scores_cut_into_pieces(dtype, head_dim, hq, hkv, batch, prompt):
+    w = workload("edge", 9100 + prompt, dtype=dtype, head_dim=head_dim, n_q_head=hq, n_kv_head=hkv, batch=batch, prompt=prompt,
                  heavy_mode="uniform4" if prompt > 8 else "none")
     ctx = H.make_ctx(w, b_init=prompt)
     for _ in range(2):                                # the second pass finds the pieces' counters as the first left them
