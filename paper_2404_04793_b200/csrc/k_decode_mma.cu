@@ -1,4 +1,5 @@
-// Tensor-core decode attention for grouped / multi-query heads (bf16): with g query heads
+// Tensor-core decode attention for grouped / multi-query heads (bf16; groups of 9 and more, smaller ones in
+// k_decode_mma_low.cu): with g query heads
 // sharing a KV head the step is a dense [g x d] . [d x tokens] contraction (g flop per byte of
 // K/V), too much for the fp32 pipes at HBM speed once g >= 4.  The g heads of a unit are
 // padded to 16-row tiles and run through mma.sync m16n8k16 (bf16 in, fp32 accumulate):
@@ -13,66 +14,10 @@
 #include "sq_decode_common.cuh"
 #include "sq_device.cuh"
 #include "sq_internal.h"
+#include "sq_mma.cuh"
 #include "sq_scores.cuh"
 
 namespace sq {
-
-namespace {
-
-constexpr int kTile = 64;  // tokens per pipeline stage
-constexpr int kScoresSmem = 110 * 1024;  // dynamic shared memory of a CTA with the score update: two CTAs per SM
-constexpr int kMaxPieces = 16;           // CTAs of a cluster (above 8: opt-in)
-// tiles of a piece when a unit of `len` slots is cut into `pieces`
-__host__ __device__ inline int piece_tiles(int len, int pieces) {
-  return ((len + kTile - 1) / kTile + pieces - 1) / pieces;
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid) {
-  const int sz = valid ? 16 : 0;  // 0: the 16 bytes are zero-filled
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(sz));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(N));
-}
-
-__device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
-                                                  uint32_t& r3) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
-               : "r"(addr));
-}
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-
-// two floats -> packed bf16x2 (lo in the low half), and the values the packing kept
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi, float& lo_r, float& hi_r) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  uint32_t u = *reinterpret_cast<uint32_t*>(&v);
-  lo_r = __uint_as_float(u << 16);
-  hi_r = __uint_as_float(u & 0xffff0000u);
-  return u;
-}
-
-template <int D>
-__device__ __forceinline__ uint32_t swz(int row, int chunk) {
-  // byte offset of 16-byte chunk `chunk` of row `row` inside a [rows][D] bf16 tile
-  return (uint32_t)(row * (D * 2) + ((chunk ^ (row & 7)) << 4));
-}
-
-}  // namespace
 
 // SCORES: H2O with the score update in the same launch (sq_scores.cuh): the pieces of a unit are the
 // CTAs of a cluster, piece_tiles(len) tiles each, and the logits stay in shared memory.
@@ -489,7 +434,8 @@ static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t log
 // 385 / 266 (at most eight pieces of two tiles or more: 281), its 16384-token caches 1309 / 560 (their
 // logits do not fit eight pieces: 1138), 4: 451 / 358, 16: 660 / 534 (four pieces per unit, more than fit at
 // once: 629), 64: 1060 / 983; 20 / 1 heads of 64, 64 sequences: 435 / 237; 80 layers of 64 / 8 heads, 4 sequences:
-// 1372 / 859.  All 32 layers in one launch, 4096 units: 322 / 446.
+// 1372 / 859.  All 32 layers in one launch, 4096 units: 322 / 446.  (With the kernel for up to 8 heads
+// k_decode_mma_low.cu gives 1 sequence 231, 4: 309, 16: 480, 64: 877.)
 cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
   const int G = a.group;
   if (G < 2 || G > 32 || (a.head_dim != 64 && a.head_dim != 128)) return cudaErrorNotSupported;
@@ -505,6 +451,7 @@ cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStrea
   while (pieces < 8 && fixed + logit_bytes(pieces) > kScoresSmem) ++pieces;
   const size_t lb = logit_bytes(pieces);
   if (fixed + lb > kScoresSmem) return cudaErrorNotSupported;
+  if (G <= 8) return launch_decode_mma_low(a, 0, pieces, lb, s);
   if (a.head_dim == 128) return G <= 16 ? launch_scores_cfg<128, 1, 3>(a, pieces, lb, s) : launch_scores_cfg<128, 2, 3>(a, pieces, lb, s);
   return G <= 16 ? launch_scores_cfg<64, 1, 4>(a, pieces, lb, s) : launch_scores_cfg<64, 2, 4>(a, pieces, lb, s);
 }
@@ -512,6 +459,7 @@ cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStrea
 // Returns cudaErrorNotSupported when no tensor-core configuration covers the shape.
 cudaError_t launch_decode_attn_mma(const DecodeArgs& a, int n_items, cudaStream_t s) {
   const int G = a.group;
+  if (G <= 8 && (a.head_dim == 64 || a.head_dim == 128)) return launch_decode_mma_low(a, n_items, 0, 0, s);
   if (a.head_dim == 128) {
     // Two stages of 32 KB let three CTAs share an SM, which wins once the launch has CTAs to
     // spare (measured: Mistral- and Llama-2-70B-shaped fused steps 5-9 % faster); a launch of

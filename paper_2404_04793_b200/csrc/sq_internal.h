@@ -175,6 +175,8 @@ cudaError_t launch_decode_attn_tc_stream(const DecodeArgs& a, const int* desc_ti
                                          cudaStream_t s);
 cudaError_t launch_h2o_gain_tc(const DecodeArgs& a, int n_items, size_t pool_bytes, size_t q_rows, cudaStream_t s);
 cudaError_t launch_decode_attn_mma(const DecodeArgs& a, int n_items, cudaStream_t s);
+// groups of at most 8 heads; pieces > 0: H2O with the score update, that many CTAs per unit
+cudaError_t launch_decode_mma_low(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s);
 cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStream_t s);
 cudaError_t launch_evict(const EvictArgs& a, cudaStream_t s);
 
