@@ -501,6 +501,8 @@ __global__ void __launch_bounds__(32 * kWarpUpdWarps, 3) h2o_update_warp_kernel(
 
 template <typename T, int D>
 static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t s) {
+  // (bf16 comes here with more than 32 heads only)
+  if constexpr (sizeof(T) == 2) return launch_chained(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, n_items, 128, 0, s, a);
   const DecodeArgsBase& base = a;
   if (a.group == 1) {
     // the register-capped kernel gets its own build for launches without split-K (which takes no table)
@@ -528,9 +530,7 @@ static cudaError_t launch_scores_kernel(const DecodeArgs& a, int pieces, int n_c
 
 // H2O with the score update in the launch.  Returns cudaErrorNotSupported where the second launch
 // (decode_combine_kernel, h2o_update_warp_kernel) is needed: a piece's logits do not fit.
-// Measured, us per token, second launch / this form: 32 layers of 32 / 32 heads of 128, one launch per layer,
-// 1 sequence 432 / 281, 8: 615 / 485, 40: 775 / 755; all layers in one launch, 8 sequences: 176 / 171; fp32, 12
-// layers of 16 / 4 heads, 8 sequences: 331 / 271.
+// Measured, us per token, second launch / this form: fp32, 12 layers of 16 / 4 heads of 128, 8 sequences: 331 / 271.
 template <typename T, int D>
 static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
   const int G = a.group;
@@ -554,9 +554,10 @@ static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStre
   return launch_scores_kernel<decode_attn_kernel<T, D, 8, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
 }
 
-// Which attention kernel serves a shape: wide bf16 groups at head_dim 64 go to the tcgen05
-// kernel, other grouped bf16 heads to the mma.sync kernel, everything else (fp32, one query head
-// per KV head, shapes those do not cover) to the fp32-pipe kernel.
+// Which attention kernel serves a shape: wide bf16 groups at head_dim 64 go to the tcgen05 kernels, other
+// bf16 heads to the mma.sync kernels (one head per KV head too: 32 layers of 32 / 32 heads of 128, us per token,
+// the kernel of this file / mma.sync: 2 sequences 305 / 198, 8: 417 / 342, 40: 1835 / 1417), fp32 and the bf16 shapes
+// those do not cover to the fp32-pipe kernel.
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
                           size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
@@ -579,12 +580,11 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need
   if (!done && a.policy == SQ_POLICY_H2O && !a.has_logits) return cudaErrorNotSupported;
   if (!done && a.policy == SQ_POLICY_H2O) {
     cudaError_t e;
-    if (dtype == SQ_BF16 && a.group > 1) e = launch_decode_mma_scores(a, max_len, s);
-    else if (dtype == SQ_F32) e = a.head_dim == 64 ? launch_attn_scores<float, 64>(a, max_len, s) : launch_attn_scores<float, 128>(a, max_len, s);
-    else e = a.head_dim == 64 ? launch_attn_scores<__nv_bfloat16, 64>(a, max_len, s) : launch_attn_scores<__nv_bfloat16, 128>(a, max_len, s);
+    if (dtype == SQ_BF16) e = launch_decode_mma_scores(a, max_len, s);
+    else e = a.head_dim == 64 ? launch_attn_scores<float, 64>(a, max_len, s) : launch_attn_scores<float, 128>(a, max_len, s);
     if (e != cudaErrorNotSupported) return e;
   }
-  if (!done && dtype == SQ_BF16 && a.group > 1) {
+  if (!done && dtype == SQ_BF16) {
     cudaError_t e = launch_decode_attn_mma(a, n_items, s);
     if (e == cudaSuccess) done = true;
     else if (e != cudaErrorNotSupported) return e;

@@ -438,7 +438,7 @@ static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t log
 // k_decode_mma_low.cu gives 1 sequence 231, 4: 309, 16: 480, 64: 877.)
 cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
   const int G = a.group;
-  if (G < 2 || G > 32 || (a.head_dim != 64 && a.head_dim != 128)) return cudaErrorNotSupported;
+  if (G > 32 || (a.head_dim != 64 && a.head_dim != 128)) return cudaErrorNotSupported;
   const int n_sm = sm_count();
   const long long units = (long long)a.n_layer_total * a.n_unit;
   if (units >= 6 * n_sm) return cudaErrorNotSupported;

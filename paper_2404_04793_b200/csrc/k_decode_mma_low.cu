@@ -1,4 +1,4 @@
-// Tensor-core decode attention for 2..8 bf16 query heads per KV head (mma.sync m16n8k16).  The heads are the
+// Tensor-core decode attention for 1..8 bf16 query heads per KV head (mma.sync m16n8k16).  The heads are the
 // N side of both products, so no row of a tile is padding (k_decode_mma.cu has them on the M side, 16 rows at
 // a time):
 //   S^T[16 tokens x 8 heads] = K Q^T      (K rows as the A operand, Q as B, kept in registers)
@@ -22,7 +22,10 @@ namespace sq {
 
 // SCORES: H2O with the score update in the same launch (sq_scores.cuh): the pieces of a unit are the CTAs of
 // a cluster and the logits stay in shared memory.
-template <int D, int STAGES, bool SCORES, class Args>
+// ONE: a single head.  Of the eight columns of P^T three are then used to keep the weights at fp32 precision: a
+// weight enters as the sum of three bf16 numbers (columns 0, 1, 2), whose results are added at the end, and
+// the normaliser is the sum of the fp32 weights.
+template <int D, int STAGES, bool SCORES, bool ONE, class Args>
 __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
   constexpr int NT = 128, WN = 4, NH = 8;
   constexpr int CH = D / 8;              // 16-byte chunks per row
@@ -148,7 +151,8 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
   for (int i = tid; i < NH * CH; i += NT) {  // query rows, zero beyond the group
     const int row = i / CH, c = i - row * CH;
     uint4 val = make_uint4(0, 0, 0, 0);
-    if (row < G) val = *reinterpret_cast<const uint4*>(qb + (size_t)row * D + c * 8);
+    // (ONE: the head once more as row 2, so that the threads of column 2 have its weights as well)
+    if (ONE ? (row == 0 || row == 2) : row < G) val = *reinterpret_cast<const uint4*>(qb + (size_t)(ONE ? 0 : row) * D + c * 8);
     *reinterpret_cast<uint4*>(q_s + swz<D>(row, c)) = val;
   }
   __syncthreads();
@@ -229,14 +233,30 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) p[j] = exp2f(v[j] - m[j & 1]);
     }
-    float pr[4];
-    const uint32_t p_lo = pack_bf16(p[0], p[1], pr[0], pr[1]), p_hi = pack_bf16(p[2], p[3], pr[2], pr[3]);
-    const uint32_t b0 = movmatrix_trans(p_lo), b1 = movmatrix_trans(p_hi);
+    uint32_t p_lo, p_hi;  // tokens gq and gq + 8
+    if constexpr (ONE) {
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      l_true[j] += p[j] + p[2 + j];
-      l_w[j] += pr[j] + pr[2 + j];
+      for (int j = 0; j < 2; ++j) {
+        const float x = p[2 * j], x1 = __bfloat162float(__float2bfloat16_rn(x)), r1 = x - x1;
+        const float x2 = __bfloat162float(__float2bfloat16_rn(r1)), x3 = r1 - x2;
+        float d0, d1;
+        const uint32_t u = pack_bf16(tq == 0 ? x1 : tq == 1 ? x3 : 0.f, tq == 0 ? x2 : 0.f, d0, d1);
+        if (j) p_hi = u;
+        else p_lo = u;
+      }
+      l_true[0] += p[0] + p[2];
+      l_w[0] = l_true[0];
+    } else {
+      float pr[4];
+      p_lo = pack_bf16(p[0], p[1], pr[0], pr[1]);
+      p_hi = pack_bf16(p[2], p[3], pr[2], pr[3]);
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        l_true[j] += p[j] + p[2 + j];
+        l_w[j] += pr[j] + pr[2 + j];
+      }
     }
+    const uint32_t b0 = movmatrix_trans(p_lo), b1 = movmatrix_trans(p_hi);
     // ---- O^T += V^T P^T ----
 #pragma unroll
     for (int d = 0; d < KS; ++d) {
@@ -295,7 +315,14 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
       f[x] = (f[x] > -INFINITY) ? exp2f(f[x] - M) : 0.f;
       Lt += row[D + 1] * f[x];
       Lw += row[D + 2] * f[x];
-      const float4 v = *reinterpret_cast<const float4*>(row + e);
+      float4 v = *reinterpret_cast<const float4*>(row + e);
+      if constexpr (ONE) {
+        const float4 v1 = *reinterpret_cast<const float4*>(row + (D + 4) + e), v2 = *reinterpret_cast<const float4*>(row + 2 * (D + 4) + e);
+        v.x += v1.x + v2.x;
+        v.y += v1.y + v2.y;
+        v.z += v1.z + v2.z;
+        v.w += v1.w + v2.w;
+      }
       O.x += v.x * f[x];
       O.y += v.y * f[x];
       O.z += v.z * f[x];
@@ -328,11 +355,11 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
   }
 }
 
-template <int D, int STAGES>
+template <int D, int STAGES, bool ONE>
 static cudaError_t launch_low_cfg(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s) {
   constexpr size_t pipe = (size_t)2 * STAGES * kTile * D * 2;
-  auto plain = decode_attn_mma_low_kernel<D, STAGES, false, DecodeArgs>;
-  auto scores = decode_attn_mma_low_kernel<D, STAGES, true, DecodeArgsBase>;
+  auto plain = decode_attn_mma_low_kernel<D, STAGES, false, ONE, DecodeArgs>;
+  auto scores = decode_attn_mma_low_kernel<D, STAGES, true, ONE, DecodeArgsBase>;
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pipe);
@@ -347,13 +374,18 @@ static cudaError_t launch_low_cfg(const DecodeArgs& a, int n_items, int pieces, 
   return launch_chained(plain, n_items, 128, pipe, s, a);
 }
 
-cudaError_t launch_decode_mma_low(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s) {
-  if (a.head_dim == 64) return launch_low_cfg<64, 4>(a, n_items, pieces, logit_bytes, s);
+template <bool ONE>
+static cudaError_t launch_low(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s) {
+  if (a.head_dim == 64) return launch_low_cfg<64, 4, ONE>(a, n_items, pieces, logit_bytes, s);
   // Two stages of 32 KB let three CTAs share an SM, which wins once the launch has CTAs to spare; a launch of
   // about one wave (one layer at a time) is better off with the deeper ring per CTA.  us per token, three /
   // two stages: 800 units per layer 305 / 277, 512: 694 / 797, 256: 2109 / 2372.
-  if (pieces == 0 && n_items >= 5 * 148) return launch_low_cfg<128, 2>(a, n_items, 0, 0, s);
-  return launch_low_cfg<128, 3>(a, n_items, pieces, logit_bytes, s);
+  if (pieces == 0 && n_items >= 5 * 148) return launch_low_cfg<128, 2, ONE>(a, n_items, 0, 0, s);
+  return launch_low_cfg<128, 3, ONE>(a, n_items, pieces, logit_bytes, s);
+}
+
+cudaError_t launch_decode_mma_low(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s) {
+  return a.group == 1 ? launch_low<true>(a, n_items, pieces, logit_bytes, s) : launch_low<false>(a, n_items, pieces, logit_bytes, s);
 }
 
 }  // namespace sq

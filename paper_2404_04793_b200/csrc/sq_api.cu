@@ -622,7 +622,7 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
       // us per token, 32 layers, (setup, merge, gain) = (8, 0, 0.90) / (8, 0, 0.95) / (4, 4, 0.95): 33 sequences of
       // 8191, 50 %, H2O 1278 / 1217 / 1217; 60 of 4000, 30 % 548 / 667 / 540; 8 of 8191, 30 %, H2O 1028 / 1098 / 1045
       tile = 128, setup = 4, merge = 4, per_sm = 2, gain = 0.95;
-    } else if (bf16 && G > 1) {                  // mma.sync kernel: 64-token tiles
+    } else if (bf16) {                           // mma.sync kernels: 64-token tiles
       tile = 64, setup = 12, per_sm = cfg.head_dim == 64 && G <= 32 ? 3 : 2;
     } else {                                     // fp32-pipe kernel
       tile = 128, setup = 1, per_sm = G == 1 ? 7 : 2;

@@ -97,6 +97,37 @@ def test_layer_by_layer_launches_match_the_whole_stack(policy, dtype, head_dim, 
     assert stack.status() == 0 and chained.status() == 0
 
 
+# One bf16 head per KV head keeps its weights at fp32 precision on the tensor cores: with fp32-exact weights
+# only the order of the fp32 sums and the bf16 output (half an ulp, 2^-9) separate it from the oracle, where
+# bf16 weights would add 2^-9 of the largest term.  Keys that make one weight dominate, after the first
+# tile too (the reference moves), lengths around a tile and a warp's share of it
+@pytest.mark.parametrize("head_dim,budget", [(128, 1), (128, 17), (128, 64), (128, 65), (64, 300), (128, 1500)])
+@pytest.mark.parametrize("hq", [3, 24])
+def test_one_and_eight_heads_per_kv_head(head_dim, budget, hq):
+    w = workload("one", 9500 + budget, policy=synth.SLIDING_WINDOW, head_dim=head_dim, n_q_head=hq, n_kv_head=3, batch=1,
+                 prompt=budget + 3, steps=2, heavy_mode="none")
+    ctx = H.make_ctx(w, b_init=budget)
+    ctx.begin_sequence_batch(1, w.prompt)
+    ctx.set_budgets([budget])
+    _, k, v = synth.prompt_qkv(w, 0, DEV, need_q=False)
+    k[:, :, 2 * w.prompt // 3:] *= 24.0
+    ctx.prefill_compress(0, k, v)
+    units = [O.UnitCache(w.policy, budget) for _ in range(3)]
+    for h, u in enumerate(units):
+        u.prefill(H.f64(k[0, h]), H.f64(v[0, h]))
+    for t in range(w.steps):
+        q, kn, vn = synth.decode_qkv(w, t, DEV)
+        out = torch.empty_like(q)
+        ctx.decode_step(0, 1, q, kn, vn, out)
+        for h, u in enumerate(units):
+            g = w.group
+            want = u.decode_step(H.f64(q[0, 0, h * g:(h + 1) * g]), H.f64(kn[0, 0, h]), H.f64(vn[0, 0, h]))
+            got = H.f64(out[0, 0, h * g:(h + 1) * g])
+            bound = np.abs(want) * 2.0 ** -8 + 1e-4 if g == 1 else np.maximum(H.TOL_OUT[w.dtype], np.abs(want) * 2.0 ** -7)
+            assert np.all(np.abs(got - want) <= bound), (t, h, np.max(np.abs(got - want)))
+    assert ctx.status() == 0
+
+
 # H2O with the score update inside the attention launch: pieces of a unit on the CTAs of a cluster, with
 # empty and ragged pieces, short and long layers, groups that are and are not multiples of four, both
 # head dims, and units too long or too many for it
