@@ -216,20 +216,24 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
     for (int j = 0; j < 4; ++j) p[j] = exp2f(v[j] - m[j & 1]);
     if (__any_sync(kFull, fmaxf(fmaxf(p[0], p[1]), fmaxf(p[2], p[3])) > 65536.f)) {
       // rare: move the references; what is there so far shrinks with them
-      float mx[2];
+      float mx[2], f[2];
       head_max(v, mx);
 #pragma unroll
       for (int j = 0; j < 2; ++j) {
-        const float m_new = fmaxf(m[j], mx[j]), f = exp2f(m[j] - m_new);
+        const float m_new = fmaxf(m[j], mx[j]);
+        f[j] = exp2f(m[j] - m_new);
         m[j] = m_new;
-        l_true[j] *= f;
-        l_w[j] *= f;
+        l_true[j] *= f[j];
+        l_w[j] *= f[j];
+      }
+      if constexpr (ONE) f[1] = f[0];  // column 1 is the head of column 0
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
 #pragma unroll
         for (int d = 0; d < KS; ++d) {
-          o[d][j] *= f;
-          o[d][2 + j] *= f;
+          o[d][j] *= f[j];
+          o[d][2 + j] *= f[j];
         }
-      }
 #pragma unroll
       for (int j = 0; j < 4; ++j) p[j] = exp2f(v[j] - m[j & 1]);
     }
