@@ -209,3 +209,29 @@ def test_prompt_selection_edges(prompt, hn, hd):
             list(range(len(pos) + 1))
         assert ctx.get_kept(l, s, 0)[0] == [(pos + [prompt])[i] for i in keep], (l, s)
     assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("hidden,tokens", [(64, 1), (128, 63), (128, 20011), (256, 65), (264, 9)])
+def test_importance_of_short_rows(dtype, hidden, tokens):
+    """Rows of up to 512 bytes, several per warp; a last group of rows that is not full; rows just longer."""
+    w = synth.Workload("short rows", 61, n_layer=1, n_q_head=2, n_kv_head=2, head_dim=64, hidden=hidden, batch=1, prompt=tokens,
+                       steps=1, dtype=dtype, policy=synth.SLIDING_WINDOW, budget_pct=100.0, p=1.0)
+    g = torch.Generator().manual_seed(tokens + hidden)
+    a, d = (torch.randn(tokens, hidden, generator=g).to(dtype) for _ in range(2))
+    stored = (a.float() + d.float()).to(dtype)
+    x, y = a.double(), stored.double()
+    want = float((x * y).sum(1).div(x.norm(dim=1) * y.norm(dim=1)).mean())
+    for fused in (False, True):
+        ctx = H.make_ctx(w)
+        ctx.begin_sequence_batch(1, tokens)
+        if fused:
+            out = torch.full((tokens, hidden), float("nan"), dtype=dtype, device=DEV)
+            ctx.layer_importance_fused(0, a.to(DEV), d.to(DEV), out)
+            assert torch.equal(out.cpu(), stored)
+        else:
+            ctx.layer_importance(0, a.to(DEV), stored.to(DEV))
+        ctx.allocate_budgets(tokens, 1.0)
+        # three fp32 sums of `hidden` products each and the mean of the fp32 cosines: at most (hidden + warps' rows) ulp
+        assert abs(float(ctx.get_cos_sim()[0]) - want) <= (hidden + 64) * 2.0 ** -23
+        assert ctx.status() == 0
