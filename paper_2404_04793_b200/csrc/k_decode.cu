@@ -1,7 +1,8 @@
 // Decode step of Algorithm 1 (steps 15-22) for a range of layers in one launch: append the new
 // token into the slot C_seq frees, attend over the kept slots (split-K flash-decode, all query
 // heads of a KV head share one pass over K/V), and for H2O add the received probabilities to
-// the per-token scores and choose the slot the next append will reuse.
+// the per-token scores and choose the slot the next append will reuse.  This file: the dispatch, and
+// the kernel on the fp32 pipes (fp32 inputs, and bf16 groups that no tensor-core kernel takes).
 #include <algorithm>
 #include <cstdlib>
 #include <cstring>
