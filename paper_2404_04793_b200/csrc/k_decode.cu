@@ -35,6 +35,9 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   constexpr int LPR = D / EPV;   // lanes per row
   constexpr int RPW = 32 / LPR;  // rows per warp per load
   constexpr int U = 4;           // rows in flight per lane
+  // Rows ahead of grid_wait() for a single head only: the registers that hold them cost a grouped head more
+  // (four heads 162 -> 184 registers, three CTAs per SM -> two) than a launch's start-up.
+  constexpr bool AHEAD = GT == 1;
   __shared__ float sm_o[NW][GT][D];
   __shared__ float sm_m[NW][GT], sm_l[NW][GT];
 
@@ -50,7 +53,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   const int unit = it.local / it.n_split;
   const int len = min(a.n_tok + 1, b);
   const bool h2o = SCORES || (a.policy == SQ_POLICY_H2O);
-  if (!a.early) grid_wait();
+  if (!AHEAD || !a.early) grid_wait();
   int w;  // slot that receives the new token
   if (h2o) {
     w = (a.n_tok < b) ? a.n_tok : __ldcg(reinterpret_cast<const int*>(a.pool + ldp->victim_off) + unit);
@@ -102,7 +105,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
       vq[u] = ld_stream(vp + sub * EPV);
     }
   };
-  if (a.early) {
+  if (AHEAD && a.early) {
     const int r0 = t0 + warp * (U * RPW);
     if (t0 < t1) load_rows(r0, false);
     grid_wait();
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
       }
     }
     for (int r0 = t0 + warp * (U * RPW); r0 < t1; r0 += NW * U * RPW) {
-      if (!(a.early && hb == 0 && r0 == t0 + warp * (U * RPW))) load_rows(r0, true);
+      if (!(AHEAD && a.early && hb == 0 && r0 == t0 + warp * (U * RPW))) load_rows(r0, true);
       float s[U][GT];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -270,7 +273,7 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
     __shared__ ScoreShared<kMaxPieces> sh;
     finish_scores<T, D, NW * 32, kMaxPieces>(a, ldp, unit, t0, t1, len, ob, logit + (size_t)t0 * a.group, part_o, part_stat, sh, nullptr, w);
   } else {
-    if (!h2o && it.n_split > 1) merge_if_last<T, (GT == 1 ? 1 : 2)>(a, it, unit, &sm_o[0][0][0]);
+    if (!h2o && it.n_split > 1) merge_if_last<T, 1>(a, it, unit, &sm_o[0][0][0]);
   }
 }
 
