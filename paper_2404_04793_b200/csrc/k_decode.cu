@@ -35,9 +35,11 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   constexpr int LPR = D / EPV;   // lanes per row
   constexpr int RPW = 32 / LPR;  // rows per warp per load
   constexpr int U = 4;           // rows in flight per lane
-  // Rows ahead of grid_wait() for a single head only: the registers that hold them cost a grouped head more
-  // (four heads 162 -> 184 registers, three CTAs per SM -> two) than a launch's start-up.
-  constexpr bool AHEAD = GT == 1;
+  // Rows ahead of grid_wait() where the registers that hold them do not cost more than a launch's start-up: with four
+  // heads and no score update they take 162 registers to 184, three CTAs per SM to two (12 layers of 16 / 4 heads,
+  // 40 sequences, one launch: 446 us with rows ahead and a wider merge, 311 without; with the score update, 8 sequences,
+  // one launch per layer: 329 with, 340 without; 80 layers of 64 / 8 heads, 2 sequences, the same: 2352 with, 2315 without).
+  constexpr bool AHEAD = GT == 1 || (GT == 4 && SCORES);
   __shared__ float sm_o[NW][GT][D];
   __shared__ float sm_m[NW][GT], sm_l[NW][GT];
 
