@@ -22,10 +22,13 @@ namespace sq {
 
 // SCORES: H2O with the score update in the same launch (sq_scores.cuh): the pieces of a unit are the CTAs of
 // a cluster and the logits stay in shared memory.
-// ONE: a single head.  Of the eight columns of P^T three are then used to keep the weights at fp32 precision: a
-// weight enters as the sum of three bf16 numbers (columns 0, 1, 2), whose results are added at the end, and
-// the normaliser is the sum of the fp32 weights.
-template <int D, int STAGES, bool SCORES, bool ONE, class Args>
+// A reference that stays leaves the largest weight anywhere up to 2^16, where a running maximum makes it 1, exact in
+// bf16.  So a weight enters the second product as a sum of bf16 numbers, and the normaliser is the sum of the
+// fp32 weights.  HEADS: 1: three parts (fp32 precision), in the columns 0, 1, 2 of P^T; 4: up to four heads, two parts, head h in
+// the columns h and h + 4; 8: two parts, the second by a product of its own.  Error of the outputs against fp64 (2-norm; bf16 rounding
+// of the outputs alone gives 1.66e-3), 32 / 8 heads of 128, caches of 5000: one part under a running maximum 1.73e-3, one
+// under a fixed reference 2.20e-3, two 1.67e-3 (80 layers of 64 / 8 heads, 32 sequences: 2142 us per token with one, 2164 with two).
+template <int D, int STAGES, bool SCORES, int HEADS, class Args>
 __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
   constexpr int NT = 128, WN = 4, NH = 8;
   constexpr int CH = D / 8;              // 16-byte chunks per row
@@ -151,8 +154,9 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
   for (int i = tid; i < NH * CH; i += NT) {  // query rows, zero beyond the group
     const int row = i / CH, c = i - row * CH;
     uint4 val = make_uint4(0, 0, 0, 0);
-    // (ONE: the head once more as row 2, so that the threads of column 2 have its weights as well)
-    if (ONE ? (row == 0 || row == 2) : row < G) val = *reinterpret_cast<const uint4*>(qb + (size_t)(ONE ? 0 : row) * D + c * 8);
+    // (a head stands once more in the row of its other parts, so that the threads of that column have its weights as well)
+    const int h = HEADS == 1 ? (row == 2 ? 0 : row) : HEADS == 4 ? row & 3 : row;
+    if (h < G) val = *reinterpret_cast<const uint4*>(qb + (size_t)h * D + c * 8);
     *reinterpret_cast<uint4*>(q_s + swz<D>(row, c)) = val;
   }
   __syncthreads();
@@ -162,7 +166,7 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
     ldmatrix_x4(smem_u32(q_s + swz<D>(r8, 2 * ks + mi)), qf[ks][0], qf[ks][1], qf[ks + 1][0], qf[ks + 1][1]);
 
   // this thread's heads are 2 tq and 2 tq + 1; of O^T it holds the rows gq and gq + 8 of each block
-  float o[KS][4], m[2] = {-INFINITY, -INFINITY}, l_true[2] = {0.f, 0.f}, l_w[2] = {0.f, 0.f};
+  float o[KS][4], m[2] = {-INFINITY, -INFINITY}, l[2] = {0.f, 0.f};
 #pragma unroll
   for (int d = 0; d < KS; ++d)
 #pragma unroll
@@ -223,10 +227,9 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
         const float m_new = fmaxf(m[j], mx[j]);
         f[j] = exp2f(m[j] - m_new);
         m[j] = m_new;
-        l_true[j] *= f[j];
-        l_w[j] *= f[j];
+        l[j] *= f[j];
       }
-      if constexpr (ONE) f[1] = f[0];  // column 1 is the head of column 0
+      if constexpr (HEADS == 1) f[1] = f[0];  // column 1 is the head of column 0
 #pragma unroll
       for (int j = 0; j < 2; ++j)
 #pragma unroll
@@ -237,46 +240,43 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
 #pragma unroll
       for (int j = 0; j < 4; ++j) p[j] = exp2f(v[j] - m[j & 1]);
     }
-    uint32_t p_lo, p_hi;  // tokens gq and gq + 8
-    if constexpr (ONE) {
+    uint32_t pa[2], pb[2];  // tokens gq and gq + 8: the weights' parts, and with HEADS == 8 their second parts
 #pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const float x = p[2 * j], x1 = __bfloat162float(__float2bfloat16_rn(x)), r1 = x - x1;
+    for (int j = 0; j < 2; ++j) {
+      const float x = p[2 * j], y = p[2 * j + 1];
+      float xr, yr, d0, d1;
+      if constexpr (HEADS == 1) {
+        const float x1 = __bfloat162float(__float2bfloat16_rn(x)), r1 = x - x1;
         const float x2 = __bfloat162float(__float2bfloat16_rn(r1)), x3 = r1 - x2;
-        float d0, d1;
-        const uint32_t u = pack_bf16(tq == 0 ? x1 : tq == 1 ? x3 : 0.f, tq == 0 ? x2 : 0.f, d0, d1);
-        if (j) p_hi = u;
-        else p_lo = u;
+        pa[j] = pack_bf16(tq == 0 ? x1 : tq == 1 ? x3 : 0.f, tq == 0 ? x2 : 0.f, d0, d1);
+      } else {
+        pa[j] = pack_bf16(x, y, xr, yr);
+        const uint32_t rest = pack_bf16(x - xr, y - yr, d0, d1);
+        if constexpr (HEADS == 4) pa[j] = tq < 2 ? pa[j] : rest;
+        else pb[j] = rest;
       }
-      l_true[0] += p[0] + p[2];
-      l_w[0] = l_true[0];
-    } else {
-      float pr[4];
-      p_lo = pack_bf16(p[0], p[1], pr[0], pr[1]);
-      p_hi = pack_bf16(p[2], p[3], pr[2], pr[3]);
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        l_true[j] += p[j] + p[2 + j];
-        l_w[j] += pr[j] + pr[2 + j];
-      }
+      l[j] += p[j] + p[2 + j];
     }
-    const uint32_t b0 = movmatrix_trans(p_lo), b1 = movmatrix_trans(p_hi);
+    const uint32_t a0 = movmatrix_trans(pa[0]), a1 = movmatrix_trans(pa[1]);
+    uint32_t b0 = 0, b1 = 0;
+    if constexpr (HEADS == 8) {
+      b0 = movmatrix_trans(pb[0]);
+      b1 = movmatrix_trans(pb[1]);
+    }
     // ---- O^T += V^T P^T ----
 #pragma unroll
     for (int d = 0; d < KS; ++d) {
       uint32_t vf[4];
       ldmatrix_x4_trans(vst + swz<D>(wn * 16 + (mi >> 1) * 8 + r8, 2 * d + (mi & 1)), vf[0], vf[1], vf[2], vf[3]);
-      mma_bf16(o[d], vf, b0, b1);
+      mma_bf16(o[d], vf, a0, a1);
+      if constexpr (HEADS == 8) mma_bf16(o[d], vf, b0, b1);
     }
   }
   cp_async_wait<0>();
 #pragma unroll
   for (int j = 0; j < 2; ++j)
 #pragma unroll
-    for (int off = 4; off < 32; off <<= 1) {
-      l_true[j] += __shfl_xor_sync(kFull, l_true[j], off);
-      l_w[j] += __shfl_xor_sync(kFull, l_w[j], off);
-    }
+    for (int off = 4; off < 32; off <<= 1) l[j] += __shfl_xor_sync(kFull, l[j], off);
   ScoreAhead ahead;
   if constexpr (SCORES)
     fetch_scores<NT>(ahead, reinterpret_cast<const float*>(a.pool + ldp->acc_off) + (size_t)unit * cap,
@@ -295,8 +295,7 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
       for (int j = 0; j < 2; ++j) {
         float* row = slot + (2 * tq + j) * (D + 4) + D;
         row[0] = m[j];
-        row[1] = l_true[j];
-        row[2] = l_w[j];
+        row[1] = l[j];
       }
   }
   __syncthreads();
@@ -311,22 +310,26 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
       f[x] = mg[x * SLOT + h * (D + 4) + D];
       M = fmaxf(M, f[x]);
     }
-    float Lt = 0.f, Lw = 0.f;
+    float L = 0.f;
     float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int x = 0; x < WN; ++x) {
       const float* row = mg + x * SLOT + h * (D + 4);
       f[x] = (f[x] > -INFINITY) ? exp2f(f[x] - M) : 0.f;
-      Lt += row[D + 1] * f[x];
-      Lw += row[D + 2] * f[x];
+      L += row[D + 1] * f[x];
       float4 v = *reinterpret_cast<const float4*>(row + e);
-      if constexpr (ONE) {
-        const float4 v1 = *reinterpret_cast<const float4*>(row + (D + 4) + e), v2 = *reinterpret_cast<const float4*>(row + 2 * (D + 4) + e);
-        v.x += v1.x + v2.x;
-        v.y += v1.y + v2.y;
-        v.z += v1.z + v2.z;
-        v.w += v1.w + v2.w;
+      [[maybe_unused]] auto add = [&](int other) {  // the result of another part of the weights
+        const float4 u = *reinterpret_cast<const float4*>(row + other * (D + 4) + e);
+        v.x += u.x;
+        v.y += u.y;
+        v.z += u.z;
+        v.w += u.w;
+      };
+      if constexpr (HEADS == 1) {
+        add(1);
+        add(2);
       }
+      if constexpr (HEADS == 4) add(4);
       O.x += v.x * f[x];
       O.y += v.y * f[x];
       O.z += v.z * f[x];
@@ -334,10 +337,10 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
     }
     if constexpr (SCORES) {
       *reinterpret_cast<float4*>(part_o + h * D + e) = O;
-      if (e == 0) *reinterpret_cast<float4*>(part_stat + h * 4) = make_float4(M, Lt, Lw, 0.f);
+      if (e == 0) *reinterpret_cast<float4*>(part_stat + h * 4) = make_float4(M, L, L, 0.f);
     } else {
       if (n_split == 1) {
-        const float inv = 1.f / Lw;
+        const float inv = 1.f / L;
         const __nv_bfloat162 lo = __floats2bfloat162_rn(O.x * inv, O.y * inv), hi = __floats2bfloat162_rn(O.z * inv, O.w * inv);
         uint2 pk;
         pk.x = *reinterpret_cast<const unsigned*>(&lo);
@@ -347,7 +350,7 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
         *reinterpret_cast<float4*>(a.part_o + (size_t)blockIdx.x * G * D + h * D + e) = O;
       }
       if (e == 0)
-        *reinterpret_cast<float4*>(a.part_stat + ((size_t)blockIdx.x * G + h) * kStatStride) = make_float4(M, Lt, Lw, 0.f);
+        *reinterpret_cast<float4*>(a.part_stat + ((size_t)blockIdx.x * G + h) * kStatStride) = make_float4(M, L, L, 0.f);
     }
   }
   if constexpr (SCORES) {
@@ -359,11 +362,11 @@ __global__ void __launch_bounds__(128) decode_attn_mma_low_kernel(Args a) {
   }
 }
 
-template <int D, int STAGES, bool ONE>
+template <int D, int STAGES, int HEADS>
 static cudaError_t launch_low_cfg(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s) {
   constexpr size_t pipe = (size_t)2 * STAGES * kTile * D * 2;
-  auto plain = decode_attn_mma_low_kernel<D, STAGES, false, ONE, DecodeArgs>;
-  auto scores = decode_attn_mma_low_kernel<D, STAGES, true, ONE, DecodeArgsBase>;
+  auto plain = decode_attn_mma_low_kernel<D, STAGES, false, HEADS, DecodeArgs>;
+  auto scores = decode_attn_mma_low_kernel<D, STAGES, true, HEADS, DecodeArgsBase>;
   static bool configured = false;
   if (!configured) {
     cudaError_t e = cudaFuncSetAttribute(plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pipe);
@@ -378,18 +381,19 @@ static cudaError_t launch_low_cfg(const DecodeArgs& a, int n_items, int pieces, 
   return launch_chained(plain, n_items, 128, pipe, s, a);
 }
 
-template <bool ONE>
+template <int HEADS>
 static cudaError_t launch_low(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s) {
-  if (a.head_dim == 64) return launch_low_cfg<64, 4, ONE>(a, n_items, pieces, logit_bytes, s);
+  if (a.head_dim == 64) return launch_low_cfg<64, 4, HEADS>(a, n_items, pieces, logit_bytes, s);
   // Two stages of 32 KB let three CTAs share an SM, which wins once the launch has CTAs to spare; a launch of
   // about one wave (one layer at a time) is better off with the deeper ring per CTA.  us per token, three /
   // two stages: 800 units per layer 305 / 277, 512: 694 / 797, 256: 2109 / 2372.
-  if (pieces == 0 && n_items >= 5 * 148) return launch_low_cfg<128, 2, ONE>(a, n_items, 0, 0, s);
-  return launch_low_cfg<128, 3, ONE>(a, n_items, pieces, logit_bytes, s);
+  if (pieces == 0 && n_items >= 5 * 148) return launch_low_cfg<128, 2, HEADS>(a, n_items, 0, 0, s);
+  return launch_low_cfg<128, 3, HEADS>(a, n_items, pieces, logit_bytes, s);
 }
 
 cudaError_t launch_decode_mma_low(const DecodeArgs& a, int n_items, int pieces, size_t logit_bytes, cudaStream_t s) {
-  return a.group == 1 ? launch_low<true>(a, n_items, pieces, logit_bytes, s) : launch_low<false>(a, n_items, pieces, logit_bytes, s);
+  if (a.group == 1) return launch_low<1>(a, n_items, pieces, logit_bytes, s);
+  return a.group <= 4 ? launch_low<4>(a, n_items, pieces, logit_bytes, s) : launch_low<8>(a, n_items, pieces, logit_bytes, s);
 }
 
 }  // namespace sq

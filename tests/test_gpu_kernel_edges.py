@@ -128,6 +128,53 @@ def test_one_and_eight_heads_per_kv_head(head_dim, budget, hq):
     assert ctx.status() == 0
 
 
+# The largest weight of a softmax enters the product exactly: it is 1 under a running maximum (or the maximum of the
+# first tile), and where the reference stays behind, the weights have more than a bf16's bits.  One key takes a
+# good half of the weight, in the second half of a wide tile and past the first tiles of the others; its value
+# and the others' nearly cancel, so that the bf16 output does not hide the weights.
+@pytest.mark.parametrize("head_dim,group", [(128, 1), (64, 2), (128, 3), (128, 4), (64, 5), (128, 8), (128, 9), (64, 32)])
+@pytest.mark.parametrize("policy", [synth.SLIDING_WINDOW, synth.H2O])
+def test_the_largest_weight_is_not_rounded(policy, head_dim, group):
+    n, at = 128, 100
+    w = workload("peak", 9600 + group, policy=policy, head_dim=head_dim, n_q_head=group, n_kv_head=1, prompt=n, steps=1, heavy_mode="none")
+    g = torch.Generator().manual_seed(group)
+    rnd = lambda *s: torch.randn(*s, generator=g)
+    u = rnd(head_dim)
+    u /= u.norm()
+    k = rnd(1, 1, n + 1, head_dim) * 0.5
+    k -= (k @ u).unsqueeze(-1) * u
+    k[0, 0, at] = u * 8.0
+    x = np.log(n) + (torch.rand(group, generator=g) - 0.5)              # its logit
+    q = rnd(1, 1, group, head_dim)
+    q += (x * head_dim ** 0.5 / 8.0).view(1, 1, group, 1) * u - (q @ u).unsqueeze(-1) * u
+    v = rnd(1, 1, n + 1, head_dim) * 0.3
+    v[0, 0, :] -= 1.0
+    v[0, 0, at] = 1.0 + rnd(head_dim) * 0.1
+    q, k, v = (t.to(torch.bfloat16).to(DEV) for t in (q, k, v))
+    ctx = H.make_ctx(w, b_init=n + 8)
+    ctx.begin_sequence_batch(1, n)
+    ctx.set_budgets([n + 8])
+    ctx.prefill_compress(0, k[:, :, :n].contiguous(), v[:, :, :n].contiguous(), None,
+                         torch.zeros(1, 1, n, device=DEV) if policy == synth.H2O else None)
+    out = torch.empty_like(q)
+    ctx.decode_step(0, 1, q, k[:, :, n:].contiguous(), v[:, :, n:].contiguous(), out)
+    s = H.f64(q[0, 0]) @ H.f64(k[0, 0]).T / head_dim ** 0.5
+    p = np.exp(s - s.max(1, keepdims=True))
+    p /= p.sum(1, keepdims=True)
+    assert np.all(s.argmax(1) == at)
+    vv = H.f64(v[0, 0])
+    want = p @ vv
+    rest = p.copy()
+    rest[:, at] = 0.0
+    # independent roundings of the other weights: 2^-8 / sqrt(3) of each at most (rms), five of them for the extreme
+    # of some thousand outputs; half an ulp of the output; fp32 sums
+    var = (rest ** 2) @ vv ** 2 - 2 * want * ((rest ** 2) @ vv) + want ** 2 * (rest ** 2).sum(1, keepdims=True)
+    bound = 5 * 2.0 ** -8 / 3 ** 0.5 * np.sqrt(np.maximum(var, 0)) + 2.0 ** -8 * np.abs(want) + 2e-5
+    err = np.abs(H.f64(out[0, 0]) - want)
+    assert np.all(err <= bound), float((err / bound).max())
+    assert ctx.status() == 0
+
+
 # H2O with the score update inside the attention launch: pieces of a unit on the CTAs of a cluster, with
 # empty and ragged pieces, short and long layers, groups that are and are not multiples of four, both
 # head dims, and units too long or too many for it
