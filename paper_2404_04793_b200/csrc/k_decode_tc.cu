@@ -15,7 +15,7 @@
 // in tensor memory (64 columns) removes 56 KB of shared-memory traffic per tile.  Inside the
 // kernel, two CTAs sharing the pipe, an MMA holds the issuing thread for about 80 cycles and a
 // tcgen05.commit for about 180.
-// A row's reference m_ref is its maximum over the first 64 tokens; later tiles reuse it and only
+// A row's reference m_ref is its maximum over the first tile; later tiles reuse it and only
 // when a weight would exceed 2^16 is the reference moved (O and the sums rescaled through
 // tcgen05.ld/st, the tile redone): every weight stays finite and the result is that of the
 // exact softmax.  Every barrier wait is bounded.

@@ -26,7 +26,7 @@
 // with the A operand in tensor memory, 68 with both operands in shared memory (whatever their
 // major-ness), and operands read from shared memory compete with the TMA writes for its
 // 128 B/clk; keeping P in tensor memory removes 56 KB of shared-memory traffic per tile.
-// A row's reference m_ref is its maximum over the segment's first 64 tokens; later tiles reuse it and
+// A row's reference m_ref is its maximum over the segment's first tile; later tiles reuse it and
 // only when a weight would exceed 2^16 is the reference moved (O and the sums rescaled through
 // tcgen05.ld/st, the tile redone): every weight stays finite and the result is that of the
 // exact softmax.  Every barrier wait is bounded.

@@ -132,7 +132,7 @@ def test_one_and_eight_heads_per_kv_head(head_dim, budget, hq):
 # first tile), and where the reference stays behind, the weights have more than a bf16's bits.  One key takes a
 # good half of the weight, in the second half of a wide tile and past the first tiles of the others; its value
 # and the others' nearly cancel, so that the bf16 output does not hide the weights.
-@pytest.mark.parametrize("head_dim,group", [(128, 1), (64, 2), (128, 3), (128, 4), (64, 5), (128, 8), (128, 9), (64, 32)])
+@pytest.mark.parametrize("head_dim,group", [(128, 1), (64, 2), (128, 3), (128, 4), (64, 5), (128, 8), (128, 9), (64, 32), (64, 36), (64, 71), (64, 128)])
 @pytest.mark.parametrize("policy", [synth.SLIDING_WINDOW, synth.H2O])
 def test_the_largest_weight_is_not_rounded(policy, head_dim, group):
     n, at = 128, 100
