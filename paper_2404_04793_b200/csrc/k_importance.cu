@@ -8,8 +8,9 @@
 namespace sq {
 
 // One warp per token: streams the token's two hidden-state rows once, keeps the three sums
-// (A.B, A.A, B.B) in fp32 registers, and adds the token's cosine to the warp's running sum.
-// CTA sums go to cta_partial; the CTA that finishes last adds them up in index order (fp64),
+// (A.B, A.A, B.B) in fp32 registers, and adds the token's cosine to the warp's running sum (fp64: with few
+// warps a sum runs over many tokens; in fp32 the mean of 3 million was off by 3.7e-8).
+// CTA sums go to cta_partial; the CTA that finishes last adds them up in index order,
 // so the result does not depend on scheduling.
 // FUSED: the rows are the residual stream (a) and the attention block's output (b); the kernel
 // writes their sum, rounded to T, to sum_out and takes the cosine between a and that sum, i.e.
@@ -34,7 +35,7 @@ __global__ void __launch_bounds__(256, ImportanceCfg<FUSED>::kCtas) cos_sim_redu
   const int nvec = a.hidden / EPV;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long n_warp = (long long)gridDim.x * 8;
-  float wsum = 0.f;
+  double wsum = 0.0;
   grid_wait();
   // one 16-byte piece of each row: its part of the three sums; FUSED: the sum's piece to *out
   auto piece = [&](const uint4& va, const uint4& vb, uint4* out, float& dot, float& na, float& nb) {
@@ -108,12 +109,12 @@ __global__ void __launch_bounds__(256, ImportanceCfg<FUSED>::kCtas) cos_sim_redu
       wsum += cosine(dot, na, nb);
     }
   }
-  __shared__ float s_w[8];
+  __shared__ double s_w[8];
   __shared__ bool s_last;
   if (lane == 0) s_w[warp] = wsum;
   __syncthreads();
   if (threadIdx.x == 0) {
-    float c = 0.f;
+    double c = 0.0;
     for (int i = 0; i < 8; ++i) c += s_w[i];
     a.cta_partial[blockIdx.x] = c;
     __threadfence();
@@ -125,7 +126,7 @@ __global__ void __launch_bounds__(256, ImportanceCfg<FUSED>::kCtas) cos_sim_redu
     __threadfence();
     __shared__ double s_acc[8];
     double acc = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) acc += (double)__ldcg(a.cta_partial + i);
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += 256) acc += __ldcg(a.cta_partial + i);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
     if (lane == 0) s_acc[warp] = acc;

@@ -140,7 +140,7 @@ WsLayout ws_layout(const sq_config& c, int64_t b_init) {
     return o;
   };
   w.cos_sum = take(8 * ND);
-  w.cta_partial = take(4 * (size_t)kMaxImportanceCtas);
+  w.cta_partial = take(8 * (size_t)kMaxImportanceCtas);
   w.ticket = take(4);
   w.cos_sim = take(4 * ND);
   w.status = take(4);
@@ -440,7 +440,7 @@ static int importance_rows(sq_ctx* c, int32_t layer, const void* row_a, const vo
     a.sum_out = sum_out ? static_cast<char*>(sum_out) + (size_t)done * row : nullptr;
     a.n_tok = n;
     a.hidden = c->cfg.hidden;
-    a.cta_partial = ws_ptr<float>(c, c->wl.cta_partial);
+    a.cta_partial = ws_ptr<double>(c, c->wl.cta_partial);
     a.ticket = ws_ptr<unsigned int>(c, c->wl.ticket);
     a.cos_sum = ws_ptr<double>(c, c->wl.cos_sum) + d;
     SQ_CUDA(c, launch_importance(a, c->cfg.dtype, c->n_sm, static_cast<cudaStream_t>(stream)));

@@ -40,7 +40,7 @@ struct ImportanceArgs {
   void* sum_out;         // fused form: receives a + b (rounded to the dtype), which then plays the part of b; else null
   long long n_tok;
   int hidden;
-  float* cta_partial;    // [n_cta]
+  double* cta_partial;   // [n_cta]
   unsigned int* ticket;  // zero on entry, zero again on exit
   double* cos_sum;       // += sum over tokens of the cosine
 };

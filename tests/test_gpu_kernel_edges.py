@@ -282,3 +282,29 @@ def test_importance_of_short_rows(dtype, hidden, tokens):
         # three fp32 sums of `hidden` products each and the mean of the fp32 cosines: at most (hidden + warps' rows) ulp
         assert abs(float(ctx.get_cos_sim()[0]) - want) <= (hidden + 64) * 2.0 ** -23
         assert ctx.status() == 0
+
+
+@pytest.mark.parametrize("hidden,tokens", [(64, 300007), (4096, 20011)])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_importance_sums_lose_nothing(dtype, hidden, tokens):
+    """Rows whose cosines the kernel's fp32 arithmetic gives exactly (3/5, 4/5, 1 in fp32): their sum over
+    many tokens is that of fp64 additions, however few warps share them."""
+    w = synth.Workload("exact rows", 62, n_layer=1, n_q_head=2, n_kv_head=2, head_dim=64, hidden=hidden, batch=1, prompt=tokens,
+                       steps=1, dtype=dtype, policy=synth.SLIDING_WINDOW, budget_pct=100.0, p=1.0)
+    kind = torch.randint(0, 3, (tokens,), generator=torch.Generator().manual_seed(hidden)).to(DEV)
+    a = torch.zeros(tokens, hidden, dtype=dtype, device=DEV)
+    b = torch.zeros_like(a)
+    a[:, 1] = 1.0
+    b[:, 1] = torch.tensor([3.0, 4.0, 2.0], device=DEV).to(dtype)[kind]
+    b[:, hidden - 1] = torch.tensor([4.0, 3.0, 0.0], device=DEV).to(dtype)[kind]
+    want = float(torch.tensor([3.0 / 5.0, 4.0 / 5.0, 1.0], device=DEV).double()[kind].sum())
+    for fused in (False, True):
+        ctx = H.make_ctx(w)
+        ctx.begin_sequence_batch(1, tokens)
+        if fused:
+            ctx.layer_importance_fused(0, a, b - a, torch.empty_like(a))
+        else:
+            ctx.layer_importance(0, a, b)
+        got, n = ctx.get_importance_state()
+        assert n == [tokens]
+        assert abs(got[0] - want) <= tokens * 2.0 ** -52 * want     # one rounding of fp64 per addition, both sides
