@@ -978,7 +978,11 @@ int sq_ctx_import_layout(sq_ctx* c, const sq_layer_layout* in, void* stream) {
         return fail(c, SQ_ERR_INVALID_ARG, "layout: budget / cap");
       if (cfg.policy == SQ_POLICY_STREAMING_LLM && e.budget <= cfg.n_sink)
         return fail(c, SQ_ERR_INVALID_ARG, "StreamingLLM needs every layer budget above n_sink");
-      c->hs.budget[l * c->n_grp + g] = e.cap;
+    }
+  // the whole table is sound: from here on the present budgets are replaced
+  for (int l = 0; l < cfg.n_layer; ++l)
+    for (int g = 0; g < c->n_grp; ++g) {
+      c->hs.budget[l * c->n_grp + g] = in[user_index(c, l, g)].cap;
       c->hs.is_g3[l * c->n_grp + g] = 0;
     }
   c->budget_state = 0;

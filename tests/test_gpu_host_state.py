@@ -1,0 +1,58 @@
+"""What the host side of a context holds: refused calls leave it as it was, read-backs wait, stream capture."""
+import pytest
+import torch
+
+from paper_2404_04793_b200 import binding as B
+from paper_2404_04793_b200 import synth
+from tests import helpers as H
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def workload(**kw):
+    base = dict(n_layer=3, n_q_head=4, n_kv_head=2, head_dim=64, hidden=64, batch=2, prompt=96, steps=4,
+                dtype=torch.bfloat16, policy=synth.SLIDING_WINDOW, budget_pct=50.0, p=0.3)
+    return synth.Workload("host state", 71, **dict(base, **kw))
+
+
+def filled(w, budgets, **over):
+    ctx = H.make_ctx(w, **over)
+    ctx.begin_sequence_batch(w.batch, w.prompt)
+    ctx.set_budgets(budgets)
+    for l in range(w.n_layer):
+        _, k, v = synth.prompt_qkv(w, l, DEV, need_q=False)
+        ctx.prefill_compress(l, k, v)
+    return ctx
+
+
+def step(ctx, w, t):
+    q, kn, vn = synth.decode_qkv(w, t, DEV)
+    out = torch.empty_like(q)
+    ctx.decode_step(0, w.n_layer, q, kn, vn, out)
+    return out
+
+
+@pytest.mark.parametrize("per_sequence", [0, 1])
+@pytest.mark.parametrize("fault", [dict(budget=0), dict(cap=7), dict(n_unit=99), dict(n_tok=1 << 30)])
+def test_a_refused_import_leaves_budgets_and_cache(per_sequence, fault):
+    w = workload()
+    one = [60, 20, 50]
+    budgets = [one, [40, 30, 61]] if per_sequence else one
+    ctx, twin = (filled(w, budgets, per_sequence_budgets=per_sequence) for _ in range(2))
+    assert torch.equal(step(ctx, w, 0), step(twin, w, 0))
+    table = ctx.export_layout()
+    for name, value in fault.items():
+        setattr(table[len(table) - 1], name, value)          # the last entry
+    with pytest.raises(B.SqError) as e:
+        ctx.import_layout(table)
+    assert e.value.code == B.SQ_ERR_INVALID_ARG
+    assert ctx.get_budgets() == twin.get_budgets()
+    assert ctx.get_budgets()[0] == budgets
+    assert torch.equal(step(ctx, w, 1), step(twin, w, 1))
+    tighter = [[b // 2 for b in r] for r in budgets] if per_sequence else [b // 2 for b in budgets]
+    for c in (ctx, twin):
+        c.evict(0, w.n_layer, tighter)
+    assert ctx.get_budgets() == twin.get_budgets()
+    assert torch.equal(step(ctx, w, 2), step(twin, w, 2))
+    assert ctx.status() == 0
