@@ -843,6 +843,7 @@ int sq_get_cos_sim(sq_ctx* c, float* cos_sim_host) {
 int sq_get_budgets(sq_ctx* c, int32_t* budgets_host, uint8_t* is_g3_host) {
   if (!c || !budgets_host) return SQ_ERR_INVALID_ARG;
   if (c->budget_state == 0) return fail(c, SQ_ERR_STATE, "budgets not set");
+  SQ_CUDA(c, cudaDeviceSynchronize());
   if (c->budget_state == 1) {
     const int rc = fetch_budgets(c);
     if (rc != SQ_OK) return rc;

@@ -56,3 +56,20 @@ def test_a_refused_import_leaves_budgets_and_cache(per_sequence, fault):
     assert ctx.get_budgets() == twin.get_budgets()
     assert torch.equal(step(ctx, w, 2), step(twin, w, 2))
     assert ctx.status() == 0
+
+
+def test_reading_budgets_waits_for_the_device():
+    w = workload()
+    ctx = filled(w, [60, 20, 50])
+    H.feed_importance(ctx, w)
+    for allocate in (False, True):
+        if allocate:
+            ctx.allocate_budgets(w.b_init, w.p)
+        else:
+            ctx.set_budgets([60, 20, 50])
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            torch.cuda._sleep(100_000_000)                   # some 50 ms
+            done = side.record_event()
+        ctx.get_budgets()
+        assert done.query()
