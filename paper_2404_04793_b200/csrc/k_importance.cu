@@ -215,7 +215,7 @@ __global__ void __launch_bounds__(kAllocThreads) allocate_budgets_kernel(Allocat
   __shared__ unsigned s_rest[kMaxLayers / 32];  // per 32 layers: those outside G3
   const int n = a.n_layer, tid = threadIdx.x;
   const int st = a.stride, off = blockIdx.x;  // this CTA's budget vector: entries i * st + off
-  const long long cnt = tid < n ? a.tok_count[tid * st + off] : 0;
+  const long long cnt = tid < n ? a.tok_count[tid] : 0;
   grid_wait();
 
   // layer averages, rounded to fp32 (the value reported to the caller), ranked by (value, layer)

@@ -28,9 +28,9 @@ struct WsLayout {
 
 // Small host <-> device tables.  "desc" = one cache descriptor: a layer of the whole batch, or with
 // per-sequence budgets a (layer, sequence) pair; arrays hold n_desc_cap entries, entry of (layer,
-// group) = layer * n_grp + group.  The host works on its own copies; what a kernel reads or a copy
-// takes is staged in one of two page-locked slots, each free again once its event has passed, so that no
-// call waits for the copies of the one before it.
+// group) = layer * n_grp + group.  The host works on its own copies; what a copy takes is staged in one
+// of two page-locked slots, each free again once its event has passed, so that no call waits for the
+// copies of the one before it.
 constexpr int kSlots = 2;
 struct HostStage {
   std::vector<int32_t> budget;
@@ -44,7 +44,7 @@ struct HostStage {
   char* block;
   int32_t* budget_down;  // written by the allocator
   uint8_t* is_g3_down;
-  char* slot[kSlots];    // image of the workspace from WsLayout::layers on, then tok_count
+  char* slot[kSlots];    // image of the workspace from WsLayout::layers on
   cudaEvent_t slot_ev[kSlots];
   int next_slot;
 };
@@ -192,7 +192,16 @@ void sort_orders(sq_ctx* c) {
   std::copy(ord.begin(), ord.end(), c->hs.order_by_layer.begin());
 }
 
-// A staging slot whose last copies or kernel are done.
+// A captured copy of host tables would read whatever the host has staged by the time of a replay: calls that
+// upload tables are refused on a capturing stream, before they change anything.
+int refuse_capture(sq_ctx* c, cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  SQ_CUDA(c, cudaStreamIsCapturing(st, &cs));
+  if (cs != cudaStreamCaptureStatusNone) return fail(c, SQ_ERR_CUDA, "this call uploads host tables and cannot be captured");
+  return SQ_OK;
+}
+
+// A staging slot whose last copy is done.
 int take_slot(sq_ctx* c, int* slot) {
   *slot = c->hs.next_slot;
   c->hs.next_slot = (*slot + 1) % kSlots;
@@ -266,19 +275,20 @@ int build_layout(sq_ctx* c, cudaStream_t st) {
   return SQ_OK;
 }
 
-// Waits for the allocator's kernel, which writes its budgets to page-locked memory.
-int fetch_budgets(sq_ctx* c) {
-  SQ_CUDA(c, cudaEventSynchronize(c->ev));
+// The budgets that the allocator's kernel, which is done, wrote to page-locked memory.
+void take_budgets(sq_ctx* c) {
   std::copy(c->hs.budget_down, c->hs.budget_down + c->n_desc, c->hs.budget.begin());
   std::copy(c->hs.is_g3_down, c->hs.is_g3_down + c->n_desc, c->hs.is_g3.begin());
-  return SQ_OK;
 }
 
 int ensure_budgets(sq_ctx* c, cudaStream_t st) {
   if (c->budget_state == 2) return SQ_OK;
   if (c->budget_state == 0) return fail(c, SQ_ERR_STATE, "budgets not set: call sq_allocate_budgets or sq_set_budgets first");
-  const int rc = fetch_budgets(c);
-  return rc != SQ_OK ? rc : build_layout(c, st);
+  int rc = refuse_capture(c, st);
+  if (rc != SQ_OK) return rc;
+  SQ_CUDA(c, cudaEventSynchronize(c->ev));  // the allocator's kernel
+  take_budgets(c);
+  return build_layout(c, st);
 }
 
 bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -339,11 +349,11 @@ int sq_ctx_create(const sq_config* cfg, int64_t b_init, void* pool, size_t pool_
   hs.order.assign(nd, 0);
   hs.order_by_layer.assign(nd, 0);
   hs.evict_tab.assign(nd, EvictLayer{});
-  const size_t image = align_up(wl.tables_end - wl.layers), counts = align_up(8 * nd), down = align_up(4 * nd) + align_up(nd);
+  const size_t image = align_up(wl.tables_end - wl.layers), down = align_up(4 * nd) + align_up(nd);
   void* blk = nullptr;
   hs.next_slot = 0;
   int n_ev = 0;
-  bool ok = cudaHostAlloc(&blk, kSlots * (image + counts) + down, cudaHostAllocDefault) == cudaSuccess;
+  bool ok = cudaHostAlloc(&blk, kSlots * image + down, cudaHostAllocDefault) == cudaSuccess;
   if (ok) ok = cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming) == cudaSuccess;
   const bool has_ev = ok;
   for (; ok && n_ev < kSlots; ++n_ev) {
@@ -360,9 +370,9 @@ int sq_ctx_create(const sq_config* cfg, int64_t b_init, void* pool, size_t pool_
     return SQ_ERR_CUDA;
   }
   hs.block = static_cast<char*>(blk);
-  std::memset(blk, 0, kSlots * (image + counts) + down);
-  for (int i = 0; i < kSlots; ++i) hs.slot[i] = hs.block + i * (image + counts);
-  hs.budget_down = reinterpret_cast<int32_t*>(hs.block + kSlots * (image + counts));
+  std::memset(blk, 0, kSlots * image + down);
+  for (int i = 0; i < kSlots; ++i) hs.slot[i] = hs.block + i * image;
+  hs.budget_down = reinterpret_cast<int32_t*>(hs.block + kSlots * image);
   hs.is_g3_down = reinterpret_cast<uint8_t*>(reinterpret_cast<char*>(hs.budget_down) + align_up(4 * nd));
   *out = c;
   return SQ_OK;
@@ -371,7 +381,7 @@ int sq_ctx_create(const sq_config* cfg, int64_t b_init, void* pool, size_t pool_
 int sq_ctx_destroy(sq_ctx* c) {
   if (!c) return SQ_ERR_INVALID_ARG;
   // nothing may still read or write the page-locked block
-  cudaEventSynchronize(c->ev);
+  if (cudaEventSynchronize(c->ev) != cudaSuccess) cudaGetLastError();  // (last recorded under capture: nothing to wait for)
   for (int i = 0; i < kSlots; ++i) {
     cudaEventSynchronize(c->hs.slot_ev[i]);
     cudaEventDestroy(c->hs.slot_ev[i]);
@@ -475,15 +485,11 @@ int sq_allocate_budgets(sq_ctx* c, int64_t b_init, double p, void* stream) {
     if (c->per_seq && c->imp_tokens[l] != (long long)c->batch * c->prompt)
       return fail(c, SQ_ERR_STATE, "per-sequence budgets need the hidden states of every prompt token of every layer");
   }
-  // the token counts go down and the budgets come up through page-locked memory, without copies
-  int slot;
-  const int rc = take_slot(c, &slot);
-  if (rc != SQ_OK) return rc;
-  long long* counts = reinterpret_cast<long long*>(c->hs.slot[slot] + align_up(c->wl.tables_end - c->wl.layers));
-  std::copy(c->hs.tok_count.begin(), c->hs.tok_count.begin() + c->n_desc, counts);
+  // the token counts go down with the launch, the budgets come up through page-locked memory: no copies, and a
+  // captured launch holds the counts it was captured with
   AllocateArgs a;
   a.cos_sum = ws_ptr<double>(c, c->wl.cos_sum);
-  a.tok_count = counts;
+  for (int l = 0; l < c->cfg.n_layer; ++l) a.tok_count[l] = c->hs.tok_count[(size_t)l * c->n_grp];  // (the same for every sequence)
   a.n_layer = c->cfg.n_layer;
   a.n_cluster = c->cfg.n_cluster;
   a.stride = c->n_grp;
@@ -494,7 +500,6 @@ int sq_allocate_budgets(sq_ctx* c, int64_t b_init, double p, void* stream) {
   a.is_g3 = c->hs.is_g3_down;
   SQ_CUDA(c, launch_allocate(a, st));
   SQ_CUDA(c, cudaEventRecord(c->ev, st));
-  SQ_CUDA(c, cudaEventRecord(c->hs.slot_ev[slot], st));
   c->budget_state = 1;
   for (int l = 0; l < c->cfg.n_layer; ++l) c->prefilled[l] = false;
   return SQ_OK;
@@ -506,6 +511,8 @@ int sq_set_budgets(sq_ctx* c, const int32_t* budgets_host, void* stream) {
   c->last_end = 0;
   if (!c->begun) return fail(c, SQ_ERR_STATE, "sq_begin_sequence_batch has not been called");
   if (!budgets_host) return fail(c, SQ_ERR_INVALID_ARG, "budgets_host is NULL");
+  const int rc = refuse_capture(c, st);
+  if (rc != SQ_OK) return rc;
   for (int l = 0; l < c->cfg.n_layer; ++l) {
     for (int g = 0; g < c->n_grp; ++g) {
       c->hs.budget[l * c->n_grp + g] = budgets_host[user_index(c, l, g)];
@@ -742,6 +749,8 @@ int sq_evict(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const int32_t* n
         return fail(c, SQ_ERR_INVALID_ARG, "StreamingLLM needs every layer budget above n_sink");
     }
   }
+  rc = refuse_capture(c, st);
+  if (rc != SQ_OK) return rc;
   int n_active = 0, max_cap = 0;
   for (int l = layer_begin; l < layer_end; ++l) {
     for (int g = 0; g < ng; ++g) {
@@ -844,10 +853,7 @@ int sq_get_budgets(sq_ctx* c, int32_t* budgets_host, uint8_t* is_g3_host) {
   if (!c || !budgets_host) return SQ_ERR_INVALID_ARG;
   if (c->budget_state == 0) return fail(c, SQ_ERR_STATE, "budgets not set");
   SQ_CUDA(c, cudaDeviceSynchronize());
-  if (c->budget_state == 1) {
-    const int rc = fetch_budgets(c);
-    if (rc != SQ_OK) return rc;
-  }
+  if (c->budget_state == 1) take_budgets(c);
   for (int l = 0; l < c->cfg.n_layer; ++l)
     for (int g = 0; g < c->n_grp; ++g) {
       budgets_host[user_index(c, l, g)] = c->hs.budget[l * c->n_grp + g];
@@ -980,6 +986,8 @@ int sq_ctx_import_layout(sq_ctx* c, const sq_layer_layout* in, void* stream) {
       if (cfg.policy == SQ_POLICY_STREAMING_LLM && e.budget <= cfg.n_sink)
         return fail(c, SQ_ERR_INVALID_ARG, "StreamingLLM needs every layer budget above n_sink");
     }
+  int rc = refuse_capture(c, st);
+  if (rc != SQ_OK) return rc;
   // the whole table is sound: from here on the present budgets are replaced
   for (int l = 0; l < cfg.n_layer; ++l)
     for (int g = 0; g < c->n_grp; ++g) {
@@ -987,7 +995,7 @@ int sq_ctx_import_layout(sq_ctx* c, const sq_layer_layout* in, void* stream) {
       c->hs.is_g3[l * c->n_grp + g] = 0;
     }
   c->budget_state = 0;
-  int rc = build_layout(c, st);
+  rc = build_layout(c, st);
   if (rc != SQ_OK) return rc;
   c->budget_state = 0;  // until the descriptors below are in place
   for (int l = 0; l < cfg.n_layer; ++l) {

@@ -45,9 +45,9 @@ struct ImportanceArgs {
   double* cos_sum;       // += sum over tokens of the cosine
 };
 
-struct AllocateArgs {  // entry of layer i: [i * stride + blockIdx.x] (one CTA per budget vector); tok_count, budget, is_g3: page-locked host memory
+struct AllocateArgs {  // entry of layer i: [i * stride + blockIdx.x] (one CTA per budget vector); budget, is_g3: page-locked host memory
   const double* cos_sum;
-  const long long* tok_count;
+  long long tok_count[kMaxLayers];  // by layer
   int n_layer, n_cluster, stride;
   long long b_init;
   double p;

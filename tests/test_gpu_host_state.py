@@ -26,8 +26,8 @@ def filled(w, budgets, **over):
     return ctx
 
 
-def step(ctx, w, t):
-    q, kn, vn = synth.decode_qkv(w, t, DEV)
+def step(ctx, w, t, inputs=None):
+    q, kn, vn = inputs or synth.decode_qkv(w, t, DEV)
     out = torch.empty_like(q)
     ctx.decode_step(0, w.n_layer, q, kn, vn, out)
     return out
@@ -73,3 +73,56 @@ def test_reading_budgets_waits_for_the_device():
             done = side.record_event()
         ctx.get_budgets()
         assert done.query()
+
+
+def test_calls_under_stream_capture():
+    """Importance and allocation can be captured and replayed (the budgets are then read back); what uploads host
+    tables is refused, changes nothing, and neither leaves anything behind that a later call stumbles on."""
+    w = workload()
+    hidden = [synth.hidden_pair(w, l, DEV) for l in range(w.n_layer)]
+
+    def measure(ctx):
+        ctx.begin_sequence_batch(w.batch, w.prompt)
+        for l, (a, b) in enumerate(hidden):
+            ctx.layer_importance(l, a, b)
+        ctx.allocate_budgets(w.b_init, w.p)
+
+    ctx, twin = filled(w, [60, 20, 50]), filled(w, [60, 20, 50])
+    budgets = ctx.get_budgets()
+    layout = ctx.export_layout()
+    inputs = synth.decode_qkv(w, 0, DEV)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for call in (lambda: ctx.set_budgets([50, 30, 40]), lambda: ctx.evict(0, 3, [30, 10, 25]), lambda: ctx.import_layout(layout)):
+            with pytest.raises(B.SqError) as e:
+                call()
+            assert e.value.code == B.SQ_ERR_CUDA
+        out = step(ctx, w, 0, inputs)
+    graph.replay()
+    assert ctx.get_budgets() == budgets
+    assert torch.equal(out, step(twin, w, 0))
+    assert torch.equal(step(ctx, w, 1), step(twin, w, 1))
+    measure(twin)
+    want = twin.get_budgets()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        measure(ctx)
+        with pytest.raises(B.SqError):                       # needs the budgets on the host
+            step(ctx, w, 0, inputs)
+    for _ in range(2):
+        graph.replay()
+        assert ctx.get_budgets() == want
+    for _ in range(3):                                       # more calls than staging slots
+        ctx.begin_sequence_batch(w.batch, w.prompt)
+        ctx.set_budgets([60, 20, 50])
+    twin = filled(w, [60, 20, 50])
+    for l in range(w.n_layer):
+        _, k, v = synth.prompt_qkv(w, l, DEV, need_q=False)
+        ctx.prefill_compress(l, k, v)
+    assert torch.equal(step(ctx, w, 0), step(twin, w, 0))
+    measure(ctx)
+    assert ctx.get_budgets() == want and ctx.status() == 0
+    del graph
+    ctx.close()
+    assert torch.zeros(1, device=DEV).item() == 0.0
