@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <exception>
 #include <new>
 #include <string>
 #include <vector>
@@ -342,18 +343,25 @@ int sq_ctx_create(const sq_config* cfg, int64_t b_init, void* pool, size_t pool_
   c->last_stream = nullptr;
   const size_t nd = wl.n_desc_cap;
   HostStage& hs = c->hs;
-  hs.budget.assign(nd, 0);
-  hs.is_g3.assign(nd, 0);
-  hs.tok_count.assign(nd, 0);
-  hs.layers.assign(nd, LayerDesc{});
-  hs.order.assign(nd, 0);
-  hs.order_by_layer.assign(nd, 0);
-  hs.evict_tab.assign(nd, EvictLayer{});
   const size_t image = align_up(wl.tables_end - wl.layers), down = align_up(4 * nd) + align_up(nd);
   void* blk = nullptr;
   hs.next_slot = 0;
   int n_ev = 0;
+  // (the page-locked block, larger than the host's own tables, comes first: a size out of reach ends here)
   bool ok = cudaHostAlloc(&blk, kSlots * image + down, cudaHostAllocDefault) == cudaSuccess;
+  if (ok) {
+    try {
+      hs.budget.assign(nd, 0);
+      hs.is_g3.assign(nd, 0);
+      hs.tok_count.assign(nd, 0);
+      hs.layers.assign(nd, LayerDesc{});
+      hs.order.assign(nd, 0);
+      hs.order_by_layer.assign(nd, 0);
+      hs.evict_tab.assign(nd, EvictLayer{});
+    } catch (const std::exception&) {  // nothing is thrown through the C interface
+      ok = false;
+    }
+  }
   if (ok) ok = cudaEventCreateWithFlags(&c->ev, cudaEventDisableTiming) == cudaSuccess;
   const bool has_ev = ok;
   for (; ok && n_ev < kSlots; ++n_ev) {

@@ -1,4 +1,8 @@
 """What the host side of a context holds: refused calls leave it as it was, read-backs wait, stream capture."""
+import os
+import subprocess
+import sys
+
 import pytest
 import torch
 
@@ -126,3 +130,24 @@ def test_calls_under_stream_capture():
     del graph
     ctx.close()
     assert torch.zeros(1, device=DEV).item() == 0.0
+
+
+_HUGE = """
+import ctypes, resource, torch
+from paper_2404_04793_b200 import binding as B
+torch.zeros(1, device="cuda")
+now = 4096 * int(open("/proc/self/statm").read().split()[0])
+resource.setrlimit(resource.RLIMIT_AS, (now + (64 << 30), now + (64 << 30)))   # no table may take the machine's memory
+cfg = B.make_config(n_layer=256, n_q_head=1, n_kv_head=1, head_dim=64, hidden=64, max_batch=2**31 - 1, max_prompt=1,
+                    max_new_tokens=1, dtype=torch.bfloat16, policy=0, page_tokens=1, per_sequence_budgets=1)
+pool, ws = B.sq_query_sizes(cfg, 1)
+h = ctypes.c_void_p()
+print("code", B.lib().sq_ctx_create(ctypes.byref(cfg), 1, 256, pool, 256, ws, ctypes.byref(h)), h.value)
+"""
+
+
+def test_a_context_out_of_reach_is_an_error():
+    """Host tables for 5e11 descriptors (the device pointers are never used): an error code, no exception through C."""
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", _HUGE], capture_output=True, text=True, cwd=root, timeout=300)
+    assert r.returncode == 0 and f"code {B.SQ_ERR_CUDA} None" in r.stdout, (r.returncode, r.stdout, r.stderr[-500:])
