@@ -525,12 +525,9 @@ static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t 
 constexpr int kScoresLimit = 96 * 1024;  // dynamic shared memory of a CTA with the score update
 template <auto KERN>
 static cudaError_t launch_scores_kernel(const DecodeArgs& a, int pieces, int n_cta, int threads, size_t smem, cudaStream_t s) {
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(KERN, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresLimit);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, kScoresLimit, KERN);
+  if (e != cudaSuccess) return e;
   return launch_chained_cluster(KERN, pieces, n_cta, threads, smem, s, static_cast<const DecodeArgsBase&>(a));
 }
 

@@ -323,13 +323,9 @@ cudaError_t launch_h2o_gain_tc(const DecodeArgs& a, int n_items, size_t pool_byt
   constexpr size_t smem = 1024 + (size_t)kTM * 128 + (size_t)kStages * kTileBytes + 18 * 8 + kTM * 4 + 8 * sizeof(Candidate);
   auto kern_u = h2o_gain_tc_kernel<kStages, kSets, kTmemCols, 2, 1, DecodeArgsBase>;
   auto kern_s = h2o_gain_tc_kernel<kStages, kSets, kTmemCols, 2, 0, DecodeArgs>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern_u, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern_s, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, smem, kern_u, kern_s);
+  if (e != cudaSuccess) return e;
   const int n_buf = kTmemCols == 128 ? 1 : (3 * n_cols <= kTmemCols ? 3 : 2);
   const DecodeArgsBase& base = a;  // without split-K: no table
   if (a.uniform) return launch_chained(kern_u, n_items, 64 + 128 * kSets, smem, s, tm_q, tm_k, base, n_cols, n_buf);

@@ -392,36 +392,22 @@ static cudaError_t launch_cfg(const DecodeArgs& a, int n_items, cudaStream_t s) 
   static_assert(merge <= pipe, "the merge area reuses the pipeline stages");
   constexpr size_t smem = (size_t)QROWS * D * 2 + pipe;
   auto kern = decode_attn_mma_kernel<D, MT, WM, WN, STAGES, false, DecodeArgs>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, smem, kern);
+  if (e != cudaSuccess) return e;
   return launch_chained(kern, n_items, 32 * WM * WN, smem, s, a);
-}
-
-static int sm_count() {
-  static int n_sm = 0;
-  if (n_sm == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      n_sm = 148;
-  }
-  return n_sm;
 }
 
 template <int D, int MT, int STAGES>
 static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t logit_bytes, cudaStream_t s) {
   const size_t smem = (size_t)2 * STAGES * kTile * D * 2 + logit_bytes;
   auto kern = decode_attn_mma_kernel<D, MT, 1, 4, STAGES, true, DecodeArgsBase>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  const cudaError_t e = set_up.once([&] {
+    const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresSmem);
+    return r == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
+  });
+  if (e != cudaSuccess) return e;
   return launch_chained_cluster(kern, pieces, a.n_layer_total * a.n_unit * pieces, 128, smem, s, static_cast<const DecodeArgsBase&>(a));
 }
 

@@ -367,14 +367,13 @@ static cudaError_t launch_low_cfg(const DecodeArgs& a, int n_items, int pieces, 
   constexpr size_t pipe = (size_t)2 * STAGES * kTile * D * 2;
   auto plain = decode_attn_mma_low_kernel<D, STAGES, false, HEADS, DecodeArgs>;
   auto scores = decode_attn_mma_low_kernel<D, STAGES, true, HEADS, DecodeArgsBase>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pipe);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(scores, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresSmem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(scores, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  const cudaError_t e = set_up.once([&] {
+    cudaError_t r = cudaFuncSetAttribute(plain, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pipe);
+    if (r == cudaSuccess) r = cudaFuncSetAttribute(scores, cudaFuncAttributeMaxDynamicSharedMemorySize, kScoresSmem);
+    return r == cudaSuccess ? cudaFuncSetAttribute(scores, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
+  });
+  if (e != cudaSuccess) return e;
   if (pieces > 0)
     return launch_chained_cluster(scores, pieces, a.n_layer_total * a.n_unit * pieces, 128, pipe + logit_bytes, s,
                                   static_cast<const DecodeArgsBase&>(a));

@@ -331,12 +331,9 @@ static cudaError_t launch_tc_cfg(const DecodeArgs& a, int n_items, const CUtenso
   constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 8 * 16 + 16;
   static_assert(2 * (smem + 1024 + 64) <= 228 * 1024, "two CTAs per SM");
   auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, smem, kern);
+  if (e != cudaSuccess) return e;
   return launch_chained(kern, n_items, 192, smem, s, tq, tk, tv, a);
 }
 

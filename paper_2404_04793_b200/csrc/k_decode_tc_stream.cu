@@ -467,12 +467,9 @@ static cudaError_t launch_tc_stream_cfg(const StreamArgs& t, int n_cta, const CU
   constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 18 * 8 + 2 * (ROWS == 120 ? 96 : 128) * 4;
   static_assert(2 * (smem + 1024) <= 228 * 1024, "two CTAs per SM");
   auto kern = decode_attn_tc_stream_kernel<STAGES, ROWS, H2O>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, smem, kern);
+  if (e != cudaSuccess) return e;
   return launch_chained(kern, n_cta, 192, smem, s, tq, tk, tv, t);
 }
 
@@ -483,13 +480,6 @@ cudaError_t launch_decode_attn_tc_stream(const DecodeArgs& a, const int* desc_ti
   if (a.head_dim != kD || a.group <= 32 || a.group > 128) return cudaErrorNotSupported;
   const long long pool_rows = (long long)(pool_bytes / (kD * 2));
   if (pool_rows + kTM > 0x7fffffffLL || (long long)q_rows + kTM > 0x7fffffffLL) return cudaErrorNotSupported;
-  static int n_sm = 0;
-  if (n_sm == 0) {
-    int dev = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e != cudaSuccess) return e;
-  }
   CUtensorMap tm_q, tm_k, tm_v;
   if (!make_tile_map(&tm_q, a.q, (long long)q_rows, kD, 8) || !make_tile_map(&tm_k, a.pool, pool_rows, kD, kTM) ||
       !make_tile_map(&tm_v, a.pool, pool_rows, kD, kTM))
@@ -497,7 +487,7 @@ cudaError_t launch_decode_attn_tc_stream(const DecodeArgs& a, const int* desc_ti
   const bool h2o = a.policy == SQ_POLICY_H2O;
   StreamArgs t;
   static_cast<DecodeArgsBase&>(t) = a;
-  const int slots = kCtasPerSm * n_sm;
+  const int slots = kCtasPerSm * sm_count();
   {
     // where this form wins (see the head of this file)
     const long long units = (long long)a.n_layer_total * a.n_unit;

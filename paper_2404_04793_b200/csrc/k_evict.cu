@@ -234,14 +234,11 @@ static cudaError_t launch_evict_cfg(const EvictArgs& a, cudaStream_t s) {
   constexpr int kMaxChunkRows = kChunkBytes / (2 * 128);
   const size_t words = ((size_t)a.max_cap + 31) / 32;
   const size_t smem = (size_t)kStages * kChunkBytes + (size_t)kStages * kMaxChunkRows * 8 + words * 8;
-  if (smem > 200 * 1024) return cudaErrorInvalidValue;  // caches beyond ~1.4 M slots per unit
-  static size_t configured = 0;
-  if (smem > configured) {
-    cudaError_t e = cudaFuncSetAttribute(evict_kernel<kChunkBytes, kStages>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = smem;
-  }
+  constexpr size_t kMaxSmem = 200 * 1024;
+  if (smem > kMaxSmem) return cudaErrorInvalidValue;  // caches beyond ~1.4 M slots per unit
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, kMaxSmem, evict_kernel<kChunkBytes, kStages>);
+  if (e != cudaSuccess) return e;
   evict_kernel<kChunkBytes, kStages><<<dim3(a.n_unit, a.n_layers), kSelThreads, smem, s>>>(a);
   return cudaGetLastError();
 }

@@ -251,13 +251,9 @@ static cudaError_t launch_scores_tq(const ScoreArgs& a, cudaStream_t s) {
   auto k1 = prefill_row_lse_kernel<T, D, TQ>;
   auto k2 = prefill_col_sum_kernel<T, D, TQ>;
   constexpr size_t smem = score_smem<D, TQ>();
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  cudaError_t e = allow_smem(set_up, smem, k1, k2);
+  if (e != cudaSuccess) return e;
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
   const int n_qt = (a.prompt + TQ - 1) / TQ, n_kt = (a.prompt + TK - 1) / TK, g = a.n_q_head / a.n_kv_head;
   const long long units = (long long)a.batch * a.n_kv_head;
@@ -267,7 +263,7 @@ static cudaError_t launch_scores_tq(const ScoreArgs& a, cudaStream_t s) {
   auto pieces = [&](long long c) { return (longest + c - 1) / c; };
   while (chunk < longest && (pieces(chunk) * units * a.prompt > (long long)a.partial_floats || pieces(chunk) * a.batch > 65535))
     chunk = std::min(longest, chunk * 2);
-  cudaError_t e = launch_chained(k1, dim3(n_qt, a.n_q_head, a.batch), 4 * TQ, smem, s, a, scale_log2);
+  e = launch_chained(k1, dim3(n_qt, a.n_q_head, a.batch), 4 * TQ, smem, s, a, scale_log2);
   if (e != cudaSuccess) return e;
   return launch_chained(k2, dim3(n_kt, a.n_kv_head, a.batch * (unsigned)pieces(chunk)), 4 * TQ, smem, s, a, scale_log2,
                         (int)pieces(chunk), (int)chunk);

@@ -447,13 +447,9 @@ static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) 
   const int n_tile = (a.prompt + kTM - 1) / kTM;
   auto k1 = prefill_scores_tc_kernel<D, STAGES, 1>;
   auto k2 = prefill_scores_tc_kernel<D, STAGES, 2>;
-  static bool configured = false;
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    configured = true;
-  }
+  static PerDevice set_up;
+  cudaError_t e = allow_smem(set_up, smem, k1, k2);
+  if (e != cudaSuccess) return e;
   // Sweep 2 walks the heads of a group one after the other.  A launch of few key tiles and many heads
   // (71 heads on one KV head) would be over when its longest CTA is: it is cut into pieces of `heads`
   // heads so that the longest CTA has at most about a quarter of a CTA slot's share of the work.
@@ -471,7 +467,7 @@ static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) 
   pc.partial = a.partial;
   pc.tickets = a.tickets;
   k1<<<dim3(a.n_q_head, a.batch, n_tile), kPrefillThreads, smem, s>>>(tm_q, tm_k, a, pc, scale_log2, status);
-  cudaError_t e = cudaGetLastError();
+  e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   k2<<<dim3(a.n_kv_head, a.batch, n_tile * pc.n_piece), kPrefillThreads, smem, s>>>(tm_k, tm_q, a, pc, scale_log2, status);
   return cudaGetLastError();

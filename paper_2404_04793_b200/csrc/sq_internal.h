@@ -7,6 +7,7 @@
 #include <utility>
 
 #include "sq.h"
+#include "sq_device_state.h"
 
 namespace sq {
 
