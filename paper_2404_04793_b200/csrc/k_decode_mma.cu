@@ -408,6 +408,8 @@ static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t log
     return r == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
   });
   if (e != cudaSuccess) return e;
+  static ClusterFit wide;
+  if (pieces > 8 && !wide.fits(reinterpret_cast<const void*>(kern), kMaxPieces, 128, kScoresSmem)) return cudaErrorNotSupported;
   return launch_chained_cluster(kern, pieces, a.n_layer_total * a.n_unit * pieces, 128, smem, s, static_cast<const DecodeArgsBase&>(a));
 }
 
@@ -429,17 +431,20 @@ cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStrea
   const long long units = (long long)a.n_layer_total * a.n_unit;
   if (units >= 6 * n_sm) return cudaErrorNotSupported;
   const int tiles = (max_len + kTile - 1) / kTile;
-  int pieces = (int)std::min<long long>(units <= 16 ? kMaxPieces : 8, std::max<long long>(1, 2 * n_sm / units));
-  pieces = std::min(pieces, tiles);
   const int stages = a.head_dim == 128 ? 3 : 4;
   const size_t fixed = (size_t)2 * stages * kTile * a.head_dim * 2;
   auto logit_bytes = [&](int p) { return (size_t)piece_tiles(max_len, p) * kTile * G * 4; };
-  while (pieces < 8 && fixed + logit_bytes(pieces) > kScoresSmem) ++pieces;
-  const size_t lb = logit_bytes(pieces);
-  if (fixed + lb > kScoresSmem) return cudaErrorNotSupported;
-  if (G <= 8) return launch_decode_mma_low(a, 0, pieces, lb, s);
-  if (a.head_dim == 128) return G <= 16 ? launch_scores_cfg<128, 1, 3>(a, pieces, lb, s) : launch_scores_cfg<128, 2, 3>(a, pieces, lb, s);
-  return G <= 16 ? launch_scores_cfg<64, 1, 4>(a, pieces, lb, s) : launch_scores_cfg<64, 2, 4>(a, pieces, lb, s);
+  auto launch = [&](int limit) {
+    int pieces = (int)std::min<long long>(limit, std::max<long long>(1, 2 * n_sm / units));
+    pieces = std::min(pieces, tiles);
+    while (pieces < 8 && fixed + logit_bytes(pieces) > kScoresSmem) ++pieces;
+    const size_t lb = logit_bytes(pieces);
+    if (fixed + lb > kScoresSmem) return cudaErrorNotSupported;
+    if (G <= 8) return launch_decode_mma_low(a, 0, pieces, lb, s);
+    if (a.head_dim == 128) return G <= 16 ? launch_scores_cfg<128, 1, 3>(a, pieces, lb, s) : launch_scores_cfg<128, 2, 3>(a, pieces, lb, s);
+    return G <= 16 ? launch_scores_cfg<64, 1, 4>(a, pieces, lb, s) : launch_scores_cfg<64, 2, 4>(a, pieces, lb, s);
+  };
+  return with_portable_clusters(units <= 16 ? kMaxPieces : 8, launch);
 }
 
 // Returns cudaErrorNotSupported when no tensor-core configuration covers the shape.

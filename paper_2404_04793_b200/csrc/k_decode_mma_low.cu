@@ -374,6 +374,8 @@ static cudaError_t launch_low_cfg(const DecodeArgs& a, int n_items, int pieces, 
     return r == cudaSuccess ? cudaFuncSetAttribute(scores, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
   });
   if (e != cudaSuccess) return e;
+  static ClusterFit wide;
+  if (pieces > 8 && !wide.fits(reinterpret_cast<const void*>(scores), kMaxPieces, 128, kScoresSmem)) return cudaErrorNotSupported;
   if (pieces > 0)
     return launch_chained_cluster(scores, pieces, a.n_layer_total * a.n_unit * pieces, 128, pipe + logit_bytes, s,
                                   static_cast<const DecodeArgsBase&>(a));

@@ -42,6 +42,47 @@ inline cudaError_t allow_smem(PerDevice& state, size_t bytes, K... kern) {
   });
 }
 
+// Whether the current device holds a cluster of `ctas` CTAs of a kernel (which is allowed that size) with `smem` bytes
+// of dynamic shared memory each.  Above the portable 8 that depends on the device and on what is left of it
+// (partitions, disabled SMs).  For static storage, one per kernel; asked once on every device, with the largest
+// ctas and smem that the kernel is launched with.
+class ClusterFit {
+ public:
+  bool fits(const void* kern, int ctas, int threads, size_t smem) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const bool known = dev >= 0 && dev < kMaxDevices;
+    const int seen = known ? state_[dev].load(std::memory_order_relaxed) : 0;
+    if (seen) return seen == 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    const bool ok = cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0;
+    if (!ok) cudaGetLastError();
+    if (known) state_[dev].store(ok ? 1 : 2, std::memory_order_relaxed);
+    return ok;
+  }
+
+ private:
+  std::atomic<int> state_[kMaxDevices] = {};
+};
+
+// launch(limit) with clusters of at most `limit` CTAs, and where the device does not hold those (or the plan does not
+// work out) with at most the portable 8.
+template <class F>
+inline cudaError_t with_portable_clusters(int limit, F launch) {
+  const cudaError_t e = launch(limit);
+  return e == cudaErrorNotSupported && limit > 8 ? launch(8) : e;
+}
+
 // SMs of the current device.
 inline int sm_count() {
   static std::atomic<int> count[kMaxDevices] = {};

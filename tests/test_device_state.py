@@ -16,8 +16,17 @@ PROGRAM = r"""
 #include "sq_device_state.h"
 static int g_dev = 0, g_fail = 0;
 static std::map<std::pair<int, const void*>, int> g_limit;   // (device, kernel) -> bytes
-static int g_sets = 0;
+static int g_sets = 0, g_asked = 0;
+static int g_room = 0;                                        // CTAs of the largest cluster that fits
 extern "C" {
+cudaError_t cudaGetLastError() { return cudaSuccess; }
+cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t* c) {
+  ++g_asked;
+  if (c->numAttrs != 1 || c->attrs[0].id != cudaLaunchAttributeClusterDimension || c->gridDim.x != c->attrs[0].val.clusterDim.x)
+    return cudaErrorInvalidValue;
+  *n = (int)c->attrs[0].val.clusterDim.x <= g_room ? 3 : 0;
+  return cudaSuccess;
+}
 cudaError_t cudaGetDevice(int* d) { *d = g_dev; return cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int d) { *v = 100 + d; return cudaSuccess; }
 cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute, int v) {
@@ -46,6 +55,30 @@ int main() {
   g_fail = 0;
   CHECK(sq::allow_smem(other, 5, kern_a) == cudaSuccess);   // a failure is not remembered as done
   CHECK((g_limit[{2, (const void*)kern_a}]) == 5);
+  static sq::ClusterFit fit;
+  const void* k = (const void*)kern_a;
+  for (int round = 0; round < 2; ++round) {
+    g_dev = 0, g_room = 16;
+    CHECK(fit.fits(k, 16, 128, 1000));
+    g_dev = 1, g_room = 8;
+    CHECK(!fit.fits(k, 16, 128, 1000));
+  }
+  CHECK(g_asked == 2);
+  // a launch that asks for 16 and finds no room is made with 8, once; other results are passed on
+  for (int d : {0, 1}) {
+    g_dev = d;
+    int made = 0, calls = 0;
+    auto launch = [&](int limit) {
+      ++calls;
+      if (limit > 8 && !fit.fits(k, 16, 128, 1000)) return cudaErrorNotSupported;
+      made = limit;
+      return cudaSuccess;
+    };
+    CHECK(sq::with_portable_clusters(16, launch) == cudaSuccess && made == (d == 0 ? 16 : 8) && calls == 1 + d);
+  }
+  int calls = 0;
+  CHECK(sq::with_portable_clusters(8, [&](int) { ++calls; return cudaErrorNotSupported; }) == cudaErrorNotSupported && calls == 1);
+  CHECK(sq::with_portable_clusters(16, [&](int) { ++calls; return cudaErrorInvalidValue; }) == cudaErrorInvalidValue && calls == 2);
   std::puts("ok");
 }
 """
@@ -63,7 +96,7 @@ def run_host_program(tmp_path, source):
 
 
 @pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
-def test_set_up_and_sm_count_are_kept_by_device(tmp_path):
+def test_set_up_clusters_and_sm_count_are_kept_by_device(tmp_path):
     assert run_host_program(tmp_path, PROGRAM) == "ok"
 
 
