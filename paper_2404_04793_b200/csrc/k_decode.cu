@@ -513,7 +513,7 @@ static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t 
   if (a.group == 1) {
     // the register-capped kernel gets its own build for launches without split-K (which takes no table)
     // few unsplit units (at most two 16-warp CTAs per SM, all resident at once): 16 warps per unit
-    if (a.uniform && n_items <= 2 * 148)
+    if (a.uniform && n_items <= 2 * sm_count())
       return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16>, n_items, 512, 0, s, base);
     if (a.uniform) return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase>, n_items, 128, 0, s, base);
     return launch_chained(decode_attn_kernel<T, D, 1, 0, DecodeArgs>, n_items, 128, 0, s, a);
@@ -538,11 +538,11 @@ template <typename T, int D>
 static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
   const int G = a.group;
   if (G > 32) return cudaErrorNotSupported;
-  constexpr int kSm = 148;
   const long long units = (long long)a.n_layer_total * a.n_unit;
   // few units: 16 warps each (two such CTAs per SM); else 4 warps, eight CTAs per SM
-  const bool wide = G == 1 && units <= 2 * kSm;
-  const long long slots = G == 1 && !wide ? 8 * kSm : 2 * kSm;
+  const int n_sm = sm_count();
+  const bool wide = G == 1 && units <= 2 * n_sm;
+  const long long slots = G == 1 && !wide ? 8LL * n_sm : 2LL * n_sm;
   int pieces = (int)std::min<long long>(kMaxPieces, std::max<long long>(1, slots / units));
   pieces = std::min(pieces, std::max(1, max_len / (wide ? 256 : 128)));
   const size_t limit = (wide || G > 1) ? kScoresLimit : 24 * 1024;
@@ -603,7 +603,7 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need
   // More units than the CTA-per-unit kernel holds in one wave (5 CTAs per SM), and nothing to
   // merge: only the scores and the next victim remain, one warp per unit.  Smaller launches
   // (one layer of a small batch) finish sooner with a CTA per unit.
-  if (a.policy == SQ_POLICY_H2O && a.uniform && a.group <= 32 && n_cta > 148 * 5) {
+  if (a.policy == SQ_POLICY_H2O && a.uniform && a.group <= 32 && n_cta > 5 * sm_count()) {
     return launch_chained(h2o_update_warp_kernel, (n_cta + kWarpUpdWarps - 1) / kWarpUpdWarps, 32 * kWarpUpdWarps, 0, s,
                           static_cast<const DecodeArgsBase&>(a));
   }

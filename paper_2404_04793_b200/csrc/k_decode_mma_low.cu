@@ -388,7 +388,7 @@ static cudaError_t launch_low(const DecodeArgs& a, int n_items, int pieces, size
   // Two stages of 32 KB let three CTAs share an SM, which wins once the launch has CTAs to spare; a launch of
   // about one wave (one layer at a time) is better off with the deeper ring per CTA.  us per token, three /
   // two stages: 800 units per layer 305 / 277, 512: 694 / 797, 256: 2109 / 2372.
-  if (pieces == 0 && n_items >= 5 * 148) return launch_low_cfg<128, 2, HEADS>(a, n_items, 0, 0, s);
+  if (pieces == 0 && n_items >= 5 * sm_count()) return launch_low_cfg<128, 2, HEADS>(a, n_items, 0, 0, s);
   return launch_low_cfg<128, 3, HEADS>(a, n_items, pieces, logit_bytes, s);
 }
 

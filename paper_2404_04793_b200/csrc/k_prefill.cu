@@ -259,7 +259,7 @@ static cudaError_t launch_scores_tq(const ScoreArgs& a, cudaStream_t s) {
   const long long units = (long long)a.batch * a.n_kv_head;
   // pieces of about an eighth of an SM's share, as far as the scratch and the grid go
   const long long longest = (long long)g * n_qt, tiles = units * longest * (n_kt + 1) / 2;
-  long long chunk = std::max(1LL, std::min(longest, tiles / (8 * 148)));
+  long long chunk = std::max(1LL, std::min(longest, tiles / (8LL * sm_count())));
   auto pieces = [&](long long c) { return (longest + c - 1) / c; };
   while (chunk < longest && (pieces(chunk) * units * a.prompt > (long long)a.partial_floats || pieces(chunk) * a.batch > 65535))
     chunk = std::min(longest, chunk * 2);
@@ -273,7 +273,7 @@ template <typename T, int D>
 static cudaError_t launch_scores_t(const ScoreArgs& a, cudaStream_t s) {
   // small problems: more and shorter CTAs
   const long long ctas = (long long)((a.prompt + 63) / 64) * a.n_q_head * a.batch;
-  return ctas < 2 * 148 ? launch_scores_tq<T, D, 32>(a, s) : launch_scores_tq<T, D, 64>(a, s);
+  return ctas < 2LL * sm_count() ? launch_scores_tq<T, D, 32>(a, s) : launch_scores_tq<T, D, 64>(a, s);
 }
 
 // fp32-pipe kernels (any dtype)

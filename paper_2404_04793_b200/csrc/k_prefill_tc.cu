@@ -458,8 +458,8 @@ static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) 
   ScorePieces pc;
   const int g = a.n_q_head / a.n_kv_head;
   const long long units = (long long)a.batch * a.n_kv_head;
-  constexpr long long kSlots = 2 * 148;  // two CTAs per SM
-  long long heads = std::max(1LL, std::min((long long)g, units * g * (n_tile + 1) / (8 * kSlots)));
+  const long long slots = 2LL * sm_count();  // two CTAs per SM
+  long long heads = std::max(1LL, std::min((long long)g, units * g * (n_tile + 1) / (8 * slots)));
   auto pieces = [&](long long h) { return (g + h - 1) / h; };
   while (heads < g && (pieces(heads) * units * a.prompt > (long long)a.partial_floats || pieces(heads) * n_tile > 65535)) ++heads;
   pc.heads = (int)heads;
