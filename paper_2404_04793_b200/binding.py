@@ -104,10 +104,14 @@ def _dptr(t):
     raise ValueError("expected a contiguous CUDA tensor")
 
 
-_raw_stream, _current_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+# torch.cuda.current_stream() without its stream object, where this torch has the names (one built without
+# CUDA does not, and sizes and argument checks work there too)
+_raw_stream, _current_device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
 
 
 def _stream():
+    if _raw_stream is None or _current_device is None:
+        return torch.cuda.current_stream().cuda_stream
     return _raw_stream(_current_device())
 
 
@@ -213,7 +217,7 @@ class Context:
 
     def decode_step(self, layer_begin, layer_end, q, k_new, v_new, out):
         rc = self._decode(self._h, layer_begin, layer_end, _dptr(q), _dptr(k_new), _dptr(v_new), _dptr(out),
-                          _raw_stream(_current_device()))
+                          _stream())
         if rc:
             self._ck(rc)
 

@@ -3,6 +3,8 @@ entry points behave (no GPU needed)."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import pytest
 
@@ -106,3 +108,18 @@ def test_null_and_bad_arguments(lib):
     assert lib.sq_last_error(None) == b"context is NULL"
     with pytest.raises(B.SqError):
         B.sq_query_sizes(cfg, 0)
+
+
+def test_the_binding_needs_no_cuda_names_of_torch_to_import():
+    """A torch built without CUDA has no torch._C._cuda_*: sizes and argument checks work there."""
+    code = ("import torch\n"
+            "for n in ('_cuda_getCurrentRawStream', '_cuda_getDevice'):\n"
+            "    if hasattr(torch._C, n): delattr(torch._C, n)\n"
+            "from paper_2404_04793_b200 import binding as B\n"
+            "cfg = B.make_config(n_layer=1, n_q_head=1, n_kv_head=1, head_dim=64, hidden=64, max_batch=1, max_prompt=8, "
+            "max_new_tokens=1, dtype=torch.float32, policy=0)\n"
+            "print(B.sq_query_sizes(cfg, 4)[0] > 0)\n"
+            "try: B._dptr(torch.zeros(1))\n"
+            "except ValueError: print('refused')\n")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, cwd=ROOT, timeout=300)
+    assert r.stdout.split() == ["True", "refused"], r.stderr[-500:]
