@@ -17,6 +17,12 @@ namespace sq {
 
 constexpr int kMaxPieces = 8;  // CTAs of a cluster (the portable limit)
 
+template <bool FIRST, class A>
+__device__ __forceinline__ A& either(A& x, A& y) {
+  if constexpr (FIRST) return x;
+  else return y;
+}
+
 // One CTA (NW warps) per (layer, unit, split).  A K or V row is D*sizeof(T) bytes = LPR lanes
 // x 16 bytes, so a warp reads 32/LPR consecutive rows per load instruction, fully coalesced.
 // Each lane keeps its 16-byte slice of up to GT query heads (pre-scaled by log2(e)/sqrt(d))
@@ -29,17 +35,13 @@ constexpr int kMaxPieces = 8;  // CTAs of a cluster (the portable limit)
 // a quarter as long.
 // SCORES: H2O with the score update in the same launch (sq_scores.cuh): the pieces of a unit are the
 // CTAs of a cluster and the logits stay in shared memory.
-template <typename T, int D, int GT, int UNIFORM, class Args, int NW = 4, bool SCORES = false>
+// AHEAD: rows are fetched ahead of grid_wait() where a.early.
+template <typename T, int D, int GT, int UNIFORM, class Args, int NW = 4, bool SCORES = false, bool AHEAD = false>
 __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 8 : 6) : 1) : 2) decode_attn_kernel(Args a) {
   constexpr int EPV = Elem<T>::kPerVec;
   constexpr int LPR = D / EPV;   // lanes per row
   constexpr int RPW = 32 / LPR;  // rows per warp per load
   constexpr int U = 4;           // rows in flight per lane
-  // Rows ahead of grid_wait() where the registers that hold them do not cost more than a launch's start-up: with four
-  // heads and no score update they take 162 registers to 184, three CTAs per SM to two (12 layers of 16 / 4 heads,
-  // 40 sequences, one launch: 446 us with rows ahead and a wider merge, 311 without; with the score update, 8 sequences,
-  // one launch per layer: 329 with, 340 without; 80 layers of 64 / 8 heads, 2 sequences, the same: 2352 with, 2315 without).
-  constexpr bool AHEAD = GT == 1 || (GT == 4 && SCORES);
   __shared__ float sm_o[NW][GT][D];
   __shared__ float sm_m[NW][GT], sm_l[NW][GT];
 
@@ -91,32 +93,29 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
   float* stat = a.part_stat + (size_t)blockIdx.x * a.group * kStatStride;
   float* po = a.part_o + (size_t)blockIdx.x * a.group * D;
 
-  // One batch of this lane's rows; the new token's come from k_new / v_new (`fresh`) or, ahead of
-  // grid_wait(), not at all (the cached row its slot still holds, replaced afterwards).
-  uint4 kq[U], vq[U];
-  bool ok[U];
-  auto load_rows = [&](int r0, bool fresh) {
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int row = r0 + u * RPW + rg;
-      ok[u] = row < t1;
-      const int rr = ok[u] ? row : t0;
-      const T* kp = (fresh && rr == w) ? kn : Kb + (size_t)rr * D;
-      const T* vp = (fresh && rr == w) ? vn : Vb + (size_t)rr * D;
-      kq[u] = ld_stream(kp + sub * EPV);
-      vq[u] = ld_stream(vp + sub * EPV);
-    }
-  };
+  // The first batch of this lane's rows, ahead of grid_wait(): the new token's slot still holds the row that it
+  // replaces, which is put right afterwards.
+  uint4 k_ahead[U], v_ahead[U];
+  bool ok_ahead[U];
   if (AHEAD && a.early) {
     const int r0 = t0 + warp * (U * RPW);
-    if (t0 < t1) load_rows(r0, false);
+    if (t0 < t1) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int row = r0 + u * RPW + rg;
+        ok_ahead[u] = row < t1;
+        const int rr = ok_ahead[u] ? row : t0;
+        k_ahead[u] = ld_stream(Kb + (size_t)rr * D + sub * EPV);
+        v_ahead[u] = ld_stream(Vb + (size_t)rr * D + sub * EPV);
+      }
+    }
     grid_wait();
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int row = r0 + u * RPW + rg, rr = ok[u] ? row : t0;
+      const int row = r0 + u * RPW + rg, rr = ok_ahead[u] ? row : t0;
       if (t0 < t1 && rr == w) {
-        kq[u] = ld_stream(kn + sub * EPV);
-        vq[u] = ld_stream(vn + sub * EPV);
+        k_ahead[u] = ld_stream(kn + sub * EPV);
+        v_ahead[u] = ld_stream(vn + sub * EPV);
       }
     }
   }
@@ -140,7 +139,25 @@ __global__ void __launch_bounds__(NW * 32, NW == 4 ? (GT == 1 ? (UNIFORM == 1 ? 
       }
     }
     for (int r0 = t0 + warp * (U * RPW); r0 < t1; r0 += NW * U * RPW) {
-      if (!(AHEAD && a.early && hb == 0 && r0 == t0 + warp * (U * RPW))) load_rows(r0, true);
+      // (arrays of the loop's own where nothing is fetched ahead, and no function for the loads: either costs the
+      // register-capped builds up to 18 spilled registers)
+      uint4 k_here[U], v_here[U];
+      bool ok_here[U];
+      auto& kq = either<AHEAD>(k_ahead, k_here);
+      auto& vq = either<AHEAD>(v_ahead, v_here);
+      auto& ok = either<AHEAD>(ok_ahead, ok_here);
+      if (!(AHEAD && a.early && hb == 0 && r0 == t0 + warp * (U * RPW))) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int row = r0 + u * RPW + rg;
+          ok[u] = row < t1;
+          const int rr = ok[u] ? row : t0;
+          const T* kp = (rr == w) ? kn : Kb + (size_t)rr * D;
+          const T* vp = (rr == w) ? vn : Vb + (size_t)rr * D;
+          kq[u] = ld_stream(kp + sub * EPV);
+          vq[u] = ld_stream(vp + sub * EPV);
+        }
+      }
       float s[U][GT];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -505,20 +522,25 @@ __global__ void __launch_bounds__(32 * kWarpUpdWarps, 3) h2o_update_warp_kernel(
   }
 }
 
+// One head: register-capped, so each form has its own build: with rows ahead of the wait or without (they
+// spill 8 to 60 bytes, which is worth it only where they hide a launch's start), with split-K (which takes the
+// table) or without, and for few unsplit units (at most two 16-warp CTAs per SM, all resident at once) 16 warps per unit.
+// More heads: no rows ahead.  With four heads they take 162 registers to 184, three CTAs per SM to two (12 layers
+// of 16 / 4 heads, 40 sequences, one launch: 446 us with rows ahead and a wider merge, 311 without).
+template <typename T, int D, bool AHEAD>
+static cudaError_t launch_attn_one(const DecodeArgs& a, int n_items, cudaStream_t s) {
+  const DecodeArgsBase& base = a;
+  if (a.uniform && n_items <= 2 * sm_count())
+    return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16, false, AHEAD>, n_items, 512, 0, s, base);
+  if (a.uniform) return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 4, false, AHEAD>, n_items, 128, 0, s, base);
+  return launch_chained(decode_attn_kernel<T, D, 1, 0, DecodeArgs, 4, false, AHEAD>, n_items, 128, 0, s, a);
+}
 template <typename T, int D>
 static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t s) {
-  // (bf16 comes here with more than 32 heads only)
-  if constexpr (sizeof(T) == 2) return launch_chained(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, n_items, 128, 0, s, a);
-  const DecodeArgsBase& base = a;
-  if (a.group == 1) {
-    // the register-capped kernel gets its own build for launches without split-K (which takes no table)
-    // few unsplit units (at most two 16-warp CTAs per SM, all resident at once): 16 warps per unit
-    if (a.uniform && n_items <= 2 * sm_count())
-      return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16>, n_items, 512, 0, s, base);
-    if (a.uniform) return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase>, n_items, 128, 0, s, base);
-    return launch_chained(decode_attn_kernel<T, D, 1, 0, DecodeArgs>, n_items, 128, 0, s, a);
+  if constexpr (sizeof(T) == 4) {  // (bf16 comes here with more than 32 heads only)
+    if (a.group == 1) return a.early ? launch_attn_one<T, D, true>(a, n_items, s) : launch_attn_one<T, D, false>(a, n_items, s);
+    if (a.group <= 4) return launch_chained(decode_attn_kernel<T, D, 4, -1, DecodeArgs>, n_items, 128, 0, s, a);
   }
-  if (a.group <= 4) return launch_chained(decode_attn_kernel<T, D, 4, -1, DecodeArgs>, n_items, 128, 0, s, a);
   return launch_chained(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, n_items, 128, 0, s, a);
 }
 
@@ -551,9 +573,11 @@ static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStre
   const size_t smem = bytes(pieces);
   if (smem > limit) return cudaErrorNotSupported;
   const int n_cta = (int)(units * pieces);
-  if (wide) return launch_scores_kernel<decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16, true>>(a, pieces, n_cta, 512, smem, s);
-  if (G == 1) return launch_scores_kernel<decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
-  if (G <= 4) return launch_scores_kernel<decode_attn_kernel<T, D, 4, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
+  // (rows ahead of the wait, us per token, one launch per layer: four heads, 12 layers, 8 sequences 329 with, 340
+  // without; 80 layers of 64 / 8 heads, 2 sequences 2352 with, 2315 without)
+  if (wide) return launch_scores_kernel<decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16, true, true>>(a, pieces, n_cta, 512, smem, s);
+  if (G == 1) return launch_scores_kernel<decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 4, true, true>>(a, pieces, n_cta, 128, smem, s);
+  if (G <= 4) return launch_scores_kernel<decode_attn_kernel<T, D, 4, 1, DecodeArgsBase, 4, true, true>>(a, pieces, n_cta, 128, smem, s);
   return launch_scores_kernel<decode_attn_kernel<T, D, 8, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
 }
 
