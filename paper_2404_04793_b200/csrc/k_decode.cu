@@ -522,6 +522,18 @@ __global__ void __launch_bounds__(32 * kWarpUpdWarps, 3) h2o_update_warp_kernel(
   }
 }
 
+// CTAs that start while the launch ahead runs out go where its short units have ended and crowd those SMs.  With long
+// pieces, or a wave or more of CTAs of unequal layers, that costs more than a launch's start.  us per token, chained /
+// not, fp32, 8 layers, 32 / 8 heads of 128: one launch, 1 sequence of 6000 tokens 141 / 132, 2 of 1500 74.6 / 70.2; one
+// per layer, 8 of 6000 1055 / 987.  Short pieces, one launch per layer, against the un-chained build: 1 of 600 180 / 160.
+template <typename K, typename A>
+static cudaError_t launch_pipe(K kern, const A& args, size_t elem, int n_items, int threads, cudaStream_t s) {
+  const size_t piece_bytes = 2 * elem * args.split_tokens * args.head_dim;
+  if ((args.early || n_items <= 2 * sm_count()) && piece_bytes <= 512 * 1024) return launch_chained(kern, n_items, threads, 0, s, args);
+  kern<<<n_items, threads, 0, s>>>(args);
+  return cudaGetLastError();
+}
+
 // One head: register-capped, so each form has its own build: with rows ahead of the wait or without (they
 // spill 8 to 60 bytes, which is worth it only where they hide a launch's start), with split-K (which takes the
 // table) or without, and for few unsplit units (at most two 16-warp CTAs per SM, all resident at once) 16 warps per unit.
@@ -531,17 +543,17 @@ template <typename T, int D, bool AHEAD>
 static cudaError_t launch_attn_one(const DecodeArgs& a, int n_items, cudaStream_t s) {
   const DecodeArgsBase& base = a;
   if (a.uniform && n_items <= 2 * sm_count())
-    return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16, false, AHEAD>, n_items, 512, 0, s, base);
-  if (a.uniform) return launch_chained(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 4, false, AHEAD>, n_items, 128, 0, s, base);
-  return launch_chained(decode_attn_kernel<T, D, 1, 0, DecodeArgs, 4, false, AHEAD>, n_items, 128, 0, s, a);
+    return launch_pipe(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16, false, AHEAD>, base, sizeof(T), n_items, 512, s);
+  if (a.uniform) return launch_pipe(decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 4, false, AHEAD>, base, sizeof(T), n_items, 128, s);
+  return launch_pipe(decode_attn_kernel<T, D, 1, 0, DecodeArgs, 4, false, AHEAD>, a, sizeof(T), n_items, 128, s);
 }
 template <typename T, int D>
 static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t s) {
   if constexpr (sizeof(T) == 4) {  // (bf16 comes here with more than 32 heads only)
     if (a.group == 1) return a.early ? launch_attn_one<T, D, true>(a, n_items, s) : launch_attn_one<T, D, false>(a, n_items, s);
-    if (a.group <= 4) return launch_chained(decode_attn_kernel<T, D, 4, -1, DecodeArgs>, n_items, 128, 0, s, a);
+    if (a.group <= 4) return launch_pipe(decode_attn_kernel<T, D, 4, -1, DecodeArgs>, a, sizeof(T), n_items, 128, s);
   }
-  return launch_chained(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, n_items, 128, 0, s, a);
+  return launch_pipe(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, a, sizeof(T), n_items, 128, s);
 }
 
 constexpr int kScoresLimit = 96 * 1024;  // dynamic shared memory of a CTA with the score update
