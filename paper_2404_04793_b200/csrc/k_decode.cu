@@ -593,6 +593,35 @@ static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStre
   return launch_scores_kernel<decode_attn_kernel<T, D, 8, 1, DecodeArgsBase, 4, true>>(a, pieces, n_cta, 128, smem, s);
 }
 
+// The second launch of H2O (scores and next victim, and for split units the merge), by a warp or a CTA per unit.
+// It walks a slot's logits four at a time and leaves the rest of their lines to L1.  A launch that starts while the
+// attention kernel runs out shares the SMs with that kernel's shared memory, which beside the bf16 kernels' tiles
+// leaves a fraction of the L1: it saves a launch's start (about 2 us) and pays by the logit.  So launches of more than a
+// million logits start after that kernel.  us per token, chained / after, 8 layers: one launch
+// for all, 16 sequences, 32 / 1 heads of 64, 12000 tokens 689 / 244, 4000: 235 / 93, 100: 15.7 / 19.0; one launch per
+// layer, 64 sequences, 32 / 1 heads of 128, 4000 tokens 887 / 687; 16 sequences, 16 / 1 heads of 64, 400 tokens 83 / 102.
+// fp32 (no tiles in shared memory) and up to four heads (one read per logit line): chained at most 6 % slower.
+static cudaError_t launch_second(const DecodeArgs& a, int dtype, const int* desc_tiles, cudaStream_t s) {
+  const int n_cta = a.n_layer_total * a.n_unit;
+  // More units than the CTA-per-unit kernel holds in one wave (5 CTAs per SM), and nothing to
+  // merge: only the scores and the next victim remain, one warp per unit.  Smaller launches
+  // (one layer of a small batch) finish sooner with a CTA per unit.
+  const bool by_warp = a.policy == SQ_POLICY_H2O && a.uniform && a.group <= 32 && n_cta > 5 * sm_count();
+  long long logits = 0;
+  for (int k = 0; k < a.n_layer_total; ++k) logits += 128LL * desc_tiles[k];
+  logits *= (long long)a.n_unit * a.group;
+  const bool chained = dtype == SQ_F32 || a.group <= 4 || logits <= 1 << 20;
+  auto go = [&](auto kern, int grid, int block, const auto& args) {
+    if (chained) return launch_chained(kern, grid, block, 0, s, args);
+    kern<<<grid, block, 0, s>>>(args);
+    return cudaGetLastError();
+  };
+  if (by_warp)
+    return go(h2o_update_warp_kernel, (n_cta + kWarpUpdWarps - 1) / kWarpUpdWarps, 32 * kWarpUpdWarps, static_cast<const DecodeArgsBase&>(a));
+  if (dtype == SQ_F32) return go(decode_combine_kernel<float>, n_cta, kSelThreads, a);
+  return go(decode_combine_kernel<__nv_bfloat16>, n_cta, kSelThreads, a);
+}
+
 // Which attention kernel serves a shape: wide bf16 groups at head_dim 64 go to the tcgen05 kernels, other
 // bf16 heads to the mma.sync kernels (one head per KV head too: 32 layers of 32 / 32 heads of 128, us per token,
 // the kernel of this file / mma.sync: 2 sequences 305 / 198, 8: 417 / 342, 40: 1835 / 1417), fp32 and the bf16 shapes
@@ -635,16 +664,7 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need
     if (e != cudaSuccess) return e;
   }
   if (!need_combine) return cudaSuccess;
-  const int n_cta = a.n_layer_total * a.n_unit;
-  // More units than the CTA-per-unit kernel holds in one wave (5 CTAs per SM), and nothing to
-  // merge: only the scores and the next victim remain, one warp per unit.  Smaller launches
-  // (one layer of a small batch) finish sooner with a CTA per unit.
-  if (a.policy == SQ_POLICY_H2O && a.uniform && a.group <= 32 && n_cta > 5 * sm_count()) {
-    return launch_chained(h2o_update_warp_kernel, (n_cta + kWarpUpdWarps - 1) / kWarpUpdWarps, 32 * kWarpUpdWarps, 0, s,
-                          static_cast<const DecodeArgsBase&>(a));
-  }
-  if (dtype == SQ_F32) return launch_chained(decode_combine_kernel<float>, n_cta, kSelThreads, 0, s, a);
-  return launch_chained(decode_combine_kernel<__nv_bfloat16>, n_cta, kSelThreads, 0, s, a);
+  return launch_second(a, dtype, desc_tiles, s);
 }
 
 }  // namespace sq

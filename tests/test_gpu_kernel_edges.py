@@ -175,15 +175,8 @@ def test_the_largest_weight_is_not_rounded(policy, head_dim, group):
     assert ctx.status() == 0
 
 
-# H2O with the score update inside the attention launch: pieces of a unit on the CTAs of a cluster, with
-# empty and ragged pieces, short and long layers, groups that are and are not multiples of four, both
-# head dims, and units too long or too many for it
-@pytest.mark.parametrize("dtype,head_dim,hq,hkv,batch,budgets", [
-    (torch.bfloat16, 128, 8, 2, 1, [1100, 70]), (torch.bfloat16, 128, 5, 1, 2, [129, 2000]), (torch.bfloat16, 64, 32, 1, 1, [513, 64]),
-    (torch.bfloat16, 128, 24, 1, 3, [700, 1]), (torch.bfloat16, 64, 6, 3, 50, [300, 290]), (torch.float32, 64, 3, 1, 1, [1400, 33]),
-    (torch.float32, 128, 16, 2, 2, [400, 31]), (torch.bfloat16, 128, 3, 3, 2, [900, 260]), (torch.bfloat16, 64, 4, 4, 40, [200, 333]),
-    (torch.bfloat16, 128, 31, 1, 1, [9000, 50])])
-def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, budgets):
+def h2o_lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack):
+    """Decode steps of all layers in one call or layer by layer, each step against the oracle from the library's state."""
     w = workload("fused", 9300 + budgets[0], dtype=dtype, head_dim=head_dim, n_q_head=hq, n_kv_head=hkv, n_layer=len(budgets),
                  batch=batch, prompt=max(budgets) + 5, steps=3, heavy_mode="zipf")
     ctx = H.make_ctx(w, b_init=max(budgets))
@@ -199,8 +192,11 @@ def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, bud
         out = torch.empty_like(q)
         # the oracle takes the library's rows and scores before the step: one step's arithmetic is compared
         before = {u: (ctx.get_kept(*u), ctx.get_kv(*u)) for u in units}
-        for l in range(w.n_layer):
-            ctx.decode_step(l, l + 1, q[l], kn[l], vn[l], out[l])
+        if stack:
+            ctx.decode_step(0, w.n_layer, q, kn, vn, out)
+        else:
+            for l in range(w.n_layer):
+                ctx.decode_step(l, l + 1, q[l], kn[l], vn[l], out[l])
         for (l, s, h), ((pos, acc), (kk, vv)) in before.items():
             u = O.UnitCache(w.policy, budgets[l], w.n_sink, w.heavy_num, w.heavy_den)
             u.pos, u.acc, u.K, u.V = list(pos), [float(x) for x in acc], list(H.f64(kk)), list(H.f64(vv))
@@ -214,6 +210,30 @@ def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, bud
             assert pos2 == u.kept_positions()
             np.testing.assert_allclose(acc2, u.acc, rtol=H.RTOL_ACC[dtype], atol=1e-6)
     assert ctx.status() == 0
+
+
+# H2O with the score update inside the attention launch: pieces of a unit on the CTAs of a cluster, with
+# empty and ragged pieces, short and long layers, groups that are and are not multiples of four, both
+# head dims, and units too long or too many for it
+@pytest.mark.parametrize("dtype,head_dim,hq,hkv,batch,budgets", [
+    (torch.bfloat16, 128, 8, 2, 1, [1100, 70]), (torch.bfloat16, 128, 5, 1, 2, [129, 2000]), (torch.bfloat16, 64, 32, 1, 1, [513, 64]),
+    (torch.bfloat16, 128, 24, 1, 3, [700, 1]), (torch.bfloat16, 64, 6, 3, 50, [300, 290]), (torch.float32, 64, 3, 1, 1, [1400, 33]),
+    (torch.float32, 128, 16, 2, 2, [400, 31]), (torch.bfloat16, 128, 3, 3, 2, [900, 260]), (torch.bfloat16, 64, 4, 4, 40, [200, 333]),
+    (torch.bfloat16, 128, 31, 1, 1, [9000, 50])])
+def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, budgets):
+    h2o_lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack=False)
+
+
+# Launches on both sides of the rules that choose between that form and the second launch (started while the attention
+# kernel runs out, or after it)
+@pytest.mark.parametrize("dtype,head_dim,hq,hkv,batch,budgets", [
+    (torch.bfloat16, 64, 32, 1, 40, [1500, 200]), (torch.bfloat16, 64, 20, 1, 64, [300, 1400]), (torch.bfloat16, 128, 32, 1, 60, [100, 40]),
+    (torch.bfloat16, 128, 16, 2, 160, [400, 130]), (torch.bfloat16, 128, 4, 1, 150, [2900, 700]), (torch.bfloat16, 128, 12, 4, 70, [333, 64]),
+    (torch.bfloat16, 64, 10, 10, 130, [60, 200]), (torch.bfloat16, 128, 30, 30, 50, [120, 3]), (torch.float32, 128, 8, 2, 1, [4000, 600]),
+    (torch.float32, 64, 16, 2, 70, [1500, 100]), (torch.float32, 64, 6, 6, 210, [200, 90])])
+@pytest.mark.parametrize("stack", [False, True])
+def test_h2o_forms_of_larger_launches(dtype, head_dim, hq, hkv, batch, budgets, stack):
+    h2o_lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack)
 
 
 # Selection over the prompt: block sizes by prompt length and the form for longer prompts, ties across the
