@@ -549,10 +549,9 @@ static cudaError_t launch_attn_one(const DecodeArgs& a, int n_items, cudaStream_
 }
 template <typename T, int D>
 static cudaError_t launch_attn_g(const DecodeArgs& a, int n_items, cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) {  // (bf16 comes here with more than 32 heads only)
-    if (a.group == 1) return a.early ? launch_attn_one<T, D, true>(a, n_items, s) : launch_attn_one<T, D, false>(a, n_items, s);
+  if (a.group == 1) return a.early ? launch_attn_one<T, D, true>(a, n_items, s) : launch_attn_one<T, D, false>(a, n_items, s);
+  if constexpr (sizeof(T) == 4)  // (bf16 comes here with one head or more than 32)
     if (a.group <= 4) return launch_pipe(decode_attn_kernel<T, D, 4, -1, DecodeArgs>, a, sizeof(T), n_items, 128, s);
-  }
   return launch_pipe(decode_attn_kernel<T, D, 8, -1, DecodeArgs>, a, sizeof(T), n_items, 128, s);
 }
 
@@ -622,10 +621,30 @@ static cudaError_t launch_second(const DecodeArgs& a, int dtype, const int* desc
   return go(decode_combine_kernel<__nv_bfloat16>, n_cta, kSelThreads, a);
 }
 
-// Which attention kernel serves a shape: wide bf16 groups at head_dim 64 go to the tcgen05 kernels, other
-// bf16 heads to the mma.sync kernels (one head per KV head too: 32 layers of 32 / 32 heads of 128, us per token,
-// the kernel of this file / mma.sync: 2 sequences 305 / 198, 8: 417 / 342, 40: 1835 / 1417), fp32 and the bf16 shapes
-// those do not cover to the fp32-pipe kernel.
+// One bf16 head per KV head: the mma.sync kernel, but for short caches, where a unit is over before its pipeline of
+// tiles pays, and for launches of very many units, where the fp32-pipe kernel's eight CTAs per SM keep as much in flight.
+// Between one and two units per SM the mma.sync kernel wins at any length.  Time of the fp32-pipe kernel over the other's,
+// 32 / 32 heads of 128 in launches of one layer: caches of 60 tokens 0.62 to 0.95, 200 0.83 to 1.08, 300 1.44 and more up to
+// 512 units, 0.98 for 2048; of 8 layers: 60 0.61 to 0.93, 200 0.77 to 0.94, 300 1.09 and more up to 1024 units, 0.93 for 4096, 700
+// 0.97 for 4096; heads of 64 cross over at twice the length.  One launch per layer, 32 layers, caches of 409 on average, us per
+// token, fp32 pipe / mma.sync: 2 sequences 305 / 198, 8: 417 / 342, 40: 1835 / 1417.
+static bool one_head_on_pipe(int n_desc, int n_unit, int head_dim, int max_len) {
+  const long long units = (long long)n_desc * n_unit, n_sm = sm_count(), row_elems = (long long)max_len * head_dim;
+  if (units <= n_sm) return max_len <= 320;
+  if (units <= 2 * n_sm) return false;
+  if (units < 8 * n_sm) return max_len <= 200;
+  return row_elems <= 64 * 1024 || (units >= 24 * n_sm && n_desc > 1 && row_elems <= 160 * 1024);
+}
+
+DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, int n_unit, int max_len) {
+  if (dtype != SQ_BF16) return DecodeKernel::kPipe;
+  if (group > 32) return head_dim == 64 ? DecodeKernel::kTcgen05 : DecodeKernel::kPipe;
+  if (group == 1 && one_head_on_pipe(n_desc, n_unit, head_dim, max_len)) return DecodeKernel::kPipe;
+  return DecodeKernel::kMma;
+}
+
+// decode_kernel_for() names the attention kernel; where the tcgen05 kernels refuse a launch (a pool or a batch
+// beyond 32-bit tile coordinates), the mma.sync kernel takes up to 96 heads of it and the fp32-pipe kernel the rest.
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
                           size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
@@ -652,7 +671,7 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need
     else e = a.head_dim == 64 ? launch_attn_scores<float, 64>(a, max_len, s) : launch_attn_scores<float, 128>(a, max_len, s);
     if (e != cudaErrorNotSupported) return e;
   }
-  if (!done && dtype == SQ_BF16) {
+  if (!done && decode_kernel_for(dtype, a.head_dim, a.group, a.n_layer_total, a.n_unit, max_len) != DecodeKernel::kPipe) {
     cudaError_t e = launch_decode_attn_mma(a, n_items, s);
     if (e == cudaSuccess) done = true;
     else if (e != cudaErrorNotSupported) return e;

@@ -630,21 +630,24 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
     // only units in several pieces pay, is 0) and a wave are depends on the kernel the shape is served by.  The running item counts of a split launch
     // travel in the kernel parameters, which hold kMaxLayers descriptors: larger launches (many
     // sequences with per-sequence budgets) are not split; they have units to spare anyway.
-    const bool bf16 = cfg.dtype == SQ_BF16;
+    int max_len = 1;
+    for (int d = d0; d < d1; ++d) max_len = std::max(max_len, std::min(n_tok + 1, c->hs.layers[d].b));
+    const DecodeKernel kern = decode_kernel_for(cfg.dtype, cfg.head_dim, G, d1 - d0, U, max_len);
     int tile, setup, per_sm, merge = 0;
     double gain = 0.90;  // more pieces only for a clear gain
-    if (bf16 && cfg.head_dim == 64 && G > 32) {  // tcgen05 kernel: 128-token tiles, 2 CTAs per SM
+    if (kern == DecodeKernel::kTcgen05) {        // 128-token tiles, 2 CTAs per SM
       // us per token, 32 layers, (setup, merge, gain) = (8, 0, 0.90) / (8, 0, 0.95) / (4, 4, 0.95): 33 sequences of
       // 8191, 50 %, H2O 1278 / 1217 / 1217; 60 of 4000, 30 % 548 / 667 / 540; 8 of 8191, 30 %, H2O 1028 / 1098 / 1045
       tile = 128, setup = 4, merge = 4, per_sm = 2, gain = 0.95;
-    } else if (bf16) {                           // mma.sync kernels: 64-token tiles
-      tile = 64, setup = 12, per_sm = cfg.head_dim == 64 && G <= 32 ? 3 : 2;
+    } else if (cfg.dtype == SQ_BF16 && (kern == DecodeKernel::kMma || G > 1)) {
+      // 64-token tiles of the mma.sync kernels.  (Also for groups above 32 at head_dim 128, which the fp32-pipe kernel
+      // takes: 40 / 1 heads, 8 layers, one launch for all, caches of 200 and 1500, 8 sequences: 68 / 157 us per token, with
+      // the constants below 101 / 182; one launch per layer, 6000: 1066, with those below 1192.)
+      tile = 64, setup = 12, per_sm = cfg.head_dim == 64 ? 3 : 2;
     } else {                                     // fp32-pipe kernel
       tile = 128, setup = 1, per_sm = G == 1 ? 7 : 2;
     }
     const long long slots = (long long)per_sm * c->n_sm;
-    int max_len = 1;
-    for (int d = d0; d < d1; ++d) max_len = std::max(max_len, std::min(n_tok + 1, c->hs.layers[d].b));
     int split = 0;
     double best_cost = 0.0;
     int prev = -1;

@@ -168,6 +168,9 @@ cudaError_t launch_prefill_scores_alu(const ScoreArgs& a, int dtype, cudaStream_
 cudaError_t launch_prefill_scores_tc(const ScoreArgs& a, int* status, cudaStream_t s);
 cudaError_t launch_select_prompt(const float* acc_prompt, int n_unit, int prompt, const LayerDesc* descs,
                                  int units_per_desc, bool any_full, char* pool, cudaStream_t s);
+// Attention kernel of a launch over n_desc descriptors of n_unit units, the longest of max_len slots.
+enum class DecodeKernel { kTcgen05, kMma, kPipe };  // wide groups; mma.sync; fp32 pipes
+DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, int n_unit, int max_len);
 // desc_tiles: per descriptor of the launch (launch order) the 128-token tiles of one unit; max_len: slots of the longest unit
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
                           size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s);

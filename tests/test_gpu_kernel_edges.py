@@ -225,7 +225,7 @@ def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, bud
 
 
 # Launches on both sides of the rules that choose between that form and the second launch (started while the attention
-# kernel runs out, or after it)
+# kernel runs out, or after it), and of the one that sends one bf16 head per KV head to the fp32 pipes
 @pytest.mark.parametrize("dtype,head_dim,hq,hkv,batch,budgets", [
     (torch.bfloat16, 64, 32, 1, 40, [1500, 200]), (torch.bfloat16, 64, 20, 1, 64, [300, 1400]), (torch.bfloat16, 128, 32, 1, 60, [100, 40]),
     (torch.bfloat16, 128, 16, 2, 160, [400, 130]), (torch.bfloat16, 128, 4, 1, 150, [2900, 700]), (torch.bfloat16, 128, 12, 4, 70, [333, 64]),
@@ -234,6 +234,41 @@ def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, bud
 @pytest.mark.parametrize("stack", [False, True])
 def test_h2o_forms_of_larger_launches(dtype, head_dim, hq, hkv, batch, budgets, stack):
     h2o_lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack)
+
+
+# One bf16 head per KV head on either kernel: few units, between one and two per SM, a few, many; lengths around the
+# limits; whole stack (with split units among them) and layer by layer
+@pytest.mark.parametrize("head_dim,hkv,batch,budgets", [
+    (128, 4, 3, [320, 17, 321]), (64, 16, 9, [320, 64]), (64, 25, 9, [150, 320]), (128, 40, 15, [200, 201]), (64, 40, 15, [190, 260]),
+    (64, 60, 20, [1024, 1025, 1]), (128, 60, 20, [512, 600])])
+@pytest.mark.parametrize("stack", [False, True])
+def test_one_bf16_head_on_either_kernel(head_dim, hkv, batch, budgets, stack):
+    w = workload("one head", 9700 + budgets[0], policy=synth.SLIDING_WINDOW, head_dim=head_dim, n_q_head=hkv, n_kv_head=hkv,
+                 n_layer=len(budgets), batch=batch, prompt=max(budgets) + 3, steps=2, heavy_mode="none")
+    ctx = H.make_ctx(w, b_init=max(budgets))
+    ctx.begin_sequence_batch(batch, w.prompt)
+    ctx.set_budgets(budgets)
+    units = {}
+    for l in range(w.n_layer):
+        _, k, v = synth.prompt_qkv(w, l, DEV, need_q=False)
+        ctx.prefill_compress(l, k, v)
+        for s in (0, batch - 1):
+            for h in (0, hkv - 1):
+                units[l, s, h] = O.UnitCache(w.policy, budgets[l])
+                units[l, s, h].prefill(H.f64(k[s, h]), H.f64(v[s, h]))
+    for t in range(w.steps):
+        q, kn, vn = synth.decode_qkv(w, t, DEV)
+        out = torch.empty_like(q)
+        if stack:
+            ctx.decode_step(0, w.n_layer, q, kn, vn, out)
+        else:
+            for l in range(w.n_layer):
+                ctx.decode_step(l, l + 1, q[l], kn[l], vn[l], out[l])
+        for (l, s, h), u in units.items():
+            want = u.decode_step(H.f64(q[l, s, h:h + 1]), H.f64(kn[l, s, h]), H.f64(vn[l, s, h]))
+            # weights at fp32 precision: the bf16 output (half an ulp, 2^-9) and fp32 sums
+            assert np.all(np.abs(H.f64(out[l, s, h:h + 1]) - want) <= np.abs(want) * 2.0 ** -8 + 1e-4), (t, l, s, h)
+    assert ctx.status() == 0
 
 
 # Selection over the prompt: block sizes by prompt length and the form for longer prompts, ties across the
