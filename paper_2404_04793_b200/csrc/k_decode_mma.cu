@@ -415,7 +415,13 @@ static cudaError_t launch_scores_cfg(const DecodeArgs& a, int pieces, size_t log
 
 // H2O with the score update in the launch.  max_len: slots of the longest unit.  Returns
 // cudaErrorNotSupported where the second launch (decode_combine_kernel, h2o_update_warp_kernel) is the
-// better form or the logits of a piece do not fit.
+// better form or the logits of a piece do not fit.  The better form it is for launches of more CTAs than are resident at
+// once, unless the pieces are equal (one layer, or few units) or the group is small and its pieces are short (one per
+// unit) or long: all units are cut into the same number of pieces, which for short layers beside long ones, and
+// where the logits ask for more pieces than the launch does, are too small.  us per token, second launch / this form, 8
+// layers: one launch, 64 sequences of 1500 tokens, 32 / 1 heads of 64 99 / 163, 16 / 1 56 / 85; 8 of 1500, 64 / 8 heads of 128 76 /
+// 97; 16 of 100, 32 / 1 of 128 19 / 24; 8 of 1500, 32 / 1 of 64 45 / 24; one launch per layer, 64 of 1500, 20 / 1 244 / 127, 64 / 8 514
+// / 637.
 // Pieces: as many as leave all CTAs resident at once (two per SM), a tile or more each; up to 16 where few
 // clusters of that size are enough (more of them do not all fit at once beside smaller ones).  Measured, us
 // per token of 32 layers of 32 / 8 heads of 128, one launch per layer, second launch / this form: 1 sequence
@@ -435,11 +441,19 @@ cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStrea
   const size_t fixed = (size_t)2 * stages * kTile * a.head_dim * 2;
   auto logit_bytes = [&](int p) { return (size_t)piece_tiles(max_len, p) * kTile * G * 4; };
   auto launch = [&](int limit) {
-    int pieces = (int)std::min<long long>(limit, std::max<long long>(1, 2 * n_sm / units));
-    pieces = std::min(pieces, tiles);
+    const int wanted = (int)std::min<long long>({limit, std::max<long long>(1, 2 * n_sm / units), tiles});
+    int pieces = wanted;
     while (pieces < 8 && fixed + logit_bytes(pieces) > kScoresSmem) ++pieces;
     const size_t lb = logit_bytes(pieces);
     if (fixed + lb > kScoresSmem) return cudaErrorNotSupported;
+    const long long ctas = units * pieces;
+    if (ctas > 2 * n_sm) {  // more than one wave
+      if (pieces > wanted && piece_tiles(max_len, pieces) == 1) return cudaErrorNotSupported;
+      const int len = max_len / pieces;
+      const bool even = units <= n_sm || a.n_layer_total == 1;
+      const bool low = G <= 4 && ((pieces == 1 && len <= 2432 && ctas <= 4 * n_sm) || (len >= 2560 && len <= 5120 && ctas <= 12 * n_sm));
+      if (!(even && ctas <= 7 * n_sm) && !low) return cudaErrorNotSupported;
+    }
     if (G <= 8) return launch_decode_mma_low(a, 0, pieces, lb, s);
     if (a.head_dim == 128) return G <= 16 ? launch_scores_cfg<128, 1, 3>(a, pieces, lb, s) : launch_scores_cfg<128, 2, 3>(a, pieces, lb, s);
     return G <= 16 ? launch_scores_cfg<64, 1, 4>(a, pieces, lb, s) : launch_scores_cfg<64, 2, 4>(a, pieces, lb, s);
