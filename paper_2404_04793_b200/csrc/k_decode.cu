@@ -565,8 +565,12 @@ static cudaError_t launch_scores_kernel(const DecodeArgs& a, int pieces, int n_c
 }
 
 // H2O with the score update in the launch.  Returns cudaErrorNotSupported where the second launch
-// (decode_combine_kernel, h2o_update_warp_kernel) is needed: a piece's logits do not fit.
-// Measured, us per token, second launch / this form: fp32, 12 layers of 16 / 4 heads of 128, 8 sequences: 331 / 271.
+// (decode_combine_kernel, h2o_update_warp_kernel) is needed, because a piece's logits do not fit, or the better form: a
+// unit has at most eight pieces here, so that long caches of few units leave the GPU idle, and the logits of long pieces
+// leave room for fewer CTAs on an SM.  us per token, second launch / this form, fp32: 12 layers of 16 / 4 heads of 128, 8
+// sequences 331 / 271; 8 layers of 32 / 8 heads of 128: one launch per layer, 1 sequence of 1500 tokens 264 / 193, 4000: 320 /
+// 379, 12000: 539 / 1018; one launch, 8 of 4000 491 / 916; 16 / 2 heads of 64, 64 of 1500, one launch per layer 501 / 444; 4 / 4
+// heads of 64, one launch, 4 of 400 14.3 / 10.6, 16 of 4000 142 / 159.
 template <typename T, int D>
 static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
   const int G = a.group;
@@ -583,7 +587,16 @@ static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStre
   while (pieces < kMaxPieces && bytes(pieces) > limit) ++pieces;
   const size_t smem = bytes(pieces);
   if (smem > limit) return cudaErrorNotSupported;
-  const int n_cta = (int)(units * pieces);
+  const long long ctas = units * pieces;
+  const int len = (max_len + pieces - 1) / pieces;
+  const bool one_layer = a.n_layer_total == 1;
+  if (G == 1) {
+    if (ctas > (one_layer ? 8 : 4) * n_sm) return cudaErrorNotSupported;
+  } else {
+    const bool filled = G > 4 && one_layer && 5 * ctas >= 8 * n_sm;  // equal pieces on nearly every slot
+    if (ctas > 4 * n_sm || (len > (G > 4 && G <= 8 ? 800 : 640) && !filled)) return cudaErrorNotSupported;
+  }
+  const int n_cta = (int)ctas;
   // (rows ahead of the wait, us per token, one launch per layer: four heads, 12 layers, 8 sequences 329 with, 340
   // without; 80 layers of 64 / 8 heads, 2 sequences 2352 with, 2315 without)
   if (wide) return launch_scores_kernel<decode_attn_kernel<T, D, 1, 1, DecodeArgsBase, 16, true, true>>(a, pieces, n_cta, 512, smem, s);
