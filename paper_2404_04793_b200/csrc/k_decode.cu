@@ -569,8 +569,9 @@ static cudaError_t launch_scores_kernel(const DecodeArgs& a, int pieces, int n_c
 // unit has at most eight pieces here, so that long caches of few units leave the GPU idle, and the logits of long pieces
 // leave room for fewer CTAs on an SM.  us per token, second launch / this form, fp32: 12 layers of 16 / 4 heads of 128, 8
 // sequences 331 / 271; 8 layers of 32 / 8 heads of 128: one launch per layer, 1 sequence of 1500 tokens 264 / 193, 4000: 320 /
-// 379, 12000: 539 / 1018; one launch, 8 of 4000 491 / 916; 16 / 2 heads of 64, 64 of 1500, one launch per layer 501 / 444; 4 / 4
-// heads of 64, one launch, 4 of 400 14.3 / 10.6, 16 of 4000 142 / 159.
+// 379, 12000: 539 / 1018; one launch, 1 of 1500 60 / 76, 8 of 4000 491 / 916; 16 / 2 heads of 64, 64 of 1500, one launch per
+// layer 501 / 444; 4 / 4 heads of 64, one launch, 4 of 400 14.3 / 10.6, 16 of 4000 142 / 159; 32 / 32 of 128, one launch, 1
+// of 1500 75 / 83, 4000: 182 / 206, 12000: 543 / 635.
 template <typename T, int D>
 static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStream_t s) {
   const int G = a.group;
@@ -591,10 +592,10 @@ static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStre
   const int len = (max_len + pieces - 1) / pieces;
   const bool one_layer = a.n_layer_total == 1;
   if (G == 1) {
-    if (ctas > (one_layer ? 8 : 4) * n_sm) return cudaErrorNotSupported;
+    if (ctas > (one_layer ? 8 : 4) * n_sm || (!one_layer && units > n_sm && len > 1200)) return cudaErrorNotSupported;
   } else {
     const bool filled = G > 4 && one_layer && 5 * ctas >= 8 * n_sm;  // equal pieces on nearly every slot
-    if (ctas > 4 * n_sm || (len > (G > 4 && G <= 8 ? 800 : 640) && !filled)) return cudaErrorNotSupported;
+    if (ctas > 4 * n_sm || (len > (one_layer ? 600 : 320) && !filled)) return cudaErrorNotSupported;
   }
   const int n_cta = (int)ctas;
   // (rows ahead of the wait, us per token, one launch per layer: four heads, 12 layers, 8 sequences 329 with, 340
@@ -608,10 +609,11 @@ static cudaError_t launch_attn_scores(const DecodeArgs& a, int max_len, cudaStre
 // The second launch of H2O (scores and next victim, and for split units the merge), by a warp or a CTA per unit.
 // It walks a slot's logits four at a time and leaves the rest of their lines to L1.  A launch that starts while the
 // attention kernel runs out shares the SMs with that kernel's shared memory, which beside the bf16 kernels' tiles
-// leaves a fraction of the L1: it saves a launch's start (about 2 us) and pays by the logit.  So launches of more than a
-// million logits start after that kernel.  us per token, chained / after, 8 layers: one launch
+// leaves a fraction of the L1: it saves a launch's start (about 2 us) and pays by the logit.  So launches of more than
+// three quarters of a million logits start after that kernel.  us per token, chained / after, 8 layers: one launch
 // for all, 16 sequences, 32 / 1 heads of 64, 12000 tokens 689 / 244, 4000: 235 / 93, 100: 15.7 / 19.0; one launch per
-// layer, 64 sequences, 32 / 1 heads of 128, 4000 tokens 887 / 687; 16 sequences, 16 / 1 heads of 64, 400 tokens 83 / 102.
+// layer, 64 sequences, 32 / 1 heads of 128, 4000 tokens 887 / 687; 16 sequences, 16 / 1 heads of 64, 400 tokens 83 / 102;
+// geometric means over groups of 9 to 32: a quarter of a million logits 0.92 to 0.97, half 0.95 to 1.2, two 1.05 to 1.12.
 // fp32 (no tiles in shared memory) and up to four heads (one read per logit line): chained at most 6 % slower.
 static cudaError_t launch_second(const DecodeArgs& a, int dtype, const int* desc_tiles, cudaStream_t s) {
   const int n_cta = a.n_layer_total * a.n_unit;
@@ -622,7 +624,7 @@ static cudaError_t launch_second(const DecodeArgs& a, int dtype, const int* desc
   long long logits = 0;
   for (int k = 0; k < a.n_layer_total; ++k) logits += 128LL * desc_tiles[k];
   logits *= (long long)a.n_unit * a.group;
-  const bool chained = dtype == SQ_F32 || a.group <= 4 || logits <= 1 << 20;
+  const bool chained = dtype == SQ_F32 || a.group <= 4 || logits <= 3 << 18;
   auto go = [&](auto kern, int grid, int block, const auto& args) {
     if (chained) return launch_chained(kern, grid, block, 0, s, args);
     kern<<<grid, block, 0, s>>>(args);
@@ -641,18 +643,22 @@ static cudaError_t launch_second(const DecodeArgs& a, int dtype, const int* desc
 // 512 units, 0.98 for 2048; of 8 layers: 60 0.61 to 0.93, 200 0.77 to 0.94, 300 1.09 and more up to 1024 units, 0.93 for 4096, 700
 // 0.97 for 4096; heads of 64 cross over at twice the length.  One launch per layer, 32 layers, caches of 409 on average, us per
 // token, fp32 pipe / mma.sync: 2 sequences 305 / 198, 8: 417 / 342, 40: 1835 / 1417.
-static bool one_head_on_pipe(int n_desc, int n_unit, int head_dim, int max_len) {
+// Under H2O the logits go to memory, where the scores are not updated in the launch: with layers of unequal length the
+// fp32-pipe kernel is then the faster one up to eight units per SM (8 layers of 8 / 8 heads of 64 in one launch, 16
+// sequences of 1500 tokens 80 / 123, 4000: 184 / 300; 32 / 32 of 128, 4 of 1500 146 / 177).
+static bool one_head_on_pipe(int n_desc, int n_unit, int head_dim, int max_len, bool h2o) {
   const long long units = (long long)n_desc * n_unit, n_sm = sm_count(), row_elems = (long long)max_len * head_dim;
   if (units <= n_sm) return max_len <= 320;
-  if (units <= 2 * n_sm) return false;
-  if (units < 8 * n_sm) return max_len <= 200;
+  const bool uneven = h2o && n_desc > 1;
+  if (units <= 2 * n_sm) return uneven && head_dim == 64 && max_len > 2048;
+  if (units < 8 * n_sm) return uneven || max_len <= 200;
   return row_elems <= 64 * 1024 || (units >= 24 * n_sm && n_desc > 1 && row_elems <= 160 * 1024);
 }
 
-DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, int n_unit, int max_len) {
+DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, int n_unit, int max_len, bool h2o) {
   if (dtype != SQ_BF16) return DecodeKernel::kPipe;
   if (group > 32) return head_dim == 64 ? DecodeKernel::kTcgen05 : DecodeKernel::kPipe;
-  if (group == 1 && one_head_on_pipe(n_desc, n_unit, head_dim, max_len)) return DecodeKernel::kPipe;
+  if (group == 1 && one_head_on_pipe(n_desc, n_unit, head_dim, max_len, h2o)) return DecodeKernel::kPipe;
   return DecodeKernel::kMma;
 }
 
@@ -684,7 +690,7 @@ cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need
     else e = a.head_dim == 64 ? launch_attn_scores<float, 64>(a, max_len, s) : launch_attn_scores<float, 128>(a, max_len, s);
     if (e != cudaErrorNotSupported) return e;
   }
-  if (!done && decode_kernel_for(dtype, a.head_dim, a.group, a.n_layer_total, a.n_unit, max_len) != DecodeKernel::kPipe) {
+  if (!done && decode_kernel_for(dtype, a.head_dim, a.group, a.n_layer_total, a.n_unit, max_len, a.policy == SQ_POLICY_H2O) != DecodeKernel::kPipe) {
     cudaError_t e = launch_decode_attn_mma(a, n_items, s);
     if (e == cudaSuccess) done = true;
     else if (e != cudaErrorNotSupported) return e;

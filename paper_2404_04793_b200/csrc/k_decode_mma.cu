@@ -447,6 +447,8 @@ cudaError_t launch_decode_mma_scores(const DecodeArgs& a, int max_len, cudaStrea
     const size_t lb = logit_bytes(pieces);
     if (fixed + lb > kScoresSmem) return cudaErrorNotSupported;
     const long long ctas = units * pieces;
+    // (one head of 64: the fp32-pipe kernel and a second launch, see one_head_on_pipe())
+    if (G == 1 && a.head_dim == 64 && a.n_layer_total > 1 && units > n_sm && max_len > 2048) return cudaErrorNotSupported;
     if (ctas > 2 * n_sm) {  // more than one wave
       if (pieces > wanted && piece_tiles(max_len, pieces) == 1) return cudaErrorNotSupported;
       const int len = max_len / pieces;

@@ -632,7 +632,7 @@ int sq_decode_step(sq_ctx* c, int32_t layer_begin, int32_t layer_end, const void
     // sequences with per-sequence budgets) are not split; they have units to spare anyway.
     int max_len = 1;
     for (int d = d0; d < d1; ++d) max_len = std::max(max_len, std::min(n_tok + 1, c->hs.layers[d].b));
-    const DecodeKernel kern = decode_kernel_for(cfg.dtype, cfg.head_dim, G, d1 - d0, U, max_len);
+    const DecodeKernel kern = decode_kernel_for(cfg.dtype, cfg.head_dim, G, d1 - d0, U, max_len, cfg.policy == SQ_POLICY_H2O);
     int tile, setup, per_sm, merge = 0;
     double gain = 0.90;  // more pieces only for a clear gain
     if (kern == DecodeKernel::kTcgen05) {        // 128-token tiles, 2 CTAs per SM

@@ -170,7 +170,7 @@ cudaError_t launch_select_prompt(const float* acc_prompt, int n_unit, int prompt
                                  int units_per_desc, bool any_full, char* pool, cudaStream_t s);
 // Attention kernel of a launch over n_desc descriptors of n_unit units, the longest of max_len slots.
 enum class DecodeKernel { kTcgen05, kMma, kPipe };  // wide groups; mma.sync; fp32 pipes
-DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, int n_unit, int max_len);
+DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, int n_unit, int max_len, bool h2o);
 // desc_tiles: per descriptor of the launch (launch order) the 128-token tiles of one unit; max_len: slots of the longest unit
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
                           size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s);

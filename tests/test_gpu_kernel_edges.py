@@ -230,7 +230,8 @@ def test_h2o_scores_in_the_attention_launch(dtype, head_dim, hq, hkv, batch, bud
     (torch.bfloat16, 64, 32, 1, 40, [1500, 200]), (torch.bfloat16, 64, 20, 1, 64, [300, 1400]), (torch.bfloat16, 128, 32, 1, 60, [100, 40]),
     (torch.bfloat16, 128, 16, 2, 160, [400, 130]), (torch.bfloat16, 128, 4, 1, 150, [2900, 700]), (torch.bfloat16, 128, 12, 4, 70, [333, 64]),
     (torch.bfloat16, 64, 10, 10, 130, [60, 200]), (torch.bfloat16, 128, 30, 30, 50, [120, 3]), (torch.float32, 128, 8, 2, 1, [4000, 600]),
-    (torch.float32, 64, 16, 2, 70, [1500, 100]), (torch.float32, 64, 6, 6, 210, [200, 90])])
+    (torch.float32, 64, 16, 2, 70, [1500, 100]), (torch.float32, 64, 6, 6, 210, [200, 90]), (torch.bfloat16, 64, 8, 8, 11, [2049, 300]),
+    (torch.bfloat16, 64, 8, 8, 60, [700, 150]), (torch.float32, 128, 8, 2, 4, [330, 80]), (torch.float32, 128, 32, 32, 3, [1300, 40])])
 @pytest.mark.parametrize("stack", [False, True])
 def test_h2o_forms_of_larger_launches(dtype, head_dim, hq, hkv, batch, budgets, stack):
     h2o_lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack)
