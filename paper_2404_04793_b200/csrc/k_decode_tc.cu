@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(192, 2)
       ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld / st are warp-wide
       if (!ok) break;
       tc_fence_after();
-      bool s_released = rows.template tile<true>(n_valid, i == 0, bar_sfree, [&]() {
+      bool s_released = rows.tile(n_valid, i == 0, bar_sfree, [&]() {
         if (i >= 1) ok = __all_sync(0xffffffffu, mbar_wait(bar_pfree, (i - 1) & 1, abort_flag));
       });
       if (!ok) break;
@@ -266,7 +266,7 @@ __global__ void __launch_bounds__(192, 2)
         if (!ok) break;
         tc_fence_after();
         rows.redo(n_valid);
-        s_released = rows.template tile<true>(n_valid, false, bar_sfree, []() {});
+        s_released = rows.tile(n_valid, false, bar_sfree, []() {});
       }
       rows.add_tile();
       tc_fence_before();

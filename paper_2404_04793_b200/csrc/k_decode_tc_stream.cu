@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
         }
         if (!ok) break;
         tc_fence_after();
-        bool s_released = rows.template tile<true>(n_valid, i == 0, bar_sfree, [&]() {
+        bool s_released = rows.tile(n_valid, i == 0, bar_sfree, [&]() {
           if (g >= 1) ok = warp_wait(bar_pfree, (g - 1) & 1, abort_flag);
         });
         if (!ok) break;
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
           if (!ok) break;
           tc_fence_after();
           rows.redo(n_valid);
-          s_released = rows.template tile<true>(n_valid, false, bar_sfree, []() {});
+          s_released = rows.tile(n_valid, false, bar_sfree, []() {});
         }
         rows.add_tile();
         tc_fence_before();

@@ -131,7 +131,7 @@ struct WideRows {
   // returns whether it was.
   // p_free() waits for the product that still reads the tile before's P: before the first store only, so
   // that the first 64 columns are worked out meanwhile.
-  template <int HF, bool TWO, bool LAST, bool EARLY, class PFree>
+  template <int HF, bool TWO, bool LAST, class PFree>
   __device__ __forceinline__ bool half(int n_valid, bool first, uint32_t bar_sfree, bool wait_p, PFree p_free) {
     constexpr int A = 2 * HF, B = TWO ? 2 * HF + 1 : 2 * HF;
     const uint32_t s = s_addr + ((uint32_t)(16 * HF) << 16), p = p_addr + ((uint32_t)(16 * HF) << 16);
@@ -157,7 +157,7 @@ struct WideRows {
     tmem_wait_ld(rb);
     if (n_valid < kTM) mask(rb, 1, n_valid);
     bool released = false;
-    if (LAST && EARLY) {
+    if (LAST) {
       // 16 weights of at most 2^10 and 2^15 before them stay below kMaxWeight
       bool safe = w[0] + w[1] <= 32768.f && fmaf(row_max(rb, 0, -INFINITY), scale_log2, -m[A]) <= 10.f;
       if (TWO) safe = safe && w[2] + w[3] <= 32768.f && fmaf(row_max(rb, 2, -INFINITY), scale_log2, -m[B]) <= 10.f;
@@ -185,13 +185,13 @@ struct WideRows {
   }
   // A whole tile; returns whether S was handed back.  A row's weights are too large when one of its
   // threads' sums is: redo() follows.
-  template <bool EARLY, class PFree>
+  template <class PFree>
   __device__ __forceinline__ bool tile(int n_valid, bool first, uint32_t bar_sfree, PFree p_free) {
     const bool upper = n_slot >= 3;
-    if (SLOTS == 4 && n_slot == 4) half<1, SLOTS == 4, false, EARLY>(n_valid, first, bar_sfree, true, p_free);
-    else if (upper) half<1, false, false, EARLY>(n_valid, first, bar_sfree, true, p_free);
-    const bool released = n_slot >= 2 ? half<0, true, true, EARLY>(n_valid, first, bar_sfree, !upper, p_free)
-                                      : half<0, false, true, EARLY>(n_valid, first, bar_sfree, !upper, p_free);
+    if (SLOTS == 4 && n_slot == 4) half<1, SLOTS == 4, false>(n_valid, first, bar_sfree, true, p_free);
+    else if (upper) half<1, false, false>(n_valid, first, bar_sfree, true, p_free);
+    const bool released = n_slot >= 2 ? half<0, true, true>(n_valid, first, bar_sfree, !upper, p_free)
+                                      : half<0, false, true>(n_valid, first, bar_sfree, !upper, p_free);
     tmem_wait_st();
     return released;
   }
