@@ -272,6 +272,66 @@ def test_one_bf16_head_on_either_kernel(head_dim, hkv, batch, budgets, stack):
     assert ctx.status() == 0
 
 
+# The even-deal form of the wide-group kernel reads ahead in launches right behind one another over different layers: each
+# CTA's first tiles, up to the one that holds the new token's slot.  The slots lie in every tile of a unit (H2O: the
+# scores decide them, one victim per step in different tiles, so that rows written a step ago are fetched ahead), at the
+# front (a full sliding window) or at the end (the last free slot).  New tokens take about half of the weight, so that a
+# stale or a missing row shows; every unit is compared.
+@pytest.mark.parametrize("policy,room", [(synth.H2O, 0), (synth.SLIDING_WINDOW, 0), (synth.SLIDING_WINDOW, 1)])
+def test_even_deal_launches_read_ahead(policy, room):
+    batch, b, n_layer, steps, hq, d = 150, 2050 + room, 4, 3, 71, 64
+    n = b - room
+    w = workload("deal ahead", 9801, policy=policy, n_q_head=hq, n_kv_head=1, n_layer=n_layer, batch=batch, prompt=n, steps=steps, heavy_mode="none")
+    ctx = H.make_ctx(w, b_init=b)
+    ctx.begin_sequence_batch(batch, n)
+    ctx.set_budgets([b] * n_layer)
+    g = torch.Generator(device=DEV).manual_seed(5)
+    rnd = lambda *sh: torch.randn(*sh, generator=g, device=DEV)
+    u = torch.nn.functional.normalize(rnd(d), dim=0)
+    keys, vals, order = [], [], []
+    for l in range(n_layer):
+        k = rnd(batch, 1, n, d) * 0.5
+        k = (k - (k @ u).unsqueeze(-1) * u).bfloat16()
+        v = rnd(batch, 1, n, d).bfloat16()
+        acc = None
+        if policy == synth.H2O:
+            # the victims of the steps, in order, among the old half: 7, 18 and 11 tiles apart over units and layers
+            first = (torch.arange(batch, device=DEV) * 128 * 7 + 128 * 3 * l + 77) % (n // 2)
+            vict = torch.stack([(first + i * 419) % (n // 2) for i in range(steps)], 1)
+            acc = torch.full((batch, 1, n), 1e4, device=DEV)
+            acc[:, 0].scatter_(1, vict, torch.tensor([0.0, 1e3, 2e3], device=DEV).expand(batch, -1))
+            order.append(vict)
+        ctx.prefill_compress(l, k, v, None, acc)
+        keys.append(k[:, 0].double())
+        vals.append(v[:, 0].double())
+    for t in range(steps):
+        q = rnd(n_layer, batch, hq, d)
+        # logit of the new token about log(n) + 1
+        q = (q + ((np.log(n) + 1) * d ** 0.5 / 8 - (q @ u)).unsqueeze(-1) * u).bfloat16()
+        kn = (8.0 * u).expand(n_layer, batch, 1, d).bfloat16().contiguous()
+        vn = rnd(n_layer, batch, 1, d).bfloat16()
+        out = torch.empty_like(q)
+        torch.cuda.synchronize()
+        for l in range(n_layer):
+            ctx.decode_step(l, l + 1, q[l], kn[l], vn[l], out[l])
+        for l in range(n_layer):
+            if room and t == 0:
+                keys[l] = torch.cat([keys[l], kn[l].double()], 1)
+                vals[l] = torch.cat([vals[l], vn[l].double()], 1)
+            else:
+                slot = order[l][:, t] if policy == synth.H2O else torch.full((batch,), t - room, device=DEV)
+                at = torch.arange(batch, device=DEV)
+                keys[l][at, slot] = kn[l, :, 0].double()
+                vals[l][at, slot] = vn[l, :, 0].double()
+            p = torch.softmax(q[l].double() @ keys[l].transpose(1, 2) / d ** 0.5, -1)
+            want = p @ vals[l]
+            # bf16 weights and output: at most 2^-8 of each term and of the sum
+            bound = 2.0 ** -7 * (p @ vals[l].abs())
+            assert bool(((out[l].double() - want).abs() <= bound).all()), (t, l, float(((out[l].double() - want).abs() / bound).max()))
+            assert float(bound.max()) < 0.1    # a missing new token moves an output by some tenths
+    assert ctx.status() == 0
+
+
 # Selection over the prompt: block sizes by prompt length and the form for longer prompts, ties across the
 # threshold, equal scores everywhere, negative scores, all slots heavy but one, none heavy, budgets around the
 # prompt; the first victim shows in which token the first append replaces
