@@ -47,8 +47,9 @@ DEFAULT_WORKLOAD = "falcon_7b_max"
 # DRAM bytes (read + write) per byte of K/V a decode launch has to read, from ncu captures of each
 # decode kernel on a small case (traffic grows in proportion to the units processed, each unit's
 # K/V being read once); None once a kernel has changed since its counters were taken.
-NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = {"decode_attn_kernel": 1.008, "decode_attn_tc_kernel": 1.018,
-                                    "decode_attn_tc_stream_kernel": 1.033, "decode_attn_mma_kernel": None}
+NCU_TRAFFIC_PER_ALGORITHMIC_BYTE = {"decode_attn_kernel": None, "decode_attn_tc_kernel": 1.017,
+                                    "decode_attn_tc_stream_kernel": 1.028, "decode_attn_mma_low_kernel": 1.006,
+                                    "decode_attn_mma_kernel": None}
 
 
 def workload_by_name(name):
@@ -356,22 +357,46 @@ def hbm_peak():
     return FALLBACK_HBM_GBS, "fallback"
 
 
-def decode_kernel_of(w, min_budget=None, per_layer=True):
-    """The attention kernel that serves the decode launches of a workload (the library picks by
-    shape; for wide groups also by launch size: long units that do not fill the CTA slots take
-    the even-deal form, the rule of k_decode_tc_stream.cu restated here for the label)."""
+def sm_count():
     import torch
-    g = w.group
-    if w.dtype == torch.bfloat16 and w.head_dim == 64 and g > 32:
-        units = w.batch * w.n_kv_head * (1 if per_layer else w.n_layer)
-        slots = 2 * torch.cuda.get_device_properties(0).multi_processor_count
-        tiles = -(-min(min_budget or w.b_init, w.prompt + 1) // 128)
+    return torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 148
+
+
+def decode_kernel_of(w, budgets, per_layer=True):
+    """The attention kernel that serves the decode launches of a workload whose caches are full (one launch per layer: that
+    of its longest layer).  The library picks by shape, wide groups and single heads also by launch size: the rules of
+    k_decode_tc_stream.cu and of one_head_on_pipe() in k_decode.cu restated here for the label."""
+    import torch
+    from paper_2404_04793_b200 import synth
+    g, n_sm = w.group, sm_count()
+    layers = 1 if per_layer else w.n_layer
+    units = w.batch * w.n_kv_head * layers
+    if w.dtype != torch.bfloat16 or (g > 32 and w.head_dim != 64):
+        return "decode_attn_kernel"
+    if g > 32:
+        slots = 2 * n_sm
+        tiles = -(-min(min(budgets), w.prompt + 1) // 128)
         if slots <= 2 * units < 4 * slots and tiles >= 16:
             return "decode_attn_tc_stream_kernel"
         return "decode_attn_tc_kernel"
-    if w.dtype == torch.bfloat16 and g > 1:
+    if g > 8:
         return "decode_attn_mma_kernel"
-    return "decode_attn_kernel"
+    if g == 1:
+        longest, h2o = min(max(budgets), w.prompt + 1), w.policy == synth.H2O
+        elems, uneven = longest * w.head_dim, h2o and layers > 1
+        if units <= n_sm:
+            pipe = longest <= 320
+        elif units <= 2 * n_sm:
+            pipe = uneven and w.head_dim == 64 and longest > 2048
+        elif units < 8 * n_sm:
+            pipe = uneven or longest <= 200
+        else:
+            pipe = elems <= 64 << 10 or (units >= 24 * n_sm and layers > 1 and elems <= 160 << 10)
+        if pipe and not h2o:    # (under H2O small launches update the scores in the mma.sync kernel whatever the length)
+            return "decode_attn_kernel"
+        if pipe and units >= 6 * n_sm:
+            return "decode_attn_kernel"
+    return "decode_attn_mma_low_kernel"
 
 
 def algorithmic_bytes_per_step(w, kv_bytes):
@@ -433,7 +458,7 @@ def decode_record(w, dev, peak, n_steps=8, reps=3, standin_scores=False, advance
     alg = algorithmic_bytes_per_step(wr, kv)
     budgets, is_g3 = job.ctx.get_budgets()
     rec = {"workload": w.name, "policy": synth.POLICY_NAMES[w.policy], "batch": w.batch, "prompt": w.prompt,
-           "b_init": w.b_init, "budgets_min_max": [min(budgets), max(budgets)], "kernel": {"per_layer": decode_kernel_of(w, min(budgets), True), "fused": decode_kernel_of(w, min(budgets), False)},
+           "b_init": w.b_init, "budgets_min_max": [min(budgets), max(budgets)], "kernel": {"per_layer": decode_kernel_of(w, budgets, True), "fused": decode_kernel_of(w, budgets, False)},
            "algorithmic_bytes_per_step": alg, "steps_timed": n_steps * reps,
            "prompt_scores": "stand-in (scoring pass skipped while filling the cache)" if standin_scores else "computed"}
     if advance:
@@ -625,7 +650,7 @@ def run_ours(args, w):
         return
 
     # ---- roofline of the dominant kernel: the per-layer decode launch ----
-    kernel = decode_kernel_of(wr, min(budgets))
+    kernel = decode_kernel_of(wr, budgets)
     n_launch = wr.steps * wr.n_layer
     sec_per_launch = ms_decode * 1e-3 / n_launch
     bytes_per_launch = alg_bytes / wr.n_layer
