@@ -26,10 +26,17 @@
  *     page-locked HOST memory (staging of the budget and layout tables, a few KB per layer) and
  *     three CUDA events; sq_ctx_destroy waits for what still uses the block and frees them.
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Work is
- *     enqueued on it and calls return without waiting, except the sq_get_* calls and
- *     sq_status, which synchronise the device, and the first call after sq_allocate_budgets
- *     that needs the budgets on the host (sq_prefill_compress / sq_decode_step / sq_evict),
- *     which waits for that one small kernel.
+ *     enqueued on it and calls return without waiting, except:
+ *       - the sq_get_* calls (but sq_get_len, which is host work) and sq_status, which synchronise the device;
+ *       - the first call after sq_allocate_budgets that needs the budgets on the host
+ *         (sq_prefill_compress / sq_decode_step / sq_evict), which waits for that one small kernel;
+ *       - calls that upload host tables (sq_set_budgets, sq_evict, sq_ctx_import_layout and the
+ *         first call after sq_allocate_budgets): two uploads can be under way, so the call waits
+ *         for the one before the last if that is still waiting in its stream.
+ *   - Stream capture: sq_begin_sequence_batch, the importance calls, sq_allocate_budgets (its
+ *     budgets are then read with sq_get_budgets after a replay), and, once the budgets are laid out,
+ *     sq_prefill_compress and sq_decode_step can be captured; a replay repeats the captured token
+ *     positions.  Calls that upload host tables return SQ_ERR_CUDA on a capturing stream and change nothing.
  *     All calls of one context must use the same stream or be ordered by the caller.
  *   - A sequence batch has `batch` sequences of the same prompt length.  A *unit* is one
  *     (sequence, KV head) pair of a layer; unit index = seq * n_kv_head + kv_head.
