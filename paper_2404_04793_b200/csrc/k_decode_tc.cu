@@ -25,15 +25,28 @@
 // it shared it with the other CTA's (the special-function unit: 128 exp2 per row and tile at one
 // warp instruction per 8 cycles), against 2780 cycles of HBM time per pair of tiles at 1.9 GHz;
 // a polynomial exp2 on the FMA pipe for a part of the weights was slower at every share tried.
+// Cluster form (up to 96 heads, launches whose units leave room for at least two CTAs each, all at a time): the
+// pieces of a unit are the CTAs of one cluster.  They read one another's row sums and un-normalised outputs over
+// distributed shared memory and each stores its share of the output, where split-K sends them through memory to the
+// last piece to arrive, which took 12 us to merge a unit of 71 heads in 8 pieces while the launch waited.  With H2O each
+// piece then knows the log-sum-exps and runs the score pass (k_decode_gain.cu has it as a launch of its own) over its
+// tokens: S^T = K_tile Q^T again, K from L2, a thread owns a token, and the first piece picks the next victim.  33
+// sequences of 8191 tokens, 50 %, H2O, one launch (before: two) per layer: 1228 to 833 us per token.  Bound now by the chain
+// of a launch: with caches of 10 tiles, 5 pieces, of 13.5 us 4 for a piece's two tiles, 1.3 its epilogue, 2 the cluster barrier
+// (pieces of unlike speed), 2.3 the row sums and the output, 2.3 the scores, 1.2 the victim.
 // Streaming K and V alone (no products, no softmax) reaches 7.3 TB/s and draws 970 W of the
 // board's 1000 W; with the products 6.4 TB/s, with the softmax as well 4.6-4.7 TB/s, both at the
 // power limit with the SM clock near 1.5-1.6 GHz: run for longer than a few milliseconds the
 // kernel is bound by power, and what helps is fewer instructions per weight.
+#include <algorithm>
+#include <numeric>
 #include <type_traits>
 
 #include "sq_decode_common.cuh"
 #include "sq_device.cuh"
 #include "sq_internal.h"
+#include "sq_scores.cuh"
+#include "sq_select.cuh"
 #include "sq_tc.cuh"
 #include "sq_tc_rows.cuh"
 
@@ -49,13 +62,241 @@ __host__ __device__ constexpr uint32_t idesc(int n, bool b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | (b_mn_major ? (1u << 16) : 0u) | ((uint32_t)(n >> 3) << 17) |
          ((uint32_t)(128 >> 4) << 24);
 }
+
+// Cluster form: what the pieces read of one another, and scratch, in the V stages once the last tile is done.
+constexpr int kMaxPieces = 14;  // CTAs of a cluster (a B200 has room for no more than 14 clusters of 13 to 16 such CTAs)
+constexpr int kClusterHeads = 96;
+constexpr int kORow = kD + 4;  // floats from one head's partial output to the next (no bank conflicts)
+struct ClusterShared {
+  float o[kClusterHeads * kORow];          // un-normalised output
+  float stat[kClusterHeads * kStatStride]; // maximum, sum, sum of the rounded weights
+  float factor[kMaxPieces][kClusterHeads]; // a piece's weight in the merged row
+  float nlse[kTM];                         // minus the row log-sum-exps, by row of the Q tile
+  ScoreCandidate offer[kMaxPieces];        // one per piece (the first CTA's is read)
+  ScoreCandidate warp_best[4];
+};
+
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// Cluster form, the four softmax warps after the last tile: the piece's partial result to shared memory, then (behind
+// the cluster's barrier) the unit's row sums from all pieces, this CTA's share of the output, and with H2O the
+// score pass over its own tokens and its candidate for the next victim.  The warps reach both cluster barriers
+// whether or not something gave up before.
+template <bool H2O, class Args, class Rows>
+__device__ __forceinline__ void finish_cluster(const Args& a, const LayerDesc* ldp, int unit, int n_tiles, int t0, int t1, int len,
+                                               size_t out_at, Rows& rows, const WideLayout& layout, bool ok, ClusterShared& sh,
+                                               uint32_t bar_odone, uint32_t bar_gfull, uint32_t bar_gfree, uint32_t tmem_base,
+                                               volatile int* abort_flag) {
+  const int tid = (int)threadIdx.x - 64, lane = tid & 31, warp = tid >> 5, quarter = (warp + 2) & 3;
+  const int G = a.group, n = cluster_size(), me = cluster_rank();
+  if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar_odone, (n_tiles - 1) & 1, abort_flag));
+  if (ok) {
+    tc_fence_after();
+    float m_ref, l, l_w;
+    rows.finish(&m_ref, &l, &l_w);
+    const int row = layout.head_of_lane(quarter, lane);
+    const bool live = row < G;
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+      float o[32];
+      tmem_ld32(rows.o_addr + c * 32, o);
+      if (!live) continue;
+#pragma unroll
+      for (int q4 = 0; q4 < 8; ++q4)
+        *reinterpret_cast<float4*>(sh.o + row * kORow + c * 32 + q4 * 4) =
+            make_float4(o[q4 * 4], o[q4 * 4 + 1], o[q4 * 4 + 2], o[q4 * 4 + 3]);
+    }
+    if (live) *reinterpret_cast<float4*>(sh.stat + row * kStatStride) = make_float4(m_ref, H2O ? l : l_w, l_w, 0.f);
+    if (H2O) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(bar_gfree);
+        mbar_arrive(bar_gfree + 8);
+      }
+    }
+  }
+  __syncwarp();
+  cluster_arrive();
+  // the first tile's scores and positions are on their way meanwhile
+  const int b = ldp->b, cap = ldp->cap;
+  const bool full = (len == b);
+  const int* pos = reinterpret_cast<const int*>(a.pool + ldp->pos_off) + (size_t)unit * cap;
+  float* acc = reinterpret_cast<float*>(a.pool + ldp->acc_off) + (size_t)unit * cap;
+  const int row = quarter * 32 + lane;
+  float old[2];
+  int p[2];
+  auto fetch = [&](int i, int u) {
+    const int slot = t0 + i * kTM + row;
+    old[u] = 0.f;
+    p[u] = 0x7fffffff;
+    if (slot < t1) {
+      old[u] = acc[slot];
+      if (full) p[u] = pos[slot];
+    }
+  };
+  if (H2O) {
+    fetch(0, 0);
+    fetch(1, 1);
+  }
+  cluster_wait();
+  // Every read crosses the cluster: several at a time, this thread's part of the output (four consecutive values of a
+  // head from every piece) on its way while the row sums are worked out.
+  const int n4 = G * kD / 4;
+  auto fetch_o = [&](int i4, int r0, float4 (&v)[8]) {
+    const float* src = sh.o + (i4 * 4 / kD) * kORow + (i4 * 4) % kD;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (i4 < n4 && r0 + u < n) v[u] = ld_cluster4(map_rank(src, r0 + u));
+    }
+  };
+  float4 v[8];
+  int i4 = (n - 1 - me) * 128 + tid;
+  fetch_o(i4, 0, v);
+  if (tid < G) {
+    float M = -INFINITY, L = 0.f, Lw = 0.f;
+    for (int r0 = 0; r0 < n; r0 += 8) {
+      float4 st[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        st[u] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
+        if (r0 + u < n) st[u] = ld_cluster4(map_rank(sh.stat + tid * kStatStride, r0 + u));
+      }
+      float m2 = M;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) m2 = fmaxf(m2, st[u].x);
+      const float f0 = M > -INFINITY ? exp2f(M - m2) : 0.f;
+      L *= f0;
+      Lw *= f0;
+      M = m2;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        if (r0 + u >= n) continue;
+        const float f = exp2f(st[u].x - M);
+        L += st[u].y * f;
+        Lw += st[u].z * f;
+        sh.factor[r0 + u][tid] = st[u].x;
+      }
+    }
+    const float inv = 1.f / Lw;
+    for (int r = 0; r < n; ++r) sh.factor[r][tid] = exp2f(sh.factor[r][tid] - M) * inv;
+    if (H2O) sh.nlse[layout.row_of_group(tid >> 3) + (tid & 7)] = -(M + log2f(L));
+  }
+  // columns past the group: their weight is exp2(-inf) = 0
+  if (H2O && tid >= G && tid < (G + 7) / 8 * 8) sh.nlse[layout.row_of_group(tid >> 3) + (tid & 7)] = -INFINITY;
+  softmax_sync();
+  for (; i4 < n4; i4 += n * 128) {
+    const int h = i4 * 4 / kD;
+    float4 O = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int r0 = 0; r0 < n; r0 += 8) {
+      if (r0 > 0) fetch_o(i4, r0, v);
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const float f = r0 + u < n ? sh.factor[r0 + u][h] : 0.f;
+        O.x += v[u].x * f;
+        O.y += v[u].y * f;
+        O.z += v[u].z * f;
+        O.w += v[u].w * f;
+      }
+    }
+    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + out_at + i4 * 4) =
+        make_uint2(pack_bf16x2(O.x, O.y), pack_bf16x2(O.z, O.w));
+    if (i4 + n * 128 < n4) fetch_o(i4 + n * 128, 0, v);
+  }
+  if constexpr (H2O) {
+    // ---------------- scores: thread = one token ----------------
+    const int thr = a.n_tok + 1 - ldp->b_recent;  // next step: positions <= thr are outside the recent window
+    const uint32_t lane_sel = (uint32_t)(quarter * 32) << 16;
+    const float c = a.scale_log2;
+    unsigned long long best = ~0ull;
+    int best_slot = -1;
+    // (a tile's scores and positions are fetched two tiles ahead: one tile takes about as long as a trip to memory)
+    auto one = [&](int i, int u) {
+      const int slot = t0 + i * kTM + row;
+      ok = __all_sync(0xffffffffu, mbar_wait(bar_gfull + 8 * u, (i >> 1) & 1, abort_flag));
+      if (!ok) return;
+      tc_fence_after();
+      const uint32_t s_addr = tmem_base + lane_sel + u * kTM;
+      float g0 = 0.f, g1 = 0.f;
+      uint32_t r[2][32];
+      tmem_ld32_nowait(s_addr, r[0]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        tmem_wait_ld(r[q & 1]);
+        if (q < 3) tmem_ld32_nowait(s_addr + (q + 1) * 32, r[(q + 1) & 1]);
+        const int live = layout.groups(q, G);
+#pragma unroll
+        for (int s = 0; s < kClusterHeads / 32; ++s) {
+          if (s >= live) continue;
+          const float4* nl = reinterpret_cast<const float4*>(sh.nlse + q * 32 + s * 8);
+#pragma unroll
+          for (int q4 = 0; q4 < 2; ++q4) {
+            const float4 l4 = nl[q4];
+            const uint32_t* x = r[q & 1] + s * 8 + q4 * 4;
+            g0 += ex2(fmaf(__uint_as_float(x[0]), c, l4.x));
+            g1 += ex2(fmaf(__uint_as_float(x[1]), c, l4.y));
+            g0 += ex2(fmaf(__uint_as_float(x[2]), c, l4.z));
+            g1 += ex2(fmaf(__uint_as_float(x[3]), c, l4.w));
+          }
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(bar_gfree + 8 * u);
+      if (slot < t1) {
+        const float v = old[u] + (g0 + g1);
+        acc[slot] = v;
+        if (full && p[u] <= thr) {
+          const unsigned long long rank = victim_rank(v, p[u]);
+          if (rank < best) {
+            best = rank;
+            best_slot = slot;
+          }
+        }
+      }
+      if (i + 2 < n_tiles) fetch(i + 2, u);
+    };
+    for (int i = 0; ok && i < n_tiles; i += 2) {
+      one(i, 0);
+      if (ok && i + 1 < n_tiles) one(i + 1, 1);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const unsigned long long r2 = __shfl_xor_sync(0xffffffffu, best, o);
+      const int s2 = __shfl_xor_sync(0xffffffffu, best_slot, o);
+      if (r2 < best) {
+        best = r2;
+        best_slot = s2;
+      }
+    }
+    if (lane == 0) {
+      sh.warp_best[warp].rank = best;
+      sh.warp_best[warp].slot = best_slot;
+    }
+    softmax_sync();
+    if (tid == 0) {
+      for (int w = 1; w < 4; ++w)
+        if (sh.warp_best[w].rank < best) {
+          best = sh.warp_best[w].rank;
+          best_slot = sh.warp_best[w].slot;
+        }
+      st_cluster_candidate(map_rank(&sh.offer[me], 0), best, best_slot);
+    }
+    __syncwarp();
+  }
+  cluster_arrive();
+}
 }  // namespace
 
 // ROWS: rows of the Q tile held in shared memory (120 for up to 96 heads, else 128; see sq_tc_rows.cuh).
-template <int STAGES, int ROWS, bool H2O>
+// CLUSTER: the pieces of a unit are the CTAs of a cluster (Args: DecodeArgsBase), see the head of the file.
+template <int STAGES, int ROWS, bool H2O, bool CLUSTER, class Args>
 __global__ void __launch_bounds__(192, 2)
     decode_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                          const __grid_constant__ CUtensorMap tm_v, DecodeArgs a) {
+                          const __grid_constant__ CUtensorMap tm_v, Args a) {
   constexpr int kQBytes = ROWS * 128;
   constexpr int kSlots = ROWS == 120 ? 3 : 4;
   extern __shared__ unsigned char smem_raw[];
@@ -67,16 +308,30 @@ __global__ void __launch_bounds__(192, 2)
   unsigned char* k_s = q_s + kQBytes;              // STAGES tiles
   unsigned char* v_s = k_s + STAGES * kTileBytes;  // STAGES tiles
   unsigned long long* bars = reinterpret_cast<unsigned long long*>(v_s + STAGES * kTileBytes);
+  static_assert(10 + 2 * STAGES <= 16 || !CLUSTER, "barrier block");
   static_assert(6 + 2 * STAGES <= 16, "barrier block");
+  static_assert(!CLUSTER || sizeof(ClusterShared) <= STAGES * kTileBytes, "scratch of the cluster form");
   const uint32_t bar_q = s_u32(bars + 0), bar_odone = s_u32(bars + 1), bar_sfull = s_u32(bars + 2),
                  bar_sfree = s_u32(bars + 3), bar_pready = s_u32(bars + 4), bar_pfree = s_u32(bars + 5);
   auto bar_full = [&](int s) { return s_u32(bars + 6 + s); };
   auto bar_empty = [&](int s) { return s_u32(bars + 6 + STAGES + s); };
+  // cluster form with scores: the score pass's two accumulator buffers
+  auto bar_gfull = [&](int j) { return s_u32(bars + 6 + 2 * STAGES + j); };
+  auto bar_gfree = [&](int j) { return s_u32(bars + 8 + 2 * STAGES + j); };
+  constexpr bool SCORES = H2O && CLUSTER;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   ItemLoc it;
-  if (!locate(a, blockIdx.x, it)) return;
+  if constexpr (CLUSTER) {
+    it.n_split = cluster_size();
+    const int k = (int)blockIdx.x / (a.n_unit * it.n_split);
+    it.layer = a.order[k];
+    it.base = k * a.n_unit * it.n_split;
+    it.local = (int)blockIdx.x - it.base;
+  } else {
+    if (!locate(a, blockIdx.x, it)) return;
+  }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const LayerDesc* ldp = a.layers + it.layer;
   const int b = ldp->b, cap = ldp->cap, G = a.group;
@@ -93,7 +348,15 @@ __global__ void __launch_bounds__(192, 2)
   } else {
     w = ring_slot(a.n_tok, b, ldp->ring_base, ldp->ring_origin);
   }
-  const int t0 = split * a.split_tokens, t1 = min(len, t0 + a.split_tokens);
+  int t0, t1;
+  if constexpr (CLUSTER) {  // the unit's tiles, dealt out evenly (the launcher sees to it that no piece is empty)
+    const int n = (len + kTM - 1) / kTM;
+    t0 = split * n / it.n_split * kTM;
+    t1 = min(len, (split + 1) * n / it.n_split * kTM);
+  } else {
+    t0 = split * a.split_tokens;
+    t1 = min(len, t0 + a.split_tokens);
+  }
   const int n_tiles = (t1 - t0 + kTM - 1) / kTM;
   const int seq = unit / a.n_kv_head, kvh = unit - seq * a.n_kv_head;
   const size_t tok = (size_t)(it.layer - a.layer_begin) * a.batch + seq;
@@ -111,6 +374,12 @@ __global__ void __launch_bounds__(192, 2)
       mbar_init(bar_full(s), 1);
       mbar_init(bar_empty(s), 1);
     }
+    if (SCORES) {
+      for (int j = 0; j < 2; ++j) {
+        mbar_init(bar_gfull(j), 1);
+        mbar_init(bar_gfree(j), 4);
+      }
+    }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -123,7 +392,7 @@ __global__ void __launch_bounds__(192, 2)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const WideLayout layout;
+  const WideLayout layout(CLUSTER ? split & 3 : WideLayout::wave());
 
   // fetch of K and V tile i (its stage is free); rows of this unit in the [rows][64] view of the pool
   auto load_tile = [&](int i) {
@@ -180,6 +449,22 @@ __global__ void __launch_bounds__(192, 2)
         if (i >= STAGES && !mbar_wait(bar_empty(i % STAGES), ((i / STAGES) - 1) & 1, abort_flag)) break;
         load_tile(i);
       }
+    }
+    if constexpr (SCORES) {
+      // the score pass reads the K tiles again (from L2), through the same ring of stages
+      cluster_arrive();
+      if (lane == 0 && !*abort_flag) {
+        for (; issued < 2 * n_tiles; ++issued) {
+          const int st = issued % STAGES;
+          if (issued >= STAGES && !mbar_wait(bar_empty(st), ((issued / STAGES) - 1) & 1, abort_flag)) break;
+          mbar_expect_tx(bar_full(st), kTileBytes);
+          tma_load_2d(s_u32(k_s + st * kTileBytes), &tm_k, 0,
+                      (int)(ldp->k_off / (kD * 2) + (long long)unit * cap + t0 + (issued - n_tiles) * kTM), bar_full(st));
+        }
+      }
+      __syncwarp();
+    }
+    if (lane == 0) {
       if (*abort_flag) {
         mbar_wait(bar_q, 0, abort_flag);
         for (int i = max(0, issued - STAGES); i < issued; ++i)
@@ -225,6 +510,27 @@ __global__ void __launch_bounds__(192, 2)
       }
     }
     __syncwarp();
+    if constexpr (SCORES) {
+      // S^T = K_tile Q^T: tokens on the lanes, rows of the Q tile (dead ones too) on the columns
+      cluster_arrive();
+      if (lane == 0 && !*abort_flag) {
+        const uint32_t q_addr = s_u32(q_s);
+        for (int i = 0; i < n_tiles; ++i) {
+          const int j = n_tiles + i, st = j % STAGES;
+          if (!mbar_wait(bar_full(st), (j / STAGES) & 1, abort_flag)) break;
+          if (!mbar_wait(bar_gfree(i & 1), (i >> 1) & 1, abort_flag)) break;
+          tc_fence_after();
+          const uint32_t k_addr = s_u32(k_s + st * kTileBytes);
+#pragma unroll
+          for (int k = 0; k < kD / 16; ++k)
+            umma_bf16(tmem_base + (i & 1) * kTM, umma_desc(k_addr + k * 32), umma_desc(q_addr + k * 32), idesc(128, false),
+                      k > 0 ? 1u : 0u);
+          umma_commit(bar_empty(st));
+          umma_commit(bar_gfull(i & 1));
+        }
+      }
+      __syncwarp();
+    }
   } else {
     // ---------------- softmax: four threads = one head row (sq_tc_rows.cuh) ----------------
     const int quarter = warp & 3;
@@ -276,43 +582,64 @@ __global__ void __launch_bounds__(192, 2)
         if (!s_released) mbar_arrive(bar_sfree);
       }
     }
-    // ---------------- epilogue: O / l -> out (or the split-K partial) ----------------
-    if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar_odone, (n_tiles - 1) & 1, abort_flag));
-    if (ok) {
-      tc_fence_after();
-      bf16* ob = reinterpret_cast<bf16*>(a.out) + (tok * a.n_q_head + (size_t)kvh * G) * kD;
-      float* stat = a.part_stat + (size_t)blockIdx.x * G * kStatStride;
-      float* po = a.part_o + (size_t)blockIdx.x * G * kD;
-      float m_ref, l, l_w;
-      rows.finish(&m_ref, &l, &l_w);
-      const int row = layout.head_of_lane(quarter, lane);
-      const bool live = row < G;  // this lane's row is a real head
-      const float inv = 1.f / l_w;
-#pragma unroll 1
-      for (int c = 0; c < 2; ++c) {
-        float o[32];
-        tmem_ld32(rows.o_addr + c * 32, o);
-        if (!live) continue;
-        if (it.n_split == 1) {
-#pragma unroll
-          for (int q4 = 0; q4 < 4; ++q4)
-            *reinterpret_cast<uint4*>(ob + (size_t)row * kD + c * 32 + q4 * 8) =
-                make_uint4(pack_bf16x2(o[q4 * 8] * inv, o[q4 * 8 + 1] * inv), pack_bf16x2(o[q4 * 8 + 2] * inv, o[q4 * 8 + 3] * inv),
-                           pack_bf16x2(o[q4 * 8 + 4] * inv, o[q4 * 8 + 5] * inv), pack_bf16x2(o[q4 * 8 + 6] * inv, o[q4 * 8 + 7] * inv));
-        } else {
-#pragma unroll
-          for (int q4 = 0; q4 < 8; ++q4)
-            *reinterpret_cast<float4*>(po + (size_t)row * kD + c * 32 + q4 * 4) =
-                make_float4(o[q4 * 4], o[q4 * 4 + 1], o[q4 * 4 + 2], o[q4 * 4 + 3]);
+    if constexpr (CLUSTER) {
+      finish_cluster<H2O>(a, ldp, unit, n_tiles, t0, t1, len, (tok * a.n_q_head + (size_t)kvh * G) * kD, rows, layout, ok,
+                          *reinterpret_cast<ClusterShared*>(v_s), bar_odone, bar_gfull(0), bar_gfree(0), tmem_base, abort_flag);
+    } else {
+      // ---------------- epilogue: O / l -> out (or the split-K partial) ----------------
+      if (ok) ok = __all_sync(0xffffffffu, mbar_wait(bar_odone, (n_tiles - 1) & 1, abort_flag));
+      if (ok) {
+        tc_fence_after();
+        bf16* ob = reinterpret_cast<bf16*>(a.out) + (tok * a.n_q_head + (size_t)kvh * G) * kD;
+        float* stat = a.part_stat + (size_t)blockIdx.x * G * kStatStride;
+        float* po = a.part_o + (size_t)blockIdx.x * G * kD;
+        float m_ref, l, l_w;
+        rows.finish(&m_ref, &l, &l_w);
+        const int row = layout.head_of_lane(quarter, lane);
+        const bool live = row < G;  // this lane's row is a real head
+        const float inv = 1.f / l_w;
+  #pragma unroll 1
+        for (int c = 0; c < 2; ++c) {
+          float o[32];
+          tmem_ld32(rows.o_addr + c * 32, o);
+          if (!live) continue;
+          if (it.n_split == 1) {
+  #pragma unroll
+            for (int q4 = 0; q4 < 4; ++q4)
+              *reinterpret_cast<uint4*>(ob + (size_t)row * kD + c * 32 + q4 * 8) =
+                  make_uint4(pack_bf16x2(o[q4 * 8] * inv, o[q4 * 8 + 1] * inv), pack_bf16x2(o[q4 * 8 + 2] * inv, o[q4 * 8 + 3] * inv),
+                             pack_bf16x2(o[q4 * 8 + 4] * inv, o[q4 * 8 + 5] * inv), pack_bf16x2(o[q4 * 8 + 6] * inv, o[q4 * 8 + 7] * inv));
+          } else {
+  #pragma unroll
+            for (int q4 = 0; q4 < 8; ++q4)
+              *reinterpret_cast<float4*>(po + (size_t)row * kD + c * 32 + q4 * 4) =
+                  make_float4(o[q4 * 4], o[q4 * 4 + 1], o[q4 * 4 + 2], o[q4 * 4 + 3]);
+          }
+        }
+        if (live) {
+          stat[row * kStatStride] = m_ref;
+          stat[row * kStatStride + 1] = H2O ? l : l_w;
+          stat[row * kStatStride + 2] = l_w;
+          // H2O: the unit's row log-sum-exps (log2 domain), read by the score-update pass that follows
+          if (H2O && it.n_split == 1) (a.logits + ldp->lse_off + (size_t)unit * G)[row] = m_ref + log2f(l);
         }
       }
-      if (live) {
-        stat[row * kStatStride] = m_ref;
-        stat[row * kStatStride + 1] = H2O ? l : l_w;
-        stat[row * kStatStride + 2] = l_w;
-        // H2O: the unit's row log-sum-exps (log2 domain), read by the score-update pass that follows
-        if (H2O && it.n_split == 1) (a.logits + ldp->lse_off + (size_t)unit * G)[row] = m_ref + log2f(l);
-      }
+    }
+  }
+  if constexpr (CLUSTER) {
+    // every offer is in; nothing of another CTA's shared memory is touched after this
+    if (warp < 2) {
+      if (!SCORES) cluster_arrive();
+      cluster_wait();
+      cluster_arrive();
+    }
+    cluster_wait();
+    if (H2O && split == 0 && tid == 64 && len == b && !*abort_flag) {
+      const ClusterShared& sh = *reinterpret_cast<const ClusterShared*>(v_s);
+      ScoreCandidate best = sh.offer[0];
+      for (int r = 1; r < it.n_split; ++r)
+        if (sh.offer[r].rank < best.rank) best = sh.offer[r];
+      reinterpret_cast<int*>(a.pool + ldp->victim_off)[unit] = best.slot;
     }
   }
   tc_fence_before();
@@ -322,7 +649,62 @@ __global__ void __launch_bounds__(192, 2)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(kTmemCols) : "memory");
   }
   if (tid == 0 && *abort_flag) atomicOr(a.status, kStatusTimeout);
-  if (it.n_split > 1) merge_if_last<bf16>(a, it, unit, reinterpret_cast<float*>(q_s), H2O ? a.logits + ldp->lse_off + (size_t)unit * G : nullptr);
+  if constexpr (!CLUSTER)
+    if (it.n_split > 1) merge_if_last<bf16>(a, it, unit, reinterpret_cast<float*>(q_s), H2O ? a.logits + ldp->lse_off + (size_t)unit * G : nullptr);
+}
+
+// The occupancy calculator takes the attention kernel's registers to leave room for one CTA per SM; two run (seen
+// by their clocks: 264 CTAs at a time).  It is asked for a kernel that has the same threads and shared memory.
+__global__ void __launch_bounds__(192) cluster_room_kernel() {}
+
+// Pieces per unit: as many as all units' clusters find room for at the same time, then as few as give the longest
+// piece as many tiles.  Measured, us per launch with 4, 5, 6, 7, 8 pieces: 33 units of 58 tiles 47, 44, 38, 36, 34; of
+// 10 tiles 17, 15, 14, 14, 15.5.
+// 0 where not even two fit, or where units of unlike length leave the longest piece too far above an even share of the
+// launch's tiles (a cluster cuts every unit into the same number of pieces; split-K cuts the long ones into more).  Time of
+// split-K, two launches with H2O, over this form, 32 layers in one launch, by the excess in tiles: without scores 4: 1.85, 7:
+// 1.16, 10: 1.05 and 1.07, 15: 0.98, 40: 0.63; H2O 4: 1.63, 5: 1.10, 7: 1.17 (8 pieces), 1.06 and 0.92 (2 pieces: the less
+// to merge, the less this form saves), 10: 0.95 and 0.96, 15: 0.85.
+// Launches of one layer, split-K / this form, us per token of 32 layers: 1 sequence of 512 tokens 289 / 246, 16384: 1621 / 470, 8
+// of 8191 1043 / 444, 33 of 1024 457 / 357, 100 of 3000 741 / 630; H2O 452 / 358, 1883 / 669, 1329 / 580, 658 / 438, 1130 / 950.
+static int cluster_pieces(const DecodeArgs& a, const int* desc_tiles, size_t smem) {
+  static PerDevice set_up;
+  static ClusterCount room;
+  const void* kern = reinterpret_cast<const void*>(cluster_room_kernel);
+  if (set_up.once([&] {
+        const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return r == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
+      }) != cudaSuccess)
+    return 0;
+  const long long units = (long long)a.n_layer_total * a.n_unit;
+  const auto [lo, hi] = std::minmax_element(desc_tiles, desc_tiles + a.n_layer_total);
+  const int min_tiles = *lo, max_tiles = *hi;
+  int n = std::min(kMaxPieces, min_tiles);
+  while (n >= 2 && units > room.active(kern, n, 192, smem)) --n;
+  if (n < 2) return 0;
+  const int longest = (max_tiles + n - 1) / n;
+  const long long total = std::accumulate(desc_tiles, desc_tiles + a.n_layer_total, 0LL) * a.n_unit;
+  const long long even = std::max(total / (2LL * sm_count()), (long long)max_tiles / kMaxPieces);
+  if (min_tiles < max_tiles && longest > even + (a.policy != SQ_POLICY_H2O ? 12 : n == 2 ? 6 : 8)) return 0;
+  while (n > 2 && (max_tiles + n - 2) / (n - 1) == longest && units <= room.active(kern, n - 1, 192, smem)) --n;
+  return n;
+}
+
+template <bool H2O>
+static cudaError_t launch_tc_cluster(const DecodeArgs& a, const int* desc_tiles, const CUtensorMap& tq, const CUtensorMap& tk,
+                                     const CUtensorMap& tv, cudaStream_t s) {
+  constexpr int STAGES = 3, ROWS = 120;
+  constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 8 * 16 + 16;
+  auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O, true, DecodeArgsBase>;
+  static PerDevice set_up;
+  const cudaError_t e = set_up.once([&] {
+    cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    return r == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
+  });
+  if (e != cudaSuccess) return e;
+  const int n = cluster_pieces(a, desc_tiles, smem);
+  if (n == 0) return cudaErrorNotSupported;
+  return launch_chained_cluster(kern, n, a.n_layer_total * a.n_unit * n, 192, smem, s, tq, tk, tv, static_cast<const DecodeArgsBase&>(a));
 }
 
 template <int STAGES, int ROWS, bool H2O>
@@ -330,22 +712,34 @@ static cudaError_t launch_tc_cfg(const DecodeArgs& a, int n_items, const CUtenso
                                  const CUtensorMap& tv, cudaStream_t s) {
   constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 8 * 16 + 16;
   static_assert(2 * (smem + 1024 + 64) <= 228 * 1024, "two CTAs per SM");
-  auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O>;
+  auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O, false, DecodeArgs>;
   static PerDevice set_up;
   const cudaError_t e = allow_smem(set_up, smem, kern);
   if (e != cudaSuccess) return e;
   return launch_chained(kern, n_items, 192, smem, s, tq, tk, tv, a);
 }
 
+static bool make_maps(const DecodeArgs& a, size_t pool_bytes, size_t q_rows, CUtensorMap* tm_q, CUtensorMap* tm_k, CUtensorMap* tm_v) {
+  if (a.head_dim != kD || a.group <= 32 || a.group > 128) return false;
+  const long long pool_rows = (long long)(pool_bytes / (kD * 2));
+  if (pool_rows + kTM > 0x7fffffffLL || (long long)q_rows + kTM > 0x7fffffffLL) return false;
+  return make_tile_map(tm_q, a.q, (long long)q_rows, kD, 8) && make_tile_map(tm_k, a.pool, pool_rows, kD, kTM) &&
+         make_tile_map(tm_v, a.pool, pool_rows, kD, kTM);
+}
+
+// The cluster form.  desc_tiles: as for the even-deal form.  Returns cudaErrorNotSupported where it is not taken.
+cudaError_t launch_decode_attn_tc_cluster(const DecodeArgs& a, const int* desc_tiles, size_t pool_bytes, size_t q_rows, cudaStream_t s) {
+  if (a.group > kClusterHeads) return cudaErrorNotSupported;
+  CUtensorMap tm_q, tm_k, tm_v;
+  if (!make_maps(a, pool_bytes, q_rows, &tm_q, &tm_k, &tm_v)) return cudaErrorNotSupported;
+  return a.policy == SQ_POLICY_H2O ? launch_tc_cluster<true>(a, desc_tiles, tm_q, tm_k, tm_v, s)
+                                   : launch_tc_cluster<false>(a, desc_tiles, tm_q, tm_k, tm_v, s);
+}
+
 // Returns cudaErrorNotSupported when the shape is outside this kernel's range.
 cudaError_t launch_decode_attn_tc(const DecodeArgs& a, int n_items, size_t pool_bytes, size_t q_rows, cudaStream_t s) {
-  if (a.head_dim != kD || a.group <= 32 || a.group > 128) return cudaErrorNotSupported;
-  const long long pool_rows = (long long)(pool_bytes / (kD * 2));
-  if (pool_rows + kTM > 0x7fffffffLL || (long long)q_rows + kTM > 0x7fffffffLL) return cudaErrorNotSupported;
   CUtensorMap tm_q, tm_k, tm_v;
-  if (!make_tile_map(&tm_q, a.q, (long long)q_rows, kD, 8) || !make_tile_map(&tm_k, a.pool, pool_rows, kD, kTM) ||
-      !make_tile_map(&tm_v, a.pool, pool_rows, kD, kTM))
-    return cudaErrorNotSupported;
+  if (!make_maps(a, pool_bytes, q_rows, &tm_q, &tm_k, &tm_v)) return cudaErrorNotSupported;
   const bool h2o = a.policy == SQ_POLICY_H2O;
   if (a.group <= 96)
     return h2o ? launch_tc_cfg<3, 120, true>(a, n_items, tm_q, tm_k, tm_v, s)

@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  const WideLayout layout;
+  const WideLayout layout(WideLayout::wave());
   SegIter it;
   it.init(a, blockIdx.x);
 

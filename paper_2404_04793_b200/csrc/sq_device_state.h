@@ -75,6 +75,40 @@ class ClusterFit {
   std::atomic<int> state_[kMaxDevices] = {};
 };
 
+// Clusters of `ctas` CTAs of a kernel that the current device runs at a time, by size (up to 16).  For static
+// storage, one per kernel and amount of shared memory; asked once for every size on every device.
+class ClusterCount {
+ public:
+  int active(const void* kern, int ctas, int threads, size_t smem) {
+    int dev = -1;
+    if (ctas < 1 || ctas > kSizes || cudaGetDevice(&dev) != cudaSuccess) return 0;
+    const bool known = dev >= 0 && dev < kMaxDevices;
+    const int seen = known ? count_[dev][ctas - 1].load(std::memory_order_relaxed) : 0;
+    if (seen) return seen - 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      n = 0;
+    }
+    if (known) count_[dev][ctas - 1].store(n + 1, std::memory_order_relaxed);
+    return n;
+  }
+
+ private:
+  static constexpr int kSizes = 16;
+  std::atomic<int> count_[kMaxDevices][kSizes] = {};
+};
+
 // launch(limit) with clusters of at most `limit` CTAs, and where the device does not hold those (or the plan does not
 // work out) with at most the portable 8.
 template <class F>

@@ -175,6 +175,8 @@ DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, i
 cudaError_t launch_decode(const DecodeArgs& a, int dtype, int n_items, bool need_combine, size_t pool_bytes,
                           size_t q_rows, const int* desc_tiles, int max_len, cudaStream_t s);
 cudaError_t launch_decode_attn_tc(const DecodeArgs& a, int n_items, size_t pool_bytes, size_t q_rows, cudaStream_t s);
+cudaError_t launch_decode_attn_tc_cluster(const DecodeArgs& a, const int* desc_tiles, size_t pool_bytes, size_t q_rows,
+                                          cudaStream_t s);
 cudaError_t launch_decode_attn_tc_stream(const DecodeArgs& a, const int* desc_tiles, size_t pool_bytes, size_t q_rows,
                                          cudaStream_t s);
 cudaError_t launch_h2o_gain_tc(const DecodeArgs& a, int n_items, size_t pool_bytes, size_t q_rows, cudaStream_t s);

@@ -29,7 +29,8 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 // results).
 struct WideLayout {
   int rot;
-  __device__ __forceinline__ WideLayout() : rot((blockIdx.x / 148) & 3) {}
+  __device__ __forceinline__ explicit WideLayout(int turn) : rot(turn & 3) {}
+  static __device__ __forceinline__ int wave() { return blockIdx.x / 148; }
   // head of tensor-memory lane `lane` of a quarter
   __device__ __forceinline__ int head_of_lane(int quarter, int lane) const {
     return 8 * (4 * (lane >> 3) + ((quarter - rot) & 3)) + (lane & 7);

@@ -237,6 +237,17 @@ def test_h2o_forms_of_larger_launches(dtype, head_dim, hq, hkv, batch, budgets, 
     h2o_lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack)
 
 
+# Wide groups with the pieces of a unit on the CTAs of a cluster: two pieces to the most there are, pieces of one tile and of
+# unlike numbers of tiles, a last tile of one slot, the smallest group and the largest that is taken and the next, groups that
+# fill no eight, a launch whose layers differ too much for it
+@pytest.mark.parametrize("hq,batch,budgets", [
+    (71, 1, [1792, 257]), (33, 2, [1921, 129]), (96, 3, [700, 1300]), (97, 2, [300, 260]), (72, 37, [260, 900]), (40, 75, [385, 290]),
+    (71, 4, [6000, 300, 260]), (65, 149, [257, 300])])
+@pytest.mark.parametrize("stack", [False, True])
+def test_wide_groups_over_a_cluster(hq, batch, budgets, stack):
+    h2o_lockstep(torch.bfloat16, 64, hq, 1, batch, budgets, stack)
+
+
 # One bf16 head per KV head on either kernel: few units, between one and two per SM, a few, many; lengths around the
 # limits; whole stack (with split units among them) and layer by layer
 @pytest.mark.parametrize("head_dim,hkv,batch,budgets", [
