@@ -2,27 +2,31 @@
 //
 // acc[t] = sum over the query heads sharing a KV head and over query rows r >= t of
 //          softmax_row_r(Q K^T / sqrt(d))[t]                       (causal)
-// is two sweeps over 128x128 tiles of the score matrix, each tile one tcgen05.mma chain
-// (M = N = 128, K = head_dim, bf16 in, fp32 accumulators in tensor memory):
+// is two sweeps over tiles of 128 rows by TN columns of the score matrix, each tile one tcgen05.mma chain
+// (M = 128, N = TN, K = head_dim, bf16 in, fp32 accumulators in tensor memory):
 //   sweep 1, CTA = (sequence, query head, 128 query rows): S = Q_tile K_tile^T for the key tiles
 //     up to the diagonal; a drain thread owns one TMEM lane = one query row and
-//     keeps its running max / sum -> row log-sum-exp.
+//     keeps its reference / sum -> row log-sum-exp.
 //   sweep 2, CTA = (sequence, KV head, 128 keys, some heads of the group): the operands swap,
 //     S^T = K_tile Q_tile^T for all query tiles from the diagonal down and the CTA's heads; thread t
 //     owns one key and adds exp2(s*scale - lse[row]) over the tile's columns -> the key's column sum,
 //     with no cross-thread reduction and no atomics; a key tile cut into several CTAs by heads is
 //     added up, in head order, by the one that finishes last (deterministic).
-// Roles per CTA (10 warps): warp 0 issues TMA tile loads (128-byte swizzle, every CTA its own tiles)
+// Roles per CTA: warp 0 issues TMA tile loads (128-byte swizzle, every CTA its own tiles)
 // into a ring of shared-memory stages; warp 1 allocates tensor memory, issues the MMAs, signalling
-// completion through tcgen05.commit -> mbarrier, and stages the row log-sum-exps of sweep 2; warps 2-9
+// completion through tcgen05.commit -> mbarrier, and stages the row log-sum-exps of sweep 2; the others
 // drain the accumulators with tcgen05.ld.  Two accumulator buffers let the next tile's MMA run under
 // this tile's exponentials.
-// Built to parity and measured slower (us of sweeps 1 / 2, 4 sequences of 4096, 32 / 8 heads of 128,
-// against 321 / 374): queries on the lanes in both sweeps with one register per key in sweep 2, which
-// takes the log-sum-exps out of shared memory (315 / 416 as one persistent CTA per SM with 128x256
-// tiles, 326 / 449 with the next tile's load in flight across the tile boundary, 334 / 511 as two CTAs
-// of nine warps); no issuing warps, the last warp to empty a buffer issues its MMAs (413 / 481: an MMA
-// holds the thread that issues it for about 80 cycles).
+// What bounds it: the drain's exponentials and what they share a scheduler with.  Per element and warp a sweep takes 9
+// cycles, the exponential arithmetic alone 7 (special-function unit 6), the rest is waits for accumulators and
+// their loads; without the exponentials a sweep still takes 60 % of its time, without loads or products 98 %; at head_dim 128 the
+// board's power limit comes first (1.7 GHz).  us per layer of sweeps 1 / 2: 4 sequences of 4096, 32 / 8 heads of 128: 313 / 366
+// with a running maximum and two loads in flight, now 286 / 352; 2 of 5003, 71 / 1 heads of 64: 499 / 508, now 455 / 482.
+// Built to parity and measured slower (sweeps 1 / 2, against 313 / 366 and 499 / 508): queries on the lanes in both sweeps, with
+// one register per key in sweep 2 (315 / 416 as one persistent CTA per SM with 128x256 tiles, 334 / 511 as two CTAs of nine
+// warps) or four queries and 16 keys per thread (356 and 515); no issuing warps, the last warp to empty a buffer issues
+// its MMAs (413 / 481: an MMA holds the thread that issues it for about 80 cycles); 16 drain warps per CTA of 32 columns
+// (310 / 409 and 496 / 556).
 // Every mbarrier wait is bounded: on expiry the CTA raises a status bit and winds down.
 #include <algorithm>
 #include <type_traits>
@@ -34,12 +38,14 @@ namespace sq {
 
 using namespace tc;
 
-// Threads per CTA: a TMA warp, an MMA warp and eight drain warps.  A warp reaches only the 32
-// tensor-memory lanes of its quarter (warp index mod 4), so each quarter of the accumulator rows
-// is drained by two warps that take 64 of the tile's 128 columns each: four drain warps per
-// scheduler (two CTAs per SM) instead of two, so the special-function pipe is fed while other
-// warps wait for an accumulator or a tensor-memory load.
-constexpr int kPrefillThreads = 64 + 256;
+// TN: columns of a tile (streamed rows), 64 or 128.  A CTA has a TMA warp, an MMA warp and TN / 16 drain warps: a warp
+// reaches only the 32 tensor-memory lanes of its quarter (warp index mod 4) and takes 64 of a tile's columns.  An SM's 16
+// drain warps are four CTAs of 64 columns, whose waits for an accumulator fall at different times, where shared memory
+// holds four (head_dim 64: 460 / 486 us against 491 / 486 with two of 128), else two of 128.
+constexpr int prefill_threads(int tn) { return 64 + 2 * tn; }
+// How far, in powers of two, a row may rise above its reference: its weights' arguments are then rounded no more coarsely than a
+// log-sum-exp of that size is when it is stored.
+constexpr float kMaxRise = 32.f, kMaxSum = 4294967296.f;
 
 // exp2 of a pair on the FMA pipe: x = n + f with n the nearest integer (the usual 1.5 * 2^23
 // addition), 2^f for |f| <= 1/2 from a degree-5 polynomial (fitted here by a Remez exchange on the
@@ -71,30 +77,26 @@ __device__ __forceinline__ unsigned long long ex2_pair_sfu(unsigned long long x2
   f32x2_split(x2, x0, x1);
   return f32x2(ex2(x0), ex2(x1));
 }
-// Of every eight pairs of score elements this many take the FMA-pipe form, spread evenly.  The drain
-// is bound by the special-function unit (16 exponentials per cycle and SM: 1024 cycles per 128x128
-// tile) with none of them, by issue slots and the FMA pipe (two cycles per packed instruction) from
-// three of eight on.  Measured on B200, us per layer of sweep 1 / sweep 2 with 0, 1, 2, 3, 4 of eight:
-// head_dim 128 (4 sequences of 4096, 32 / 8 heads) 334/395, 321/374, 322/377, 337/380, 380/402;
-// head_dim 64 (2 sequences of 5003, 71 / 1 heads) 539/559, 512/520, 506/513, 533/523, 610/579.
-template <int D>
-__device__ __forceinline__ constexpr bool on_fma(int pair) {
-  constexpr int n = D == 64 ? 2 : 1;
-  return ((pair & 7) * n) % 8 + n >= 8;  // `pair` is a constant after unrolling
-}
+// Of every eight pairs of score elements two take the FMA-pipe form, spread evenly.  With none the special-function
+// unit bounds the drain (16 exponentials per cycle and SM: 1024 cycles per 128 x 128 elements); an FMA-pipe pair costs 25 cycles of
+// a scheduler where the unit's takes 16.  Measured on B200, us per layer of sweep 1 / sweep 2 with 1, 2, 3 of eight: head_dim
+// 128 (4 sequences of 4096, 32 / 8 heads) 296 / 364, 289 / 360, 301 / 374; head_dim 64 (2 sequences of 5003, 71 / 1 heads) 480 / 501,
+// 460 / 485, 475 / 505.
+__device__ __forceinline__ constexpr bool on_fma(int pair) { return (pair & 3) == 3; }  // `pair` is a constant after unrolling
 
 // SWEEP 1: rows = queries, streamed tiles = keys; SWEEP 2: rows = keys, streamed tiles = queries.
-template <int D, int STAGES, int SWEEP>
-__global__ void __launch_bounds__(kPrefillThreads, 2)
+template <int D, int TN, int STAGES, int SWEEP>
+__global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
     prefill_scores_tc_kernel(const __grid_constant__ CUtensorMap tm_rows, const __grid_constant__ CUtensorMap tm_stream,
                              ScoreArgs a, ScorePieces pc, float scale_log2, int* status) {
-  constexpr int SUB = D / 64;                  // 64-column sub-tiles per operand tile
-  constexpr int TILE_BYTES = SUB * kSubBytes;  // one operand tile
-  constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTM >> 3) << 17) | ((uint32_t)(kTM >> 4) << 24);
+  constexpr int SUB = D / 64;               // 64-column sub-tiles per operand tile
+  constexpr int STREAM_SUB = TN * 128;      // one [TN rows x 64 bf16] swizzled sub-tile
+  constexpr int ROWS_BYTES = SUB * kSubBytes, TILE_BYTES = SUB * STREAM_SUB;  // the fixed tile, a streamed tile
+  constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TN >> 3) << 17) | ((uint32_t)(kTM >> 4) << 24);
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* a_s = smem;
-  unsigned char* b_s = smem + TILE_BYTES;
+  unsigned char* b_s = smem + ROWS_BYTES;
   unsigned long long* bars = reinterpret_cast<unsigned long long*>(b_s + STAGES * TILE_BYTES);
   // barriers (at most 15 of the 16 slots), then the TMEM base, the abort flag and the lse staging
   static_assert(7 + 2 * STAGES <= 16, "barrier block");
@@ -106,11 +108,12 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
   auto bar_lse = [&](int b) { return s_u32(bars + 5 + 2 * STAGES + b); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* redo_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
   float* lse_s = reinterpret_cast<float*>(tmem_slot + 4);  // [2][128]: sweep 2, minus the row log-sum-exps
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int P = a.prompt, g = a.n_q_head / a.n_kv_head;
-  const int n_tile = (P + kTM - 1) / kTM;
+  const int n_tile = (P + kTM - 1) / kTM, n_col_tile = (P + TN - 1) / TN;
   // grid = (head, sequence, tile): the tile index varies slowest, so the CTAs with the most streamed
   // tiles of every head and sequence start first and the short ones fill the tail of the launch
   const int bi = blockIdx.y;
@@ -121,14 +124,14 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
     hq = blockIdx.x;
     hk = hq / g;
     row_tile = n_tile - 1 - blockIdx.z;  // longest rows first
-    n_stream = row_tile + 1;
+    n_stream = min(kTM / TN * (row_tile + 1), n_col_tile);
     rows0 = ((long long)bi * a.n_q_head + hq) * P + (long long)row_tile * kTM;
   } else {
     hk = blockIdx.x;
     row_tile = blockIdx.z / pc.n_piece;  // key tile 0 sees every query tile: longest first
     piece = blockIdx.z - row_tile * pc.n_piece;
     head0 = piece * pc.heads;            // this piece's heads of the group
-    n_stream = min(pc.heads, g - head0) * (n_tile - row_tile);
+    n_stream = min(pc.heads, g - head0) * (n_col_tile - kTM / TN * row_tile);
     rows0 = ((long long)bi * a.n_kv_head + hk) * P + (long long)row_tile * kTM;
   }
   // Walks the streamed tiles in order: (sweep 1) key tiles 0..row_tile, (sweep 2) per head of the
@@ -140,18 +143,18 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
   auto walk_begin = [&]() {
     Walk w;
     w.h = head0;
-    w.qt = SWEEP == 1 ? 0 : row_tile;
+    w.qt = SWEEP == 1 ? 0 : kTM / TN * row_tile;
     w.row0 = SWEEP == 1 ? ((long long)bi * a.n_kv_head + hk) * P
                         : ((long long)bi * a.n_q_head + hk * g + head0) * P + (long long)row_tile * kTM;
     return w;
   };
   auto walk_next = [&](Walk& w) {
     ++w.qt;
-    w.row0 += kTM;
-    if (SWEEP == 2 && w.qt == n_tile) {
-      w.qt = row_tile;
+    w.row0 += TN;
+    if (SWEEP == 2 && w.qt == n_col_tile) {
+      w.qt = kTM / TN * row_tile;
       ++w.h;
-      w.row0 += P - (long long)(n_tile - row_tile) * kTM;
+      w.row0 += P - (long long)(n_col_tile - kTM / TN * row_tile) * TN;
     }
   };
 
@@ -163,14 +166,16 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(bar_sfull(b), 1);
-      mbar_init(bar_sfree(b), 8);  // one arrival per drain warp
+      mbar_init(bar_sfree(b), TN / 16);  // one arrival per drain warp
       mbar_init(bar_lse(b), 1);
     }
     *abort_flag = 0;
+    *redo_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(s_u32(tmem_slot)) : "memory");
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(s_u32(tmem_slot)), "n"(2 * TN)
+                 : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -178,135 +183,160 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem_base = *tmem_slot;
 
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
-      mbar_expect_tx(bar_a, TILE_BYTES);
+  // drain threads: sweep 1: reference of the row and the sum of its weights; sweep 2: the key's sum (even and odd columns)
+  // (a tile's 64 weights are added up by themselves, so that a sum over thousands of tiles is no less precise than they are)
+  float m = -INFINITY, sum = 0.f;
+  bool ok = true;
+  // tiles are numbered through both passes of sweep 1 (the second one is rare, see the drain)
+  int tile0 = 0;
+#pragma unroll 1
+  for (;;) {
+    const int tile1 = tile0 + n_stream;
+    if (warp == 0) {
+      // ---------------- TMA producer ----------------
+      if (lane == 0) {
+        if (tile0 == 0) {
+          mbar_expect_tx(bar_a, ROWS_BYTES);
 #pragma unroll
-      for (int sb = 0; sb < SUB; ++sb) tma_load_2d(s_u32(a_s + sb * kSubBytes), &tm_rows, sb * 64, (int)rows0, bar_a);
-      int issued = 0;
-      Walk w = walk_begin();
-      for (int i = 0; i < n_stream; ++i) {
-        const int st = i % STAGES;
-        if (i >= STAGES && !mbar_wait(bar_empty(st), ((i / STAGES) - 1) & 1, abort_flag)) break;
-        mbar_expect_tx(bar_full(st), TILE_BYTES);
+          for (int sb = 0; sb < SUB; ++sb) tma_load_2d(s_u32(a_s + sb * kSubBytes), &tm_rows, sb * 64, (int)rows0, bar_a);
+        }
+        int issued = tile0;
+        Walk w = walk_begin();
+        for (int i = tile0; i < tile1; ++i) {
+          const int st = i % STAGES;
+          if (i >= STAGES && !mbar_wait(bar_empty(st), ((i / STAGES) - 1) & 1, abort_flag)) break;
+          mbar_expect_tx(bar_full(st), TILE_BYTES);
 #pragma unroll
-        for (int sb = 0; sb < SUB; ++sb)
-          tma_load_2d(s_u32(b_s + st * TILE_BYTES + sb * kSubBytes), &tm_stream, sb * 64, (int)w.row0, bar_full(st));
-        issued = i + 1;
-        walk_next(w);
-      }
-      if (*abort_flag) {
-        // winding down early: let the copies already in flight land before the CTA exits
-        mbar_wait(bar_a, 0, abort_flag);
-        for (int i = max(0, issued - STAGES); i < issued; ++i) {
-          for (int k = 0; k < kSpinLimit && !mbar_try_wait(bar_full(i % STAGES), (i / STAGES) & 1); ++k) {
+          for (int sb = 0; sb < SUB; ++sb)
+            tma_load_2d(s_u32(b_s + st * TILE_BYTES + sb * STREAM_SUB), &tm_stream, sb * 64, (int)w.row0, bar_full(st));
+          issued = i + 1;
+          walk_next(w);
+        }
+        if (*abort_flag) {
+          // winding down early: let the copies already in flight land before the CTA exits
+          mbar_wait(bar_a, 0, abort_flag);
+          for (int i = max(0, issued - STAGES); i < issued; ++i) {
+            for (int k = 0; k < kSpinLimit && !mbar_try_wait(bar_full(i % STAGES), (i / STAGES) & 1); ++k) {
+            }
           }
         }
       }
-    }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer; sweep 2: also stages the tile's row log-sum-exps ----------------
-    // (fetched one tile ahead, so that the trip to memory runs under the tile before)
-    auto fetch_lse = [&](const Walk& w) {
-      const float* src = a.lse2 + ((size_t)bi * a.n_q_head + hk * g + w.h) * P;
-      const int q = w.qt * kTM + lane * 4;
-      float4 v;
-      v.x = (q + 0 < P) ? -src[q + 0] : -INFINITY;  // a query past the end attends to nothing
-      v.y = (q + 1 < P) ? -src[q + 1] : -INFINITY;
-      v.z = (q + 2 < P) ? -src[q + 2] : -INFINITY;
-      v.w = (q + 3 < P) ? -src[q + 3] : -INFINITY;
-      return v;
-    };
-    Walk w = walk_begin();
-    float4 lse_next = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (SWEEP == 2) lse_next = fetch_lse(w);
-    bool ok = mbar_wait(bar_a, 0, abort_flag);
-    for (int i = 0; ok && i < n_stream; ++i) {
-      const int st = i % STAGES, buf = i & 1;
-      ok = mbar_wait(bar_full(st), (i / STAGES) & 1, abort_flag);
-      if (ok && i >= 2) ok = mbar_wait(bar_sfree(buf), ((i >> 1) - 1) & 1, abort_flag);
-      if (!ok) break;
-      if (SWEEP == 2) {
-        *reinterpret_cast<float4*>(lse_s + buf * kTM + lane * 4) = lse_next;
-        __syncwarp();
-      }
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      if (lane == 0) {
-        if (SWEEP == 2) mbar_arrive(bar_lse(buf));
-        const uint32_t d_tmem = tmem_base + buf * kTM;
+    } else if (warp == 1) {
+      // ---------------- MMA issuer; sweep 2: also stages the tile's row log-sum-exps ----------------
+      // (fetched one tile ahead, so that the trip to memory runs under the tile before)
+      constexpr int kLse = TN / 32;  // per lane
+      struct alignas(4 * kLse) Lse {
+        float x[kLse];
+      };
+      auto fetch_lse = [&](const Walk& w) {
+        const float* src = a.lse2 + ((size_t)bi * a.n_q_head + hk * g + w.h) * P;
+        const int q = w.qt * TN + lane * kLse;
+        Lse v;
 #pragma unroll
-        for (int k = 0; k < D / 16; ++k) {
-          const uint32_t a_addr = s_u32(a_s + (k / 4) * kSubBytes) + (k % 4) * 32;
-          const uint32_t b_addr = s_u32(b_s + st * TILE_BYTES + (k / 4) * kSubBytes) + (k % 4) * 32;
-          umma_bf16(d_tmem, umma_desc(a_addr), umma_desc(b_addr), kIdesc, k > 0 ? 1u : 0u);
+        for (int e = 0; e < kLse; ++e) v.x[e] = (q + e < P) ? -src[q + e] : -INFINITY;  // a query past the end attends to nothing
+        return v;
+      };
+      Walk w = walk_begin();
+      Lse lse_next = {};
+      if (SWEEP == 2) lse_next = fetch_lse(w);
+      ok = mbar_wait(bar_a, 0, abort_flag);
+      for (int i = tile0; ok && i < tile1; ++i) {
+        const int st = i % STAGES, buf = i & 1;
+        ok = mbar_wait(bar_full(st), (i / STAGES) & 1, abort_flag);
+        if (ok && i >= 2) ok = mbar_wait(bar_sfree(buf), ((i >> 1) - 1) & 1, abort_flag);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (lane == 0) {
+          const uint32_t d_tmem = tmem_base + buf * TN;
+#pragma unroll
+          for (int k = 0; k < D / 16; ++k) {
+            const uint32_t a_addr = s_u32(a_s + (k / 4) * kSubBytes) + (k % 4) * 32;
+            const uint32_t b_addr = s_u32(b_s + st * TILE_BYTES + (k / 4) * STREAM_SUB) + (k % 4) * 32;
+            umma_bf16(d_tmem, umma_desc(a_addr), umma_desc(b_addr), kIdesc, k > 0 ? 1u : 0u);
+          }
+          umma_commit(bar_empty(st));  // the stage may be refilled once these MMAs have read it
+          umma_commit(bar_sfull(buf)); // the accumulator buffer is complete
         }
-        umma_commit(bar_empty(st));  // the stage may be refilled once these MMAs have read it
-        umma_commit(bar_sfull(buf)); // the accumulator buffer is complete
+        __syncwarp();
+        if (SWEEP == 2) {
+          // (behind the products, which do not wait for them)
+          *reinterpret_cast<Lse*>(lse_s + buf * TN + lane * kLse) = lse_next;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_lse(buf));
+          if (i + 1 < tile1) {
+            walk_next(w);
+            lse_next = fetch_lse(w);
+          }
+        }
       }
-      __syncwarp();
-      if (SWEEP == 2 && i + 1 < n_stream) {
-        walk_next(w);
-        lse_next = fetch_lse(w);
-      }
-    }
-  } else {
-    // ---------------- accumulator drain: thread = one row of the fixed tile ----------------
-    const int quarter = warp & 3;
-    const int half = (warp - 2) >> 2;  // which 64 columns of every tile this warp drains
-    const int row = quarter * 32 + lane;
-    const int row_idx = row_tile * kTM + row;  // query index (sweep 1) / key index (sweep 2)
-    const uint32_t s_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + half * 64;
-    const unsigned long long scale2 = f32x2(scale_log2, scale_log2);
-    // sweep 1: running reference of the row and its sum; sweep 2: the key's sum (even and odd columns)
-    float m = -INFINITY, l = 0.f;
-    unsigned long long acc_a = f32x2(0.f, 0.f), acc_b = acc_a;
-    bool ok = true;
-    Walk w = walk_begin();
-    for (int i = 0; ok && i < n_stream; ++i) {
-      const int buf = i & 1;
-      const bool diag = w.qt == row_tile;
-      walk_next(w);
-      if (SWEEP == 2) ok = mbar_wait(bar_lse(buf), (i >> 1) & 1, abort_flag);
-      if (ok) ok = mbar_wait(bar_sfull(buf), (i >> 1) & 1, abort_flag);
-      if (!ok) break;
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      // The tile on the diagonal masks half of its elements; every other tile masks none.  The two
-      // cases are separate instantiations of the drain, so that tiles off the diagonal (all but one
-      // per row of tiles) carry no compare / select per element.
-      auto chunk = [&](auto diag_c, uint32_t (&r)[32], int c0) {  // columns c0 .. c0+31 of the tile
-        constexpr bool DIAG = decltype(diag_c)::value;
-        if (SWEEP == 1) {
-          if (DIAG) {
+    } else {
+      // ---------------- accumulator drain: thread = one row of the fixed tile, 64 columns ----------------
+      const int quarter = warp & 3;
+      const int col0 = TN == 64 ? 0 : ((warp - 2) >> 2) * 64;  // of the 64 columns of every tile that this warp drains
+      const int row = quarter * 32 + lane;
+      const uint32_t s_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + col0;
+      const unsigned long long scale2 = f32x2(scale_log2, scale_log2);
+      m = -INFINITY;
+      sum = 0.f;
+      unsigned long long acc_a, acc_b;  // of the tile, even and odd columns
+      float top = -INFINITY, m_first = 0.f;  // of the FMA-pipe form's scores; reference of the plain tiles
+      Walk w = walk_begin();
+      // The tiles on the diagonal mask a part of their elements, the others none: they are separate
+      // instantiations of the drain, so that tiles off the diagonal carry no compare / select per element.
+      // Sweep 1 has a third: a row's reference is its maximum over the first tile (and over those on the diagonal), so
+      // that most tiles carry no maximum.  A weight above 2^kMaxRise shows in the sum, but for the FMA-pipe form, which
+      // may overflow without a trace and whose scores are therefore looked at: a CTA with such a row walks its tiles again
+      // with a running maximum.  (Redone on the spot, chunk by chunk, the code that hardly ever runs cost 456 against 440
+      // us a sweep; a reference that follows the FMA-pipe form's scores 488 against 460, at the same precision.)
+      enum { kPlain, kDiagonal, kFirst };
+      struct Tile {
+        int buf, off;  // off: of the tile's first column from the fixed tile's first row
+      };
+      // weights of 32 columns under the reference m
+      auto row_weights = [&](auto exact_c, const uint32_t (&r)[32]) {
+        const unsigned long long neg_m2 = f32x2(-m, -m);
+#pragma unroll
+        for (int jp = 0; jp < 16; ++jp) {
+          const unsigned long long x2 =
+              fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])), scale2, neg_m2);
+          // (a masked tile keeps to the form that gives an exact 0)
+          const unsigned long long e2 = !decltype(exact_c)::value && on_fma(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
+          if (jp & 1) acc_b = add_f32x2(acc_b, e2);
+          else acc_a = add_f32x2(acc_a, e2);
+        }
+      };
+      auto move_reference = [&](const uint32_t (&r)[32]) {
+        float mx = __uint_as_float(r[0]);
+#pragma unroll
+        for (int j = 1; j + 1 < 32; j += 2) mx = max3(mx, __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
+        const float m_new = fmaxf(m, fmaxf(mx, __uint_as_float(r[31])) * scale_log2);
+        if (m_new > m) {
+          const float f = ex2(m - m_new);
+          const unsigned long long f2 = f32x2(f, f), zero = f32x2(0.f, 0.f);
+          acc_a = fma_f32x2(acc_a, f2, zero);
+          acc_b = fma_f32x2(acc_b, f2, zero);
+          sum *= f;
+          m = m_new;
+        }
+      };
+      auto chunk = [&](auto kind_c, const Tile& t, uint32_t (&r)[32], int c0) {  // columns c0 .. c0+31 of the tile
+        constexpr int KIND = decltype(kind_c)::value;
+        if constexpr (SWEEP == 1 && KIND == kPlain) {
+          row_weights(std::false_type{}, r);
+#pragma unroll
+          for (int jp = 0; jp < 16; ++jp)
+            if (on_fma(jp)) top = max3(top, __uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1]));
+        } else if constexpr (SWEEP == 1) {
+          if (KIND == kDiagonal) {
 #pragma unroll
             for (int j = 0; j < 32; ++j)
-              if (c0 + j > row) r[j] = 0xff800000u;  // key after the query: -inf
+              if (t.off + c0 + j > row) r[j] = 0xff800000u;  // key after the query: -inf
           }
-          float mx = __uint_as_float(r[0]);
-#pragma unroll
-          for (int j = 1; j + 1 < 32; j += 2) mx = max3(mx, __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
-          mx = fmaxf(mx, __uint_as_float(r[31]));
-          const float m_new = fmaxf(m, mx * scale_log2);
-          if (DIAG && m_new == -INFINITY) return;  // nothing of the row so far (second half of the first rows)
-          if (m_new > m) {
-            const float f = ex2(m - m_new);
-            const unsigned long long f2 = f32x2(f, f), zero = f32x2(0.f, 0.f);
-            acc_a = fma_f32x2(acc_a, f2, zero);
-            acc_b = fma_f32x2(acc_b, f2, zero);
-            m = m_new;
-          }
-          const unsigned long long neg_m2 = f32x2(-m, -m);
-#pragma unroll
-          for (int jp = 0; jp < 16; ++jp) {
-            const unsigned long long x2 =
-                fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])), scale2, neg_m2);
-            // (the masked tile keeps to the form that gives an exact 0)
-            const unsigned long long e2 = !DIAG && on_fma<D>(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
-            if (jp & 1) acc_b = add_f32x2(acc_b, e2);
-            else acc_a = add_f32x2(acc_a, e2);
-          }
+          move_reference(r);
+          if (KIND == kDiagonal && m == -INFINITY) return;  // nothing of the row so far (second half of the first rows)
+          row_weights(std::bool_constant<KIND == kDiagonal>{}, r);
         } else {
-          const ulonglong2* ls = reinterpret_cast<const ulonglong2*>(lse_s + buf * kTM + c0);
+          const ulonglong2* ls = reinterpret_cast<const ulonglong2*>(lse_s + t.buf * TN + c0);
 #pragma unroll
           for (int j4 = 0; j4 < 8; ++j4) {
             const ulonglong2 lv = ls[j4];
@@ -315,11 +345,11 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
               const int jp = 2 * j4 + q;
               const unsigned long long x2 = fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])),
                                                       scale2, q ? lv.y : lv.x);
-              unsigned long long e2 = on_fma<D>(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
-              if (DIAG) {  // query before the key: no attention
+              unsigned long long e2 = on_fma(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
+              if (KIND == kDiagonal) {  // query before the key: no attention
                 float e0, e1;
                 f32x2_split(e2, e0, e1);
-                e2 = f32x2(c0 + 2 * jp >= row ? e0 : 0.f, c0 + 2 * jp + 1 >= row ? e1 : 0.f);
+                e2 = f32x2(t.off + c0 + 2 * jp >= row ? e0 : 0.f, t.off + c0 + 2 * jp + 1 >= row ? e1 : 0.f);
               }
               if (q) acc_b = add_f32x2(acc_b, e2);
               else acc_a = add_f32x2(acc_a, e2);
@@ -327,50 +357,78 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
           }
         }
       };
-      auto hand_back = [&]() {
-        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      auto drain_tile = [&](auto kind_c, const Tile& t) {
+        auto hand_back = [&]() {
+          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+          __syncwarp();
+          if (lane == 0) mbar_arrive(bar_sfree(t.buf));
+        };
+        // (32 columns at a time: with the second half's load in flight under the first's exponentials the registers
+        // held the FMA-pipe form back, 497 against 482 us a sweep at head_dim 64)
+        acc_a = acc_b = f32x2(0.f, 0.f);
+        uint32_t r[32];
+        tmem_ld32_nowait(s_addr + t.buf * TN, r);
+        tmem_wait_ld(r);
+        chunk(kind_c, t, r, col0);
         __syncwarp();
-        if (lane == 0) mbar_arrive(bar_sfree(buf));
-      };
-      auto drain_tile = [&](auto diag_c) {
-        uint32_t ra[32], rb[32];
-        tmem_ld32_nowait(s_addr + buf * kTM, ra);
-        tmem_wait_ld(ra);
-        tmem_ld32_nowait(s_addr + buf * kTM + 32, rb);
-        chunk(diag_c, ra, half * 64);
-        __syncwarp();
-        tmem_wait_ld(rb);
+        tmem_ld32_nowait(s_addr + t.buf * TN + 32, r);
+        tmem_wait_ld(r);
         if (SWEEP == 1) hand_back();  // the tile is in registers: the tensor core may have the buffer back
-        chunk(diag_c, rb, half * 64 + 32);
+        chunk(kind_c, t, r, col0 + 32);
         if (SWEEP == 2) hand_back();  // the buffer's lse staging is in use until here
+        float a0, a1;
+        f32x2_split(add_f32x2(acc_a, acc_b), a0, a1);
+        sum += a0 + a1;
       };
-      if (diag) drain_tile(std::true_type{});
-      else drain_tile(std::false_type{});
+      for (int i = tile0; ok && i < tile1; ++i) {
+        const Tile t{i & 1, (w.qt - kTM / TN * row_tile) * TN};
+        const bool diag = (unsigned)t.off < (unsigned)kTM;
+        walk_next(w);
+        if (SWEEP == 2) ok = mbar_wait(bar_lse(t.buf), (i >> 1) & 1, abort_flag);
+        if (ok) ok = mbar_wait(bar_sfull(t.buf), (i >> 1) & 1, abort_flag);
+        if (!ok) break;
+        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+        if (SWEEP == 1 && i == 1) m_first = m;
+        if (diag) drain_tile(std::integral_constant<int, kDiagonal>{}, t);
+        else if (SWEEP == 1 && (i == 0 || tile0 > 0)) drain_tile(std::integral_constant<int, kFirst>{}, t);
+        else drain_tile(std::integral_constant<int, kPlain>{}, t);
+      }
+      if (SWEEP == 1 && tile0 == 0 && (fmaf(top, scale_log2, -m_first) > kMaxRise || !(sum <= kMaxSum))) *redo_flag = 1;
     }
-    {
-      float a0, a1, b0, b1;
-      f32x2_split(acc_a, a0, a1);
-      f32x2_split(acc_b, b0, b1);
-      l = (a0 + a1) + (b0 + b1);
-    }
-    // the two halves of a row meet in shared memory (the staging area is free once every drain
-    // thread is past its last tile); every drain thread reaches both barriers, aborted or not
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (half == 1) {
-      lse_s[2 * row] = m;
-      lse_s[2 * row + 1] = l;
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (half == 0 && ok && !*abort_flag && row_idx < P) {
+    if (SWEEP == 2) break;
+    __syncthreads();
+    if (tile0 > 0 || !*redo_flag || *abort_flag) break;
+    tile0 = tile1;
+  }
+  if (warp >= 2) {
+    const int row = (warp & 3) * 32 + lane, row_idx = row_tile * kTM + row;  // query (sweep 1) / key (sweep 2)
+    const bool second_half = warp >= 6;
+    float l = sum;
+    if constexpr (TN == 128) {
+      // the two halves of a row meet in shared memory (the staging area is free once every drain
+      // thread is past its last tile); every drain thread reaches both barriers, aborted or not
+      asm volatile("bar.sync 1, 256;" ::: "memory");
+      if (second_half) {
+        lse_s[2 * row] = m;
+        lse_s[2 * row + 1] = l;
+      }
+      asm volatile("bar.sync 1, 256;" ::: "memory");
       const float o0 = lse_s[2 * row], o1 = lse_s[2 * row + 1];
       if (SWEEP == 1) {
         // this half holds column 0 of every tile, so m is finite; the other half may be empty
         const float mm = fmaxf(m, o0);
-        const float ll = l * ex2(m - mm) + o1 * ex2(o0 - mm);
-        a.lse2[((size_t)bi * a.n_q_head + hq) * P + row_idx] = mm + log2f(ll);
+        l = l * ex2(m - mm) + o1 * ex2(o0 - mm);
+        m = mm;
+      } else {
+        l += o1;
+      }
+    }
+    if (!second_half && ok && !*abort_flag && row_idx < P) {
+      if (SWEEP == 1) {
+        a.lse2[((size_t)bi * a.n_q_head + hq) * P + row_idx] = m + log2f(l);
       } else {
         float* dst = pc.n_piece == 1 ? a.acc_prompt : pc.partial + (size_t)piece * a.batch * a.n_kv_head * P;
-        dst[((size_t)bi * a.n_kv_head + hk) * P + row_idx] = l + o1;
+        dst[((size_t)bi * a.n_kv_head + hk) * P + row_idx] = l;
       }
     }
   }
@@ -378,7 +436,7 @@ __global__ void __launch_bounds__(kPrefillThreads, 2)
   __syncthreads();
   if (warp == 1) {
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem_base) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "n"(2 * TN) : "memory");
   }
   if (tid == 0 && *abort_flag) atomicOr(status, kStatusTimeout);
   if (SWEEP == 2 && pc.n_piece > 1) {
@@ -436,17 +494,19 @@ bool make_tile_map(CUtensorMap* tm, const void* base, long long rows, int d, int
 }
 }  // namespace tc
 
-template <int D, int STAGES>
+template <int D, int TN, int STAGES>
 static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) {
   CUtensorMap tm_q, tm_k;
   const long long q_rows = (long long)a.batch * a.n_q_head * a.prompt, k_rows = (long long)a.batch * a.n_kv_head * a.prompt;
   if (q_rows + kTM > 0x7fffffffLL) return cudaErrorNotSupported;  // TMA coordinates are 32-bit
+  CUtensorMap ts_q, ts_k;  // streamed
   if (!tc::make_tile_map(&tm_q, a.q, q_rows, D, kTM) || !tc::make_tile_map(&tm_k, a.k, k_rows, D, kTM)) return cudaErrorNotSupported;
-  constexpr size_t smem = 1024 + (size_t)(1 + STAGES) * (D / 64) * kSubBytes + 8 * 16 + 16 + 2 * kTM * 4;
+  if (!tc::make_tile_map(&ts_q, a.q, q_rows, D, TN) || !tc::make_tile_map(&ts_k, a.k, k_rows, D, TN)) return cudaErrorNotSupported;
+  constexpr size_t smem = 1024 + (size_t)(D / 64) * (kSubBytes + STAGES * TN * 128) + 8 * 16 + 16 + 2 * TN * 4;
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
   const int n_tile = (a.prompt + kTM - 1) / kTM;
-  auto k1 = prefill_scores_tc_kernel<D, STAGES, 1>;
-  auto k2 = prefill_scores_tc_kernel<D, STAGES, 2>;
+  auto k1 = prefill_scores_tc_kernel<D, TN, STAGES, 1>;
+  auto k2 = prefill_scores_tc_kernel<D, TN, STAGES, 2>;
   static PerDevice set_up;
   cudaError_t e = allow_smem(set_up, smem, k1, k2);
   if (e != cudaSuccess) return e;
@@ -458,7 +518,7 @@ static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) 
   ScorePieces pc;
   const int g = a.n_q_head / a.n_kv_head;
   const long long units = (long long)a.batch * a.n_kv_head;
-  const long long slots = 2LL * sm_count();  // two CTAs per SM
+  const long long slots = 2LL * sm_count();  // (of 128 columns; finer pieces for the CTAs of 64 were slower, 497 against 488 us)
   long long heads = std::max(1LL, std::min((long long)g, units * g * (n_tile + 1) / (8 * slots)));
   auto pieces = [&](long long h) { return (g + h - 1) / h; };
   while (heads < g && (pieces(heads) * units * a.prompt > (long long)a.partial_floats || pieces(heads) * n_tile > 65535)) ++heads;
@@ -466,10 +526,10 @@ static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) 
   pc.n_piece = (int)pieces(heads);
   pc.partial = a.partial;
   pc.tickets = a.tickets;
-  k1<<<dim3(a.n_q_head, a.batch, n_tile), kPrefillThreads, smem, s>>>(tm_q, tm_k, a, pc, scale_log2, status);
+  k1<<<dim3(a.n_q_head, a.batch, n_tile), prefill_threads(TN), smem, s>>>(tm_q, ts_k, a, pc, scale_log2, status);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k2<<<dim3(a.n_kv_head, a.batch, n_tile * pc.n_piece), kPrefillThreads, smem, s>>>(tm_k, tm_q, a, pc, scale_log2, status);
+  k2<<<dim3(a.n_kv_head, a.batch, n_tile * pc.n_piece), prefill_threads(TN), smem, s>>>(tm_k, ts_q, a, pc, scale_log2, status);
   return cudaGetLastError();
 }
 
@@ -477,8 +537,8 @@ static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) 
 cudaError_t launch_prefill_scores_tc(const ScoreArgs& a, int* status, cudaStream_t s) {
   if (a.n_q_head > 65535 || a.batch > 65535 || (a.prompt + kTM - 1) / kTM > 65535) return cudaErrorNotSupported;
   if ((reinterpret_cast<uintptr_t>(a.q) | reinterpret_cast<uintptr_t>(a.k)) & 15u) return cudaErrorNotSupported;
-  if (a.head_dim == 64) return launch_tc_t<64, 4>(a, status, s);
-  if (a.head_dim == 128) return launch_tc_t<128, 2>(a, status, s);
+  if (a.head_dim == 64) return launch_tc_t<64, 64, 3>(a, status, s);
+  if (a.head_dim == 128) return launch_tc_t<128, 128, 2>(a, status, s);
   return cudaErrorNotSupported;
 }
 

@@ -43,6 +43,29 @@ def test_prompt_scores_cut_into_pieces(dtype, head_dim, hq, hkv, batch, prompt):
     assert ctx.status() == 0
 
 
+# A row's reference is its maximum over the first keys and stays unless a row rises 2^32 above it: some rows do, by overflowing
+# amounts too, some rise less, some not at all; both tile widths, both halves of a wide tile, the last tile ragged
+@pytest.mark.parametrize("head_dim,hq", [(64, 3), (128, 2)])
+@pytest.mark.parametrize("prompt", [200, 700])
+def test_prompt_scores_of_rising_rows(head_dim, hq, prompt):
+    w = workload("rising", 9150 + prompt, head_dim=head_dim, n_q_head=hq, n_kv_head=1, batch=3, prompt=prompt, heavy_mode="none")
+    ctx = H.make_ctx(w, b_init=prompt)
+    ctx.begin_sequence_batch(3, prompt)
+    ctx.set_budgets([prompt])
+    q, k, v = synth.prompt_qkv(w, 0, DEV)
+    k[1, :, 140:] *= 12.0          # logits of some tens
+    k[2, :, 150:170] *= 100.0      # beyond 2^128
+    ctx.prefill_compress(0, k, v, q)
+    for s in range(3):
+        pos, acc = ctx.get_kept(0, s, 0)
+        assert pos == list(range(prompt))
+        want = O.prefill_scores(H.f64(q[s]), H.f64(k[s, 0]))
+        # logits of up to L = 100 * 6 are fp32 sums of head_dim products and meet the stored log-sum-exp at that size: 2^-23 L
+        # each in the exponent, twice; scores below 2^-126 of a row count as that
+        np.testing.assert_allclose(acc, want, rtol=H.RTOL_ACC[w.dtype] * (10 if s == 2 else 1), atol=1e-6)
+    assert ctx.status() == 0
+
+
 # Decode launches of one layer right behind one another start before the launch ahead is done and fetch
 # their first rows ahead of it, all but the new token's: its slot goes through every row of the cache,
 # and one layer behind itself (n_layer 1) or a stream change must not read ahead
