@@ -4,16 +4,13 @@
 //      over the scores) and record the decisions as a bitmask in shared memory with a running
 //      count per 32 slots, so that any thread knows a row's new slot without touching memory;
 //   2. close the gaps by moving the kept rows towards slot 0 in slot order.  A row's new slot
-//      is never behind its old one, so a chunk of rows (with its positions and scores) is
-//      fetched into shared memory with cp.async and stored to its new slots once it has
+//      is never behind its old one, so a chunk of kept rows (with its positions and scores) is
+//      fetched into shared memory with cp.async and stored to its new slots, which are consecutive, once it has
 //      landed; chunks go in slot order, so a store never overwrites a row not yet read.
-// The kernel is templated on the chunk size and on the number of chunks in flight per CTA.
-// Measured (budgets halved on full caches, GB/s of rows read + written, Llama-2-7B- /
-// Mistral-7B-H2O- / Llama-2-70B-shaped): 32 KB x 3 in flight (2 CTAs per SM) 2837 / 1868 / 3343;
-// 16 KB x 3: 3727 / 2573 / 4513; 8 KB x 4: 3812 / 2776 / 4582; 16 KB x 2: 4180 / 2947 / 4901;
-// 16 KB x 1: 4148 / 2987 / 5024; 32 KB x 1 (7 CTAs per SM): 4176 / 2982 / 5124.  The overlap
-// that matters comes from many resident CTAs, not from a deep ring inside one, so the build
-// uses one 32 KB chunk per CTA.
+// A chunk is 32 KB of rows that stay: with chunks of slots a budget cut to half filled half of each, and a CTA took
+// twice the trips to memory, one after the other (32 layers of 8 KV heads of 128, 16 sequences, H2O, 20 % of 4096 halved:
+// 411 us, now 360).  The overlap that matters comes from many resident CTAs (7 per SM), not from a deep ring inside
+// one: 32 KB x 3 in flight (2 CTAs per SM) moved 2.8 to 3.3 TB/s where 32 KB x 1 moved 4.2 to 5.1.
 #include "sq_device.cuh"
 #include "sq_internal.h"
 #include "sq_select.cuh"
@@ -30,16 +27,21 @@ __device__ __forceinline__ void cp_async(void* dst_smem, const void* src, int by
   else
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src));
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;"); }
-__device__ __forceinline__ void cp_async_wait_all_but(int n) {
-  switch (n) {
-    case 0: asm volatile("cp.async.wait_group 0;"); break;
-    case 1: asm volatile("cp.async.wait_group 1;"); break;
-    case 2: asm volatile("cp.async.wait_group 2;"); break;
-    case 3: asm volatile("cp.async.wait_group 3;"); break;
-    case 4: asm volatile("cp.async.wait_group 4;"); break;
-    default: asm volatile("cp.async.wait_group 5;"); break;
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// index of the r-th set bit of m (r < popc(m))
+__device__ __forceinline__ int nth_set_bit(unsigned m, int r) {
+  int at = 0;
+#pragma unroll
+  for (int s = 16; s > 0; s >>= 1) {
+    const int c = __popc(m & ((1u << s) - 1u));
+    if (r >= c) {
+      r -= c;
+      m >>= s;
+      at += s;
+    }
   }
+  return at;
 }
 
 // H2O: among the first b slots, the token outside the recent window (position <= last_old) that
@@ -61,17 +63,18 @@ __device__ __forceinline__ int h2o_next_victim(SelScratch& sc, const int* pos, c
 }
 }  // namespace
 
-// Dynamic shared memory: kStages chunks of rows, then per stage the chunk's positions and
-// scores, then the keep bitmask (one word per 32 slots) and its running count.
-template <int kChunkBytes, int kStages>
+// Dynamic shared memory: a chunk of rows, its positions and scores, the slots that this chunk and the next come from, then
+// the keep bitmask (one word per 32 slots) and its running count.
+template <int kChunkBytes>
 __global__ void __launch_bounds__(kSelThreads) evict_kernel(EvictArgs a) {
   constexpr int kMaxChunkRows = kChunkBytes / (2 * 128);  // 128-byte rows (bf16, head_dim 64)
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ SelScratch sc;
   uint4* stage = reinterpret_cast<uint4*>(dyn);
-  int* s_pos = reinterpret_cast<int*>(dyn + (size_t)kStages * kChunkBytes);
-  float* s_acc = reinterpret_cast<float*>(s_pos + kStages * kMaxChunkRows);
-  unsigned* s_mask = reinterpret_cast<unsigned*>(s_acc + kStages * kMaxChunkRows);
+  int* s_pos = reinterpret_cast<int*>(dyn + kChunkBytes);
+  float* s_acc = reinterpret_cast<float*>(s_pos + kMaxChunkRows);
+  int* s_src = reinterpret_cast<int*>(s_acc + kMaxChunkRows);
+  unsigned* s_mask = reinterpret_cast<unsigned*>(s_src + 2 * kMaxChunkRows);
   const int unit = blockIdx.x, tid = threadIdx.x;
   const EvictLayer& ev = a.tab[blockIdx.y];
   const LayerDesc& lo = ev.ld_old;
@@ -158,33 +161,26 @@ __global__ void __launch_bounds__(kSelThreads) evict_kernel(EvictArgs a) {
   }
   __syncthreads();
   const int written = sc.total;
-  auto kept = [&](int slot) { return (s_mask[slot >> 5] >> (slot & 31)) & 1u; };
-  auto new_slot = [&](int slot) { return s_before[slot >> 5] + __popc(s_mask[slot >> 5] & ((1u << (slot & 31)) - 1u)); };
+  if (tid == 0 && written > b) atomicOr(a.status, 4);
 
-  // --- 2. stable compaction through the cp.async ring ---
+  // --- 2. stable compaction ---
   const int vpr = a.row_bytes / 16;                  // 8, 16 or 32 sixteen-byte pieces per row
   const int lv = 31 - __clz(2 * vpr);                // a slot's K and V pieces: 1 << lv
-  const int rows = kChunkBytes / (2 * a.row_bytes);  // slots per chunk
-  const int n_chunks = (n + rows - 1) / rows;
+  const int rows = kChunkBytes / (2 * a.row_bytes);  // rows per chunk
+  const int n_out = min(written, b), n_chunks = (n_out + rows - 1) / rows;
   uint4* kb = reinterpret_cast<uint4*>(a.pool + lo.k_off) + (size_t)unit * cap * vpr;
   uint4* vb = reinterpret_cast<uint4*>(a.pool + lo.v_off) + (size_t)unit * cap * vpr;
-  auto issue = [&](int c) {
-    if (c < n_chunks) {
-      const int s0 = c * rows, st = c % kStages;
-      uint4* sg = stage + (size_t)st * (kChunkBytes / 16);
-      for (int idx = tid; idx < rows * 2 * vpr; idx += kSelThreads) {
-        const int j = idx >> lv, r = idx & ((1 << lv) - 1);
-        const int slot = s0 + j;
-        if (slot >= n || !kept(slot)) continue;
-        const size_t src = (size_t)slot * vpr;
-        cp_async(sg + idx, (r < vpr) ? (kb + src + r) : (vb + src + r - vpr), 1);
-        if (r == 0) {
-          cp_async(s_pos + st * kMaxChunkRows + j, pos + slot, 0);
-          if (h2o) cp_async(s_acc + st * kMaxChunkRows + j, acc + slot, 0);
-        }
-      }
+  // the slots that the rows of chunk c come from: the word whose running count reaches the row, then the bit
+  auto find_sources = [&](int c) {
+    const int k = c * rows + tid;
+    if (tid >= rows || k >= n_out) return;
+    int w0 = 0, w1 = n_words;  // s_before[w0] <= k < s_before[w1]
+    while (w1 - w0 > 1) {
+      const int mid = (w0 + w1) >> 1;
+      if (s_before[mid] <= k) w0 = mid;
+      else w1 = mid;
     }
-    cp_async_commit();  // one group per chunk, empty past the end, so the wait counts stay aligned
+    s_src[(c & 1) * kMaxChunkRows + tid] = w0 * 32 + nth_set_bit(s_mask[w0], k - s_before[w0]);
   };
   // chunks before the first kept row that moves hold nothing to do
   int c_begin = n_chunks;
@@ -195,31 +191,35 @@ __global__ void __launch_bounds__(kSelThreads) evict_kernel(EvictArgs a) {
       break;
     }
   }
-  for (int c = c_begin; c < c_begin + kStages - 1; ++c) issue(c);
+  find_sources(c_begin);
   for (int c = c_begin; c < n_chunks; ++c) {
-    issue(c + kStages - 1);
-    cp_async_wait_all_but(kStages - 1);
-    __syncthreads();
-    const int s0 = c * rows, st = c % kStages;
-    const uint4* sg = stage + (size_t)st * (kChunkBytes / 16);
-    for (int idx = tid; idx < rows * 2 * vpr; idx += kSelThreads) {
+    __syncthreads();  // the chunk's sources are known, the staging area is free
+    const int s0 = c * rows, n_row = min(rows, n_out - s0);
+    const int* src = s_src + (c & 1) * kMaxChunkRows;
+    for (int idx = tid; idx < n_row << lv; idx += kSelThreads) {
       const int j = idx >> lv, r = idx & ((1 << lv) - 1);
-      const int slot = s0 + j;
-      if (slot >= n || !kept(slot)) continue;
-      const int d = new_slot(slot);
-      if (d >= b) {
-        atomicOr(a.status, 4);
-        continue;
-      }
-      if (r < vpr) kb[(size_t)d * vpr + r] = sg[idx];
-      else vb[(size_t)d * vpr + r - vpr] = sg[idx];
+      const size_t from = (size_t)src[j] * vpr;
+      cp_async(stage + idx, (r < vpr) ? (kb + from + r) : (vb + from + r - vpr), 1);
       if (r == 0) {
-        pos[d] = s_pos[st * kMaxChunkRows + j];
-        if (h2o) acc[d] = s_acc[st * kMaxChunkRows + j];
+        cp_async(s_pos + j, pos + src[j], 0);
+        if (h2o) cp_async(s_acc + j, acc + src[j], 0);
       }
     }
-    __syncthreads();  // the stage is refilled by the next iteration's loads
+    find_sources(c + 1);
+    cp_async_wait();
+    __syncthreads();
+    for (int idx = tid; idx < n_row << lv; idx += kSelThreads) {
+      const int j = idx >> lv, r = idx & ((1 << lv) - 1);
+      const size_t to = (size_t)(s0 + j) * vpr;
+      if (r < vpr) kb[to + r] = stage[idx];
+      else vb[to + r - vpr] = stage[idx];
+      if (r == 0) {
+        pos[s0 + j] = s_pos[j];
+        if (h2o) acc[s0 + j] = s_acc[j];
+      }
+    }
   }
+  __syncthreads();
   if (tid == 0 && written != b) atomicOr(a.status, 8);
 
   // --- H2O: the slot the next append replaces ---
@@ -229,24 +229,19 @@ __global__ void __launch_bounds__(kSelThreads) evict_kernel(EvictArgs a) {
   }
 }
 
-template <int kChunkBytes, int kStages>
-static cudaError_t launch_evict_cfg(const EvictArgs& a, cudaStream_t s) {
-  constexpr int kMaxChunkRows = kChunkBytes / (2 * 128);
-  const size_t words = ((size_t)a.max_cap + 31) / 32;
-  const size_t smem = (size_t)kStages * kChunkBytes + (size_t)kStages * kMaxChunkRows * 8 + words * 8;
-  constexpr size_t kMaxSmem = 200 * 1024;
-  if (smem > kMaxSmem) return cudaErrorInvalidValue;  // caches beyond ~1.4 M slots per unit
-  static PerDevice set_up;
-  const cudaError_t e = allow_smem(set_up, kMaxSmem, evict_kernel<kChunkBytes, kStages>);
-  if (e != cudaSuccess) return e;
-  evict_kernel<kChunkBytes, kStages><<<dim3(a.n_unit, a.n_layers), kSelThreads, smem, s>>>(a);
-  return cudaGetLastError();
-}
-
 cudaError_t launch_evict(const EvictArgs& a, cudaStream_t s) {
   if (a.row_bytes / 16 > kMaxVecPerRow || a.row_bytes < 128 || (a.row_bytes & (a.row_bytes - 1)))
     return cudaErrorInvalidValue;
-  return launch_evict_cfg<32 * 1024, 1>(a, s);
+  constexpr int kChunkBytes = 32 * 1024, kMaxChunkRows = kChunkBytes / (2 * 128);
+  const size_t words = ((size_t)a.max_cap + 31) / 32;
+  const size_t smem = (size_t)kChunkBytes + (size_t)kMaxChunkRows * 16 + words * 8;
+  constexpr size_t kMaxSmem = 201 * 1024;
+  if (smem > kMaxSmem) return cudaErrorInvalidValue;  // caches of more than 684,000 slots per unit
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, kMaxSmem, evict_kernel<kChunkBytes>);
+  if (e != cudaSuccess) return e;
+  evict_kernel<kChunkBytes><<<dim3(a.n_unit, a.n_layers), kSelThreads, smem, s>>>(a);
+  return cudaGetLastError();
 }
 
 }  // namespace sq

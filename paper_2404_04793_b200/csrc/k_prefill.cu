@@ -295,6 +295,58 @@ cudaError_t launch_prefill_scores(const ScoreArgs& a, int dtype, int* status, cu
 }
 
 // ---------------------------------------------------------------------------------------
+// Copies of kept prompt rows of K and V into the unit's slots (16-byte vectors).
+// Bound by HBM (a kept row is read and written once).  Each thread moves 16-byte pieces of K and V of
+// several slots, all loads before the first store.  Measured, 256 units of 409 rows of 256 bytes on average
+// per layer (107 MB read + written): 20.1 us with one piece of K and V per thread, 18 with this.
+// ---------------------------------------------------------------------------------------
+__host__ __device__ constexpr int copy_slots(int nt) { return nt / 4; }  // slots per CTA of nt threads
+
+// The slots s0 .. s0 + copy_slots(NT) - 1 of a unit; pos_of(j): the prompt position of slot s0 + j, -1 past the last.
+// ug: unit of the batch (sequence, KV head), unit: its index within the descriptor.
+template <int ROW_BYTES, int NT, class Pos>
+__device__ __forceinline__ void copy_rows(const GatherArgs& a, const LayerDesc& ld, int ug, int unit, int s0, Pos pos_of) {
+  constexpr int VPR = ROW_BYTES / 16;            // 16-byte pieces per row
+  constexpr int N = copy_slots(NT) * VPR / NT;   // pieces of K (and of V) per thread
+  constexpr int B = N < 4 ? N : 4;               // of them in flight
+  const uint4* ksrc = reinterpret_cast<const uint4*>(a.k_prompt) + (size_t)ug * a.prompt * VPR;
+  const uint4* vsrc = reinterpret_cast<const uint4*>(a.v_prompt) + (size_t)ug * a.prompt * VPR;
+  uint4* kdst = reinterpret_cast<uint4*>(a.pool + ld.k_off) + ((size_t)unit * ld.cap + s0) * VPR;
+  uint4* vdst = reinterpret_cast<uint4*>(a.pool + ld.v_off) + ((size_t)unit * ld.cap + s0) * VPR;
+#pragma unroll
+  for (int n0 = 0; n0 < N; n0 += B) {
+    uint4 kv[B], vv[B];
+    int p[B];
+#pragma unroll
+    for (int n = 0; n < B; ++n) {
+      const int idx = threadIdx.x + (n0 + n) * NT;
+      p[n] = pos_of(idx / VPR);
+      if (p[n] >= 0) {
+        kv[n] = ld_stream(ksrc + (size_t)p[n] * VPR + idx % VPR);
+        vv[n] = ld_stream(vsrc + (size_t)p[n] * VPR + idx % VPR);
+      }
+    }
+#pragma unroll
+    for (int n = 0; n < B; ++n) {
+      const int idx = threadIdx.x + (n0 + n) * NT;
+      if (p[n] >= 0) {
+        kdst[idx] = kv[n];
+        vdst[idx] = vv[n];
+      }
+    }
+  }
+}
+
+// The slots of an H2O cache whose position needs no selection: the recent window behind the heavy slots, or the whole prompt
+// where the budget holds it.  Slot s of them has position s + prompt - min(prompt, b).
+struct FixedSlots {
+  int begin, end;
+};
+__host__ __device__ inline FixedSlots fixed_slots(int prompt, int b, int b_heavy) {
+  return prompt > b ? FixedSlots{b_heavy, b} : FixedSlots{0, prompt};
+}
+
+// ---------------------------------------------------------------------------------------
 // C_seq over the prompt for H2O (one block per unit): keeps the b_recent highest positions
 // and, of the others, the b_heavy with the largest score (equal scores: lower position).
 // Writes the kept positions, ascending, and their scores to the layer's tables.
@@ -364,20 +416,32 @@ __global__ void __launch_bounds__(kSelThreads) select_prompt_kernel(const float*
 // cache's first victim come out of the same registers.
 // Measured, us per layer of 128 units, 4096 tokens (16 sequences, 8 KV heads): 17.8 with the histogram
 // form and its victim launch, about 5 with this one (one sq_evict pass over 32 layers: 2275 -> 1930).
-template <int NT, int KPT>
-__global__ void __launch_bounds__(NT) select_prompt_regs_kernel(const float* __restrict__ acc_prompt, int P,
-                                                                const LayerDesc* __restrict__ descs, int units_per_desc,
-                                                                char* pool) {
+// The CTAs behind one per unit copy the rows of the slots that need no selection (with the default split of a budget half
+// of them) meanwhile: the selection is a chain of block-wide steps on one CTA per unit, 12 us in which HBM idled.
+// Measured, us per layer, selection and copy one after the other / this, 16 sequences of 4096, 8 KV heads of 128: 1423 rows kept
+// 45 / 36, 286 rows 21 / 20; 33 of 8191, one head of 64, 7000 rows 43 / 35.
+template <int NT, int KPT, int ROW_BYTES>
+__global__ void __launch_bounds__(NT) select_prompt_regs_kernel(const GatherArgs a) {
   constexpr int NW = NT / 32;
+  const LayerDesc* descs = a.descs;
+  const int P = a.prompt, units_per_desc = a.units_per_desc;
+  char* pool = a.pool;
   __shared__ unsigned s_cnt[2][NW];
   __shared__ int s_off[KPT * NW];
   __shared__ unsigned long long s_best[NW];
   __shared__ int s_slot[NW];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   grid_wait();
-  const LayerDesc ld = descs[blockIdx.x / units_per_desc];
-  const int unit = blockIdx.x % units_per_desc;
-  const float* acc = acc_prompt + (size_t)blockIdx.x * P;
+  const int ug = blockIdx.x % a.n_unit;
+  const LayerDesc ld = descs[ug / units_per_desc];
+  const int unit = ug % units_per_desc;
+  if (blockIdx.x >= a.n_unit) {
+    const FixedSlots f = fixed_slots(P, ld.b, ld.b_heavy);
+    const int s0 = f.begin + ((int)blockIdx.x / a.n_unit - 1) * copy_slots(NT), shift = P - min(P, ld.b);
+    if (s0 < f.end) copy_rows<ROW_BYTES, NT>(a, ld, ug, unit, s0, [&](int j) { return s0 + j < f.end ? s0 + j + shift : -1; });
+    return;
+  }
+  const float* acc = a.scores + (size_t)ug * P;
   int* pos_out = reinterpret_cast<int*>(pool + ld.pos_off) + (size_t)unit * ld.cap;
   float* acc_out = reinterpret_cast<float*>(pool + ld.acc_off) + (size_t)unit * ld.cap;
   const bool drop = P > ld.b;
@@ -553,49 +617,22 @@ __global__ void __launch_bounds__(kSelThreads) pick_victim_kernel(char* pool, co
   if (threadIdx.x == 0) reinterpret_cast<int*>(pool + ld.victim_off)[unit] = slot;
 }
 
-// Selection over the prompt and the first victim of the caches it fills.  The register form covers
-// prompts of up to 16384 tokens; its block is sized by the prompt, so that short prompts of many units
-// do not start warps that hold nothing.
-cudaError_t launch_select_prompt(const float* acc_prompt, int n_unit, int prompt, const LayerDesc* descs,
-                                 int units_per_desc, bool any_full, char* pool, cudaStream_t s) {
-  if (prompt <= 1024)
-    return launch_chained(select_prompt_regs_kernel<256, 4>, n_unit, 256, 0, s, acc_prompt, prompt, descs, units_per_desc, pool);
-  if (prompt <= 4096)
-    return launch_chained(select_prompt_regs_kernel<512, 8>, n_unit, 512, 0, s, acc_prompt, prompt, descs, units_per_desc, pool);
-  if (prompt <= 16384)
-    return launch_chained(select_prompt_regs_kernel<1024, 16>, n_unit, 1024, 0, s, acc_prompt, prompt, descs, units_per_desc, pool);
-  select_prompt_kernel<<<n_unit, kSelThreads, 0, s>>>(acc_prompt, prompt, descs, units_per_desc, pool);
-  if (any_full) pick_victim_kernel<<<n_unit, kSelThreads, 0, s>>>(pool, descs, units_per_desc, prompt, prompt);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------------------------------
-// Gather: copies the kept prompt rows of K and V into the unit's slots (16-byte vectors) and, but for
-// H2O, fills the position table.  Sliding Window / StreamingLLM compute the
-// kept position of a slot in closed form; H2O reads it from the table the selection wrote.
-// ---------------------------------------------------------------------------------------
-// Bound by HBM (a kept row is read and written once).  Each thread moves 16-byte pieces of K and V of
-// several slots, all loads before the first store.  Measured, 256 units of 409 rows of 256 bytes on average
-// per layer (107 MB read + written): 20.1 us with one piece of K and V per thread, 18 with this.
-constexpr int kGatherSlots = 64;
-
+// The rows of the slots [0, n) of a unit.  Sliding Window / StreamingLLM: all, the kept position of a slot in closed form, which
+// also goes to the position table; H2O: those whose position the selection wrote there, with `heavy` only the heavy ones.
 template <int ROW_BYTES>
-__global__ void __launch_bounds__(256) gather_kernel(GatherArgs a) {
-  constexpr int VPR = ROW_BYTES / 16;                         // 16-byte pieces per row
-  constexpr int N = kGatherSlots * VPR / 256;                 // pieces of K (and of V) per thread
-  constexpr int B = N < 4 ? N : 4;                            // of them in flight
-  __shared__ int s_pos[kGatherSlots];
-  const int ug = blockIdx.x, s0 = blockIdx.y * kGatherSlots;  // ug: unit of the batch (sequence, KV head)
+__global__ void __launch_bounds__(256) gather_kernel(const GatherArgs a, bool heavy) {
+  __shared__ int s_pos[copy_slots(256)];
+  const int ug = blockIdx.x, s0 = blockIdx.y * copy_slots(256);
   grid_wait();
   const LayerDesc ld = a.descs[ug / a.units_per_desc];
-  const int unit = ug % a.units_per_desc;                     // its index within the descriptor
-  const int n_keep = min(a.prompt, ld.b);
-  if (s0 >= n_keep) return;                                   // the grid covers the longest descriptor
+  const int unit = ug % a.units_per_desc;
+  const int n = heavy ? fixed_slots(a.prompt, ld.b, ld.b_heavy).begin : min(a.prompt, ld.b);
+  if (s0 >= n) return;                                   // the grid covers the longest descriptor
   int* pos_tab = reinterpret_cast<int*>(a.pool + ld.pos_off) + (size_t)unit * ld.cap;
-  if (threadIdx.x < kGatherSlots) {
+  if (threadIdx.x < copy_slots(256)) {
     const int slot = s0 + threadIdx.x;
     int p = -1;
-    if (slot < n_keep) {
+    if (slot < n) {
       if (a.policy == SQ_POLICY_H2O) {
         p = pos_tab[slot];
       } else {
@@ -606,41 +643,44 @@ __global__ void __launch_bounds__(256) gather_kernel(GatherArgs a) {
     s_pos[threadIdx.x] = p;
   }
   __syncthreads();
-  const uint4* ksrc = reinterpret_cast<const uint4*>(a.k_prompt) + (size_t)ug * a.prompt * VPR;
-  const uint4* vsrc = reinterpret_cast<const uint4*>(a.v_prompt) + (size_t)ug * a.prompt * VPR;
-  uint4* kdst = reinterpret_cast<uint4*>(a.pool + ld.k_off) + ((size_t)unit * ld.cap + s0) * VPR;
-  uint4* vdst = reinterpret_cast<uint4*>(a.pool + ld.v_off) + ((size_t)unit * ld.cap + s0) * VPR;
-#pragma unroll
-  for (int n0 = 0; n0 < N; n0 += B) {
-    uint4 kv[B], vv[B];
-    int p[B];
-#pragma unroll
-    for (int n = 0; n < B; ++n) {
-      const int idx = threadIdx.x + (n0 + n) * 256;
-      p[n] = s_pos[idx / VPR];
-      if (p[n] >= 0) {
-        kv[n] = ld_stream(ksrc + (size_t)p[n] * VPR + idx % VPR);
-        vv[n] = ld_stream(vsrc + (size_t)p[n] * VPR + idx % VPR);
-      }
-    }
-#pragma unroll
-    for (int n = 0; n < B; ++n) {
-      const int idx = threadIdx.x + (n0 + n) * 256;
-      if (p[n] >= 0) {
-        kdst[idx] = kv[n];
-        vdst[idx] = vv[n];
-      }
-    }
-  }
+  copy_rows<ROW_BYTES, 256>(a, ld, ug, unit, s0, [&](int j) { return s_pos[j]; });
 }
 
-cudaError_t launch_gather(const GatherArgs& a, int dtype, cudaStream_t s) {
-  if (a.max_keep <= 0) return cudaSuccess;
+template <int ROW_BYTES>
+static cudaError_t launch_gather(const GatherArgs& a, int max_slots, bool heavy, cudaStream_t s) {
+  if (max_slots <= 0) return cudaSuccess;
+  return launch_chained(gather_kernel<ROW_BYTES>, dim3(a.n_unit, (max_slots + copy_slots(256) - 1) / copy_slots(256)), 256, 0, s, a, heavy);
+}
+
+template <int NT, int KPT, int ROW_BYTES>
+static cudaError_t launch_select(const GatherArgs& a, cudaStream_t s) {
+  const long long chunks = (a.max_fixed + copy_slots(NT) - 1) / copy_slots(NT);
+  return launch_chained(select_prompt_regs_kernel<NT, KPT, ROW_BYTES>, (unsigned)(a.n_unit * (1 + chunks)), NT, 0, s, a);
+}
+
+// H2O: selection over the prompt and the first victim of the caches it fills.  The register form covers
+// prompts of up to 16384 tokens; its block is sized by the prompt, so that short prompts of many units
+// do not start warps that hold nothing.
+template <int ROW_BYTES>
+static cudaError_t launch_fill(const GatherArgs& a, bool any_full, cudaStream_t s) {
+  if (a.policy != SQ_POLICY_H2O) return launch_gather<ROW_BYTES>(a, a.max_keep, false, s);
+  if (a.prompt > 16384) {
+    select_prompt_kernel<<<a.n_unit, kSelThreads, 0, s>>>(a.scores, a.prompt, a.descs, a.units_per_desc, a.pool);
+    if (any_full) pick_victim_kernel<<<a.n_unit, kSelThreads, 0, s>>>(a.pool, a.descs, a.units_per_desc, a.prompt, a.prompt);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e : launch_gather<ROW_BYTES>(a, a.max_keep, false, s);
+  }
+  const cudaError_t e = a.prompt <= 1024   ? launch_select<256, 4, ROW_BYTES>(a, s)
+                        : a.prompt <= 4096 ? launch_select<512, 8, ROW_BYTES>(a, s)
+                                           : launch_select<1024, 16, ROW_BYTES>(a, s);
+  return e != cudaSuccess ? e : launch_gather<ROW_BYTES>(a, a.max_heavy, true, s);
+}
+
+cudaError_t launch_fill_cache(const GatherArgs& a, int dtype, bool any_full, cudaStream_t s) {
   const int row_bytes = a.head_dim * (dtype == SQ_F32 ? 4 : 2);
-  const dim3 grid(a.n_unit, (a.max_keep + kGatherSlots - 1) / kGatherSlots);
-  if (row_bytes == 128) return launch_chained(gather_kernel<128>, grid, 256, 0, s, a);
-  if (row_bytes == 256) return launch_chained(gather_kernel<256>, grid, 256, 0, s, a);
-  if (row_bytes == 512) return launch_chained(gather_kernel<512>, grid, 256, 0, s, a);
+  if (row_bytes == 128) return launch_fill<128>(a, any_full, s);
+  if (row_bytes == 256) return launch_fill<256>(a, any_full, s);
+  if (row_bytes == 512) return launch_fill<512>(a, any_full, s);
   return cudaErrorInvalidValue;
 }
 

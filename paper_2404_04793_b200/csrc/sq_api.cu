@@ -569,17 +569,19 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
       acc = s.acc_prompt;
     }
   }
-  // selection (with the first victim) and gather: one launch each over all descriptors of the layer
+  // selection (with the first victim) and copies, over all descriptors of the layer
   const LayerDesc* descs_dev = ws_ptr<LayerDesc>(c, c->wl.layers) + layer * c->n_grp;
   const int n_unit = c->batch * c->cfg.n_kv_head;
-  int max_keep = 0;
+  int max_keep = 0, max_fixed = 0, max_heavy = 0;
   bool any_full = false;
   for (int g = 0; g < c->n_grp; ++g) {
     const LayerDesc& ld = c->hs.layers[layer * c->n_grp + g];
     max_keep = std::max(max_keep, std::min(P, ld.b));
     any_full |= P >= ld.b;
+    const int heavy = P > ld.b ? ld.b_heavy : 0;
+    max_heavy = std::max(max_heavy, heavy);
+    max_fixed = std::max(max_fixed, std::min(P, ld.b) - heavy);
   }
-  if (h2o) SQ_CUDA(c, launch_select_prompt(acc, n_unit, P, descs_dev, U, any_full, c->pool, st));
   GatherArgs ga;
   ga.k_prompt = k_prompt;
   ga.v_prompt = v_prompt;
@@ -591,7 +593,10 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
   ga.max_keep = max_keep;
   ga.policy = c->cfg.policy;
   ga.head_dim = c->cfg.head_dim;
-  SQ_CUDA(c, launch_gather(ga, c->cfg.dtype, st));
+  ga.scores = acc;
+  ga.max_fixed = max_fixed;
+  ga.max_heavy = max_heavy;
+  SQ_CUDA(c, launch_fill_cache(ga, c->cfg.dtype, any_full, st));
   c->n_tok[layer] = P;
   c->prefilled[layer] = true;
   return SQ_OK;

@@ -64,6 +64,8 @@ struct GatherArgs {  // prompt rows -> cache slots of one layer (all its descrip
   const LayerDesc* descs;   // the layer's descriptors (device); unit u belongs to descs[u / units_per_desc]
   int units_per_desc;
   int n_unit, prompt, max_keep, policy, head_dim;
+  const float* scores;      // H2O: [n_unit][prompt]
+  int max_fixed, max_heavy; // H2O: most slots of a descriptor that need no selection, and that do
 };
 
 struct ScoreArgs {  // H2O prompt scores of one layer
@@ -162,12 +164,10 @@ inline cudaError_t launch_chained(void (*kern)(P...), dim3 grid, dim3 block, siz
 // Launchers: each returns the cudaError_t of its launches.
 cudaError_t launch_importance(const ImportanceArgs& a, int dtype, int n_sm, cudaStream_t s);
 cudaError_t launch_allocate(const AllocateArgs& a, cudaStream_t s);
-cudaError_t launch_gather(const GatherArgs& a, int dtype, cudaStream_t s);
+cudaError_t launch_fill_cache(const GatherArgs& a, int dtype, bool any_full, cudaStream_t s);
 cudaError_t launch_prefill_scores(const ScoreArgs& a, int dtype, int* status, cudaStream_t s);
 cudaError_t launch_prefill_scores_alu(const ScoreArgs& a, int dtype, cudaStream_t s);
 cudaError_t launch_prefill_scores_tc(const ScoreArgs& a, int* status, cudaStream_t s);
-cudaError_t launch_select_prompt(const float* acc_prompt, int n_unit, int prompt, const LayerDesc* descs,
-                                 int units_per_desc, bool any_full, char* pool, cudaStream_t s);
 // Attention kernel of a launch over n_desc descriptors of n_unit units, the longest of max_len slots.
 enum class DecodeKernel { kTcgen05, kMma, kPipe };  // wide groups; mma.sync; fp32 pipes
 DecodeKernel decode_kernel_for(int dtype, int head_dim, int group, int n_desc, int n_unit, int max_len, bool h2o);
