@@ -45,7 +45,7 @@ def test_prompt_scores_cut_into_pieces(dtype, head_dim, hq, hkv, batch, prompt):
 
 # A row's reference is its maximum over the first keys and stays unless a row rises 2^32 above it: some rows do, by overflowing
 # amounts too, some rise less, some not at all; both tile widths, both halves of a wide tile, the last tile ragged
-@pytest.mark.parametrize("head_dim,hq", [(64, 3), (128, 2)])
+@pytest.mark.parametrize("head_dim,hq", [(64, 3), (64, 60), (128, 2)])   # (60 heads: enough CTAs for the narrow tiles)
 @pytest.mark.parametrize("prompt", [200, 700])
 def test_prompt_scores_of_rising_rows(head_dim, hq, prompt):
     w = workload("rising", 9150 + prompt, head_dim=head_dim, n_q_head=hq, n_kv_head=1, batch=3, prompt=prompt, heavy_mode="none")
