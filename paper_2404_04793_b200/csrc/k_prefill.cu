@@ -337,6 +337,13 @@ __device__ __forceinline__ void copy_rows(const GatherArgs& a, const LayerDesc& 
   }
 }
 
+// Where a unit's heavy rows are few, the CTA that selects them copies them too: up to 100 KB of K and V, in less time than a launch
+// takes to start, and no launch follows.  us per layer, copied by a launch / here: fp32, 1 sequence of 256, two heads, 102 kept
+// 11.4 / 7.1; 8 KV heads of 128, 16 sequences, 286 kept 20.0 / 17.2, 180: 18.0 / 14.7, 4 sequences, 140: 12.2 / 10.4; 32 KV heads, 8
+// sequences, 240 kept 21.7 / 17.3; one head of 64, 33 sequences, 400 kept 12.7 / 11.5.
+constexpr int kOwnSlots = 256;
+constexpr int kOwnBytes = 100 * 1024;
+
 // The slots of an H2O cache whose position needs no selection: the recent window behind the heavy slots, or the whole prompt
 // where the budget holds it.  Slot s of them has position s + prompt - min(prompt, b).
 struct FixedSlots {
@@ -430,6 +437,7 @@ __global__ void __launch_bounds__(NT) select_prompt_regs_kernel(const GatherArgs
   __shared__ int s_off[KPT * NW];
   __shared__ unsigned long long s_best[NW];
   __shared__ int s_slot[NW];
+  __shared__ int s_heavy[kOwnSlots];  // own_copy: the heavy slots' positions
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   grid_wait();
   const int ug = blockIdx.x % a.n_unit;
@@ -556,6 +564,7 @@ __global__ void __launch_bounds__(NT) select_prompt_regs_kernel(const GatherArgs
     if (keep[j] && rank[j] < ld.b) {
       pos_out[rank[j]] = i;
       acc_out[rank[j]] = val[j];
+      if (a.own_copy && rank[j] < kOwnSlots) s_heavy[rank[j]] = i;
       if (i <= last_old) {
         const unsigned long long r = victim_rank(val[j], i);
         if (r < best) {
@@ -565,7 +574,7 @@ __global__ void __launch_bounds__(NT) select_prompt_regs_kernel(const GatherArgs
       }
     }
   }
-  if (!full) return;  // the cache still grows: the next token takes a fresh slot
+  if (!full) return;  // the cache still grows: the next token takes a fresh slot (and nothing was selected)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const unsigned long long r2 = __shfl_xor_sync(0xffffffffu, best, o);
@@ -580,6 +589,11 @@ __global__ void __launch_bounds__(NT) select_prompt_regs_kernel(const GatherArgs
     s_slot[warp] = best_slot;
   }
   __syncthreads();
+  if (a.own_copy) {
+    const int n = drop ? ld.b_heavy : 0;
+    for (int s0 = 0; s0 < n; s0 += copy_slots(NT))
+      copy_rows<ROW_BYTES, NT>(a, ld, ug, unit, s0, [&](int j) { return s0 + j < n ? s_heavy[s0 + j] : -1; });
+  }
   if (tid == 0) {
     for (int w = 1; w < NW; ++w)
       if (s_best[w] < best) {
@@ -670,10 +684,12 @@ static cudaError_t launch_fill(const GatherArgs& a, bool any_full, cudaStream_t 
     const cudaError_t e = cudaGetLastError();
     return e != cudaSuccess ? e : launch_gather<ROW_BYTES>(a, a.max_keep, false, s);
   }
-  const cudaError_t e = a.prompt <= 1024   ? launch_select<256, 4, ROW_BYTES>(a, s)
-                        : a.prompt <= 4096 ? launch_select<512, 8, ROW_BYTES>(a, s)
-                                           : launch_select<1024, 16, ROW_BYTES>(a, s);
-  return e != cudaSuccess ? e : launch_gather<ROW_BYTES>(a, a.max_heavy, true, s);
+  GatherArgs b = a;
+  b.own_copy = a.max_heavy <= kOwnSlots && a.max_heavy * 2 * ROW_BYTES <= kOwnBytes;
+  const cudaError_t e = b.prompt <= 1024   ? launch_select<256, 4, ROW_BYTES>(b, s)
+                        : b.prompt <= 4096 ? launch_select<512, 8, ROW_BYTES>(b, s)
+                                           : launch_select<1024, 16, ROW_BYTES>(b, s);
+  return e != cudaSuccess || b.own_copy ? e : launch_gather<ROW_BYTES>(b, b.max_heavy, true, s);
 }
 
 cudaError_t launch_fill_cache(const GatherArgs& a, int dtype, bool any_full, cudaStream_t s) {

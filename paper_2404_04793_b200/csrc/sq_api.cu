@@ -596,6 +596,7 @@ int sq_prefill_compress(sq_ctx* c, int32_t layer, const void* k_prompt, const vo
   ga.scores = acc;
   ga.max_fixed = max_fixed;
   ga.max_heavy = max_heavy;
+  ga.own_copy = false;
   SQ_CUDA(c, launch_fill_cache(ga, c->cfg.dtype, any_full, st));
   c->n_tok[layer] = P;
   c->prefilled[layer] = true;

@@ -66,6 +66,7 @@ struct GatherArgs {  // prompt rows -> cache slots of one layer (all its descrip
   int n_unit, prompt, max_keep, policy, head_dim;
   const float* scores;      // H2O: [n_unit][prompt]
   int max_fixed, max_heavy; // H2O: most slots of a descriptor that need no selection, and that do
+  bool own_copy;            // H2O: the selecting CTA copies the heavy rows of its unit
 };
 
 struct ScoreArgs {  // H2O prompt scores of one layer
