@@ -702,8 +702,9 @@ static cudaError_t launch_tc_cluster(const DecodeArgs& a, const int* desc_tiles,
     return r == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
   });
   if (e != cudaSuccess) return e;
+  static ClusterCount own;  // (a device that holds no cluster of that size at all)
   const int n = cluster_pieces(a, desc_tiles, smem);
-  if (n == 0) return cudaErrorNotSupported;
+  if (n == 0 || own.active(reinterpret_cast<const void*>(kern), n, 192, smem) == 0) return cudaErrorNotSupported;
   return launch_chained_cluster(kern, n, a.n_layer_total * a.n_unit * n, 192, smem, s, tq, tk, tv, static_cast<const DecodeArgsBase&>(a));
 }
 

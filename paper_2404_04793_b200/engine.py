@@ -150,15 +150,15 @@ class Job:
 
     def kernel_launches_per_pass(self, inp: ResidentInputs, per_layer_decode=None) -> int:
         """Kernels of the library launched by one pass: importance per layer and chunk feed, one
-        allocator, prefill kernels per layer, decode kernels per step."""
+        allocator, prefill kernels per layer, decode kernels per step.  At least: H2O copies many heavy rows by a
+        launch of its own, and some of its decode steps take two."""
         w = self.w
         per_layer = self.per_layer_decode if per_layer_decode is None else per_layer_decode
         h2o = w.policy == synth.H2O
-        # H2O: two scoring sweeps (unless stand-in scores are given), selection, gather
-        per_layer_prefill = ((0 if inp.acc is not None else 2) + 1 + 1) if h2o else 1
+        # H2O: two scoring sweeps (unless stand-in scores are given), selection with copies
+        per_layer_prefill = ((0 if inp.acc is not None else 2) + 1) if h2o else 1
         groups = w.n_layer if per_layer else 1
-        per_step = groups * (2 if h2o and w.group > 32 else 1)   # at least: H2O launches of many units take two as well
-        return w.n_layer * inp.hidden_repeat + 1 + w.n_layer * per_layer_prefill + w.steps * per_step
+        return w.n_layer * inp.hidden_repeat + 1 + w.n_layer * per_layer_prefill + w.steps * groups
 
     # ---- the same pass fed from page-locked host memory ----
     def run_from_host(self, host: ResidentInputs, out_host: torch.Tensor):
