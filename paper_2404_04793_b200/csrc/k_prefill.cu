@@ -246,6 +246,136 @@ __global__ void __launch_bounds__(4 * TQ) prefill_col_sum_kernel(ScoreArgs a, fl
   }
 }
 
+// Short prompts in one launch: a CTA has a query tile of one head and keeps its logits of all keys in shared memory, so
+// that once the row sums are known it adds up its rows' weights per key.  The sums of a KV head's (head, query tile)
+// pairs go to scratch, pair by pair; a key tile's last pair to finish adds them in order (no pair waits).  Against the
+// two sweeps that is one launch and one product less.  us per layer of scores, selection and copies, fp32, two sweeps / this:
+// 2 / 2 heads of 64: 1 sequence of 128 tokens 17.2 / 13.3, 256: 23.4 / 19.7, 30 of 256: 59.4 / 36.9; 32 / 32 of 128, 1 of 256: 70.1 /
+// 43.8, 500: 165 / 133; 16 / 4 of 128, 6 of 150: 69.6 / 54.2; 8 / 8 of 128, 2 of 600: 144 / 113.
+// The chain of a CTA (all keys of its rows) and of the last pair grow with the prompt: of more than 20 pairs per KV head
+// launches of few CTAs are no faster (1 sequence of 700, 2 / 2 heads of 64, 45.8 / 46.5).
+constexpr int kRowsPairs = 20;
+constexpr size_t kRowsSmem = 160 * 1024;
+template <int D>
+constexpr size_t rows_smem(int n_kt) {
+  return score_smem<D, 32>() + (size_t)32 * (n_kt * TK + 4) * 4;
+}
+
+template <typename T, int D>
+__global__ void __launch_bounds__(128) prefill_rows_kernel(ScoreArgs a, float scale_log2) {
+  constexpr int TQ = 32, NT = 4 * TQ;
+  extern __shared__ __align__(16) float sm[];
+  __shared__ float s_lse[TQ];
+  __shared__ int s_last[NT];
+  float* qs = sm;
+  float* ks = qs + D * (TQ + 4);
+  float* logit = ks + D * (TK + 4);  // [TQ][row_len]
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int P = a.prompt, n_qt = (P + TQ - 1) / TQ, n_kt_all = (P + TK - 1) / TK, row_len = n_kt_all * TK + 4;
+  const int qt = n_qt - 1 - blockIdx.x, hq = blockIdx.y, bi = blockIdx.z;  // longest rows first
+  const int g = a.n_q_head / a.n_kv_head, hk = hq / g;
+  const T* qbase = reinterpret_cast<const T*>(a.q) + ((size_t)bi * a.n_q_head + hq) * P * D;
+  const T* kbase = reinterpret_cast<const T*>(a.k) + ((size_t)bi * a.n_kv_head + hk) * P * D;
+  const int q0 = qt * TQ, n_kt = (min(q0 + TQ, P) + TK - 1) / TK;
+  grid_wait();
+  {
+    TileLoad<T, D, TQ, NT> ql;
+    ql.fetch(qbase, q0, P);
+    ql.store(qs);
+  }
+  TileLoad<T, D, TK, NT> kl;
+  kl.fetch(kbase, 0, P);
+  float m[4], l[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    m[r] = -INFINITY;
+    l[r] = 0.f;
+  }
+  for (int kt = 0; kt < n_kt; ++kt) {
+    const int k0 = kt * TK;
+    __syncthreads();
+    kl.store(ks);
+    __syncthreads();
+    if (kt + 1 < n_kt) kl.fetch(kbase, k0 + TK, P);
+    float s[4][4];
+    score_tile<D, TQ>(qs, ks, s);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int qr = q0 + 4 * ty + r;
+      float tmax = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        const int kr = k0 + 4 * tx + c;
+        s[r][c] = (kr <= qr && qr < P) ? s[r][c] * scale_log2 : -INFINITY;
+        tmax = fmaxf(tmax, s[r][c]);
+      }
+      *reinterpret_cast<float4*>(logit + (4 * ty + r) * row_len + k0 + 4 * tx) = make_float4(s[r][0], s[r][1], s[r][2], s[r][3]);
+      const float m_new = fmaxf(m[r], tmax);
+      if (m_new > -INFINITY) {
+        float sum = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) sum += exp2f(s[r][c] - m_new);
+        l[r] = l[r] * exp2f(m[r] - m_new) + sum;
+        m[r] = m_new;
+      }
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    float mm = m[r];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) mm = fmaxf(mm, __shfl_xor_sync(0xffffffffu, mm, o));
+    float ll = (m[r] > -INFINITY) ? l[r] * exp2f(m[r] - mm) : 0.f;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) ll += __shfl_xor_sync(0xffffffffu, ll, o);
+    if (tx == 0) s_lse[4 * ty + r] = q0 + 4 * ty + r < P ? mm + log2f(ll) : INFINITY;  // a query past the end attends to nothing
+  }
+  __syncthreads();
+  const size_t unit = (size_t)bi * a.n_kv_head + hk, stride = (size_t)a.batch * a.n_kv_head * P;
+  const int pair = (hq - hk * g) * n_qt + qt;
+  float* mine = a.partial + pair * stride + unit * P;
+  const int n_key = min(n_kt * TK, P);
+  for (int key = tid; key < n_key; key += NT) {
+    float sum = 0.f;
+#pragma unroll 8
+    for (int r = 0; r < TQ; ++r) sum += exp2f(logit[r * row_len + key] - s_lse[r]);  // (-inf before the key: 0)
+    mine[key] = sum;
+  }
+  // the pair's key tiles: a ticket each, query tiles from kt * TK / TQ on see tile kt
+  __threadfence();
+  __syncthreads();
+  if (tid < n_kt) {
+    int* ticket = a.tickets + unit * n_kt_all + tid;
+    s_last[tid] = atomicAdd(ticket, 1) == g * (n_qt - tid * TK / TQ) - 1;
+    if (s_last[tid]) *ticket = 0;
+  }
+  __syncthreads();
+  for (int key = tid; key < n_key; key += NT) {
+    if (!s_last[key / TK]) continue;
+    __threadfence();
+    float sum = 0.f;
+    for (int h = 0; h < g; ++h)
+#pragma unroll 8
+      for (int t = key / TK * TK / TQ; t < n_qt; ++t) sum += __ldcg(a.partial + (size_t)(h * n_qt + t) * stride + unit * P + key);
+    a.acc_prompt[unit * P + key] = sum;
+  }
+}
+
+template <typename T, int D>
+static cudaError_t launch_scores_rows(const ScoreArgs& a, cudaStream_t s) {
+  const int n_qt = (a.prompt + 31) / 32, n_kt = (a.prompt + TK - 1) / TK, g = a.n_q_head / a.n_kv_head;
+  const long long pairs = (long long)g * n_qt;
+  if (pairs > kRowsPairs) return cudaErrorNotSupported;
+  const size_t smem = rows_smem<D>(n_kt);
+  if (smem > kRowsSmem) return cudaErrorNotSupported;
+  if (pairs * a.batch * a.n_kv_head * a.prompt > (long long)a.partial_floats) return cudaErrorNotSupported;
+  auto kern = prefill_rows_kernel<T, D>;
+  static PerDevice set_up;
+  const cudaError_t e = allow_smem(set_up, kRowsSmem, kern);
+  if (e != cudaSuccess) return e;
+  return launch_chained(kern, dim3(n_qt, a.n_q_head, a.batch), 128, smem, s, a, 1.4426950408889634f / sqrtf((float)D));
+}
+
 template <typename T, int D, int TQ>
 static cudaError_t launch_scores_tq(const ScoreArgs& a, cudaStream_t s) {
   auto k1 = prefill_row_lse_kernel<T, D, TQ>;
@@ -271,6 +401,8 @@ static cudaError_t launch_scores_tq(const ScoreArgs& a, cudaStream_t s) {
 
 template <typename T, int D>
 static cudaError_t launch_scores_t(const ScoreArgs& a, cudaStream_t s) {
+  const cudaError_t e = launch_scores_rows<T, D>(a, s);
+  if (e != cudaErrorNotSupported) return e;
   // small problems: more and shorter CTAs
   const long long ctas = (long long)((a.prompt + 63) / 64) * a.n_q_head * a.batch;
   return ctas < 2LL * sm_count() ? launch_scores_tq<T, D, 32>(a, s) : launch_scores_tq<T, D, 64>(a, s);

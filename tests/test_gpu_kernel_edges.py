@@ -43,6 +43,15 @@ def test_prompt_scores_cut_into_pieces(dtype, head_dim, hq, hkv, batch, prompt):
     assert ctx.status() == 0
 
 
+# fp32 prompts that go in one launch, and just not: one query, edges of a query tile and of a key tile, the most (head, query
+# tile) pairs of a KV head with one head and with several, one more than that
+@pytest.mark.parametrize("head_dim,hq,hkv,batch,prompt", [
+    (64, 2, 2, 1, 1), (64, 2, 1, 3, 31), (128, 1, 1, 2, 32), (64, 6, 3, 2, 65), (128, 2, 2, 2, 127), (64, 5, 1, 2, 128),
+    (128, 5, 1, 1, 129), (64, 1, 1, 2, 640), (128, 2, 2, 1, 639), (64, 1, 1, 1, 641)])
+def test_prompt_scores_of_short_fp32_prompts(head_dim, hq, hkv, batch, prompt):
+    test_prompt_scores_cut_into_pieces(torch.float32, head_dim, hq, hkv, batch, prompt)
+
+
 # A row's reference is its maximum over the first keys and stays unless a row rises 2^32 above it: some rows do, by overflowing
 # amounts too, some rise less, some not at all; both tile widths, both halves of a wide tile, the last tile ragged
 @pytest.mark.parametrize("head_dim,hq", [(64, 3), (64, 60), (128, 2)])   # (60 heads: enough CTAs for the narrow tiles)
