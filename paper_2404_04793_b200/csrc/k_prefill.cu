@@ -306,10 +306,15 @@ __global__ void __launch_bounds__(128) prefill_rows_kernel(ScoreArgs a, float sc
 #pragma unroll
       for (int c = 0; c < 4; ++c) {
         const int kr = k0 + 4 * tx + c;
-        s[r][c] = (kr <= qr && qr < P) ? s[r][c] * scale_log2 : -INFINITY;
+        if (kr > qr || qr >= P) s[r][c] = -INFINITY;
+      }
+      // (unscaled: the scaling is rounded once, with the subtraction of the log-sum-exp)
+      *reinterpret_cast<float4*>(logit + (4 * ty + r) * row_len + k0 + 4 * tx) = make_float4(s[r][0], s[r][1], s[r][2], s[r][3]);
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        s[r][c] *= scale_log2;
         tmax = fmaxf(tmax, s[r][c]);
       }
-      *reinterpret_cast<float4*>(logit + (4 * ty + r) * row_len + k0 + 4 * tx) = make_float4(s[r][0], s[r][1], s[r][2], s[r][3]);
       const float m_new = fmaxf(m[r], tmax);
       if (m_new > -INFINITY) {
         float sum = 0.f;
@@ -336,10 +341,12 @@ __global__ void __launch_bounds__(128) prefill_rows_kernel(ScoreArgs a, float sc
   float* mine = a.partial + pair * stride + unit * P;
   const int n_key = min(n_kt * TK, P);
   for (int key = tid; key < n_key; key += NT) {
-    float sum = 0.f;
-#pragma unroll 8
-    for (int r = 0; r < TQ; ++r) sum += exp2f(logit[r * row_len + key] - s_lse[r]);  // (-inf before the key: 0)
-    mine[key] = sum;
+    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+    for (int r = 0; r < TQ; r += 4)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) sum[u] += exp2f(fmaf(logit[(r + u) * row_len + key], scale_log2, -s_lse[r + u]));  // (-inf before the key: 0)
+    mine[key] = (sum[0] + sum[1]) + (sum[2] + sum[3]);
   }
   // the pair's key tiles: a ticket each, query tiles from kt * TK / TQ on see tile kt
   __threadfence();
@@ -354,9 +361,12 @@ __global__ void __launch_bounds__(128) prefill_rows_kernel(ScoreArgs a, float sc
     if (!s_last[key / TK]) continue;
     __threadfence();
     float sum = 0.f;
-    for (int h = 0; h < g; ++h)
+    for (int h = 0; h < g; ++h) {
+      float part = 0.f;  // of the head
 #pragma unroll 8
-      for (int t = key / TK * TK / TQ; t < n_qt; ++t) sum += __ldcg(a.partial + (size_t)(h * n_qt + t) * stride + unit * P + key);
+      for (int t = key / TK * TK / TQ; t < n_qt; ++t) part += __ldcg(a.partial + (size_t)(h * n_qt + t) * stride + unit * P + key);
+      sum += part;
+    }
     a.acc_prompt[unit * P + key] = sum;
   }
 }
