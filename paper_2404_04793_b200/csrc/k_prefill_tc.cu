@@ -6,7 +6,7 @@
 // (M = 128, N = TN, K = head_dim, bf16 in, fp32 accumulators in tensor memory):
 //   sweep 1, CTA = (sequence, query head, 128 query rows): S = Q_tile K_tile^T for the key tiles
 //     up to the diagonal; a drain thread owns one TMEM lane = one query row and
-//     keeps its reference / sum -> row log-sum-exp.
+//     keeps its running maximum / sum -> row log-sum-exp.
 //   sweep 2, CTA = (sequence, KV head, 128 keys, some heads of the group): the operands swap,
 //     S^T = K_tile Q_tile^T for all query tiles from the diagonal down and the CTA's heads; thread t
 //     owns one key and adds exp2(s*scale - lse[row]) over the tile's columns -> the key's column sum,
@@ -20,8 +20,11 @@
 // What bounds it: the drain's exponentials and what they share a scheduler with.  Per element and warp a sweep takes 9
 // cycles, the exponential arithmetic alone 7 (special-function unit 6), the rest is waits for accumulators and
 // their loads; without the exponentials a sweep still takes 60 % of its time, without loads or products 98 %; at head_dim 128 the
-// board's power limit comes first (1.7 GHz).  us per layer of sweeps 1 / 2: 4 sequences of 4096, 32 / 8 heads of 128: 313 / 366
-// with a running maximum and two loads in flight, now 286 / 352; 2 of 5003, 71 / 1 heads of 64: 499 / 508, now 455 / 482.
+// board's power limit comes first (1.7 GHz).  us per layer of sweeps 1 / 2: 4 sequences of 4096, 32 / 8 heads of 128: 314 / 367
+// with two loads in flight and tiles of 128 columns only, now 305 / 363; 2 of 5003, 71 / 1 heads of 64: 499 / 507, now 482 / 483.
+// Built and taken back: in sweep 1 a row's maximum over its first tile as its reference throughout (298 and 457 us).  Rows that
+// rise above it then have their exponents formed at the size of the rise, 31 for a key of 2^1 after keys of 2^-30: such
+// a key's score was off by up to 1.3e-6, where under a running maximum roundings come to 3.8e-7 at most.
 // Built to parity and measured slower (sweeps 1 / 2, against 313 / 366 and 499 / 508): queries on the lanes in both sweeps, with
 // one register per key in sweep 2 (315 / 416 as one persistent CTA per SM with 128x256 tiles, 334 / 511 as two CTAs of nine
 // warps) or four queries and 16 keys per thread (356 and 515); no issuing warps, the last warp to empty a buffer issues
@@ -42,11 +45,9 @@ using namespace tc;
 // TN: columns of a tile (streamed rows), 64 or 128.  A CTA has a TMA warp, an MMA warp and TN / 16 drain warps: a warp
 // reaches only the 32 tensor-memory lanes of its quarter (warp index mod 4) and takes 64 of a tile's columns.  An SM's 16
 // drain warps are four CTAs of 64 columns, whose waits for an accumulator fall at different times, where shared memory
-// holds four (head_dim 64: 460 / 486 us against 491 / 486 with two of 128), else two of 128.
+// holds four (head_dim 64, 2 sequences of 5003, 71 / 1 heads: 992 us a layer against 998 with two of 128; 1136 CTAs 73 against 80), else
+// two of 128.
 constexpr int prefill_threads(int tn) { return 64 + 2 * tn; }
-// How far, in powers of two, a row may rise above its reference: its weights' arguments are then rounded no more coarsely than a
-// log-sum-exp of that size is when it is stored.
-constexpr float kMaxRise = 32.f, kMaxSum = 4294967296.f;
 
 // exp2 of a pair on the FMA pipe: x = n + f with n the nearest integer (the usual 1.5 * 2^23
 // addition), 2^f for |f| <= 1/2 from a degree-5 polynomial (fitted here by a Remez exchange on the
@@ -78,12 +79,15 @@ __device__ __forceinline__ unsigned long long ex2_pair_sfu(unsigned long long x2
   f32x2_split(x2, x0, x1);
   return f32x2(ex2(x0), ex2(x1));
 }
-// Of every eight pairs of score elements two take the FMA-pipe form, spread evenly.  With none the special-function
-// unit bounds the drain (16 exponentials per cycle and SM: 1024 cycles per 128 x 128 elements); an FMA-pipe pair costs 25 cycles of
-// a scheduler where the unit's takes 16.  Measured on B200, us per layer of sweep 1 / sweep 2 with 1, 2, 3 of eight: head_dim
-// 128 (4 sequences of 4096, 32 / 8 heads) 296 / 364, 289 / 360, 301 / 374; head_dim 64 (2 sequences of 5003, 71 / 1 heads) 480 / 501,
-// 460 / 485, 475 / 505.
-__device__ __forceinline__ constexpr bool on_fma(int pair) { return (pair & 3) == 3; }  // `pair` is a constant after unrolling
+// Of every eight pairs of score elements two take the FMA-pipe form, spread evenly, in sweep 1 at head_dim 128 one.  With none the
+// special-function unit bounds the drain (16 exponentials per cycle and SM: 1024 cycles per 128 x 128 elements); an FMA-pipe
+// pair costs 25 cycles of a scheduler where the unit's takes 16.  Measured on B200, us per layer with 1, 2, 3 of eight: head_dim 128 (4
+// sequences of 4096, 32 / 8 heads), sweep 1 305, 320, 321, sweep 2 364, 360, 374; head_dim 64 (2 sequences of 5003, 71 / 1 heads)
+// 485, 482, 504 and 501, 485, 505.
+template <int D, int SWEEP>
+__device__ __forceinline__ constexpr bool on_fma(int pair) {  // `pair` is a constant after unrolling
+  return SWEEP == 1 && D == 128 ? (pair & 7) == 7 : (pair & 3) == 3;
+}
 
 // SWEEP 1: rows = queries, streamed tiles = keys; SWEEP 2: rows = keys, streamed tiles = queries.
 template <int D, int TN, int STAGES, int SWEEP>
@@ -109,7 +113,6 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
   auto bar_lse = [&](int b) { return s_u32(bars + 5 + 2 * STAGES + b); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* redo_flag = reinterpret_cast<volatile int*>(tmem_slot + 2);
   float* lse_s = reinterpret_cast<float*>(tmem_slot + 4);  // [2][128]: sweep 2, minus the row log-sum-exps
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -171,7 +174,6 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
       mbar_init(bar_lse(b), 1);
     }
     *abort_flag = 0;
-    *redo_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) {
@@ -185,133 +187,112 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
   const uint32_t tmem_base = *tmem_slot;
   grid_wait();
 
-  // drain threads: sweep 1: reference of the row and the sum of its weights; sweep 2: the key's sum (even and odd columns)
+  // drain threads: sweep 1: running maximum of the row and the sum of its weights; sweep 2: the key's sum (even and odd columns)
   // (a tile's 64 weights are added up by themselves, so that a sum over thousands of tiles is no less precise than they are)
   float m = -INFINITY, sum = 0.f;
   bool ok = true;
-  // tiles are numbered through both passes of sweep 1 (the second one is rare, see the drain)
-  int tile0 = 0;
-#pragma unroll 1
-  for (;;) {
-    const int tile1 = tile0 + n_stream;
-    if (warp == 0) {
-      // ---------------- TMA producer ----------------
+  if (warp == 0) {
+    // ---------------- TMA producer ----------------
+    if (lane == 0) {
+      mbar_expect_tx(bar_a, ROWS_BYTES);
+#pragma unroll
+      for (int sb = 0; sb < SUB; ++sb) tma_load_2d(s_u32(a_s + sb * kSubBytes), &tm_rows, sb * 64, (int)rows0, bar_a);
+      int issued = 0;
+      Walk w = walk_begin();
+      for (int i = 0; i < n_stream; ++i) {
+        const int st = i % STAGES;
+        if (i >= STAGES && !mbar_wait(bar_empty(st), ((i / STAGES) - 1) & 1, abort_flag)) break;
+        mbar_expect_tx(bar_full(st), TILE_BYTES);
+#pragma unroll
+        for (int sb = 0; sb < SUB; ++sb)
+          tma_load_2d(s_u32(b_s + st * TILE_BYTES + sb * STREAM_SUB), &tm_stream, sb * 64, (int)w.row0, bar_full(st));
+        issued = i + 1;
+        walk_next(w);
+      }
+      if (*abort_flag) {
+        // winding down early: let the copies already in flight land before the CTA exits
+        mbar_wait(bar_a, 0, abort_flag);
+        for (int i = max(0, issued - STAGES); i < issued; ++i) {
+          for (int k = 0; k < kSpinLimit && !mbar_try_wait(bar_full(i % STAGES), (i / STAGES) & 1); ++k) {
+          }
+        }
+      }
+    }
+  } else if (warp == 1) {
+    // ---------------- MMA issuer; sweep 2: also stages the tile's row log-sum-exps ----------------
+    // (fetched one tile ahead, so that the trip to memory runs under the tile before)
+    constexpr int kLse = TN / 32;  // per lane
+    struct alignas(4 * kLse) Lse {
+      float x[kLse];
+    };
+    auto fetch_lse = [&](const Walk& w) {
+      const float* src = a.lse2 + ((size_t)bi * a.n_q_head + hk * g + w.h) * P;
+      const int q = w.qt * TN + lane * kLse;
+      Lse v;
+#pragma unroll
+      for (int e = 0; e < kLse; ++e) v.x[e] = (q + e < P) ? -src[q + e] : -INFINITY;  // a query past the end attends to nothing
+      return v;
+    };
+    Walk w = walk_begin();
+    Lse lse_next = {};
+    if (SWEEP == 2) lse_next = fetch_lse(w);
+    ok = mbar_wait(bar_a, 0, abort_flag);
+    for (int i = 0; ok && i < n_stream; ++i) {
+      const int st = i % STAGES, buf = i & 1;
+      ok = mbar_wait(bar_full(st), (i / STAGES) & 1, abort_flag);
+      if (ok && i >= 2) ok = mbar_wait(bar_sfree(buf), ((i >> 1) - 1) & 1, abort_flag);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (lane == 0) {
-        if (tile0 == 0) {
-          mbar_expect_tx(bar_a, ROWS_BYTES);
+        const uint32_t d_tmem = tmem_base + buf * TN;
 #pragma unroll
-          for (int sb = 0; sb < SUB; ++sb) tma_load_2d(s_u32(a_s + sb * kSubBytes), &tm_rows, sb * 64, (int)rows0, bar_a);
+        for (int k = 0; k < D / 16; ++k) {
+          const uint32_t a_addr = s_u32(a_s + (k / 4) * kSubBytes) + (k % 4) * 32;
+          const uint32_t b_addr = s_u32(b_s + st * TILE_BYTES + (k / 4) * STREAM_SUB) + (k % 4) * 32;
+          umma_bf16(d_tmem, umma_desc(a_addr), umma_desc(b_addr), kIdesc, k > 0 ? 1u : 0u);
         }
-        int issued = tile0;
-        Walk w = walk_begin();
-        for (int i = tile0; i < tile1; ++i) {
-          const int st = i % STAGES;
-          if (i >= STAGES && !mbar_wait(bar_empty(st), ((i / STAGES) - 1) & 1, abort_flag)) break;
-          mbar_expect_tx(bar_full(st), TILE_BYTES);
-#pragma unroll
-          for (int sb = 0; sb < SUB; ++sb)
-            tma_load_2d(s_u32(b_s + st * TILE_BYTES + sb * STREAM_SUB), &tm_stream, sb * 64, (int)w.row0, bar_full(st));
-          issued = i + 1;
-          walk_next(w);
-        }
-        if (*abort_flag) {
-          // winding down early: let the copies already in flight land before the CTA exits
-          mbar_wait(bar_a, 0, abort_flag);
-          for (int i = max(0, issued - STAGES); i < issued; ++i) {
-            for (int k = 0; k < kSpinLimit && !mbar_try_wait(bar_full(i % STAGES), (i / STAGES) & 1); ++k) {
-            }
-          }
-        }
+        umma_commit(bar_empty(st));  // the stage may be refilled once these MMAs have read it
+        umma_commit(bar_sfull(buf)); // the accumulator buffer is complete
       }
-    } else if (warp == 1) {
-      // ---------------- MMA issuer; sweep 2: also stages the tile's row log-sum-exps ----------------
-      // (fetched one tile ahead, so that the trip to memory runs under the tile before)
-      constexpr int kLse = TN / 32;  // per lane
-      struct alignas(4 * kLse) Lse {
-        float x[kLse];
-      };
-      auto fetch_lse = [&](const Walk& w) {
-        const float* src = a.lse2 + ((size_t)bi * a.n_q_head + hk * g + w.h) * P;
-        const int q = w.qt * TN + lane * kLse;
-        Lse v;
-#pragma unroll
-        for (int e = 0; e < kLse; ++e) v.x[e] = (q + e < P) ? -src[q + e] : -INFINITY;  // a query past the end attends to nothing
-        return v;
-      };
-      Walk w = walk_begin();
-      Lse lse_next = {};
-      if (SWEEP == 2) lse_next = fetch_lse(w);
-      ok = mbar_wait(bar_a, 0, abort_flag);
-      for (int i = tile0; ok && i < tile1; ++i) {
-        const int st = i % STAGES, buf = i & 1;
-        ok = mbar_wait(bar_full(st), (i / STAGES) & 1, abort_flag);
-        if (ok && i >= 2) ok = mbar_wait(bar_sfree(buf), ((i >> 1) - 1) & 1, abort_flag);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (lane == 0) {
-          const uint32_t d_tmem = tmem_base + buf * TN;
-#pragma unroll
-          for (int k = 0; k < D / 16; ++k) {
-            const uint32_t a_addr = s_u32(a_s + (k / 4) * kSubBytes) + (k % 4) * 32;
-            const uint32_t b_addr = s_u32(b_s + st * TILE_BYTES + (k / 4) * STREAM_SUB) + (k % 4) * 32;
-            umma_bf16(d_tmem, umma_desc(a_addr), umma_desc(b_addr), kIdesc, k > 0 ? 1u : 0u);
-          }
-          umma_commit(bar_empty(st));  // the stage may be refilled once these MMAs have read it
-          umma_commit(bar_sfull(buf)); // the accumulator buffer is complete
-        }
+      __syncwarp();
+      if (SWEEP == 2) {
+        // (behind the products, which do not wait for them)
+        *reinterpret_cast<Lse*>(lse_s + buf * TN + lane * kLse) = lse_next;
         __syncwarp();
-        if (SWEEP == 2) {
-          // (behind the products, which do not wait for them)
-          *reinterpret_cast<Lse*>(lse_s + buf * TN + lane * kLse) = lse_next;
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_lse(buf));
-          if (i + 1 < tile1) {
-            walk_next(w);
-            lse_next = fetch_lse(w);
-          }
+        if (lane == 0) mbar_arrive(bar_lse(buf));
+        if (i + 1 < n_stream) {
+          walk_next(w);
+          lse_next = fetch_lse(w);
         }
       }
-    } else {
-      // ---------------- accumulator drain: thread = one row of the fixed tile, 64 columns ----------------
-      const int quarter = warp & 3;
-      const int col0 = TN == 64 ? 0 : ((warp - 2) >> 2) * 64;  // of the 64 columns of every tile that this warp drains
-      const int row = quarter * 32 + lane;
-      const uint32_t s_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + col0;
-      const unsigned long long scale2 = f32x2(scale_log2, scale_log2);
-      m = -INFINITY;
-      sum = 0.f;
-      unsigned long long acc_a, acc_b;  // of the tile, even and odd columns
-      float top = -INFINITY, m_first = 0.f;  // of the FMA-pipe form's scores; reference of the plain tiles
-      Walk w = walk_begin();
-      // The tiles on the diagonal mask a part of their elements, the others none: they are separate
-      // instantiations of the drain, so that tiles off the diagonal carry no compare / select per element.
-      // Sweep 1 has a third: a row's reference is its maximum over the first tile (and over those on the diagonal), so
-      // that most tiles carry no maximum.  A weight above 2^kMaxRise shows in the sum, but for the FMA-pipe form, which
-      // may overflow without a trace and whose scores are therefore looked at: a CTA with such a row walks its tiles again
-      // with a running maximum.  (Redone on the spot, chunk by chunk, the code that hardly ever runs cost 456 against 440
-      // us a sweep; a reference that follows the FMA-pipe form's scores 488 against 460, at the same precision.)
-      enum { kPlain, kDiagonal, kFirst };
-      struct Tile {
-        int buf, off;  // off: of the tile's first column from the fixed tile's first row
-      };
-      // weights of 32 columns under the reference m
-      auto row_weights = [&](auto exact_c, const uint32_t (&r)[32]) {
-        const unsigned long long neg_m2 = f32x2(-m, -m);
+    }
+  } else {
+    // ---------------- accumulator drain: thread = one row of the fixed tile, 64 columns ----------------
+    const int quarter = warp & 3;
+    const int col0 = TN == 64 ? 0 : ((warp - 2) >> 2) * 64;  // of the 64 columns of every tile that this warp drains
+    const int row = quarter * 32 + lane;
+    const uint32_t s_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + col0;
+    const unsigned long long scale2 = f32x2(scale_log2, scale_log2);
+    unsigned long long acc_a, acc_b;  // of the tile, even and odd columns
+    Walk w = walk_begin();
+    // The tiles on the diagonal mask a part of their elements, the others none: they are separate
+    // instantiations of the drain, so that tiles off the diagonal carry no compare / select per element.
+    struct Tile {
+      int buf, off;  // off: of the tile's first column from the fixed tile's first row
+    };
+    auto chunk = [&](auto diag_c, const Tile& t, uint32_t (&r)[32], int c0) {  // columns c0 .. c0+31 of the tile
+      constexpr bool DIAG = decltype(diag_c)::value;
+      if (SWEEP == 1) {
+        if (DIAG) {
 #pragma unroll
-        for (int jp = 0; jp < 16; ++jp) {
-          const unsigned long long x2 =
-              fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])), scale2, neg_m2);
-          // (a masked tile keeps to the form that gives an exact 0)
-          const unsigned long long e2 = !decltype(exact_c)::value && on_fma(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
-          if (jp & 1) acc_b = add_f32x2(acc_b, e2);
-          else acc_a = add_f32x2(acc_a, e2);
+          for (int j = 0; j < 32; ++j)
+            if (t.off + c0 + j > row) r[j] = 0xff800000u;  // key after the query: -inf
         }
-      };
-      auto move_reference = [&](const uint32_t (&r)[32]) {
         float mx = __uint_as_float(r[0]);
 #pragma unroll
         for (int j = 1; j + 1 < 32; j += 2) mx = max3(mx, __uint_as_float(r[j]), __uint_as_float(r[j + 1]));
         const float m_new = fmaxf(m, fmaxf(mx, __uint_as_float(r[31])) * scale_log2);
+        if (DIAG && m_new == -INFINITY) return;  // nothing of the row so far (second half of the first rows)
         if (m_new > m) {
           const float f = ex2(m - m_new);
           const unsigned long long f2 = f32x2(f, f), zero = f32x2(0.f, 0.f);
@@ -320,87 +301,72 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
           sum *= f;
           m = m_new;
         }
-      };
-      auto chunk = [&](auto kind_c, const Tile& t, uint32_t (&r)[32], int c0) {  // columns c0 .. c0+31 of the tile
-        constexpr int KIND = decltype(kind_c)::value;
-        if constexpr (SWEEP == 1 && KIND == kPlain) {
-          row_weights(std::false_type{}, r);
+        const unsigned long long neg_m2 = f32x2(-m, -m);
 #pragma unroll
-          for (int jp = 0; jp < 16; ++jp)
-            if (on_fma(jp)) top = max3(top, __uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1]));
-        } else if constexpr (SWEEP == 1) {
-          if (KIND == kDiagonal) {
+        for (int jp = 0; jp < 16; ++jp) {
+          const unsigned long long x2 =
+              fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])), scale2, neg_m2);
+          // (a masked tile keeps to the form that gives an exact 0)
+          const unsigned long long e2 = !DIAG && on_fma<D, SWEEP>(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
+          if (jp & 1) acc_b = add_f32x2(acc_b, e2);
+          else acc_a = add_f32x2(acc_a, e2);
+        }
+      } else {
+        const ulonglong2* ls = reinterpret_cast<const ulonglong2*>(lse_s + t.buf * TN + c0);
 #pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (t.off + c0 + j > row) r[j] = 0xff800000u;  // key after the query: -inf
-          }
-          move_reference(r);
-          if (KIND == kDiagonal && m == -INFINITY) return;  // nothing of the row so far (second half of the first rows)
-          row_weights(std::bool_constant<KIND == kDiagonal>{}, r);
-        } else {
-          const ulonglong2* ls = reinterpret_cast<const ulonglong2*>(lse_s + t.buf * TN + c0);
+        for (int j4 = 0; j4 < 8; ++j4) {
+          const ulonglong2 lv = ls[j4];
 #pragma unroll
-          for (int j4 = 0; j4 < 8; ++j4) {
-            const ulonglong2 lv = ls[j4];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-              const int jp = 2 * j4 + q;
-              const unsigned long long x2 = fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])),
-                                                      scale2, q ? lv.y : lv.x);
-              unsigned long long e2 = on_fma(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
-              if (KIND == kDiagonal) {  // query before the key: no attention
-                float e0, e1;
-                f32x2_split(e2, e0, e1);
-                e2 = f32x2(t.off + c0 + 2 * jp >= row ? e0 : 0.f, t.off + c0 + 2 * jp + 1 >= row ? e1 : 0.f);
-              }
-              if (q) acc_b = add_f32x2(acc_b, e2);
-              else acc_a = add_f32x2(acc_a, e2);
+          for (int q = 0; q < 2; ++q) {
+            const int jp = 2 * j4 + q;
+            const unsigned long long x2 = fma_f32x2(f32x2(__uint_as_float(r[2 * jp]), __uint_as_float(r[2 * jp + 1])),
+                                                    scale2, q ? lv.y : lv.x);
+            unsigned long long e2 = on_fma<D, SWEEP>(jp) ? ex2_pair_fma(x2) : ex2_pair_sfu(x2);
+            if (DIAG) {  // query before the key: no attention
+              float e0, e1;
+              f32x2_split(e2, e0, e1);
+              e2 = f32x2(t.off + c0 + 2 * jp >= row ? e0 : 0.f, t.off + c0 + 2 * jp + 1 >= row ? e1 : 0.f);
             }
+            if (q) acc_b = add_f32x2(acc_b, e2);
+            else acc_a = add_f32x2(acc_a, e2);
           }
         }
-      };
-      auto drain_tile = [&](auto kind_c, const Tile& t) {
-        auto hand_back = [&]() {
-          asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-          __syncwarp();
-          if (lane == 0) mbar_arrive(bar_sfree(t.buf));
-        };
-        // (32 columns at a time: with the second half's load in flight under the first's exponentials the registers
-        // held the FMA-pipe form back, 497 against 482 us a sweep at head_dim 64)
-        acc_a = acc_b = f32x2(0.f, 0.f);
-        uint32_t r[32];
-        tmem_ld32_nowait(s_addr + t.buf * TN, r);
-        tmem_wait_ld(r);
-        chunk(kind_c, t, r, col0);
-        __syncwarp();
-        tmem_ld32_nowait(s_addr + t.buf * TN + 32, r);
-        tmem_wait_ld(r);
-        if (SWEEP == 1) hand_back();  // the tile is in registers: the tensor core may have the buffer back
-        chunk(kind_c, t, r, col0 + 32);
-        if (SWEEP == 2) hand_back();  // the buffer's lse staging is in use until here
-        float a0, a1;
-        f32x2_split(add_f32x2(acc_a, acc_b), a0, a1);
-        sum += a0 + a1;
-      };
-      for (int i = tile0; ok && i < tile1; ++i) {
-        const Tile t{i & 1, (w.qt - kTM / TN * row_tile) * TN};
-        const bool diag = (unsigned)t.off < (unsigned)kTM;
-        walk_next(w);
-        if (SWEEP == 2) ok = mbar_wait(bar_lse(t.buf), (i >> 1) & 1, abort_flag);
-        if (ok) ok = mbar_wait(bar_sfull(t.buf), (i >> 1) & 1, abort_flag);
-        if (!ok) break;
-        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        if (SWEEP == 1 && i == 1) m_first = m;
-        if (diag) drain_tile(std::integral_constant<int, kDiagonal>{}, t);
-        else if (SWEEP == 1 && (i == 0 || tile0 > 0)) drain_tile(std::integral_constant<int, kFirst>{}, t);
-        else drain_tile(std::integral_constant<int, kPlain>{}, t);
       }
-      if (SWEEP == 1 && tile0 == 0 && (fmaf(top, scale_log2, -m_first) > kMaxRise || !(sum <= kMaxSum))) *redo_flag = 1;
+    };
+    auto drain_tile = [&](auto diag_c, const Tile& t) {
+      auto hand_back = [&]() {
+        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar_sfree(t.buf));
+      };
+      // (32 columns at a time: with the second half's load in flight under the first's exponentials the registers
+      // held the FMA-pipe form back, 497 against 482 us a sweep at head_dim 64)
+      acc_a = acc_b = f32x2(0.f, 0.f);
+      uint32_t r[32];
+      tmem_ld32_nowait(s_addr + t.buf * TN, r);
+      tmem_wait_ld(r);
+      chunk(diag_c, t, r, col0);
+      __syncwarp();
+      tmem_ld32_nowait(s_addr + t.buf * TN + 32, r);
+      tmem_wait_ld(r);
+      if (SWEEP == 1) hand_back();  // the tile is in registers: the tensor core may have the buffer back
+      chunk(diag_c, t, r, col0 + 32);
+      if (SWEEP == 2) hand_back();  // the buffer's lse staging is in use until here
+      float a0, a1;
+      f32x2_split(add_f32x2(acc_a, acc_b), a0, a1);
+      sum += a0 + a1;
+    };
+    for (int i = 0; ok && i < n_stream; ++i) {
+      const Tile t{i & 1, (w.qt - kTM / TN * row_tile) * TN};
+      const bool diag = (unsigned)t.off < (unsigned)kTM;
+      walk_next(w);
+      if (SWEEP == 2) ok = mbar_wait(bar_lse(t.buf), (i >> 1) & 1, abort_flag);
+      if (ok) ok = mbar_wait(bar_sfull(t.buf), (i >> 1) & 1, abort_flag);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      if (diag) drain_tile(std::true_type{}, t);
+      else drain_tile(std::false_type{}, t);
     }
-    if (SWEEP == 2) break;
-    __syncthreads();
-    if (tile0 > 0 || !*redo_flag || *abort_flag) break;
-    tile0 = tile1;
   }
   if (warp >= 2) {
     const int row = (warp & 3) * 32 + lane, row_idx = row_tile * kTM + row;  // query (sweep 1) / key (sweep 2)
@@ -546,8 +512,8 @@ cudaError_t launch_prefill_scores_tc(const ScoreArgs& a, int* status, cudaStream
   if (a.n_q_head > 65535 || a.batch > 65535 || (a.prompt + kTM - 1) / kTM > 65535) return cudaErrorNotSupported;
   if ((reinterpret_cast<uintptr_t>(a.q) | reinterpret_cast<uintptr_t>(a.k)) & 15u) return cudaErrorNotSupported;
   // Tiles of 64 columns put four CTAs with four drain warps each on an SM; a launch that fills no more than two of them is over
-  // sooner with eight warps per CTA.  us per layer, 64 / 128 columns: 256 CTAs in sweep 1 (4 sequences of 4000, two heads) 100 /
-  // 72, 32: 22.5 / 19.4, 284: 32.8 / 31.1, 568: 49.4 / 51.2, 1136: 74.7 / 80.2.
+  // sooner with eight warps per CTA.  us per layer, 64 / 128 columns, by CTAs of sweep 1: 32 (1 sequence of 4096, one head) 95 / 66, 256
+  // (4 of 4000, two) 101 / 79, 284 28.1 / 26.6, 296 40 / 34, 300 27.9 / 28.1, 568 48.0 / 49.4, 1136 73 / 80.
   const long long ctas = (long long)a.n_q_head * a.batch * ((a.prompt + kTM - 1) / kTM);
   if (a.head_dim == 64) return ctas > 2LL * sm_count() ? launch_tc_t<64, 64, 3>(a, status, s) : launch_tc_t<64, 128, 4>(a, status, s);
   if (a.head_dim == 128) return launch_tc_t<128, 128, 2>(a, status, s);

@@ -52,8 +52,8 @@ def test_prompt_scores_of_short_fp32_prompts(head_dim, hq, hkv, batch, prompt):
     test_prompt_scores_cut_into_pieces(torch.float32, head_dim, hq, hkv, batch, prompt)
 
 
-# A row's reference is its maximum over the first keys and stays unless a row rises 2^32 above it: some rows do, by overflowing
-# amounts too, some rise less, some not at all; both tile widths, both halves of a wide tile, the last tile ragged
+# A row's reference is its maximum so far: some rows rise far above their first keys, by amounts beyond fp32's range too, some
+# less, some not at all; both tile widths, both halves of a wide tile, the last tile ragged
 @pytest.mark.parametrize("head_dim,hq", [(64, 3), (64, 60), (128, 2)])   # (60 heads: enough CTAs for the narrow tiles)
 @pytest.mark.parametrize("prompt", [200, 700])
 def test_prompt_scores_of_rising_rows(head_dim, hq, prompt):
@@ -72,6 +72,36 @@ def test_prompt_scores_of_rising_rows(head_dim, hq, prompt):
         # logits of up to L = 100 * 6 are fp32 sums of head_dim products and meet the stored log-sum-exp at that size: 2^-23 L
         # each in the exponent, twice; scores below 2^-126 of a row count as that
         np.testing.assert_allclose(acc, want, rtol=H.RTOL_ACC[w.dtype] * (10 if s == 2 else 1), atol=1e-6)
+    assert ctx.status() == 0
+
+
+# Rows whose first keys weigh next to nothing and one later key nearly everything, each such key alone seen by one row of one head,
+# so that its score is that row's weight and no sum over rows evens the rounding out
+@pytest.mark.parametrize("head_dim,hq,batch", [(64, 3, 1), (64, 60, 3), (128, 2, 2)])   # wide tiles, narrow tiles, head_dim 128
+def test_prompt_score_of_one_late_key_per_row(head_dim, hq, batch):
+    prompt, n = 700, 32
+    w = workload("late key", 9180, head_dim=head_dim, n_q_head=hq, n_kv_head=1, batch=batch, prompt=prompt, heavy_mode="none")
+    q, k, v = (t.zero_() for t in synth.prompt_qkv(w, 0, DEV))
+    gen = torch.Generator().manual_seed(9180 + head_dim)
+    scale = 1.4426950408889634 / head_dim ** 0.5               # logits in powers of two
+    late = 300 + 7 * torch.arange(n)                           # every place of a tile's pairs; in tiles off the diagonal
+    k[:, 0, :, :n] = -26.0 / 4 / scale                         # a late row's other keys: 2^-26 and less
+    k[:, 0, late, torch.arange(n)] = ((1 + torch.rand(n, generator=gen)) / 4.25 / scale).to(k)
+    k[:, 0, late, 40] = -60.0 / 4 / scale                      # the other rows do not see the late keys
+    q[:, :, :, 40] = 4.0
+    rows = torch.arange(prompt - n, prompt)
+    q[:, 0, rows, 40] = 0.0
+    q[:, 0, rows, torch.arange(n)] = (4 + torch.arange(n) % 9 / 32).to(q)
+    ctx = H.make_ctx(w, b_init=prompt)
+    ctx.begin_sequence_batch(batch, prompt)
+    ctx.set_budgets([prompt])
+    ctx.prefill_compress(0, k, v, q)
+    for s in range(batch):
+        _, acc = ctx.get_kept(0, s, 0)
+        want = O.prefill_scores(H.f64(q[s]), H.f64(k[s, 0]))
+        # The late key's logit and the log-sum-exp lie between 1 and 2 (in powers of two): each is rounded by 2^-24 once it is
+        # scaled and once more when it is stored, so the weight by 4 * 2^-24 * ln 2 = 1.7e-7; its exponential by 2.1e-7
+        np.testing.assert_allclose(np.asarray(acc)[late], want[late], rtol=3.8e-7, atol=0)
     assert ctx.status() == 0
 
 
