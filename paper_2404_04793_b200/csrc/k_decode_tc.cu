@@ -76,9 +76,11 @@ struct ClusterShared {
   ScoreCandidate warp_best[4];
 };
 
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
-__device__ __forceinline__ void softmax_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+// (bar.sync is an .aligned form as well)
+__device__ __forceinline__ void softmax_sync() {
+  __syncwarp();
+  asm volatile("bar.sync 1, 128;" ::: "memory");
+}
 
 // Cluster form, the four softmax warps after the last tile: the piece's partial result to shared memory, then (behind
 // the cluster's barrier) the unit's row sums from all pieces, this CTA's share of the output, and with H2O the
@@ -102,11 +104,13 @@ __device__ __forceinline__ void finish_cluster(const Args& a, const LayerDesc* l
     for (int c = 0; c < 2; ++c) {
       float o[32];
       tmem_ld32(rows.o_addr + c * 32, o);
-      if (!live) continue;
+      if (live) {
 #pragma unroll
-      for (int q4 = 0; q4 < 8; ++q4)
-        *reinterpret_cast<float4*>(sh.o + row * kORow + c * 32 + q4 * 4) =
-            make_float4(o[q4 * 4], o[q4 * 4 + 1], o[q4 * 4 + 2], o[q4 * 4 + 3]);
+        for (int q4 = 0; q4 < 8; ++q4)
+          *reinterpret_cast<float4*>(sh.o + row * kORow + c * 32 + q4 * 4) =
+              make_float4(o[q4 * 4], o[q4 * 4 + 1], o[q4 * 4 + 2], o[q4 * 4 + 3]);
+      }
+      __syncwarp();  // the loads of tensor memory are warp-wide
     }
     if (live) *reinterpret_cast<float4*>(sh.stat + row * kStatStride) = make_float4(m_ref, H2O ? l : l_w, l_w, 0.f);
     if (H2O) {
@@ -118,7 +122,6 @@ __device__ __forceinline__ void finish_cluster(const Args& a, const LayerDesc* l
       }
     }
   }
-  __syncwarp();
   cluster_arrive();
   // the first tile's scores and positions are on their way meanwhile
   const int b = ldp->b, cap = ldp->cap;
@@ -285,7 +288,6 @@ __device__ __forceinline__ void finish_cluster(const Args& a, const LayerDesc* l
         }
       st_cluster_candidate(map_rank(&sh.offer[me], 0), best, best_slot);
     }
-    __syncwarp();
   }
   cluster_arrive();
 }
@@ -598,23 +600,23 @@ __global__ void __launch_bounds__(192, 2)
         const int row = layout.head_of_lane(quarter, lane);
         const bool live = row < G;  // this lane's row is a real head
         const float inv = 1.f / l_w;
-  #pragma unroll 1
+#pragma unroll 1
         for (int c = 0; c < 2; ++c) {
           float o[32];
           tmem_ld32(rows.o_addr + c * 32, o);
-          if (!live) continue;
-          if (it.n_split == 1) {
-  #pragma unroll
+          if (live && it.n_split == 1) {
+#pragma unroll
             for (int q4 = 0; q4 < 4; ++q4)
               *reinterpret_cast<uint4*>(ob + (size_t)row * kD + c * 32 + q4 * 8) =
                   make_uint4(pack_bf16x2(o[q4 * 8] * inv, o[q4 * 8 + 1] * inv), pack_bf16x2(o[q4 * 8 + 2] * inv, o[q4 * 8 + 3] * inv),
                              pack_bf16x2(o[q4 * 8 + 4] * inv, o[q4 * 8 + 5] * inv), pack_bf16x2(o[q4 * 8 + 6] * inv, o[q4 * 8 + 7] * inv));
-          } else {
-  #pragma unroll
+          } else if (live) {
+#pragma unroll
             for (int q4 = 0; q4 < 8; ++q4)
               *reinterpret_cast<float4*>(po + (size_t)row * kD + c * 32 + q4 * 4) =
                   make_float4(o[q4 * 4], o[q4 * 4 + 1], o[q4 * 4 + 2], o[q4 * 4 + 3]);
           }
+          __syncwarp();  // the loads of tensor memory are warp-wide
         }
         if (live) {
           stat[row * kStatStride] = m_ref;

@@ -409,18 +409,18 @@ __global__ void __launch_bounds__(192, kCtasPerSm)
         for (int c = 0; c < 2; ++c) {
           float o[32];
           tmem_ld32(rows.o_addr + c * 32, o);
-          if (!live) continue;
-          if (n_piece == 1) {
+          if (live && n_piece == 1) {
 #pragma unroll
             for (int q4 = 0; q4 < 4; ++q4)
               *reinterpret_cast<uint4*>(orow + c * 32 + q4 * 8) =
                   make_uint4(pack_bf16x2(o[q4 * 8] * inv, o[q4 * 8 + 1] * inv), pack_bf16x2(o[q4 * 8 + 2] * inv, o[q4 * 8 + 3] * inv),
                              pack_bf16x2(o[q4 * 8 + 4] * inv, o[q4 * 8 + 5] * inv), pack_bf16x2(o[q4 * 8 + 6] * inv, o[q4 * 8 + 7] * inv));
-          } else {
+          } else if (live) {
 #pragma unroll
             for (int q4 = 0; q4 < 8; ++q4)
               *reinterpret_cast<float4*>(prow + c * 32 + q4 * 4) = make_float4(o[q4 * 4], o[q4 * 4 + 1], o[q4 * 4 + 2], o[q4 * 4 + 3]);
           }
+          __syncwarp();  // the loads of tensor memory are warp-wide
         }
         if (live) {
           if (n_piece == 1) {

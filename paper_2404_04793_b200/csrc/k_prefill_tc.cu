@@ -375,11 +375,13 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
     if constexpr (TN == 128) {
       // the two halves of a row meet in shared memory (the staging area is free once every drain
       // thread is past its last tile); every drain thread reaches both barriers, aborted or not
+      __syncwarp();
       asm volatile("bar.sync 1, 256;" ::: "memory");
       if (second_half) {
         lse_s[2 * row] = m;
         lse_s[2 * row + 1] = l;
       }
+      __syncwarp();
       asm volatile("bar.sync 1, 256;" ::: "memory");
       const float o0 = lse_s[2 * row], o1 = lse_s[2 * row + 1];
       if (SWEEP == 1) {

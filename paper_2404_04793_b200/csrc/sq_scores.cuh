@@ -25,10 +25,20 @@ __device__ __forceinline__ int cluster_size() {
   asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
   return (int)r;
 }
-// Barrier over the cluster's threads; shared memory written before it is visible to the others after it.
-__device__ __forceinline__ void cluster_sync() {
+// Barrier over the cluster's threads, in two parts; shared memory written before it is visible to the others after it.  The
+// .aligned forms want a warp's threads together, so the warp meets first: loops and branches ahead may end in its lanes at
+// different times.
+__device__ __forceinline__ void cluster_arrive() {
+  __syncwarp();
   asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  __syncwarp();
   asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_sync() {
+  cluster_arrive();
+  cluster_wait();
 }
 // Address, in the cluster's shared window, of this CTA's shared-memory location p in CTA `rank`.
 __device__ __forceinline__ uint32_t map_rank(const void* p, int rank) {
