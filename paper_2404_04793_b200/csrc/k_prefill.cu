@@ -597,14 +597,16 @@ __global__ void __launch_bounds__(NT) select_prompt_regs_kernel(const GatherArgs
   const bool drop = P > ld.b;
   const int n_cand = drop ? P - ld.b_recent : 0;  // positions [0, n_cand) compete for the heavy slots
   float val[KPT];
-  uint32_t key[KPT];  // of the competing tokens; 0, below every finite score's, for the others
+  // of the competing tokens; 0 for the others.  (A score with every bit set, a NaN, has key 0 as well: it takes the lowest other, since
+  // there have to be as many competing tokens as the heavy slots were reckoned to get.)
+  uint32_t key[KPT];
 #pragma unroll
   for (int j = 0; j < KPT; ++j) {
     const int i = j * NT + tid;
     val[j] = (i < P) ? acc[i] : 0.f;
   }
 #pragma unroll
-  for (int j = 0; j < KPT; ++j) key[j] = (j * NT + tid < n_cand) ? score_key(val[j]) : 0u;
+  for (int j = 0; j < KPT; ++j) key[j] = (j * NT + tid < n_cand) ? max(score_key(val[j]), 1u) : 0u;
 
   // Competing tokens with key >= lo stay: the largest lo that leaves at least b_heavy of them.  With
   // ties at lo (need_ties < all of them) the lowest positions among those stay.

@@ -105,6 +105,27 @@ def test_prompt_score_of_one_late_key_per_row(head_dim, hq, batch):
     assert ctx.status() == 0
 
 
+# Given scores with every bit set (NaN, which no selection has to make sense of): every slot still gets a token of its own and that
+# token's rows.  Few heavy rows, copied by the selecting CTA, and more than it copies
+@pytest.mark.parametrize("prompt,budget", [(300, 100), (1200, 900), (3000, 1024)])
+def test_prompt_selection_with_scores_of_all_ones(prompt, budget):
+    w = workload("all ones", 9190 + prompt, prompt=prompt, heavy_mode="none")
+    ctx = H.make_ctx(w, b_init=budget)
+    ctx.begin_sequence_batch(1, prompt)
+    ctx.set_budgets([budget])
+    _, k, v = synth.prompt_qkv(w, 0, DEV, need_q=False)
+    acc = torch.full((w.n_kv_head, prompt), -1, dtype=torch.int32, device=DEV).view(torch.float32)
+    acc[:, 17:budget // 4 + 17:2] = 1.0            # fewer than there are heavy slots
+    ctx.prefill_compress(0, k, v, None, acc)
+    for h in range(w.n_kv_head):
+        pos, _ = ctx.get_kept(0, 0, h)
+        assert len(pos) == budget and sorted(set(pos)) == pos and pos[0] >= 0 and pos[-1] == prompt - 1
+        assert set(range(17, budget // 4 + 17, 2)) <= set(pos)
+        kk, vv = ctx.get_kv(0, 0, h)
+        assert torch.equal(kk, k[0, h, pos].cpu()) and torch.equal(vv, v[0, h, pos].cpu())
+    assert ctx.status() == 0
+
+
 # Decode launches of one layer right behind one another start before the launch ahead is done and fetch
 # their first rows ahead of it, all but the new token's: its slot goes through every row of the cache,
 # and one layer behind itself (n_layer 1) or a stream change must not read ahead
