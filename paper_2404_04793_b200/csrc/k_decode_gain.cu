@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(64 + 128 * SETS, CTAS)
   if (tid >= 64 && tid < 64 + kTM) {
     const int h = tid - 64;
     const float* lse = a.logits + ldp->lse_off + (size_t)unit * G;
-    // columns past the group read +inf here, so their weight is exp2(-inf) = 0
+    // columns past the group: a query of zeros (tm_q), so their weight is exp2(0 - inf) = 0
     s_nlse[h] = (h < G) ? -lse[h] : -INFINITY;
   }
   __syncthreads();
@@ -131,9 +131,8 @@ __global__ void __launch_bounds__(64 + 128 * SETS, CTAS)
   if (warp == 0) {
     // ---------------- TMA producer ----------------
     if (lane == 0) {
-      const long long q_row0 = (long long)(tok * a.n_q_head + (size_t)kvh * G);
       mbar_expect_tx(bar_q, n_cols * 128);
-      tma_load_2d(s_u32(q_s), &tm_q, 0, (int)q_row0, bar_q);
+      tma_load_3d(s_u32(q_s), &tm_q, 0, 0, (int)(tok * a.n_kv_head) + kvh, bar_q);
       for (; issued < n_tiles; ++issued) {
         const int i = issued;
         if (i >= STAGES && !mbar_wait(bar_empty(i % STAGES), ((i / STAGES) - 1) & 1, abort_flag)) break;
@@ -317,7 +316,7 @@ cudaError_t launch_h2o_gain_tc(const DecodeArgs& a, int n_items, size_t pool_byt
   if (pool_rows + kTM > 0x7fffffffLL || (long long)q_rows + kTM > 0x7fffffffLL) return cudaErrorNotSupported;
   const int n_cols = (a.group + 15) & ~15;
   CUtensorMap tm_q, tm_k;
-  if (!make_tile_map(&tm_q, a.q, (long long)q_rows, kD, n_cols) || !make_tile_map(&tm_k, a.pool, pool_rows, kD, kTM))
+  if (!make_block_tile_map(&tm_q, a.q, (long long)q_rows / a.group, a.group, kD, n_cols) || !make_tile_map(&tm_k, a.pool, pool_rows, kD, kTM))
     return cudaErrorNotSupported;
   constexpr int kStages = 4, kSets = 2, kTmemCols = 256;
   constexpr size_t smem = 1024 + (size_t)kTM * 128 + (size_t)kStages * kTileBytes + 18 * 8 + kTM * 4 + 8 * sizeof(Candidate);

@@ -188,7 +188,7 @@ __device__ __forceinline__ void finish_cluster(const Args& a, const LayerDesc* l
     for (int r = 0; r < n; ++r) sh.factor[r][tid] = exp2f(sh.factor[r][tid] - M) * inv;
     if (H2O) sh.nlse[layout.row_of_group(tid >> 3) + (tid & 7)] = -(M + log2f(L));
   }
-  // columns past the group: their weight is exp2(-inf) = 0
+  // columns past the group: a query of zeros (tm_q), so their weight is exp2(0 - inf) = 0
   if (H2O && tid >= G && tid < (G + 7) / 8 * 8) sh.nlse[layout.row_of_group(tid >> 3) + (tid & 7)] = -INFINITY;
   softmax_sync();
   for (; i4 < n4; i4 += n * 128) {
@@ -419,7 +419,7 @@ __global__ void __launch_bounds__(192, 2)
     if (lane == 0) mbar_expect_tx(bar_q, n_group * 1024);
     __syncwarp();
     if (lane < n_group)
-      tma_load_2d(s_u32(q_s + layout.row_of_group(lane) * 128), &tm_q, 0, (int)(tok * a.n_q_head + (size_t)kvh * G) + 8 * lane, bar_q);
+      tma_load_3d(s_u32(q_s + layout.row_of_group(lane) * 128), &tm_q, 0, 8 * lane, (int)(tok * a.n_kv_head) + kvh, bar_q);
   }
   // the CTA whose range holds slot w stores the new token (generic proxy), then lets the TMA reads
   // (async proxy) see it
@@ -726,7 +726,7 @@ static bool make_maps(const DecodeArgs& a, size_t pool_bytes, size_t q_rows, CUt
   if (a.head_dim != kD || a.group <= 32 || a.group > 128) return false;
   const long long pool_rows = (long long)(pool_bytes / (kD * 2));
   if (pool_rows + kTM > 0x7fffffffLL || (long long)q_rows + kTM > 0x7fffffffLL) return false;
-  return make_tile_map(tm_q, a.q, (long long)q_rows, kD, 8) && make_tile_map(tm_k, a.pool, pool_rows, kD, kTM) &&
+  return make_block_tile_map(tm_q, a.q, (long long)q_rows / a.group, a.group, kD, 8) && make_tile_map(tm_k, a.pool, pool_rows, kD, kTM) &&
          make_tile_map(tm_v, a.pool, pool_rows, kD, kTM);
 }
 

@@ -122,43 +122,40 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
   // tiles of every head and sequence start first and the short ones fill the tail of the launch
   const int bi = blockIdx.y;
   int row_tile, n_stream, piece = 0, head0 = 0;
-  long long rows0;  // first row of this CTA's fixed tile in the rows tensor
+  int rows_head, stream_head;  // (sequence, head) of the fixed tile in the rows tensor, of the first streamed one in the other
   int hq = 0, hk = 0;
   if (SWEEP == 1) {
     hq = blockIdx.x;
     hk = hq / g;
     row_tile = n_tile - 1 - blockIdx.z;  // longest rows first
     n_stream = min(kTM / TN * (row_tile + 1), n_col_tile);
-    rows0 = ((long long)bi * a.n_q_head + hq) * P + (long long)row_tile * kTM;
+    rows_head = bi * a.n_q_head + hq;
+    stream_head = bi * a.n_kv_head + hk;
   } else {
     hk = blockIdx.x;
     row_tile = blockIdx.z / pc.n_piece;  // key tile 0 sees every query tile: longest first
     piece = blockIdx.z - row_tile * pc.n_piece;
     head0 = piece * pc.heads;            // this piece's heads of the group
     n_stream = min(pc.heads, g - head0) * (n_col_tile - kTM / TN * row_tile);
-    rows0 = ((long long)bi * a.n_kv_head + hk) * P + (long long)row_tile * kTM;
+    rows_head = bi * a.n_kv_head + hk;
+    stream_head = bi * a.n_q_head + hk * g;
   }
   // Walks the streamed tiles in order: (sweep 1) key tiles 0..row_tile, (sweep 2) per head of the
   // piece the query tiles from the diagonal down.
   struct Walk {
     int h, qt;
-    long long row0;
   };
   auto walk_begin = [&]() {
     Walk w;
     w.h = head0;
     w.qt = SWEEP == 1 ? 0 : kTM / TN * row_tile;
-    w.row0 = SWEEP == 1 ? ((long long)bi * a.n_kv_head + hk) * P
-                        : ((long long)bi * a.n_q_head + hk * g + head0) * P + (long long)row_tile * kTM;
     return w;
   };
   auto walk_next = [&](Walk& w) {
     ++w.qt;
-    w.row0 += TN;
     if (SWEEP == 2 && w.qt == n_col_tile) {
       w.qt = kTM / TN * row_tile;
       ++w.h;
-      w.row0 += P - (long long)(n_col_tile - kTM / TN * row_tile) * TN;
     }
   };
 
@@ -196,7 +193,7 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
     if (lane == 0) {
       mbar_expect_tx(bar_a, ROWS_BYTES);
 #pragma unroll
-      for (int sb = 0; sb < SUB; ++sb) tma_load_2d(s_u32(a_s + sb * kSubBytes), &tm_rows, sb * 64, (int)rows0, bar_a);
+      for (int sb = 0; sb < SUB; ++sb) tma_load_3d(s_u32(a_s + sb * kSubBytes), &tm_rows, sb * 64, row_tile * kTM, rows_head, bar_a);
       int issued = 0;
       Walk w = walk_begin();
       for (int i = 0; i < n_stream; ++i) {
@@ -205,7 +202,7 @@ __global__ void __launch_bounds__(prefill_threads(TN), TN == 64 ? 4 : 2)
         mbar_expect_tx(bar_full(st), TILE_BYTES);
 #pragma unroll
         for (int sb = 0; sb < SUB; ++sb)
-          tma_load_2d(s_u32(b_s + st * TILE_BYTES + sb * STREAM_SUB), &tm_stream, sb * 64, (int)w.row0, bar_full(st));
+          tma_load_3d(s_u32(b_s + st * TILE_BYTES + sb * STREAM_SUB), &tm_stream, sb * 64, w.qt * TN, stream_head + w.h, bar_full(st));
         issued = i + 1;
         walk_next(w);
       }
@@ -462,16 +459,32 @@ bool make_tile_map(CUtensorMap* tm, const void* base, long long rows, int d, int
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
+bool make_block_tile_map(CUtensorMap* tm, const void* base, long long blocks, int rows, int d, int box_rows) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)rows, (cuuint64_t)blocks};
+  cuuint64_t strides[2] = {(cuuint64_t)d * 2, (cuuint64_t)rows * d * 2};
+  cuuint32_t box[3] = {64, (cuuint32_t)box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 }  // namespace tc
 
 template <int D, int TN, int STAGES>
 static cudaError_t launch_tc_t(const ScoreArgs& a, int* status, cudaStream_t s) {
+  // Blocks of the maps: a head's prompt.  (A query past the end of one has weight exp2(x - inf), which is 0 for a row of zeros; the
+  // next head's query, if it is NaN or inf, would make it NaN.)
   CUtensorMap tm_q, tm_k;
-  const long long q_rows = (long long)a.batch * a.n_q_head * a.prompt, k_rows = (long long)a.batch * a.n_kv_head * a.prompt;
-  if (q_rows + kTM > 0x7fffffffLL) return cudaErrorNotSupported;  // TMA coordinates are 32-bit
+  const long long q_heads = (long long)a.batch * a.n_q_head, k_heads = (long long)a.batch * a.n_kv_head;
+  if (q_heads * a.prompt + kTM > 0x7fffffffLL) return cudaErrorNotSupported;
   CUtensorMap ts_q, ts_k;  // streamed
-  if (!tc::make_tile_map(&tm_q, a.q, q_rows, D, kTM) || !tc::make_tile_map(&tm_k, a.k, k_rows, D, kTM)) return cudaErrorNotSupported;
-  if (!tc::make_tile_map(&ts_q, a.q, q_rows, D, TN) || !tc::make_tile_map(&ts_k, a.k, k_rows, D, TN)) return cudaErrorNotSupported;
+  auto map = [&](CUtensorMap* tm, const void* base, long long heads, int rows) {
+    return tc::make_block_tile_map(tm, base, heads, a.prompt, D, rows);
+  };
+  if (!map(&tm_q, a.q, q_heads, kTM) || !map(&tm_k, a.k, k_heads, kTM)) return cudaErrorNotSupported;
+  if (!map(&ts_q, a.q, q_heads, TN) || !map(&ts_k, a.k, k_heads, TN)) return cudaErrorNotSupported;
   constexpr size_t smem = 1024 + (size_t)(D / 64) * (kSubBytes + STAGES * TN * 128) + 8 * 16 + 16 + 2 * TN * 4;
   const float scale_log2 = 1.4426950408889634f / sqrtf((float)D);
   const int n_tile = (a.prompt + kTM - 1) / kTM;

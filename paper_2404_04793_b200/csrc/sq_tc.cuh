@@ -61,6 +61,12 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* tm,
       "l"(reinterpret_cast<unsigned long long>(tm)), "r"(x), "r"(y), "r"(bar)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, int x, int y, int z, uint32_t bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(dst),
+      "l"(reinterpret_cast<unsigned long long>(tm)), "r"(x), "r"(y), "r"(z), "r"(bar)
+      : "memory");
+}
 // shared-memory matrix descriptor: K-major, 128-byte swizzle, 8-row groups 1024 bytes apart
 __device__ __forceinline__ unsigned long long umma_desc(uint32_t saddr) {
   return (unsigned long long)((saddr & 0x3ffffu) >> 4) | (1ull << 16) | ((unsigned long long)(1024 >> 4) << 32) |
@@ -218,6 +224,8 @@ __device__ __forceinline__ unsigned long long add_f32x2(unsigned long long a, un
 // Host: tensor map over a [rows, 64*k] bf16 row-major tensor, box = box_rows x 64 columns,
 // 128-byte swizzle.  Returns false when the driver entry point is unavailable.
 bool make_tile_map(CUtensorMap* tm, const void* base, long long rows, int cols, int box_rows);
+// The same over [blocks, rows, 64*k]: rows of a box past the end of its block read as 0, not as the next block's.
+bool make_block_tile_map(CUtensorMap* tm, const void* base, long long blocks, int rows, int cols, int box_rows);
 
 }  // namespace tc
 }  // namespace sq

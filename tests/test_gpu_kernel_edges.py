@@ -321,6 +321,46 @@ def test_h2o_forms_of_larger_launches(dtype, head_dim, hq, hkv, batch, budgets, 
     lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack)
 
 
+# Rows of a tile past a unit's heads (decode) or a head's prompt (prompt scores) are the next sequence's: a NaN or an infinity there
+# changes no bit of this one's scores.  Wide groups with the scores in the attention launch and in one of their own
+@pytest.mark.parametrize("hq,batch,budget", [(71, 3, 400), (33, 2, 150), (97, 2, 300), (65, 160, 140)])
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+def test_decode_scores_of_a_sequence_stand_alone(hq, batch, budget, bad):
+    got = []
+    for spoilt in (False, True):
+        w = workload("alone", 9250 + hq, n_q_head=hq, n_kv_head=1, batch=batch, prompt=budget + 9, heavy_mode="none")
+        ctx = H.make_ctx(w, b_init=budget)
+        ctx.begin_sequence_batch(batch, w.prompt)
+        ctx.set_budgets([budget])
+        _, k, v = synth.prompt_qkv(w, 0, DEV, need_q=False)
+        ctx.prefill_compress(0, k, v, None, synth.prompt_scores_standin(w, 0, DEV))
+        q, kn, vn = synth.decode_qkv(w, 0, DEV)
+        if spoilt:
+            q[:, 1] = bad
+        out = torch.empty_like(q)
+        ctx.decode_step(0, 1, q, kn, vn, out)
+        got.append((ctx.get_kept(0, 0, 0), out[0, 0].clone()))
+    assert got[0][0] == got[1][0] and torch.equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("head_dim,hq,hkv,prompt", [(64, 4, 2, 333), (64, 130, 2, 333), (128, 4, 2, 200), (64, 2, 2, 31)])
+def test_prompt_scores_of_a_sequence_stand_alone(dtype, head_dim, hq, hkv, prompt):
+    got = []
+    for spoilt in (False, True):
+        w = workload("alone", 9260, dtype=dtype, head_dim=head_dim, n_q_head=hq, n_kv_head=hkv, batch=2, prompt=prompt, heavy_mode="none")
+        ctx = H.make_ctx(w, b_init=prompt)
+        ctx.begin_sequence_batch(2, prompt)
+        ctx.set_budgets([prompt])
+        q, k, v = synth.prompt_qkv(w, 0, DEV)
+        if spoilt:
+            q[0, hq // hkv:] = float("nan")
+            q[1, 0] = float("inf")
+        ctx.prefill_compress(0, k, v, q)
+        got.append([ctx.get_kept(0, s, h)[1] for s, h in ((0, 0), (1, hkv - 1))])
+    assert got[0] == got[1]
+
+
 # Wide groups with the pieces of a unit on the CTAs of a cluster: two pieces to the most there are, pieces of one tile and of
 # unlike numbers of tiles, a last tile of one slot, the smallest group and the largest that is taken and the next, groups that
 # fill no eight, a launch whose layers differ too much for it (split-K); with the scores and without
