@@ -294,11 +294,14 @@ __device__ __forceinline__ void finish_cluster(const Args& a, const LayerDesc* l
 }  // namespace
 
 // ROWS: rows of the Q tile held in shared memory (120 for up to 96 heads, else 128; see sq_tc_rows.cuh).
-// CLUSTER: the pieces of a unit are the CTAs of a cluster (Args: DecodeArgsBase), see the head of the file.
-template <int STAGES, int ROWS, bool H2O, bool CLUSTER, class Args>
+// FORM: split-K, or the pieces of a unit as the CTAs of a cluster (Args: DecodeArgsBase), see the head of the file; kClusterMax: with a
+// row's maximum so far as its reference throughout.
+enum WideForm { kSplitK, kCluster, kClusterMax };
+template <int STAGES, int ROWS, bool H2O, WideForm FORM, class Args>
 __global__ void __launch_bounds__(192, 2)
     decode_attn_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                           const __grid_constant__ CUtensorMap tm_v, Args a) {
+  constexpr bool CLUSTER = FORM != kSplitK;
   constexpr int kQBytes = ROWS * 128;
   constexpr int kSlots = ROWS == 120 ? 3 : 4;
   extern __shared__ unsigned char smem_raw[];
@@ -565,11 +568,17 @@ __global__ void __launch_bounds__(192, 2)
       ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld / st are warp-wide
       if (!ok) break;
       tc_fence_after();
-      bool s_released = rows.tile(n_valid, i == 0, bar_sfree, [&]() {
+      float f_o = 1.f;
+      const bool moved = FORM == kClusterMax && i > 0 && rows.follow(n_valid, &f_o);
+      bool s_released = rows.template tile<FORM == kClusterMax>(n_valid, i == 0, bar_sfree, [&]() {
         if (i >= 1) ok = __all_sync(0xffffffffu, mbar_wait(bar_pfree, (i - 1) & 1, abort_flag));
+        if (FORM == kClusterMax && ok && moved) {  // (P is free once the product that O is waiting for is complete)
+          tc_fence_after();
+          rows.scale_o(f_o);
+        }
       });
       if (!ok) break;
-      if (rows.too_large()) {
+      if (FORM != kClusterMax && rows.too_large()) {
         ok = __all_sync(0xffffffffu, mbar_wait(bar_odone, (i - 1) & 1, abort_flag));
         if (!ok) break;
         tc_fence_after();
@@ -662,14 +671,21 @@ __global__ void __launch_bounds__(192) cluster_room_kernel() {}
 // Pieces per unit: as many as all units' clusters find room for at the same time, then as few as give the longest
 // piece as many tiles.  Measured, us per launch with 4, 5, 6, 7, 8 pieces: 33 units of 58 tiles 47, 44, 38, 36, 34; of
 // 10 tiles 17, 15, 14, 14, 15.5.
+// *follow: bf16 holds the weight of a piece's reference exactly, so that the more pieces a unit has, the closer its outputs are
+// to fp64.  Where split-K would cut shorter pieces than these, the references follow the rows' maxima instead (kClusterMax).  Error
+// against fp64 of 8 sequences of 8191 tokens, logits of standard deviation 1, 2, 3, split-K / a fixed reference / this: 2.25e-3 /
+// 2.32e-3 / 2.21e-3, 2.01e-3 / 2.17e-3 / 1.79e-3, 1.89e-3 / 2.00e-3 / 1.70e-3; us per launch 49.8 / 17.5 / 20.1.
 // 0 where not even two fit, or where units of unlike length leave the longest piece too far above an even share of the
 // launch's tiles (a cluster cuts every unit into the same number of pieces; split-K cuts the long ones into more).  Time of
 // split-K, two launches with H2O, over this form, 32 layers in one launch, by the excess in tiles: without scores 4: 1.85, 7:
 // 1.16, 10: 1.05 and 1.07, 15: 0.98, 40: 0.63; H2O 4: 1.63, 5: 1.10, 7: 1.17 (8 pieces), 1.06 and 0.92 (2 pieces: the less
-// to merge, the less this form saves), 10: 0.95 and 0.96, 15: 0.85.
-// Launches of one layer, split-K / this form, us per token of 32 layers: 1 sequence of 512 tokens 289 / 246, 16384: 1621 / 470, 8
-// of 8191 1043 / 444, 33 of 1024 457 / 357, 100 of 3000 741 / 630; H2O 452 / 358, 1883 / 669, 1329 / 580, 658 / 438, 1130 / 950.
-static int cluster_pieces(const DecodeArgs& a, const int* desc_tiles, size_t smem) {
+// to merge, the less this form saves), 10: 0.95 and 0.96, 15: 0.85.  With references that follow the line falls with the pieces, by
+// pieces and excess: without scores 2 pieces 4: 1.10, 5: 0.99, 6: 0.93; 3: 4: 1.01, 7: 0.93; 4: 5: 1.07, 6: 0.99, 8: 0.92; 5: 7: 1.18, 9:
+// 1.05 and 0.97; 6: 6: 1.10, 8: 0.99; 8: 8: 1.30; H2O 2: 3: 1.06, 5: 0.97; 3: 4: 0.87; 4: 4: 1.09, 5: 0.95; 5: 5: 1.14, 7: 0.95; 6: 3: 1.12, 6: 0.98; 8:
+// 4: 1.18 and 1.40, 8: 1.07.
+// Launches of one layer, split-K / this form, us: 1 sequence of 4096 tokens 28.0 / 12.9, 16384: 84 / 25.5, 16 of 8191 35.6 / 22.6, 20 of 4000
+// 29.5 / 16.4, 33 of 8191 32.3 / 24.3; H2O 1 of 16384 96 / 37.6, 8 of 8191 61 / 28.6, 33 of 8191 49.6 / 38.4, of 2457 34.4 / 20.0.
+static int cluster_pieces(const DecodeArgs& a, const int* desc_tiles, size_t smem, bool* follow) {
   static PerDevice set_up;
   static ClusterCount room;
   const void* kern = reinterpret_cast<const void*>(cluster_room_kernel);
@@ -687,17 +703,22 @@ static int cluster_pieces(const DecodeArgs& a, const int* desc_tiles, size_t sme
   const int longest = (max_tiles + n - 1) / n;
   const long long total = std::accumulate(desc_tiles, desc_tiles + a.n_layer_total, 0LL) * a.n_unit;
   const long long even = std::max(total / (2LL * sm_count()), (long long)max_tiles / kMaxPieces);
-  if (min_tiles < max_tiles && longest > even + (a.policy != SQ_POLICY_H2O ? 12 : n == 2 ? 6 : 8)) return 0;
+  const bool h2o = a.policy == SQ_POLICY_H2O;
+  *follow = longest * kTM > a.split_tokens;
+  const int excess = *follow ? (h2o ? n : n + 2) : !h2o ? 12 : n == 2 ? 6 : 8;
+  if (min_tiles < max_tiles && longest > even + excess) return 0;
   while (n > 2 && (max_tiles + n - 2) / (n - 1) == longest && units <= room.active(kern, n - 1, 192, smem)) --n;
   return n;
 }
 
-template <bool H2O>
-static cudaError_t launch_tc_cluster(const DecodeArgs& a, const int* desc_tiles, const CUtensorMap& tq, const CUtensorMap& tk,
-                                     const CUtensorMap& tv, cudaStream_t s) {
-  constexpr int STAGES = 3, ROWS = 120;
-  constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 8 * 16 + 16;
-  auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O, true, DecodeArgsBase>;
+constexpr int kClusterStages = 3, kClusterRows = 120;
+constexpr size_t kClusterSmem = 1024 + (size_t)kClusterRows * 128 + (size_t)2 * kClusterStages * kTileBytes + 8 * 16 + 16;
+
+template <bool H2O, WideForm FORM>
+static cudaError_t launch_tc_cluster(const DecodeArgs& a, int n, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                                     cudaStream_t s) {
+  constexpr size_t smem = kClusterSmem;
+  auto kern = decode_attn_tc_kernel<kClusterStages, kClusterRows, H2O, FORM, DecodeArgsBase>;
   static PerDevice set_up;
   const cudaError_t e = set_up.once([&] {
     cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -705,8 +726,7 @@ static cudaError_t launch_tc_cluster(const DecodeArgs& a, const int* desc_tiles,
   });
   if (e != cudaSuccess) return e;
   static ClusterCount own;  // (a device that holds no cluster of that size at all)
-  const int n = cluster_pieces(a, desc_tiles, smem);
-  if (n == 0 || own.active(reinterpret_cast<const void*>(kern), n, 192, smem) == 0) return cudaErrorNotSupported;
+  if (own.active(reinterpret_cast<const void*>(kern), n, 192, smem) == 0) return cudaErrorNotSupported;
   return launch_chained_cluster(kern, n, a.n_layer_total * a.n_unit * n, 192, smem, s, tq, tk, tv, static_cast<const DecodeArgsBase&>(a));
 }
 
@@ -715,7 +735,7 @@ static cudaError_t launch_tc_cfg(const DecodeArgs& a, int n_items, const CUtenso
                                  const CUtensorMap& tv, cudaStream_t s) {
   constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 8 * 16 + 16;
   static_assert(2 * (smem + 1024 + 64) <= 228 * 1024, "two CTAs per SM");
-  auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O, false, DecodeArgs>;
+  auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O, kSplitK, DecodeArgs>;
   static PerDevice set_up;
   const cudaError_t e = allow_smem(set_up, smem, kern);
   if (e != cudaSuccess) return e;
@@ -735,8 +755,12 @@ cudaError_t launch_decode_attn_tc_cluster(const DecodeArgs& a, const int* desc_t
   if (a.group > kClusterHeads) return cudaErrorNotSupported;
   CUtensorMap tm_q, tm_k, tm_v;
   if (!make_maps(a, pool_bytes, q_rows, &tm_q, &tm_k, &tm_v)) return cudaErrorNotSupported;
-  return a.policy == SQ_POLICY_H2O ? launch_tc_cluster<true>(a, desc_tiles, tm_q, tm_k, tm_v, s)
-                                   : launch_tc_cluster<false>(a, desc_tiles, tm_q, tm_k, tm_v, s);
+  bool follow = false;
+  const int n = cluster_pieces(a, desc_tiles, kClusterSmem, &follow);
+  if (n == 0) return cudaErrorNotSupported;
+  auto launch = a.policy == SQ_POLICY_H2O ? follow ? launch_tc_cluster<true, kClusterMax> : launch_tc_cluster<true, kCluster>
+                : follow ? launch_tc_cluster<false, kClusterMax> : launch_tc_cluster<false, kCluster>;
+  return launch(a, n, tm_q, tm_k, tm_v, s);
 }
 
 // Returns cudaErrorNotSupported when the shape is outside this kernel's range.

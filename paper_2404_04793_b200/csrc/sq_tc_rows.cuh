@@ -132,7 +132,8 @@ struct WideRows {
   // returns whether it was.
   // p_free() waits for the product that still reads the tile before's P: before the first store only, so
   // that the first 64 columns are worked out meanwhile.
-  template <int HF, bool TWO, bool LAST, class PFree>
+  // SCALES: p_free() may also have O to scale, for which the load in flight has to be complete.
+  template <int HF, bool TWO, bool LAST, bool SCALES, class PFree>
   __device__ __forceinline__ bool half(int n_valid, bool first, uint32_t bar_sfree, bool wait_p, PFree p_free) {
     constexpr int A = 2 * HF, B = TWO ? 2 * HF + 1 : 2 * HF;
     const uint32_t s = s_addr + ((uint32_t)(16 * HF) << 16), p = p_addr + ((uint32_t)(16 * HF) << 16);
@@ -153,6 +154,7 @@ struct WideRows {
     }
     uint32_t pk[16];
     chunk<TWO>(ra, pk, m[A], m[B], la, lb, w);
+    if (SCALES && wait_p) tmem_wait_ld(rb);
     if (wait_p) p_free();
     tmem_st16x128_x8_u32(p, pk);
     tmem_wait_ld(rb);
@@ -186,13 +188,13 @@ struct WideRows {
   }
   // A whole tile; returns whether S was handed back.  A row's weights are too large when one of its
   // threads' sums is: redo() follows.
-  template <class PFree>
+  template <bool SCALES = false, class PFree>
   __device__ __forceinline__ bool tile(int n_valid, bool first, uint32_t bar_sfree, PFree p_free) {
     const bool upper = n_slot >= 3;
-    if (SLOTS == 4 && n_slot == 4) half<1, SLOTS == 4, false>(n_valid, first, bar_sfree, true, p_free);
-    else if (upper) half<1, false, false>(n_valid, first, bar_sfree, true, p_free);
-    const bool released = n_slot >= 2 ? half<0, true, true>(n_valid, first, bar_sfree, !upper, p_free)
-                                      : half<0, false, true>(n_valid, first, bar_sfree, !upper, p_free);
+    if (SLOTS == 4 && n_slot == 4) half<1, SLOTS == 4, false, SCALES>(n_valid, first, bar_sfree, true, p_free);
+    else if (upper) half<1, false, false, SCALES>(n_valid, first, bar_sfree, true, p_free);
+    const bool released = n_slot >= 2 ? half<0, true, true, SCALES>(n_valid, first, bar_sfree, !upper, p_free)
+                                      : half<0, false, true, SCALES>(n_valid, first, bar_sfree, !upper, p_free);
     tmem_wait_st();
     return released;
   }
@@ -234,6 +236,28 @@ struct WideRows {
     }
     float f_o = of_lane(f);
     if ((lane >> 3) >= n_slot) f_o = 1.f;
+    scale_o(f_o);
+  }
+  // Ahead of a tile: the references of the rows that have their largest logit so far in it move there, and the sums shrink with
+  // them.  Returns whether any did; O is to be multiplied by f_o once the tile before's product is complete.
+  __device__ __forceinline__ bool follow(int n_valid, float* f_o) {
+    float mx[SLOTS], f[SLOTS];
+    bool up = false;
+    tile_max(n_valid, mx);
+#pragma unroll
+    for (int s = 0; s < SLOTS; ++s) {
+      const bool rise = s < n_slot && mx[s] > m[s];
+      f[s] = rise ? ex2(m[s] - mx[s]) : 1.f;
+      l[s] *= f[s];
+      l_w[s] *= f[s];
+      if (rise) m[s] = mx[s];
+      up = up || rise;
+    }
+    *f_o = of_lane(f);
+    return __any_sync(0xffffffffu, up);
+  }
+  // O times this lane's factor
+  __device__ __forceinline__ void scale_o(float f_o) {
 #pragma unroll 1
     for (int c = 0; c < 2; ++c) {
       float o[32];

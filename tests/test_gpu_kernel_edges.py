@@ -217,8 +217,7 @@ def test_one_and_eight_heads_per_kv_head(head_dim, budget, hq):
 # and the others' nearly cancel, so that the bf16 output does not hide the weights.
 @pytest.mark.parametrize("head_dim,group", [(128, 1), (64, 2), (128, 3), (128, 4), (64, 5), (128, 8), (128, 9), (64, 32), (64, 36), (64, 71), (64, 128)])
 @pytest.mark.parametrize("policy", [synth.SLIDING_WINDOW, synth.H2O])
-def test_the_largest_weight_is_not_rounded(policy, head_dim, group):
-    n, at = 128, 100
+def test_the_largest_weight_is_not_rounded(policy, head_dim, group, n=128, at=100):
     w = workload("peak", 9600 + group, policy=policy, head_dim=head_dim, n_q_head=group, n_kv_head=1, prompt=n, steps=1, heavy_mode="none")
     g = torch.Generator().manual_seed(group)
     rnd = lambda *s: torch.randn(*s, generator=g)
@@ -256,6 +255,14 @@ def test_the_largest_weight_is_not_rounded(policy, head_dim, group):
     err = np.abs(H.f64(out[0, 0]) - want)
     assert np.all(err <= bound), float((err / bound).max())
     assert ctx.status() == 0
+
+
+# Wide groups, few long units: pieces of several tiles on the CTAs of a cluster.  The key lies in a piece's first tile, a later one
+# and the new token's tile
+@pytest.mark.parametrize("group,at", [(71, 100), (71, 700), (71, 3333), (71, 7980), (33, 1900), (96, 4500)])
+@pytest.mark.parametrize("policy", [synth.SLIDING_WINDOW, synth.H2O])
+def test_the_largest_weight_of_a_long_unit_is_not_rounded(policy, group, at):
+    test_the_largest_weight_is_not_rounded(policy, 64, group, 8000, at)
 
 
 def lockstep(dtype, head_dim, hq, hkv, batch, budgets, stack, policy=synth.H2O):
