@@ -685,21 +685,13 @@ __global__ void __launch_bounds__(192) cluster_room_kernel() {}
 // 4: 1.18 and 1.40, 8: 1.07.
 // Launches of one layer, split-K / this form, us: 1 sequence of 4096 tokens 28.0 / 12.9, 16384: 84 / 25.5, 16 of 8191 35.6 / 22.6, 20 of 4000
 // 29.5 / 16.4, 33 of 8191 32.3 / 24.3; H2O 1 of 16384 96 / 37.6, 8 of 8191 61 / 28.6, 33 of 8191 49.6 / 38.4, of 2457 34.4 / 20.0.
-static int cluster_pieces(const DecodeArgs& a, const int* desc_tiles, size_t smem, bool* follow) {
-  static PerDevice set_up;
-  static ClusterCount room;
-  const void* kern = reinterpret_cast<const void*>(cluster_room_kernel);
-  if (set_up.once([&] {
-        const cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        return r == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
-      }) != cudaSuccess)
-    return 0;
+template <class Room>
+static int cluster_pieces(const DecodeArgs& a, const int* desc_tiles, Room room, bool* follow) {
   const long long units = (long long)a.n_layer_total * a.n_unit;
   const auto [lo, hi] = std::minmax_element(desc_tiles, desc_tiles + a.n_layer_total);
   const int min_tiles = *lo, max_tiles = *hi;
-  int n = std::min(kMaxPieces, min_tiles);
-  while (n >= 2 && units > room.active(kern, n, 192, smem)) --n;
-  if (n < 2) return 0;
+  int n = most_ctas(std::min(kMaxPieces, min_tiles), units, room);
+  if (n == 0) return 0;
   const int longest = (max_tiles + n - 1) / n;
   const long long total = std::accumulate(desc_tiles, desc_tiles + a.n_layer_total, 0LL) * a.n_unit;
   const long long even = std::max(total / (2LL * sm_count()), (long long)max_tiles / kMaxPieces);
@@ -707,27 +699,41 @@ static int cluster_pieces(const DecodeArgs& a, const int* desc_tiles, size_t sme
   *follow = longest * kTM > a.split_tokens;
   const int excess = *follow ? (h2o ? n : n + 2) : !h2o ? 12 : n == 2 ? 6 : 8;
   if (min_tiles < max_tiles && longest > even + excess) return 0;
-  while (n > 2 && (max_tiles + n - 2) / (n - 1) == longest && units <= room.active(kern, n - 1, 192, smem)) --n;
+  while (n > 2 && (max_tiles + n - 2) / (n - 1) == longest && units <= room(n - 1)) --n;
   return n;
 }
 
-constexpr int kClusterStages = 3, kClusterRows = 120;
-constexpr size_t kClusterSmem = 1024 + (size_t)kClusterRows * 128 + (size_t)2 * kClusterStages * kTileBytes + 8 * 16 + 16;
-
-template <bool H2O, WideForm FORM>
-static cudaError_t launch_tc_cluster(const DecodeArgs& a, int n, const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                                     cudaStream_t s) {
-  constexpr size_t smem = kClusterSmem;
-  auto kern = decode_attn_tc_kernel<kClusterStages, kClusterRows, H2O, FORM, DecodeArgsBase>;
+template <bool H2O>
+static cudaError_t launch_tc_cluster(const DecodeArgs& a, const int* desc_tiles, const CUtensorMap& tq, const CUtensorMap& tk,
+                                     const CUtensorMap& tv, cudaStream_t s) {
+  constexpr int STAGES = 3, ROWS = 120;
+  constexpr size_t smem = 1024 + (size_t)ROWS * 128 + (size_t)2 * STAGES * kTileBytes + 8 * 16 + 16;
+  auto kern = decode_attn_tc_kernel<STAGES, ROWS, H2O, kCluster, DecodeArgsBase>;
+  auto kern_max = decode_attn_tc_kernel<STAGES, ROWS, H2O, kClusterMax, DecodeArgsBase>;
+  const void* const all[3] = {reinterpret_cast<const void*>(cluster_room_kernel), reinterpret_cast<const void*>(kern),
+                              reinterpret_cast<const void*>(kern_max)};
   static PerDevice set_up;
   const cudaError_t e = set_up.once([&] {
-    cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return r == cudaSuccess ? cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) : r;
+    cudaError_t r = cudaSuccess;
+    for (const void* k : all) {
+      if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      if (r == cudaSuccess) r = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    }
+    return r;
   });
   if (e != cudaSuccess) return e;
-  static ClusterCount own;  // (a device that holds no cluster of that size at all)
-  if (own.active(reinterpret_cast<const void*>(kern), n, 192, smem) == 0) return cudaErrorNotSupported;
-  return launch_chained_cluster(kern, n, a.n_layer_total * a.n_unit * n, 192, smem, s, tq, tk, tv, static_cast<const DecodeArgsBase&>(a));
+  static ClusterCount count[3];
+  auto room = [&](int ctas) {  // (none of a size that the device does not hold for one of the kernels at all)
+    int n = count[0].active(all[0], ctas, 192, smem);
+    for (int k = 1; k < 3; ++k)
+      if (count[k].active(all[k], ctas, 192, smem) == 0) n = 0;
+    return n;
+  };
+  bool follow = false;
+  const int n = cluster_pieces(a, desc_tiles, room, &follow);
+  if (n == 0) return cudaErrorNotSupported;
+  return launch_chained_cluster(follow ? kern_max : kern, n, a.n_layer_total * a.n_unit * n, 192, smem, s, tq, tk, tv,
+                                static_cast<const DecodeArgsBase&>(a));
 }
 
 template <int STAGES, int ROWS, bool H2O>
@@ -755,12 +761,8 @@ cudaError_t launch_decode_attn_tc_cluster(const DecodeArgs& a, const int* desc_t
   if (a.group > kClusterHeads) return cudaErrorNotSupported;
   CUtensorMap tm_q, tm_k, tm_v;
   if (!make_maps(a, pool_bytes, q_rows, &tm_q, &tm_k, &tm_v)) return cudaErrorNotSupported;
-  bool follow = false;
-  const int n = cluster_pieces(a, desc_tiles, kClusterSmem, &follow);
-  if (n == 0) return cudaErrorNotSupported;
-  auto launch = a.policy == SQ_POLICY_H2O ? follow ? launch_tc_cluster<true, kClusterMax> : launch_tc_cluster<true, kCluster>
-                : follow ? launch_tc_cluster<false, kClusterMax> : launch_tc_cluster<false, kCluster>;
-  return launch(a, n, tm_q, tm_k, tm_v, s);
+  return a.policy == SQ_POLICY_H2O ? launch_tc_cluster<true>(a, desc_tiles, tm_q, tm_k, tm_v, s)
+                                   : launch_tc_cluster<false>(a, desc_tiles, tm_q, tm_k, tm_v, s);
 }
 
 // Returns cudaErrorNotSupported when the shape is outside this kernel's range.

@@ -42,39 +42,6 @@ inline cudaError_t allow_smem(PerDevice& state, size_t bytes, K... kern) {
   });
 }
 
-// Whether the current device holds a cluster of `ctas` CTAs of a kernel (which is allowed that size) with `smem` bytes
-// of dynamic shared memory each.  Above the portable 8 that depends on the device and on what is left of it
-// (partitions, disabled SMs).  For static storage, one per kernel; asked once on every device, with the largest
-// ctas and smem that the kernel is launched with.
-class ClusterFit {
- public:
-  bool fits(const void* kern, int ctas, int threads, size_t smem) {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    const bool known = dev >= 0 && dev < kMaxDevices;
-    const int seen = known ? state_[dev].load(std::memory_order_relaxed) : 0;
-    if (seen) return seen == 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(ctas);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = ctas;
-    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int n = 0;
-    const bool ok = cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0;
-    if (!ok) cudaGetLastError();
-    if (known) state_[dev].store(ok ? 1 : 2, std::memory_order_relaxed);
-    return ok;
-  }
-
- private:
-  std::atomic<int> state_[kMaxDevices] = {};
-};
-
 // Clusters of `ctas` CTAs of a kernel that the current device runs at a time, by size (up to 16).  For static
 // storage, one per kernel and amount of shared memory; asked once for every size on every device.
 class ClusterCount {
@@ -108,6 +75,26 @@ class ClusterCount {
   static constexpr int kSizes = 16;
   std::atomic<int> count_[kMaxDevices][kSizes] = {};
 };
+
+// Whether the current device holds a cluster of `ctas` CTAs of a kernel (which is allowed that size) with `smem` bytes
+// of dynamic shared memory each.  Above the portable 8 that depends on the device and on what is left of it
+// (partitions, disabled SMs).  For static storage, one per kernel; asked once for every size on every device, with the most smem
+// that the kernel is launched with.
+class ClusterFit {
+ public:
+  bool fits(const void* kern, int ctas, int threads, size_t smem) { return count_.active(kern, ctas, threads, smem) > 0; }
+
+ private:
+  ClusterCount count_;
+};
+
+// The most CTAs per cluster, up to `limit` and at least two, with room for `units` clusters at a time; 0 where there is none.
+// room(ctas): how many clusters of that size the device runs at a time.
+template <class Room>
+inline int most_ctas(int limit, long long units, Room room) {
+  while (limit >= 2 && room(limit) < units) --limit;
+  return limit >= 2 ? limit : 0;
+}
 
 // launch(limit) with clusters of at most `limit` CTAs, and where the device does not hold those (or the plan does not
 // work out) with at most the portable 8.

@@ -95,6 +95,29 @@ def run_host_program(tmp_path, source):
     return subprocess.run([str(exe)], capture_output=True, text=True, timeout=60).stdout.strip()
 
 
+PIECES = r"""
+#include <cstdio>
+#include "sq_device_state.h"
+int main() {
+  // room of a device by cluster size: as many CTAs as there are slots, none of more than `largest`
+  int slots = 264, largest = 16;
+  auto room = [&](int ctas) { return ctas <= largest ? slots / ctas : 0; };
+  bool ok = sq::most_ctas(14, 1, room) == 14 && sq::most_ctas(14, 33, room) == 8 && sq::most_ctas(14, 132, room) == 2 &&
+            sq::most_ctas(14, 133, room) == 0 && sq::most_ctas(1, 1, room) == 0 && sq::most_ctas(3, 1, room) == 3;
+  largest = 8;   // a device without the larger sizes: the portable ones are still taken
+  ok = ok && sq::most_ctas(14, 1, room) == 8 && sq::most_ctas(14, 33, room) == 8 && sq::most_ctas(14, 60, room) == 4;
+  largest = 0;
+  ok = ok && sq::most_ctas(14, 1, room) == 0;
+  std::puts(ok ? "ok" : "wrong");
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
+def test_pieces_of_a_unit_shrink_to_the_clusters_that_a_device_holds(tmp_path):
+    assert run_host_program(tmp_path, PIECES) == "ok"
+
+
 @pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
 def test_set_up_clusters_and_sm_count_are_kept_by_device(tmp_path):
     assert run_host_program(tmp_path, PROGRAM) == "ok"
