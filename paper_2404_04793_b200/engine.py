@@ -155,8 +155,10 @@ class Job:
         w = self.w
         per_layer = self.per_layer_decode if per_layer_decode is None else per_layer_decode
         h2o = w.policy == synth.H2O
-        # H2O: two scoring sweeps (unless stand-in scores are given), selection with copies
-        per_layer_prefill = ((0 if inp.acc is not None else 2) + 1) if h2o else 1
+        # H2O: two scoring sweeps (unless stand-in scores are given), selection with copies; short fp32 prompts (up to 20
+        # pairs of a head and 32 queries per KV head) are scored by one launch
+        short = w.dtype == torch.float32 and w.group * -(-w.prompt // 32) <= 20
+        per_layer_prefill = ((0 if inp.acc is not None else 1 if short else 2) + 1) if h2o else 1
         groups = w.n_layer if per_layer else 1
         return w.n_layer * inp.hidden_repeat + 1 + w.n_layer * per_layer_prefill + w.steps * groups
 

@@ -47,3 +47,20 @@ def test_kernel_names_are_those_launched(hq, hkv, head_dim, batch, budgets, dtyp
         torch.cuda.synchronize()
     names = {e.key.split("<")[0].split("::")[-1] for e in prof.key_averages() if "decode_attn" in e.key}
     assert names == {bench.decode_kernel_of(w, budgets, per_layer)}
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("over", [{}, dict(prompt=700), dict(dtype=torch.bfloat16), dict(policy=synth.SLIDING_WINDOW)])
+def test_counted_launches_are_made(over):
+    """The launches of a pass that the bench counts are at least made, and no more are counted."""
+    from paper_2404_04793_b200 import engine
+    w = synth.tiny().replace(steps=3, **over)
+    job, inp = engine.Job(w, "cuda"), engine.ResidentInputs(w, "cuda")
+    job.run(inp)
+    torch.cuda.synchronize()
+    with torch.profiler.profile(activities=[torch.profiler.ProfilerActivity.CUDA]) as prof:
+        job.run(inp)
+        torch.cuda.synchronize()
+    made = sum(e.count for e in prof.key_averages() if "sq::" in e.key)
+    counted = job.kernel_launches_per_pass(inp)
+    assert counted <= made <= counted + w.n_layer + w.steps   # copies of many heavy rows, a second launch of a decode step
