@@ -21,8 +21,8 @@ namespace sq {
 // prompts and by the chain of tiles of a CTA for small ones: there TQ is 32, and the second sweep's
 // stream is cut into pieces whose column sums the last to finish adds up in order (deterministic).
 // Measured, us per layer of scores, selection and gather, fp32, 64 x 64 tiles with scalar reads and one CTA per
-// key tile / this: 1 sequence of 256 tokens, 2 / 2 heads of 64: 79.6 / 25.9; 2 of 777, 16 / 4 heads of 128: 798 /
-// 286; 20 of 500, 20 / 1 heads of 64: 1627 / 585; 1 of 2048, 32 / 32 heads of 128: 2143 / 1395.
+// key tile / this: 2 sequences of 777 tokens, 16 / 4 heads of 128: 798 / 286; 20 of 500, 20 / 1 heads of 64: 1627 / 585; 1 of
+// 2048, 32 / 32 heads of 128: 2143 / 1395.  (Short prompts: prefill_rows_kernel.)
 // ---------------------------------------------------------------------------------------
 constexpr int TK = 64;
 
@@ -255,7 +255,6 @@ __global__ void __launch_bounds__(4 * TQ) prefill_col_sum_kernel(ScoreArgs a, fl
 // The chain of a CTA (all keys of its rows) and of the last pair grow with the prompt: of more than 20 pairs per KV head
 // launches of few CTAs are no faster (1 sequence of 700, 2 / 2 heads of 64, 45.8 / 46.5).
 constexpr int kRowsPairs = 20;
-constexpr size_t kRowsSmem = 160 * 1024;
 template <int D>
 constexpr size_t rows_smem(int n_kt) {
   return score_smem<D, 32>() + (size_t)32 * (n_kt * TK + 4) * 4;
@@ -376,14 +375,14 @@ static cudaError_t launch_scores_rows(const ScoreArgs& a, cudaStream_t s) {
   const int n_qt = (a.prompt + 31) / 32, n_kt = (a.prompt + TK - 1) / TK, g = a.n_q_head / a.n_kv_head;
   const long long pairs = (long long)g * n_qt;
   if (pairs > kRowsPairs) return cudaErrorNotSupported;
-  const size_t smem = rows_smem<D>(n_kt);
-  if (smem > kRowsSmem) return cudaErrorNotSupported;
+  constexpr size_t kMost = rows_smem<D>((kRowsPairs * 32 + TK - 1) / TK);  // of one head per KV head
+  static_assert(kMost <= 227 * 1024, "shared memory of a CTA");
   if (pairs * a.batch * a.n_kv_head * a.prompt > (long long)a.partial_floats) return cudaErrorNotSupported;
   auto kern = prefill_rows_kernel<T, D>;
   static PerDevice set_up;
-  const cudaError_t e = allow_smem(set_up, kRowsSmem, kern);
+  const cudaError_t e = allow_smem(set_up, kMost, kern);
   if (e != cudaSuccess) return e;
-  return launch_chained(kern, dim3(n_qt, a.n_q_head, a.batch), 128, smem, s, a, 1.4426950408889634f / sqrtf((float)D));
+  return launch_chained(kern, dim3(n_qt, a.n_q_head, a.batch), 128, rows_smem<D>(n_kt), s, a, 1.4426950408889634f / sqrtf((float)D));
 }
 
 template <typename T, int D, int TQ>
