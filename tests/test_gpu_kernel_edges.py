@@ -370,14 +370,46 @@ def test_prompt_scores_of_a_sequence_stand_alone(dtype, head_dim, hq, hkv, promp
 
 # Wide groups with the pieces of a unit on the CTAs of a cluster: two pieces to the most there are, pieces of one tile and of
 # unlike numbers of tiles, a last tile of one slot, the smallest group and the largest that is taken and the next, groups that
-# fill no eight, a launch whose layers differ too much for it (split-K); with the scores and without
+# fill no eight, pieces of several tiles whose references follow the maxima, launches whose layers differ too much for the
+# form in one call (split-K; the smallest group and the largest too); with the scores and without
 @pytest.mark.parametrize("hq,batch,budgets", [
     (71, 1, [1792, 257]), (33, 2, [1921, 129]), (96, 3, [700, 1300]), (97, 2, [300, 260]), (72, 37, [260, 900]), (40, 75, [385, 290]),
-    (71, 4, [6000, 300, 260]), (65, 149, [257, 300])])
+    (71, 4, [6000, 300, 260]), (65, 149, [257, 300]), (33, 3, [4000, 150]), (96, 2, [3000, 129, 1000]), (71, 2, [5000, 2600])])
 @pytest.mark.parametrize("stack", [False, True])
 @pytest.mark.parametrize("policy", [synth.H2O, synth.SLIDING_WINDOW])
 def test_wide_groups_over_a_cluster(hq, batch, budgets, stack, policy):
     lockstep(torch.bfloat16, 64, hq, 1, batch, budgets, stack, policy)
+
+
+# Keys that grow within every piece, so that references move after a piece's first tile: to the maximum of each tile (one long
+# unit), or where a weight would be too large (pieces as long as split-K's)
+@pytest.mark.parametrize("batch,prompt", [(1, 6000), (33, 2400)])
+@pytest.mark.parametrize("policy", [synth.H2O, synth.SLIDING_WINDOW])
+def test_growing_logits_over_a_cluster(policy, batch, prompt):
+    w = workload("grow", 9280, policy=policy, n_q_head=71, n_kv_head=1, batch=batch, prompt=prompt, steps=2, heavy_mode="none")
+    b = prompt + 40
+    ctx = H.make_ctx(w, b_init=b)
+    ctx.begin_sequence_batch(batch, prompt)
+    ctx.set_budgets([b])
+    _, k, v = synth.prompt_qkv(w, 0, DEV, need_q=False)
+    k *= (1 + torch.arange(prompt, device=DEV) % 384 / 16).to(k)[:, None]
+    acc = torch.zeros(batch, 1, prompt, device=DEV) if policy == synth.H2O else None
+    ctx.prefill_compress(0, k, v, None, acc)
+    units = {s: O.UnitCache(policy, b, w.n_sink, w.heavy_num, w.heavy_den) for s in sorted({0, batch - 1})}
+    for s, u in units.items():
+        u.prefill(H.f64(k[s, 0]), H.f64(v[s, 0]), None, np.zeros(prompt))
+    for t in range(w.steps):
+        q, kn, vn = synth.decode_qkv(w, t, DEV)
+        out = torch.empty_like(q)
+        ctx.decode_step(0, 1, q, kn, vn, out)
+        for s, u in units.items():
+            want = u.decode_step(H.f64(q[0, s]), H.f64(kn[0, s, 0]), H.f64(vn[0, s, 0]))
+            # so peaked that an output is close to one V row: half an ulp of the output, 2^-9 of the weights
+            assert np.all(np.abs(H.f64(out[0, s]) - want) <= np.maximum(H.TOL_OUT[w.dtype], 2.0 ** -7 * np.abs(want))), (t, s)
+            if policy == synth.H2O:
+                # logits of up to 25 * 5, fp32 sums of 64 products: 2^-24 of their size in the exponent, some of them
+                np.testing.assert_allclose(ctx.get_kept(0, s, 0)[1], u.acc, rtol=H.RTOL_ACC[w.dtype], atol=1e-6)
+    assert ctx.status() == 0
 
 
 # One bf16 head per KV head on either kernel: few units, between one and two per SM, a few, many; lengths around the

@@ -356,8 +356,8 @@ def test_decode_split_k_long_context(policy):
 
 @pytest.mark.parametrize("policy", [synth.SLIDING_WINDOW, synth.STREAMING_LLM, synth.H2O])
 def test_decode_wide_mqa_long_context(policy):
-    # Falcon-shaped group (71 query heads on one KV head): several 128-token tiles, ragged tail,
-    # with and without split-K
+    # Falcon-shaped group (71 query heads on one KV head): several 128-token tiles, ragged tail; the pieces of a unit are the
+    # CTAs of a cluster here (split-K: test_wide_groups_over_a_cluster's unlike layers)
     w = small("mqa", 28, policy=policy, dtype=torch.bfloat16, head_dim=64, n_q_head=71, n_kv_head=1, batch=2,
               n_layer=2, prompt=1500, steps=3, hidden=64, heavy_mode="zipf")
     _run_decode_and_compare(w, budgets=[1300, 700], check_every_step=False)
@@ -369,8 +369,8 @@ def test_decode_wide_mqa_long_context(policy):
 @pytest.mark.parametrize("policy", [synth.SLIDING_WINDOW, synth.H2O])
 def test_decode_wide_mqa_sparsely_filled_quarter(policy, hq):
     """Group sizes that leave 4 head rows in the second, third or fourth quarter of the 128-row
-    tile (worked four threads to a row), over several tiles with a ragged tail, with and without
-    split-K."""
+    tile (worked four threads to a row), over several tiles with a ragged tail, in pieces over a cluster (above 96
+    heads: split-K)."""
     w = small("mqa_quad", 32 + hq, policy=policy, dtype=torch.bfloat16, head_dim=64, n_q_head=hq, n_kv_head=1, batch=2,
               n_layer=2, prompt=1500, steps=3, hidden=64, heavy_mode="zipf")
     _run_decode_and_compare(w, budgets=[1300, 900], check_every_step=False)
