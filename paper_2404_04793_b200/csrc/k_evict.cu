@@ -9,8 +9,9 @@
 //      landed; chunks go in slot order, so a store never overwrites a row not yet read.
 // A chunk is 32 KB of rows that stay: with chunks of slots a budget cut to half filled half of each, and a CTA took
 // twice the trips to memory, one after the other (32 layers of 8 KV heads of 128, 16 sequences, H2O, 20 % of 4096 halved:
-// 411 us, now 360).  The overlap that matters comes from many resident CTAs (7 per SM), not from a deep ring inside
-// one: 32 KB x 3 in flight (2 CTAs per SM) moved 2.8 to 3.3 TB/s where 32 KB x 1 moved 4.2 to 5.1.
+// 411 us, now 360).  The overlap that matters comes from many resident CTAs (6 per SM of 37 KB each, fewer
+// where the bitmask of a long cache adds to that), not from a deep ring inside one: 32 KB x 3 in flight (2 CTAs per SM) moved 2.8 to
+// 3.3 TB/s where 32 KB x 1 moved 4.2 to 5.1.
 #include "sq_device.cuh"
 #include "sq_internal.h"
 #include "sq_select.cuh"
